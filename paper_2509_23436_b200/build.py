@@ -11,6 +11,8 @@ import glob
 import os
 import subprocess
 import sys
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -20,7 +22,7 @@ LIB_DEBUG = os.path.join(PKG, "liblot_debug.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
-    "-shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
+    "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
     "-cudart", "static", "-diag-suppress", "128",
 ]
 
@@ -40,9 +42,16 @@ def build_lib(force: bool = False, verbose: bool = False, debug: bool = False) -
     if not force and os.path.exists(lib) and os.path.getmtime(lib) >= newest:
         return lib
     nvcc = os.environ.get("NVCC", "nvcc")
-    cmd = [nvcc] + NVCC_FLAGS + (["-DLOT_DEBUG"] if debug else []) + (["-Xptxas", "-v"] if verbose else []) + \
-        ["-o", lib] + sources() + ["-lcuda"]
-    subprocess.run(cmd, check=True)
+    extra = (["-DLOT_DEBUG"] if debug else []) + (["-Xptxas", "-v"] if verbose else [])
+    with tempfile.TemporaryDirectory() as tmp:
+        def compile_one(src):
+            obj = os.path.join(tmp, os.path.basename(src) + ".o")
+            subprocess.run([nvcc] + NVCC_FLAGS + extra + ["-c", "-o", obj, src], check=True)
+            return obj
+
+        with ThreadPoolExecutor(max_workers=os.cpu_count() or 4) as pool:      # one nvcc per source file
+            objs = list(pool.map(compile_one, sources()))
+        subprocess.run([nvcc] + NVCC_FLAGS + ["-shared", "-o", lib] + objs + ["-lcuda"], check=True)
     return lib
 
 

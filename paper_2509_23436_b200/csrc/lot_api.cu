@@ -2,6 +2,7 @@
 // launch sequence.  No arithmetic of the method lives here.
 #include "../../include/lot.h"
 #include "lot_internal.h"
+#include "lot_sweep.h"
 
 #include <math.h>
 #include <atomic>
@@ -61,64 +62,45 @@ SinkLayout sink_layout(int nprob, int n, int r, size_t base, size_t lt)
     return L;
 }
 
-struct AttnLayout {
-    SinkLayout s;
-    size_t counter2, cost, wpart, Wp, total;
+// Workspace of a forward on the general path (queries and keys may differ in number): the head (status word, tickets of
+// the apply stage, exchange words of the sweep) is one region cleared at the start of every call.
+struct ForwardLayout {
+    SweepPlan plan;
+    int rounds;              // problems a group works through per launch
+    size_t counter, xbuf, ybuf, head_end, w[2], gref[2], inv[2], kt[2], scores, wpart, Wp, total;
     int achunks, arows;
 };
 
-AttnLayout attn_layout(int B, int H, int n, int d, int r, int dtype)
+ForwardLayout forward_layout(int B, int H, int nq, int nk, int d, int r, int dtype, bool variant)
 {
-    AttnLayout A;
-    const size_t lt = dtype == LOT_F32 ? 8 : 4;
-    const int BH = B * H;
-    // tickets of the apply stage sit right behind the status word so one memset clears all
-    size_t o = 0;
-    int tiles = ((r + 63) / 64) * ((d + 63) / 64) * BH;
-    A.counter2 = 256;
-    o = 256 + up256((size_t)tiles * 4);
-    A.s = sink_layout(2 * BH, n, r, o, lt);
-    A.s.status = 0; // shared status word at the very start
-    o = A.s.total;
-    A.cost = o; o += up256((size_t)2 * BH * n * r * lt);
-    A.achunks = apply_chunks(BH > 0 ? BH : 1, n > 0 ? n : 1, r, d);
-    A.arows = (n + A.achunks - 1) / A.achunks;
-    A.wpart = o; o += up256((size_t)BH * A.achunks * r * d * 4);
-    A.Wp = o; o += up256((size_t)BH * r * d * 4);
-    A.total = o;
-    return A;
-}
-
-// Workspace of lot_attention_fwd_var: the two sides have their own token counts, so each gets a Sinkhorn block.
-struct VarLayout {
-    SinkLayout s1, s2;
-    size_t counter2, cost1, cost2, wa, wb, scores, wpart, Wp, total;
-    int achunks, arows;
-};
-
-VarLayout var_layout(int B, int H, int nq, int nk, int d, int r, int dtype)
-{
-    VarLayout V;
-    const size_t lt = dtype == LOT_F32 ? 8 : 4;
-    const int BH = B * H;
-    const int tiles = ((r + 63) / 64) * ((d + 63) / 64) * BH;
-    V.counter2 = 256;
-    size_t o = 256 + up256((size_t)tiles * 4);
-    // one cleared head for both sides: status word at 0, then tickets and potentials
-    V.s1 = sink_layout(BH, nq, r, o, lt);
-    V.s2 = sink_layout(BH, nk, r, V.s1.total, lt);
-    o = V.s2.total;
-    V.cost1 = o; o += up256((size_t)BH * nq * r * lt);
-    V.cost2 = o; o += up256((size_t)BH * nk * r * lt);
-    V.wa = o; o += up256((size_t)BH * nq * 4);
-    V.wb = o; o += up256((size_t)BH * nk * 4);
-    V.scores = o; o += up256((size_t)BH * nk * 4);
-    V.achunks = apply_chunks(BH > 0 ? BH : 1, nk > 0 ? nk : 1, r, d);
-    V.arows = (nk + V.achunks - 1) / V.achunks;
-    V.wpart = o; o += up256((size_t)BH * V.achunks * r * d * 4);
-    V.Wp = o; o += up256((size_t)BH * r * d * 4);
-    V.total = o;
-    return V;
+    ForwardLayout L;
+    const int BH = B * H, n[2] = {nq, nk};
+    L.plan = sweep_plan(dtype, BH > 0 ? BH : 1, nq > 0 ? nq : 1, nk > 0 ? nk : 1, d, r);
+    const int RP = L.plan.RP;
+    L.rounds = (2 * BH + L.plan.groups - 1) / L.plan.groups;
+    size_t o = 256;                                                   // status word at 0
+    L.counter = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
+    L.xbuf = o;
+    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * L.plan.C * RP * 8);
+    L.ybuf = o;
+    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * kSweepCopies * RP * 8);
+    L.head_end = o;
+    for (int side = 0; side < 2; ++side) {
+        L.w[side] = o; o += up256((size_t)BH * RP * 4);
+        L.gref[side] = o; o += up256((size_t)BH * RP * 8);
+        L.inv[side] = o; o += up256((size_t)BH * n[side] * 4);
+        L.kt[side] = o; o += up256((size_t)BH * n[side] * RP * 4);
+    }
+    L.scores = o;
+    if (variant) o += up256((size_t)BH * nk * 4);
+    L.achunks = apply_chunks(BH > 0 ? BH : 1, nk > 0 ? nk : 1, r, dtype == LOT_F32 ? d : 64);   // bf16: all channels in a block
+    L.arows = (nk + L.achunks - 1) / L.achunks;
+    L.wpart = o; o += up256((size_t)BH * L.achunks * r * d * 4);
+    L.Wp = o; o += up256((size_t)BH * r * d * 4);
+    // float32 tensors: never less than eight bytes per similarity, the size the interface has always asked for there
+    const size_t least = dtype == LOT_F32 ? up256((size_t)BH * ((size_t)nq + nk) * r * 8) : 0;
+    L.total = o > least ? o : least;
+    return L;
 }
 
 // Workspace of lot_attention_bwd: the general path's blocks plus the kept potentials of every iteration, the
@@ -208,6 +190,48 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
         if (G.whole && (long long)B * H <= (long long)G.ctas * G.wave_slices) return kPathResident;
     }
     return kPathStreamed;
+}
+
+// Both Sinkhorn problems and the apply stages on the general path, behind the clearing of the workspace head.
+cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, const void *v, const float *z, const float *beta,
+                        const float *mass_q, const float *mass_k, int skip, const int32_t *key_len, const float *g1_in, const float *g2_in,
+                        int dtype, int B, int H, int nq, int nk, int d, int r, float eps, int iters, void *out, float *g1_out,
+                        float *g2_out, void *ws, cudaStream_t s)
+{
+    SweepArgs a{};
+    SweepApplyArgs ap{};
+    for (int side = 0; side < 2; ++side) {
+        a.kt[side] = at<float>(ws, L.kt[side]); a.inv[side] = at<float>(ws, L.inv[side]);
+        a.w[side] = at<float>(ws, L.w[side]); a.gref[side] = at<double>(ws, L.gref[side]);
+        ap.kt[side] = a.kt[side]; ap.inv[side] = a.inv[side]; ap.w[side] = a.w[side];
+    }
+    a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
+    a.mass[0] = mass_q; a.mass[1] = mass_k; a.g_in[0] = g1_in; a.g_in[1] = g2_in; a.g_out[0] = g1_out; a.g_out[1] = g2_out;
+    a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf); a.status = at<int>(ws, 0);
+    a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip;
+    a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
+    a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
+    a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
+    cudaError_t e;
+    if (!L.plan.steps) {
+        if ((e = launch_build(L.plan.RP, a, dtype, 3, s)) != cudaSuccess) return e;
+        if ((e = launch_sweep(L.plan, a, dtype, s)) != cudaSuccess) return e;
+    } else {
+        // one launch per side and pass: 4 sequence numbers per pass and problem of a group cover its exchanges
+        if ((e = launch_build(L.plan.RP, a, dtype, 2, s)) != cudaSuccess) return e;
+        if ((e = launch_build(L.plan.RP, a, dtype, 1, s)) != cudaSuccess) return e;
+        for (int it = 0; it <= iters; ++it) {
+            a.it0 = it; a.it1 = it < iters ? it + 1 : it; a.first = it == 0; a.close = it == iters;
+            a.seq0 = 4u * (unsigned)it * (unsigned)L.rounds;
+            if ((e = launch_sweep(L.plan, a, dtype, s)) != cudaSuccess) return e;
+        }
+    }
+    ap.beta = beta; ap.key_len = key_len; ap.mass2 = mass_k; ap.v = v; ap.out = out;
+    ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
+    ap.B = B; ap.H = H; ap.nq = nq; ap.nk = nk; ap.d = d; ap.r = r; ap.RP = L.plan.RP; ap.skip = skip;
+    ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
+    if ((e = launch_sweep_apply_w(ap, dtype, s)) != cudaSuccess) return e;
+    return launch_sweep_apply_out(ap, dtype, s);
 }
 
 // Scratch of lot_sinkhorn_static: part of the library image, present on every device that loads
@@ -341,7 +365,7 @@ size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
     if (path == kPathResident) return up256(resident_layout(B, H, n, d, r).total) + fused_layout(B, H, n, d, r).total;
     if (path == kPathStreamed) return fused_layout(B, H, n, d, r).total;
     if (path == kPathSlice) return 256;                              // the status word
-    return attn_layout(B, H, n, d, r, dtype).total;
+    return forward_layout(B, H, n, n, d, r, dtype, false).total;
 }
 
 int lot_path(int dtype, int B, int H, int n, int d, int r, int iters)
@@ -359,7 +383,7 @@ int lot_launch_count(int dtype, int B, int H, int n, int d, int r, int iters)
     if (path == kPathResident) return 1 + 2;                        // the two streamed kernels return at once unless asked to redo
     if (path == kPathStreamed) return fused_launches(B, H, n, r, iters);
     if (path == kPathSlice) return 1;
-    return 2 + iters + 1 + 2;
+    return sweep_plan(dtype, B * H > 0 ? B * H : 1, n, n, d, r).steps ? 2 + iters + 1 + 2 : 4;
 }
 
 int lot_debug_hook(int what, long long value)
@@ -419,49 +443,12 @@ int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
         return e == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
     }
     remember_ws(ws, kPathGeneral, 0, 0);
-    AttnLayout A = attn_layout(B, H, n, d, r, dtype);
-    const bool wide = dtype == LOT_F32;
-    const size_t lt = wide ? 8 : 4;
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < A.total) return LOT_ERR_WORKSPACE;
+    const ForwardLayout L = forward_layout(B, H, n, n, d, r, dtype, false);
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    const int BH = B * H;
-    if (cudaMemsetAsync(ws, 0, A.s.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
-
-    char *cost1 = at<char>(ws, A.cost);
-    char *cost2 = cost1 + (size_t)BH * n * r * lt;
-    if (launch_cost(q, z, dtype, BH, H, n, d, r, cost1, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_cost(k, z, dtype, BH, H, n, d, r, cost2, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-
-    PassArgs a{};
-    a.cost = cost1; a.beta = beta; a.len = key_len; a.len_from = BH;
-    a.G = at<void>(ws, A.s.G); a.part = at<float>(ws, A.s.part); a.counter = at<unsigned>(ws, A.s.counter);
-    a.M = at<void>(ws, A.s.M); a.g_out = at<float>(ws, A.s.gnat); a.f_out = nullptr; a.plan_out = nullptr;
-    a.status = at<int>(ws, 0);
-    a.nprob = 2 * BH; a.B = B; a.H = H; a.n = n; a.r = r;
-    a.chunks = A.s.chunks; a.rows_per_chunk = A.s.rows_per_chunk;
-    a.mode = wide ? kModeWide : kModeF32;
-    a.scale_d = 1.4426950408889634 / (double)eps;
-    a.eps_ln2 = (float)((double)eps * 0.6931471805599453);
-    for (int it = 0; it < iters; ++it)
-        if (launch_sinkhorn_pass(a, false, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_sinkhorn_pass(a, true, s) != cudaSuccess) return LOT_ERR_CUDA;
-
-    ApplyArgs ap{};
-    ap.cost1 = cost1; ap.cost2 = cost2;
-    ap.G1 = a.G; ap.G2 = static_cast<char *>(a.G) + (size_t)BH * r * lt;
-    ap.M1 = a.M; ap.M2 = static_cast<char *>(a.M) + (size_t)BH * n * lt;
-    ap.beta = beta; ap.key_len = key_len; ap.v = v; ap.out = out;
-    ap.wpart = at<float>(ws, A.wpart); ap.Wp = at<float>(ws, A.Wp); ap.counter = at<unsigned>(ws, A.counter2);
-    ap.B = B; ap.H = H; ap.n = n; ap.nk = n; ap.d = d; ap.r = r;
-    ap.chunks = A.achunks; ap.rows_per_chunk = A.arows; ap.scale_d = a.scale_d;
-    if (launch_apply_w(ap, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_apply_out(ap, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;
-
-    const size_t gb = (size_t)BH * r * sizeof(float);
-    if (g1_out && cudaMemcpyAsync(g1_out, a.g_out, gb, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (g2_out && cudaMemcpyAsync(g2_out, a.g_out + (size_t)BH * r, gb, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return LOT_ERR_CUDA;
-    return LOT_OK;
+    if (cudaMemsetAsync(ws, 0, L.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
+    return run_forward(L, q, k, v, z, beta, nullptr, nullptr, 0, key_len, nullptr, nullptr, dtype, B, H, n, n, d, r, eps, iters, out,
+                       g1_out, g2_out, ws, s) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
 }
 
 size_t lot_var_workspace_bytes(int B, int H, int nq, int nk, int d, int r, int dtype)
@@ -469,7 +456,7 @@ size_t lot_var_workspace_bytes(int B, int H, int nq, int nk, int d, int r, int d
     if (dtype != LOT_F32 && dtype != LOT_BF16) return 0;
     if (check_dims(B, H, nq, r) != LOT_OK || check_dims(B, H, nk, r) != LOT_OK) return 0;
     if (check_d(nq, d) != LOT_OK || check_d(nk, d) != LOT_OK) return 0;
-    return var_layout(B, H, nq, nk, d, r, dtype).total;
+    return forward_layout(B, H, nq, nk, d, r, dtype, true).total;
 }
 
 int lot_attention_fwd_var(const void *q, const void *k, const void *v, const float *z, const float *beta,
@@ -495,65 +482,17 @@ int lot_attention_fwd_var(const void *q, const void *k, const void *v, const flo
         !aligned16(g1_out) || !aligned16(g2_out) || !aligned16(g1_in) || !aligned16(g2_in) || !aligned16(a) ||
         !aligned16(b) || (key_len && (reinterpret_cast<uintptr_t>(key_len) & 3u)))
         return LOT_ERR_INVALID_ARG;
-    VarLayout V = var_layout(B, H, nq, nk, d, r, dtype);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < V.total) return LOT_ERR_WORKSPACE;
-    const bool wide = dtype == LOT_F32;
-    const size_t lt = wide ? 8 : 4;
+    const ForwardLayout L = forward_layout(B, H, nq, nk, d, r, dtype, true);
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    const int BH = B * H;
     remember_ws(ws, kPathGeneral, 0, 0);
-    // the head (status word, tickets) starts at zero; the potentials start at the given ones
-    if (cudaMemsetAsync(ws, 0, V.s1.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (cudaMemsetAsync(at<char>(ws, V.s2.status), 0, V.s2.head_end - V.s2.status, s) != cudaSuccess) return LOT_ERR_CUDA;
-    const double scale = 1.4426950408889634 / (double)eps;
-    if (g1_in && launch_g_init(g1_in, at<void>(ws, V.s1.G), (size_t)BH * r, scale, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (g2_in && launch_g_init(g2_in, at<void>(ws, V.s2.G), (size_t)BH * r, scale, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    const float *wa = a, *wb = b;
-    if (cls) {
-        if (launch_cls_marginals(at<float>(ws, V.wa), at<float>(ws, V.wb), key_len, B, H, nq, nk, at<int>(ws, 0), s) != cudaSuccess)
-            return LOT_ERR_CUDA;
-        wa = at<float>(ws, V.wa);
-        wb = at<float>(ws, V.wb);
-    }
-
-    char *cost1 = at<char>(ws, V.cost1), *cost2 = at<char>(ws, V.cost2);
-    if (launch_cost(q, z, dtype, BH, H, nq, d, r, cost1, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_cost(k, z, dtype, BH, H, nk, d, r, cost2, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-
-    PassArgs pa[2] = {};
-    for (int side = 0; side < 2; ++side) {
-        const SinkLayout &L = side ? V.s2 : V.s1;
-        PassArgs &x = pa[side];
-        x = PassArgs{};
-        x.cost = side ? cost2 : cost1; x.beta = beta;
-        // a key length is a mask on the key side only; with explicit weights it only bounds the rows that are read
-        x.len = side ? key_len : nullptr; x.len_from = 0;
-        x.mass = side ? wb : wa;
-        x.G = at<void>(ws, L.G); x.part = at<float>(ws, L.part); x.counter = at<unsigned>(ws, L.counter);
-        x.M = at<void>(ws, L.M); x.g_out = side ? g2_out : g1_out;
-        x.status = at<int>(ws, 0);
-        x.nprob = BH; x.B = B; x.H = H; x.n = side ? nk : nq; x.r = r;
-        x.chunks = L.chunks; x.rows_per_chunk = L.rows_per_chunk;
-        x.mode = wide ? kModeWide : kModeF32;
-        x.scale_d = scale;
-        x.eps_ln2 = (float)((double)eps * 0.6931471805599453);
-        for (int it = 0; it < iters; ++it)
-            if (launch_sinkhorn_pass(x, false, s) != cudaSuccess) return LOT_ERR_CUDA;
-        if (launch_sinkhorn_pass(x, true, s) != cudaSuccess) return LOT_ERR_CUDA;
-    }
-
-    ApplyArgs ap{};
-    ap.cost1 = cost1; ap.cost2 = cost2;
-    ap.G1 = pa[0].G; ap.G2 = pa[1].G; ap.M1 = pa[0].M; ap.M2 = pa[1].M;
-    ap.beta = beta; ap.key_len = key_len; ap.mass2 = wb; ap.v = v; ap.out = out;
-    ap.wpart = at<float>(ws, V.wpart); ap.Wp = at<float>(ws, V.Wp); ap.counter = at<unsigned>(ws, V.counter2);
-    ap.B = B; ap.H = H; ap.n = nq; ap.nk = nk; ap.d = d; ap.r = r;
-    ap.chunks = V.achunks; ap.rows_per_chunk = V.arows; ap.scale_d = scale;
-    if (launch_apply_w(ap, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_apply_out(ap, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (cls && launch_cls_row(q, k, v, key_len, dtype, B, H, nq, nk, d, cls_tau, at<float>(ws, V.scores), out, s) != cudaSuccess)
+    if (cudaMemsetAsync(ws, 0, L.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
+    // the class token is neither a query nor a key of the transport problem: it is skipped on both sides
+    if (run_forward(L, q, k, v, z, beta, a, b, cls, key_len, g1_in, g2_in, dtype, B, H, nq, nk, d, r, eps, iters, out, g1_out, g2_out,
+                    ws, s) != cudaSuccess)
         return LOT_ERR_CUDA;
-    (void)lt;
+    if (cls && launch_cls_row(q, k, v, key_len, dtype, B, H, nq, nk, d, cls_tau, at<float>(ws, L.scores), out, s) != cudaSuccess)
+        return LOT_ERR_CUDA;
     return LOT_OK;
 }
 
@@ -567,7 +506,7 @@ int lot_attention_fwd(const float *q, const float *k, const float *v,
     st = check_d(n, d);
     if (st != LOT_OK) return st;
     if (B == 0 || n == 0) return LOT_OK;
-    const size_t need = attn_layout(B, H, n, d, r, LOT_F32).total;
+    const size_t need = forward_layout(B, H, n, n, d, r, LOT_F32, false).total;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LOT_ERR_CUDA;
     void *ws = nullptr;

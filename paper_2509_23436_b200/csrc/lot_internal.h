@@ -70,11 +70,6 @@ cudaError_t launch_cost(const void *x, const float *z, int dtype, int BH, int H,
 cudaError_t launch_sinkhorn_pass(const PassArgs &a, bool final_pass, cudaStream_t st);
 cudaError_t launch_apply_w(const ApplyArgs &a, int dtype, cudaStream_t st);
 cudaError_t launch_apply_out(const ApplyArgs &a, int dtype, cudaStream_t st);
-// starting potentials: G = g_in * scale (float or double per `wide`), zeros when g_in == nullptr
-cudaError_t launch_g_init(const float *g_in, void *G, size_t count, double scale, bool wide, cudaStream_t st);
-// weights of the [CLS] treatment, Eq. (5): a = (0, 1/(nq-1), ...), b = (0, 1/(kv-1), ... up to the key length, 0 ...)
-cudaError_t launch_cls_marginals(float *a, float *b, const int32_t *key_len, int B, int H, int nq, int nk, int *status,
-                                 cudaStream_t st);
 // row 0 of every slice: softmax_j(tau <q_0, k_j>) over the valid keys, applied to v; scores: [BH][nk] scratch
 cudaError_t launch_cls_row(const void *q, const void *k, const void *v, const int32_t *key_len, int dtype, int B, int H,
                            int nq, int nk, int d, float tau, float *scores, void *out, cudaStream_t st);

@@ -539,102 +539,100 @@ cudaError_t launch_apply_out(const ApplyArgs &a, int dtype, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------------------------
-// Forward variants: starting potentials, the weights and the softmax row of the [CLS] treatment
-// ------------------------------------------------------------------------------------
-template <typename LT>
-__global__ void g_init_kernel(const float *__restrict__ g_in, LT *__restrict__ G, size_t count, double scale)
+// Eq. (5): row 0 of every slice is the plain softmax over the valid keys.  One block per slice: eight lanes a key for the
+// scores (kept in shared memory while they fit, else in global scratch), their maximum, the exponentials and their sum,
+// then d / 8 threads a key for the weighted values, the threads' parts added in a fixed order.
+constexpr int kClsKeys = 4096;
+
+template <typename T> __device__ __forceinline__ void load8(const T *p, float (&o)[8])
 {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-        G[i] = g_in ? (LT)((double)g_in[i] * scale) : (LT)0;
+    float a[4], b[4];
+    load4(p, a);
+    load4(p + 4, b);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { o[i] = a[i]; o[4 + i] = b[i]; }
 }
 
-cudaError_t launch_g_init(const float *g_in, void *G, size_t count, double scale, bool wide, cudaStream_t st)
+template <bool MAX> __device__ __forceinline__ float cls_block(float v, float *red)
 {
-    if (count == 0) return cudaSuccess;
-    const int blocks = (int)((count + 255) / 256 < 1024 ? (count + 255) / 256 : 1024);
-    if (wide) g_init_kernel<double><<<blocks, 256, 0, st>>>(g_in, static_cast<double *>(G), count, scale);
-    else g_init_kernel<float><<<blocks, 256, 0, st>>>(g_in, static_cast<float *>(G), count, scale);
-    return cudaGetLastError();
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const float o = __shfl_xor_sync(0xffffffffu, v, off);
+        v = MAX ? fmaxf(v, o) : v + o;
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = red[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v = MAX ? fmaxf(v, red[w]) : v + red[w];
+    return v;
 }
 
-// Eq. (5) keeps the [CLS] token (index 0) out of the transport problem: zero weight for it on both sides, uniform
-// weights over the other queries and over the other valid keys.
-__global__ void cls_marginals_kernel(float *__restrict__ a, float *__restrict__ b, const int32_t *key_len, int H, int nq,
-                                     int nk, int *status)
-{
-    const int bh = blockIdx.x, bb = bh / H;
-    int kv = nk;
-    if (key_len != nullptr) kv = min(max(key_len[bb], 0), nk);
-    if (threadIdx.x == 0 && (kv <= 1 || nq <= 1)) atomicOr(status, 2 /* LOT_DEV_EMPTY */);
-    const float wa = nq > 1 ? 1.f / (float)(nq - 1) : 0.f, wb = kv > 1 ? 1.f / (float)(kv - 1) : 0.f;
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) a[(size_t)bh * nq + i] = i == 0 ? 0.f : wa;
-    for (int j = threadIdx.x; j < nk; j += blockDim.x) b[(size_t)bh * nk + j] = (j == 0 || j >= kv) ? 0.f : wb;
-}
-
-cudaError_t launch_cls_marginals(float *a, float *b, const int32_t *key_len, int B, int H, int nq, int nk, int *status,
-                                 cudaStream_t st)
-{
-    cls_marginals_kernel<<<B * H, 256, 0, st>>>(a, b, key_len, H, nq, nk, status);
-    return cudaGetLastError();
-}
-
-// One block per slice: scores tau <q_0, k_j> of the valid keys (kept in global scratch), their maximum, the
-// exponentials and their sum, then one thread per channel adds up the weighted values.
 template <typename T>
 __global__ void __launch_bounds__(256)
 cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, const int32_t *key_len, int H,
-               int nq, int nk, int d, float tau, float *__restrict__ scores, T *__restrict__ out)
+               int nq, int nk, int d, float tau, float *scores, T *__restrict__ out)
 {
-    __shared__ float red[256];
-    __shared__ float q0[256];
-    const int bh = blockIdx.x, bb = bh / H;
+    __shared__ float sc_s[kClsKeys];
+    __shared__ __align__(16) float part[256 * 8];
+    __shared__ float red[8];
+    const int bh = blockIdx.x, bb = bh / H, tid = threadIdx.x;
     int kv = nk;
     if (key_len != nullptr) kv = min(max(key_len[bb], 0), nk);
     const T *qb = q + (size_t)bh * nq * d, *kb = k + (size_t)bh * nk * d, *vb = v + (size_t)bh * nk * d;
-    float *sc = scores + (size_t)bh * nk;
-    for (int c = threadIdx.x; c < d; c += blockDim.x) q0[c] = Elem<T>::load(qb + c);
-    __syncthreads();
+    float *sc = kv <= kClsKeys ? sc_s : scores + (size_t)bh * nk;
+    const int l8 = tid & 7;
     float mx = neg_inf();
-    for (int j = threadIdx.x; j < kv; j += blockDim.x) {
+#pragma unroll 4
+    for (int j0 = 0; j0 < kv; j0 += 32) {
+        const int j = j0 + (tid >> 3);
         float acc = 0.f;
-        for (int c = 0; c < d; c += 4) {
-            float kk[4];
-            load4(kb + (size_t)j * d + c, kk);
-            acc = fmaf(q0[c], kk[0], acc); acc = fmaf(q0[c + 1], kk[1], acc);
-            acc = fmaf(q0[c + 2], kk[2], acc); acc = fmaf(q0[c + 3], kk[3], acc);
-        }
+        if (j < kv)
+            for (int c = l8 * 8; c < d; c += 64) {
+                float qq[8], kk[8];
+                load8(qb + c, qq);
+                load8(kb + (size_t)j * d + c, kk);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc = fmaf(qq[i], kk[i], acc);
+            }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         acc *= tau;
-        sc[j] = acc;
-        mx = fmaxf(mx, acc);
+        if (j < kv) {
+            if (l8 == 0) sc[j] = acc;
+            mx = fmaxf(mx, acc);
+        }
     }
-    red[threadIdx.x] = mx;
-    __syncthreads();
-    for (int off = 128; off > 0; off >>= 1) {
-        if (threadIdx.x < off) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + off]);
-        __syncthreads();
-    }
-    mx = red[0];
-    __syncthreads();
+    mx = cls_block<true>(mx, red);
     float den = 0.f;
-    for (int j = threadIdx.x; j < kv; j += blockDim.x) {
+    for (int j = tid; j < kv; j += 256) {
         const float e = __expf(sc[j] - mx);
         sc[j] = e;
         den += e;
     }
-    red[threadIdx.x] = den;
-    __syncthreads();
-    for (int off = 128; off > 0; off >>= 1) {
-        if (threadIdx.x < off) red[threadIdx.x] += red[threadIdx.x + off];
-        __syncthreads();
-    }
-    den = red[0];
+    den = cls_block<false>(den, red);
     __threadfence_block();
     __syncthreads();
-    for (int c = threadIdx.x; c < d; c += blockDim.x) {
-        float acc = 0.f;
-        for (int j = 0; j < kv; ++j) acc = fmaf(sc[j], Elem<T>::load(vb + (size_t)j * d + c), acc);
-        Elem<T>::store(out + (size_t)bh * nq * d + c, kv > 0 ? acc / den : 0.f);
+    const int groups = d / 8, parts = 256 / groups, c = (tid % groups) * 8, p = tid / groups;
+    float acc[8] = {};
+    if (p < parts) {
+#pragma unroll 4
+        for (int j = p; j < kv; j += parts) {
+            float vv[8];
+            load8(vb + (size_t)j * d + c, vv);
+            const float w = sc[j];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i] = fmaf(w, vv[i], acc[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) part[p * d + c + i] = acc[i];
+    }
+    __syncthreads();
+    for (int cc = tid; cc < d; cc += 256) {
+        float s = 0.f;
+        for (int i = 0; i < parts; ++i) s += part[i * d + cc];
+        Elem<T>::store(out + (size_t)bh * nq * d + cc, kv > 0 ? s / den : 0.f);
     }
 }
 
