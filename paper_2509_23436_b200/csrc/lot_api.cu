@@ -103,7 +103,7 @@ ForwardLayout forward_layout(int B, int H, int nq, int nk, int d, int r, int dty
     return L;
 }
 
-// Workspace of lot_attention_bwd: the general path's blocks plus the kept potentials of every iteration, the
+// Workspace of lot_attention_bwd for float32 tensors: similarities in float64, the row blocks of the log-domain passes plus the kept potentials of every iteration, the
 // gradient with respect to the similarities and the small reduction buffers.
 struct BwdLayout {
     size_t counter, counter2, hist, gamma, dbeta_acc, head_end, part, M, cost, dC, wpart, Wp, Xw, dWm, dbeta_direct, zt,
@@ -111,10 +111,10 @@ struct BwdLayout {
     int chunks, rows_per_chunk, achunks, arows, dzchunks;
 };
 
-BwdLayout bwd_layout(int B, int H, int n, int d, int r, int dtype, int iters)
+BwdLayout bwd_layout(int B, int H, int n, int d, int r, int iters)
 {
     BwdLayout L;
-    const size_t lt = dtype == LOT_F32 ? 8 : 4;
+    const size_t lt = 8;
     const int BH = B * H, np = 2 * BH;
     const int tiles = ((r + 63) / 64) * ((d + 63) / 64) * BH;
     L.chunks = pass_chunks(np > 0 ? np : 1, n > 0 ? n : 1);
@@ -140,6 +140,58 @@ BwdLayout bwd_layout(int B, int H, int n, int d, int r, int dtype, int iters)
     L.dbeta_direct = o; o += up256((size_t)BH * r * 4);
     L.zt = o; o += up256((size_t)H * r * d * 4);
     L.dzpart = o; o += up256((size_t)np * L.dzchunks * r * d * lt);
+    L.total = o;
+    return L;
+}
+
+// Workspace of lot_attention_bwd for bf16 tensors: the forward's blocks (kernel and weights of both sides), the kept
+// weights of every iteration, the row and column coefficients of the reverse steps and the gradient with respect to the
+// similarities.
+struct BwdSweepLayout {
+    SweepPlan plan;
+    int rounds, tiles, achunks, arows;
+    size_t counter, xbuf, ybuf, head_end, w[2], gref[2], inv[2], kt[2], dC[2], hist, hist_g, wide, coef, fk, gpart, dbeta_acc, wpart,
+        Wp, Xw, dWm, dbeta_direct, zpart[2], total;
+};
+
+BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
+{
+    BwdSweepLayout L;
+    const int BH = B * H > 0 ? B * H : 1, NP = 2 * BH;
+    if (n < 1) n = 1;
+    L.plan = sweep_plan(LOT_BF16, BH, n, n, d, r);
+    const int RP = L.plan.RP;
+    L.rounds = (NP + L.plan.groups - 1) / L.plan.groups;
+    L.tiles = (n + 127) / 128;
+    size_t o = 256;                                                   // status word at 0
+    L.counter = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
+    L.xbuf = o;
+    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * L.plan.C * RP * 8);
+    L.ybuf = o;
+    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * kSweepCopies * RP * 8);
+    L.head_end = o;
+    for (int side = 0; side < 2; ++side) {
+        L.w[side] = o; o += up256((size_t)BH * RP * 4);
+        L.gref[side] = o; o += up256((size_t)BH * RP * 8);
+        L.inv[side] = o; o += up256((size_t)BH * n * 4);
+        L.kt[side] = o; o += up256((size_t)BH * n * RP * 4);
+        L.dC[side] = o; o += up256((size_t)BH * n * RP * 4);
+    }
+    L.hist = o; o += up256((size_t)(iters + 1) * NP * RP * 4);
+    L.hist_g = o; o += up256((size_t)(iters + 1) * NP * RP * 8);
+    L.wide = o; o += up256((size_t)NP * 4);
+    L.coef = o; o += up256((size_t)NP * iters * n * 8);
+    L.fk = o; o += up256((size_t)iters * NP * RP * 4);
+    L.gpart = o; o += up256((size_t)NP * L.tiles * RP * 4);
+    L.dbeta_acc = o; o += up256((size_t)NP * RP * 4);
+    L.achunks = apply_chunks(BH, n, r, 64);
+    L.arows = (n + L.achunks - 1) / L.achunks;
+    L.wpart = o; o += up256((size_t)BH * L.achunks * r * d * 4);
+    L.Wp = o; o += up256((size_t)BH * r * d * 4);
+    L.Xw = o; o += up256((size_t)BH * r * d * 4);
+    L.dWm = o; o += up256((size_t)BH * r * d * 4);
+    L.dbeta_direct = o; o += up256((size_t)BH * r * 4);
+    for (int side = 0; side < 2; ++side) { L.zpart[side] = o; o += up256((size_t)BH * L.achunks * r * d * 4); }
     L.total = o;
     return L;
 }
@@ -232,6 +284,70 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
     ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
     if ((e = launch_sweep_apply_w(ap, dtype, s)) != cudaSuccess) return e;
     return launch_sweep_apply_out(ap, dtype, s);
+}
+
+// lot_attention_bwd for bf16 tensors, behind the argument checks.
+cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, const void *v, const float *z, const float *beta,
+                         const int32_t *key_len, const void *dout, int B, int H, int n, int d, int r, float eps, int iters, void *dq,
+                         void *dk, void *dv, float *dz, float *dbeta, void *ws, cudaStream_t st)
+{
+    const int dt = LOT_BF16, RP = L.plan.RP;
+    cudaError_t e = cudaMemsetAsync(ws, 0, L.head_end, st);
+    if (e != cudaSuccess) return e;
+    SweepBwdArgs b{};
+    SweepArgs &a = b.s;
+    SweepApplyArgs ap{};
+    for (int side = 0; side < 2; ++side) {
+        a.kt[side] = at<float>(ws, L.kt[side]); a.inv[side] = at<float>(ws, L.inv[side]);
+        a.w[side] = at<float>(ws, L.w[side]); a.gref[side] = at<double>(ws, L.gref[side]);
+        ap.kt[side] = a.kt[side]; ap.inv[side] = a.inv[side]; ap.w[side] = a.w[side];
+        b.dC[side] = at<float>(ws, L.dC[side]);
+        a.n[side] = n;
+    }
+    a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
+    a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf);
+    a.hist = at<float>(ws, L.hist); a.hist_g = at<double>(ws, L.hist_g); a.wide = at<int>(ws, L.wide); a.status = at<int>(ws, 0);
+    a.B = B; a.H = H; a.d = d; a.r = r;
+    a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
+    a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
+    a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
+    // ---- the forward, keeping the weights of every iteration
+    if ((e = launch_build(RP, a, dt, 3, st)) != cudaSuccess) return e;
+    if ((e = launch_sweep(L.plan, a, dt, st)) != cudaSuccess) return e;
+    ap.beta = beta; ap.key_len = key_len; ap.v = v;
+    ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
+    ap.B = B; ap.H = H; ap.nq = n; ap.nk = n; ap.d = d; ap.r = r; ap.RP = RP;
+    ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
+    if ((e = launch_sweep_apply_w(ap, dt, st)) != cudaSuccess) return e;              // W' = Diag(1/beta) Gamma2 V
+    // ---- reverse of the read-out, Eq. (4): out = R1 W'
+    SweepApplyArgs aq = ap;                                                             // R1^T dout / (n beta): the key-side product on the query side
+    aq.kt[1] = ap.kt[0]; aq.inv[1] = ap.inv[0]; aq.w[1] = ap.w[0]; aq.key_len = nullptr; aq.v = dout; aq.Wp = at<float>(ws, L.Xw);
+    if ((e = launch_sweep_apply_w(aq, dt, st)) != cudaSuccess) return e;
+    float *dbd = at<float>(ws, L.dbeta_direct), *dWm = at<float>(ws, L.dWm);
+    if ((e = launch_bwd_w_fix(at<float>(ws, L.Xw), ap.Wp, key_len, dWm, dbd, B, H, n, d, r, st)) != cudaSuccess) return e;
+    SweepApplyArgs av = ap;                                                             // dV = Gamma2 dW: the query-side product on the key side
+    av.kt[0] = ap.kt[1]; av.inv[0] = ap.inv[1]; av.w[0] = ap.w[1]; av.Wp = dWm; av.out = dv; av.out_len = key_len;
+    if ((e = launch_sweep_apply_out(av, dt, st)) != cudaSuccess) return e;
+    b.g[0] = dout; b.g[1] = v; b.wmat[0] = ap.Wp; b.wmat[1] = dWm;
+    b.coef = at<float2>(ws, L.coef); b.fk = at<float>(ws, L.fk); b.gpart = at<float>(ws, L.gpart); b.dbeta_acc = at<float>(ws, L.dbeta_acc);
+    b.T = iters; b.tiles = L.tiles; b.eps = (double)eps;
+    if ((e = launch_bwd_close(RP, b, st)) != cudaSuccess) return e;
+    // ---- the iterations, last first
+    a.seq0 = 4u * (unsigned)(iters + 1) * (unsigned)L.rounds;
+    if ((e = launch_bwd_reverse(L.plan, b, st)) != cudaSuccess) return e;
+    if (iters > 0 && (e = launch_bwd_assemble(RP, b, st)) != cudaSuccess) return e;
+    // ---- C = X Z^T: dX = dC Z, dZ = dC^T X, the same two products with the gradient in place of the plan
+    for (int side = 0; side < 2; ++side) {
+        SweepApplyArgs x = ap;
+        x.kt[0] = b.dC[side]; x.inv[0] = nullptr; x.w[0] = nullptr; x.Wp = const_cast<float *>(z); x.per_head = 1;
+        x.out = side ? dk : dq; x.out_len = side ? key_len : nullptr;
+        if ((e = launch_sweep_apply_out(x, dt, st)) != cudaSuccess) return e;
+        SweepApplyArgs y = ap;
+        y.kt[1] = b.dC[side]; y.inv[1] = nullptr; y.w[1] = nullptr; y.beta = nullptr; y.key_len = side ? key_len : nullptr;
+        y.v = side ? k : q; y.Wp = nullptr; y.wpart = at<float>(ws, L.zpart[side]);
+        if ((e = launch_sweep_apply_w(y, dt, st)) != cudaSuccess) return e;
+    }
+    return launch_bwd_merge(at<float>(ws, L.zpart[0]), at<float>(ws, L.zpart[1]), dbd, b.dbeta_acc, dz, dbeta, B, H, d, r, RP, L.achunks, st);
 }
 
 // Scratch of lot_sinkhorn_static: part of the library image, present on every device that loads
@@ -567,7 +683,7 @@ size_t lot_bwd_workspace_bytes(int B, int H, int n, int d, int r, int dtype, int
 {
     if (dtype != LOT_F32 && dtype != LOT_BF16) return 0;
     if (check_dims(B, H, n, r) != LOT_OK || check_d(n, d) != LOT_OK || iters < 0) return 0;
-    return bwd_layout(B, H, n, d, r, dtype, iters).total;
+    return dtype == LOT_BF16 ? bwd_sweep_layout(B, H, n, d, r, iters).total : bwd_layout(B, H, n, d, r, iters).total;
 }
 
 int lot_attention_bwd(const void *q, const void *k, const void *v, const float *z, const float *beta,
@@ -595,7 +711,14 @@ int lot_attention_bwd(const void *q, const void *k, const void *v, const float *
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(dout) || !aligned16(dq) || !aligned16(dk) ||
         !aligned16(dv) || (key_len && (reinterpret_cast<uintptr_t>(key_len) & 3u)))
         return LOT_ERR_INVALID_ARG;
-    const BwdLayout L = bwd_layout(B, H, n, d, r, dtype, iters);
+    if (dtype == LOT_BF16) {
+        const BwdSweepLayout L = bwd_sweep_layout(B, H, n, d, r, iters);
+        if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
+        remember_ws(ws, kPathGeneral, 0, 0);
+        return run_backward(L, q, k, v, z, beta, key_len, dout, B, H, n, d, r, eps, iters, dq, dk, dv, dz, dbeta, ws, s) == cudaSuccess
+                   ? LOT_OK : LOT_ERR_CUDA;
+    }
+    const BwdLayout L = bwd_layout(B, H, n, d, r, iters);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     remember_ws(ws, kPathGeneral, 0, 0);
     const bool wide = dtype == LOT_F32;

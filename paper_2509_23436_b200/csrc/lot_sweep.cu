@@ -12,617 +12,12 @@
 // spread of the potentials is exact.
 // What bounds a pass: shared-memory reads (4 bytes per entry at 128 bytes per clock and SM) and, for C > 1, one or two
 // round trips through L2 for the exchange, which other blocks on the SM (other groups) hide.
-#include "lot_common.cuh"
-#include "lot_internal.h"
-#include "lot_logits.cuh"
-#include "lot_sm100.cuh"
-#include "lot_sweep.h"
+#include "lot_sweep_core.cuh"
 
-#include <math.h>
-#include <string.h>
 #include <mutex>
 
 namespace lot {
 namespace sweep {
-
-typedef unsigned long long u64;
-using sm100::global_timer_ns;
-
-__host__ __device__ constexpr int kTileRows(int threads) { return threads / 2; }   // 16 rows per warp
-constexpr float kLostLo = 1e-30f, kLostHi = 1e38f;
-constexpr float kFarLo = 7.7037198e-34f, kFarHi = 1.1258999e15f;   // 2^-110, 2^50
-constexpr float kStart = 8.8817842e-16f;                            // 2^kStartLog2
-constexpr int kDirectWords = 4096, kCopies = kSweepCopies;
-constexpr unsigned long long kWaitNs = 1000000000ull;
-
-// floats <-> packed pairs for fma.rn.f32x2
-__device__ __forceinline__ u64 pack_f2(float lo, float hi)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack_f2(u64 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ u64 fma_f2(u64 a, u64 b, u64 c)
-{
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void lds2(u64 &a, u64 &b, uint32_t addr)
-{
-    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ float lds(uint32_t addr)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void sts(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
-
-// A row of RP columns lies over LPR = RP / CPL adjacent lanes, CPL columns (CPL / 4 chunks of 16 bytes) per lane: chunk v of
-// lane cl is v * LPR + cl.  In shared memory the chunks of a row are permuted so that the eight lanes of a 128-byte
-// phase, which cover 8 / LPR rows, fall on different banks.
-template <int RP, int CPL> struct Lay {
-    static constexpr int LPR = RP / CPL, RPW = 32 / LPR, CH = RP / 4, NV = CPL / 4;
-    static constexpr int RPL = RP >= 32 ? 1 : 32 / RP, SG = LPR >= 8 ? 1 : (8 / LPR / RPL < 1 ? 1 : 8 / LPR / RPL);
-    static __device__ __forceinline__ int swz(int row, int chunk) { return chunk ^ (((row / RPL) & (SG - 1)) * LPR); }
-};
-
-// columns per lane where a pass is bound by issue and shared-memory reads, not by latency
-constexpr int wide_cols(int RP) { return RP <= 32 ? 8 : 16; }
-
-// blocks per SM that the registers allow (80 a thread, 128 with sixteen columns per lane)
-__host__ __device__ constexpr int max_blocks(int cpl, int threads) { return (cpl == 16 ? 512 : 768) / threads; }
-
-// shared memory: [kernel rows | gref | work area (staged pivots, or the column reduction) | refs | weights, targets | flags]
-__host__ __device__ constexpr int rebuild_cols(int RP) { return RP < 32 ? RP : 32; }      // columns per step of a rebuild
-template <typename T> __host__ __device__ constexpr size_t work_bytes(int RP, int threads)
-{
-    const size_t red = (size_t)2 * (threads / 32) * RP * 4, st = logits::stage_bytes<T>(rebuild_cols(RP));
-    return red > st ? red : st;
-}
-__host__ __device__ constexpr size_t ref_bytes(int RP, int threads)
-{
-    const size_t refs = (size_t)kTileRows(threads) * (RP / rebuild_cols(RP)) * 4, cols = (size_t)threads * 4;
-    return refs > cols ? refs : cols;
-}
-template <typename T> __host__ __device__ constexpr size_t fixed_bytes(int RP, int threads)
-{
-    return work_bytes<T>(RP, threads) + ref_bytes(RP, threads) + (size_t)RP * (4 + 4 + 8) + 64;
-}
-
-struct Shared {
-    float *K;                // kernel rows; up to a multiple of the block's rows per step, the last ones zero
-    uint8_t *work;
-    float *ref, *w, *tgt;
-    double *gref;
-    volatile int *flag;      // [0] a wait gave up, [1] a weight left its range
-};
-
-// A block's share of one problem.
-struct Share {
-    float *g;                // its rows in global memory, [nrows][RP]
-    const float *mass;       // its tokens' weights or nullptr
-    int nrows, ns, steps;    // rows, of which the first ns are in shared memory too, in `steps` steps of the block
-};
-
-template <int RP, int CPL> __device__ __forceinline__ float4 *chunk_ptr(const Shared &S, const Share &R, int i, int chunk)
-{
-    return i < R.ns ? reinterpret_cast<float4 *>(S.K + (size_t)i * RP) + Lay<RP, CPL>::swz(i, chunk)
-                    : reinterpret_cast<float4 *>(R.g + (size_t)i * RP) + chunk;
-}
-
-// The block's kernel rows again, around the reference potentials S.gref: exponents e_it = L_it + Gref_t - max_t(.) (EXPS),
-// or the kernel.  Columns come in chunks of 32, which keeps the accumulators few beside the pass's registers: a chunk is
-// stored relative to its own maximum first (the float32 rounding of an exponent must not depend on far-away columns)
-// and the chunks of a row are combined in a second sweep.  Rare: see the exponent range in lot_sweep.h.
-template <typename T, int RP, int CPL, int THREADS, bool EXPS>
-__device__ __forceinline__ void build(const Shared &S, const Share &R, const T *x, const float *z, int d, int r, double scale)
-{
-    constexpr int CC = rebuild_cols(RP), NCH = RP / CC, ROWS = kTileRows(THREADS);
-    typedef logits::Logits<T, CC, 16, THREADS> Lg;
-    typedef typename Lg::LT LT;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
-    for (int rt = 0; rt < R.nrows; rt += ROWS) {
-        const int w0 = rt + warp * 16, wrows = min(max(R.nrows - w0, 0), 16);
-#pragma unroll 1
-        for (int ch = 0; ch < NCH; ++ch) {
-            Lg lg;
-            lg.run(x + (size_t)w0 * d, wrows, d, z + (size_t)ch * CC * d, min(max(r - ch * CC, 0), CC), S.work, lane);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                LT m = (LT)neg_inf();
-#pragma unroll
-                for (int j = 0; j < CC / 8; ++j)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int t = ch * CC + 8 * j + 2 * q + e;
-                        const LT l = t < r ? fma(lg.at(j, h, e), (LT)scale, (LT)S.gref[t]) : (LT)neg_inf();
-                        lg.at(j, h, e) = l;
-                        m = fmax(m, l);
-                    }
-                m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 1));
-                m = fmax(m, __shfl_xor_sync(0xffffffffu, m, 2));
-                const float mf = (float)m;
-                const int i = w0 + g + 8 * h;
-                if (NCH > 1 && q == 0) S.ref[(warp * 16 + g + 8 * h) * NCH + ch] = mf;
-                if (i < R.nrows) {
-#pragma unroll
-                    for (int j = 0; j < CC / 8; ++j) {
-                        float2 v;
-                        v.x = mf == neg_inf() ? neg_inf() : (float)(lg.at(j, h, 0) - (LT)mf);
-                        v.y = mf == neg_inf() ? neg_inf() : (float)(lg.at(j, h, 1) - (LT)mf);
-                        if (NCH == 1 && !EXPS) { v.x = ex2(v.x + kKernelTop); v.y = ex2(v.y + kKernelTop); }
-                        const int c0 = ch * CC + 8 * j + 2 * q;
-                        float *p = reinterpret_cast<float *>(chunk_ptr<RP, CPL>(S, R, i, c0 >> 2)) + (c0 & 3);
-                        *reinterpret_cast<float2 *>(p) = v;
-                        if (NCH == 1 && !EXPS && i < R.ns) *reinterpret_cast<float2 *>(R.g + (size_t)i * RP + c0) = v;
-                    }
-                }
-            }
-        }
-        if (NCH > 1) {
-            __syncwarp();
-            for (int i = w0; i < w0 + wrows; ++i) {
-                const float *rf = S.ref + (i - rt) * NCH;
-                float M = rf[0];
-#pragma unroll
-                for (int c = 1; c < NCH; ++c) M = fmaxf(M, rf[c]);
-                for (int ck = lane; ck < RP / 4; ck += 32) {
-                    float4 *p = chunk_ptr<RP, CPL>(S, R, i, ck);
-                    const float off = rf[ck / (CC / 4)] - M + (EXPS ? 0.f : kKernelTop);
-                    float4 v = *p;
-                    v.x += off; v.y += off; v.z += off; v.w += off;
-                    if (!EXPS) { v.x = ex2(v.x); v.y = ex2(v.y); v.z = ex2(v.z); v.w = ex2(v.w); }
-                    *p = v;
-                    if (!EXPS && i < R.ns) reinterpret_cast<float4 *>(R.g + (size_t)i * RP)[ck] = v;
-                }
-            }
-        }
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ float group_sum(float v, int lpr)
-{
-    for (int off = lpr / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-
-__device__ __forceinline__ float rcp(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-template <int CPL> struct Row { u64 k[CPL / 2]; };       // a lane's columns of a row
-
-// One row's step of a pass: row sum against the weights, its reciprocal (times the token's weight), column sums.  A row of
-// zeros adds nothing.
-template <int RP, int CPL, bool SUMS>
-__device__ __forceinline__ float row_step(const Row<CPL> &k, const u64 (&w)[CPL / 2], u64 (&acc)[CPL / 2], float mass)
-{
-    u64 s0 = 0, s1 = 0;
-#pragma unroll
-    for (int j = 0; j < CPL / 2; j += 2) { s0 = fma_f2(k.k[j], w[j], s0); s1 = fma_f2(k.k[j + 1], w[j + 1], s1); }
-    float a, b, c, e;
-    unpack_f2(s0, a, b);
-    unpack_f2(s1, c, e);
-    float s = (a + b) + (c + e);
-#pragma unroll
-    for (int off = Lay<RP, CPL>::LPR / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    const float inv = rcp(fmaxf(s, 1e-37f)) * mass;
-    if (SUMS) {
-        const u64 ii = pack_f2(inv, inv);
-#pragma unroll
-        for (int j = 0; j < CPL / 2; ++j) acc[j] = fma_f2(k.k[j], ii, acc[j]);
-    }
-    return inv;
-}
-
-// What a thread needs in every iteration, worked out once per problem: shared-memory addresses of its columns of its
-// first row, of its weights and of the column it owns.
-template <int RP, int CPL> struct Lane {
-    uint32_t k[CPL / 4], w, red, own;
-    int i0, cl;
-};
-
-template <int RP, int CPL>
-__device__ __forceinline__ Lane<RP, CPL> make_lane(const Shared &S)
-{
-    typedef Lay<RP, CPL> Y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    Lane<RP, CPL> L;
-    L.cl = lane % Y::LPR;
-    L.i0 = warp * Y::RPW + lane / Y::LPR;
-#pragma unroll
-    for (int v = 0; v < Y::NV; ++v) L.k[v] = smem_addr(S.K) + (L.i0 * Y::CH + Y::swz(L.i0, v * Y::LPR + L.cl)) * 16;
-    L.w = smem_addr(S.w) + L.cl * 16;
-    // after the halving the lane holds its columns off .. off + LEFT - 1 (warp_columns)
-    int off = 0;
-#pragma unroll
-    for (int bit = Y::LPR, h = CPL / 2; bit < 32; bit <<= 1, h >>= 1) off += (lane & bit) ? h : 0;
-    L.red = smem_addr(S.work) + (warp * RP + ((off >> 2) * Y::LPR + L.cl) * 4 + (off & 3)) * 4;
-    L.own = smem_addr(S.work) + threadIdx.x * 4;
-    return L;
-}
-
-// One pass over the block's rows: the lane's column sums.  CLOSE: the reciprocal row sums go to inv_out instead (0 for a
-// token without weight).  WEIGHTED: the tokens bring weights of their own.
-template <int RP, int CPL, int THREADS, bool CLOSE, bool WEIGHTED>
-__device__ __forceinline__ void pass_t(const Lane<RP, CPL> &L, const Share &R, const u64 (&w)[CPL / 2], u64 (&acc)[CPL / 2], float *inv_out)
-{
-    typedef Lay<RP, CPL> Y;
-    constexpr int STEP = (THREADS / 32) * Y::RPW;        // a multiple of 8: a lane's chunk permutation never changes
-#pragma unroll
-    for (int j = 0; j < CPL / 2; ++j) acc[j] = 0;
-    auto one = [&](const Row<CPL> &k, int i, int end) {
-        float m = 1.f;
-        if (WEIGHTED) m = i < end ? __ldg(R.mass + i) : 0.f;
-        if (!CLOSE) {
-            row_step<RP, CPL, true>(k, w, acc, m);
-        } else {
-            const float inv = row_step<RP, CPL, false>(k, w, acc, 1.f);
-            if (i < end && L.cl == 0) inv_out[i] = m > 0.f ? inv : 0.f;
-        }
-    };
-    auto load = [&](Row<CPL> &k, int st) {
-#pragma unroll
-        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.k[v] + st * (STEP * RP * 4));
-    };
-    if (R.steps & 1) {
-        Row<CPL> k;
-        load(k, 0);
-        one(k, L.i0, R.ns);
-    }
-    for (int st = R.steps & 1; st < R.steps; st += 2) {
-        Row<CPL> k[2];
-        load(k[0], st);
-        load(k[1], st + 1);
-        one(k[0], L.i0 + st * STEP, R.ns);
-        one(k[1], L.i0 + (st + 1) * STEP, R.ns);
-    }
-    // rows that do not fit: streamed from L2
-    if (R.ns < R.nrows)
-        for (int i = R.ns + L.i0; i - L.i0 < R.nrows; i += 2 * STEP) {
-            Row<CPL> k[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-#pragma unroll
-                for (int v = 0; v < Y::NV; ++v) {
-                    const ulonglong2 t = i + u * STEP < R.nrows
-                                             ? __ldcg(reinterpret_cast<const ulonglong2 *>(R.g + (size_t)(i + u * STEP) * RP) + v * Y::LPR + L.cl)
-                                             : make_ulonglong2(0, 0);
-                    k[u].k[2 * v] = t.x;
-                    k[u].k[2 * v + 1] = t.y;
-                }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) one(k[u], i + u * STEP, R.nrows);
-        }
-}
-
-template <int RP, int CPL, int THREADS, bool CLOSE>
-__device__ __forceinline__ void pass(const Lane<RP, CPL> &L, const Share &R, const u64 (&w)[CPL / 2], u64 (&acc)[CPL / 2], float *inv_out)
-{
-    if (R.mass == nullptr) pass_t<RP, CPL, THREADS, CLOSE, false>(L, R, w, acc, inv_out);
-    else pass_t<RP, CPL, THREADS, CLOSE, true>(L, R, w, acc, inv_out);
-}
-
-template <int RP, int CPL>
-__device__ __forceinline__ void load_weights(const Lane<RP, CPL> &L, u64 (&w)[CPL / 2])
-{
-#pragma unroll
-    for (int v = 0; v < CPL / 4; ++v) lds2(w[2 * v], w[2 * v + 1], L.w + v * (Lay<RP, CPL>::LPR * 16));
-}
-
-template <int CNT, int N, int BIT, bool MAX>
-__device__ __forceinline__ void halve_lanes(float (&v)[N], int lane, int &off)
-{
-    if constexpr (BIT < 32) {
-        constexpr int H = CNT > 1 ? CNT / 2 : 1;
-        const bool up = CNT > 1 && (lane & BIT) != 0;
-#pragma unroll
-        for (int i = 0; i < H; ++i) {
-            const float give = up || CNT == 1 ? v[i] : v[i + H < N ? i + H : i], keep = up ? v[i + H < N ? i + H : i] : v[i];
-            const float got = __shfl_xor_sync(0xffffffffu, give, BIT);
-            v[i] = MAX ? fmaxf(keep, got) : keep + got;
-        }
-        off += up ? H : 0;
-        halve_lanes<H, N, BIT * 2, MAX>(v, lane, off);
-    }
-}
-
-// The warp's column values into red[warp][RP], in a fixed order: lanes that hold the same columns halve them among them.
-template <int RP, int CPL, bool MAX>
-__device__ __forceinline__ void warp_columns(float *red, float (&v)[CPL])
-{
-    typedef Lay<RP, CPL> Y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cl = lane % Y::LPR;
-    int off = 0;
-    halve_lanes<CPL, CPL, Y::LPR, MAX>(v, lane, off);
-    constexpr int LEFT = CPL / Y::RPW < 1 ? 1 : CPL / Y::RPW;
-#pragma unroll
-    for (int i = 0; i < LEFT; ++i) {
-        const int k = off + i;
-        red[warp * RP + ((k >> 2) * Y::LPR + cl) * 4 + (k & 3)] = v[i];
-    }
-}
-
-// ... and the block's: thread t < RP returns column t's.  One barrier inside; the work area is free again after the
-// caller's next barrier.
-template <int RP, int CPL, int THREADS, bool MAX>
-__device__ __forceinline__ float block_columns(const Shared &S, float (&v)[CPL])
-{
-    float *red = reinterpret_cast<float *>(S.work);
-    warp_columns<RP, CPL, MAX>(red, v);
-    __syncthreads();
-    float tot = MAX ? neg_inf() : 0.f;
-    if (threadIdx.x < RP) {
-#pragma unroll
-        for (int wv = 0; wv < THREADS / 32; ++wv) {
-            const float o = red[wv * RP + threadIdx.x];
-            tot = MAX ? fmaxf(tot, o) : tot + o;
-        }
-    }
-    return tot;
-}
-
-__device__ __forceinline__ void put_word(u64 *p, float v, unsigned tag)
-{
-    const u64 word = ((u64)tag << 32) | __float_as_uint(v);
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(word) : "memory");
-}
-__device__ __forceinline__ u64 peek_word(const u64 *p)
-{
-    u64 v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-// Wait until the word carries `tag` (at most a second, then the call is flagged and every later wait gives up at once).
-__device__ __forceinline__ float take_word(const u64 *p, u64 first, unsigned tag, volatile int *dead, int *status)
-{
-    u64 v = first;
-    if ((unsigned)(v >> 32) != tag && !*dead) {
-        const u64 start = global_timer_ns();
-        unsigned spin = 0;
-        while (true) {
-            v = peek_word(p);
-            if ((unsigned)(v >> 32) == tag) break;
-            if ((++spin & 255u) == 0 && (*dead || global_timer_ns() - start > kWaitNs)) {
-                if (!*dead) atomicOr(status, 4 /* LOT_DEV_TIMEOUT */);
-                *dead = 1;
-                break;
-            }
-        }
-    }
-    return __uint_as_float((unsigned)v);
-}
-
-// Totals of the group's column values: thread t < RP gives its block's value of column t and gets the group's.
-// Small groups: every block reads every block's words.  Large ones (C * RP > kDirectWords): block t % C adds up column t
-// and leaves the total in kCopies places, each read by a share of the blocks (one place for all of 148 blocks to poll
-// took 5.9 us per exchange at RP = 256, eight take 4.4; reading every block's words takes 12.9 there, but 2.1 for 16
-// blocks and 0.7 for two).  Two buffers by parity: a block can be at most one exchange ahead of the others.
-template <int RP, int THREADS, bool MAX>
-__device__ __forceinline__ float group_columns(const SweepArgs &a, const Shared &S, float part, int group, int c, unsigned &seq)
-{
-    const int C = a.C, tid = threadIdx.x;
-    if (C == 1) return part;
-    ++seq;
-    const unsigned tag = seq;
-    u64 *X = a.xbuf + (size_t)(group * 2 + (seq & 1)) * C * RP;
-    if (C * RP <= kDirectWords) {
-        constexpr int NS = THREADS / RP;                     // threads that share a column
-        if (tid < RP) put_word(X + (size_t)c * RP + tid, part, tag);
-        const int t = tid % RP, sb = tid / RP;
-        float tot = MAX ? neg_inf() : 0.f;
-        for (int c0 = sb; c0 < C; c0 += 4 * NS) {
-            u64 wd[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * NS < C) wd[u] = peek_word(X + (size_t)(c0 + u * NS) * RP + t);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * NS < C) {
-                    const float o = take_word(X + (size_t)(c0 + u * NS) * RP + t, wd[u], tag, S.flag, a.status);
-                    tot = MAX ? fmaxf(tot, o) : tot + o;
-                }
-        }
-        if (NS > 1) {
-            float *r2 = reinterpret_cast<float *>(S.ref);    // NS * RP = THREADS floats; refs are in use only while building
-            r2[tid] = tot;
-            __syncthreads();
-            if (tid < RP) {
-                tot = r2[tid];
-                for (int s2 = 1; s2 < NS; ++s2) tot = MAX ? fmaxf(tot, r2[s2 * RP + tid]) : tot + r2[s2 * RP + tid];
-            }
-        }
-        return tot;
-    }
-    if (tid < RP) put_word(X + (size_t)tid * C + c, part, tag);
-    u64 *Y = a.ybuf + (size_t)(group * 2 + (seq & 1)) * kCopies * RP;
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int t = c + warp * C; t < RP; t += (THREADS / 32) * C) {
-        float tot = MAX ? neg_inf() : 0.f;
-        for (int c0 = lane; c0 < C; c0 += 128) {
-            u64 wd[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * 32 < C) wd[u] = peek_word(X + (size_t)t * C + c0 + u * 32);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * 32 < C) {
-                    const float o = take_word(X + (size_t)t * C + c0 + u * 32, wd[u], tag, S.flag, a.status);
-                    tot = MAX ? fmaxf(tot, o) : tot + o;
-                }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float o = __shfl_xor_sync(0xffffffffu, tot, off);
-            tot = MAX ? fmaxf(tot, o) : tot + o;
-        }
-        if (lane < kCopies) put_word(Y + lane * RP + t, tot, tag);
-    }
-    float tot = 0.f;
-    Y += (c % kCopies) * RP;
-    if (tid < RP) tot = take_word(Y + tid, peek_word(Y + tid), tag, S.flag, a.status);
-    return tot;
-}
-
-// Column sums in the log domain, from stored exponents e_it: with x_it = e_it - log2 sum_t 2^e_it + log2 m_i the
-// thread t < RP returns log2 sum_i 2^x_it over the group, taken relative to the column's maximum.
-template <int RP, int CPL, int THREADS>
-__device__ __forceinline__ float log_columns(const SweepArgs &a, const Shared &S, const Share &R, int group, int c, unsigned &seq)
-{
-    typedef Lay<RP, CPL> Y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane / Y::LPR, cl = lane % Y::LPR;
-    constexpr int STEP = (THREADS / 32) * Y::RPW;
-    float v[CPL];
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) v[k] = neg_inf();
-    for (int base = warp * Y::RPW; base < R.nrows; base += STEP) {
-        const int i = base + sub;
-        const bool ok = i < R.nrows;
-        float e[CPL];
-        float s = 0.f;
-#pragma unroll
-        for (int u = 0; u < Y::NV; ++u) {
-            const float4 t = ok ? *chunk_ptr<RP, CPL>(S, R, i, u * Y::LPR + cl) : make_float4(0.f, 0.f, 0.f, 0.f);
-            e[4 * u] = t.x; e[4 * u + 1] = t.y; e[4 * u + 2] = t.z; e[4 * u + 3] = t.w;
-        }
-#pragma unroll
-        for (int k = 0; k < CPL; ++k) s += ex2(e[k]);
-        s = group_sum(s, Y::LPR);
-        const float m = ok ? (R.mass ? __ldg(R.mass + i) : 1.f) : 0.f;
-        const float shift = m > 0.f ? lg2(m) - lg2(s) : neg_inf();
-#pragma unroll
-        for (int k = 0; k < CPL; ++k) {
-            e[k] = e[k] + shift;
-            v[k] = fmaxf(v[k], e[k]);
-        }
-        if (ok) {
-#pragma unroll
-            for (int u = 0; u < Y::NV; ++u)
-                *chunk_ptr<RP, CPL>(S, R, i, u * Y::LPR + cl) = make_float4(e[4 * u], e[4 * u + 1], e[4 * u + 2], e[4 * u + 3]);
-        }
-    }
-    const float kap = group_columns<RP, THREADS, true>(a, S, block_columns<RP, CPL, THREADS, true>(S, v), group, c, seq);
-    if (threadIdx.x < RP) S.w[threadIdx.x] = kap;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) v[k] = 0.f;
-    for (int base = warp * Y::RPW; base < R.nrows; base += STEP) {
-        const int i = base + sub;
-        if (i >= R.nrows) continue;
-#pragma unroll
-        for (int u = 0; u < Y::NV; ++u) {
-            const float4 t = *chunk_ptr<RP, CPL>(S, R, i, u * Y::LPR + cl), kk = *reinterpret_cast<const float4 *>(S.w + (u * Y::LPR + cl) * 4);
-            if (kk.x > neg_inf()) v[4 * u] += ex2(t.x - kk.x);
-            if (kk.y > neg_inf()) v[4 * u + 1] += ex2(t.y - kk.y);
-            if (kk.z > neg_inf()) v[4 * u + 2] += ex2(t.z - kk.z);
-            if (kk.w > neg_inf()) v[4 * u + 3] += ex2(t.w - kk.w);
-        }
-    }
-    __syncthreads();
-    const float sum = group_columns<RP, THREADS, false>(a, S, block_columns<RP, CPL, THREADS, false>(S, v), group, c, seq);
-    return kap + lg2(sum);
-}
-
-// The group's share of problem p for block c, and the block's shared memory.
-template <typename T, int RP, int THREADS>
-__device__ __forceinline__ Shared carve(uint8_t *p, int srows)
-{
-    Shared S;
-    S.K = reinterpret_cast<float *>(p); p += (size_t)srows * RP * 4;
-    S.gref = reinterpret_cast<double *>(p); p += RP * 8;
-    S.work = p; p += work_bytes<T>(RP, THREADS);
-    S.ref = reinterpret_cast<float *>(p); p += ref_bytes(RP, THREADS);
-    S.w = reinterpret_cast<float *>(p); p += RP * 4;
-    S.tgt = reinterpret_cast<float *>(p); p += RP * 4;
-    S.flag = reinterpret_cast<volatile int *>(p);
-    return S;
-}
-
-struct Problem {
-    int slice, side, h, n, nv, row0;
-};
-
-template <int RP, int CPL, int THREADS>
-__device__ __forceinline__ Problem locate(const SweepArgs &a, int p, int c, Share &R)
-{
-    constexpr int STEP = (THREADS / 32) * Lay<RP, CPL>::RPW;
-    Problem P;
-    P.slice = p >> 1;
-    P.side = (p & 1) ^ 1;
-    P.h = P.slice % a.H;
-    P.n = a.n[P.side];
-    P.nv = P.n;
-    if (P.side == 1 && a.key_len != nullptr) P.nv = min(max(__ldg(a.key_len + P.slice / a.H), 0), P.n);
-    P.nv = max(P.nv - a.skip, 0);
-    const int per = (P.nv + a.C - 1) / a.C;
-    P.row0 = min(c * per, P.nv);
-    R.nrows = min(per, P.nv - P.row0);
-    P.row0 += a.skip;                                        // from here on within the slice's tokens
-    R.ns = min(R.nrows, a.srows);
-    R.steps = (R.ns + STEP - 1) / STEP;
-    R.g = a.kt[P.side] + ((size_t)P.slice * P.n + P.row0) * RP;
-    R.mass = a.mass[P.side] ? a.mass[P.side] + (size_t)P.slice * P.n + P.row0 : nullptr;
-    return P;
-}
-
-// Whether a weight is outside the kernel's range, and whether that is because its column sum (target / weight) left
-// float32's.
-__device__ __forceinline__ bool out_of_range(float w) { return !(w >= kFarLo && w <= kFarHi); }
-__device__ __forceinline__ bool sum_lost(float tgt, float w) { return !(tgt >= kLostLo * w && tgt <= kLostHi * w); }
-
-// One iteration of the block's problem: thread t < r gets its column's weight before and after; true where the update
-// leaves the range (block-uniform; the weights in shared memory are then the new ones all the same).  The chain of an
-// iteration is what a short problem takes: two plain barriers, the range flag read beside the weights of the next
-// iteration (a voting barrier took 50 cycles more).
-template <int RP, int CPL, int THREADS, bool GROUP>
-__device__ __forceinline__ bool iterate(const SweepArgs &a, const Shared &S, const Share &R, const Lane<RP, CPL> &L, u64 (&w)[CPL / 2],
-                                        float tgt, int group, int c, unsigned &seq, float &wold, float &wnew)
-{
-    typedef Lay<RP, CPL> Y;
-    u64 acc[CPL / 2];
-    pass<RP, CPL, THREADS, false>(L, R, w, acc, nullptr);
-    float v[CPL];
-#pragma unroll
-    for (int j = 0; j < CPL / 2; ++j) unpack_f2(acc[j], v[2 * j], v[2 * j + 1]);
-    int off = 0;
-    halve_lanes<CPL, CPL, Y::LPR, false>(v, threadIdx.x & 31, off);
-    constexpr int LEFT = CPL / Y::RPW < 1 ? 1 : CPL / Y::RPW;
-#pragma unroll
-    for (int i = 0; i < LEFT; ++i) sts(L.red + ((i >> 2) * Y::LPR * 4 + (i & 3)) * 4, v[i]);
-    __syncthreads();
-    float tot = 0.f;
-    if (threadIdx.x < RP) {
-        float o[THREADS / 32];
-#pragma unroll
-        for (int i = 0; i < THREADS / 32; ++i) o[i] = lds(L.own + i * (RP * 4));
-#pragma unroll
-        for (int h = THREADS / 64; h > 0; h >>= 1)
-#pragma unroll
-            for (int i = 0; i < h; ++i) o[i] += o[i + h];
-        tot = o[0];
-    }
-    if (GROUP) tot = group_columns<RP, THREADS, false>(a, S, tot, group, c, seq);
-    if ((int)threadIdx.x < a.r) {
-        wold = wnew;
-        wnew = tgt * rcp(tot);
-        if (out_of_range(wnew)) S.flag[1] = 1;
-        S.w[threadIdx.x] = wnew;
-    }
-    __syncthreads();
-    load_weights<RP, CPL>(L, w);
-    return S.flag[1] != 0;
-}
 
 template <int RP, int CPL, int THREADS>
 __device__ __forceinline__ void finish(const SweepArgs &a, const Shared &S, const Share &R, const Problem &P, int c)
@@ -644,66 +39,11 @@ __device__ __forceinline__ void finish(const SweepArgs &a, const Shared &S, cons
     }
 }
 
-// The rest of a problem from iteration `it` on, whose update left the kernel's range (wold, wnew: thread t < r's weight
-// before and after it): the kernel is rebuilt around the new potentials, after the update has been redone in the log
-// domain where a column sum was lost.  Out of line and last in a problem's life, so that it costs the iteration loop of
-// the kernel no registers.  Returns the sequence number.
-template <typename T, int RP, int CPL, int THREADS, bool GROUP>
-__device__ __noinline__ unsigned finish_slow(const SweepArgs *ap, int p, int group, int c, int it, unsigned seq, float wold, float wnew)
-{
-    extern __shared__ __align__(128) uint8_t smem[];
-    const SweepArgs &a = *ap;
-    const Shared S = carve<T, RP, THREADS>(smem, a.srows);
-    Share R;
-    const Problem P = locate<RP, CPL, THREADS>(a, p, c, R);
-    const T *x = static_cast<const T *>(a.x[P.side]) + ((size_t)P.slice * P.n + P.row0) * a.d;
-    const float *z = a.z + (size_t)P.h * a.r * a.d;
-    const Lane<RP, CPL> L = make_lane<RP, CPL>(S);
-    const int tid = threadIdx.x, r = a.r;
-    while (true) {
-        double gn = 0.0;
-        if (__syncthreads_or(tid < r && sum_lost(S.tgt[tid < RP ? tid : 0], wnew))) {
-            if (tid < r) {
-                gn = S.gref[tid] + log2((double)wold);
-                S.gref[tid] = gn;
-            }
-            __syncthreads();
-            build<T, RP, CPL, THREADS, true>(S, R, x, z, a.d, r, a.scale);
-            const float lam = log_columns<RP, CPL, THREADS>(a, S, R, group, c, seq);
-            if (tid < r) gn += log2((double)S.tgt[tid]) - (double)lam;
-        } else if (tid < r) {
-            gn = S.gref[tid] + log2((double)wnew);
-        }
-        __syncthreads();
-        if (tid < r) {
-            if (!isfinite(gn)) atomicOr(a.status, 1 /* LOT_DEV_NONFINITE */);
-            S.gref[tid] = gn - (double)kStartLog2;
-            S.w[tid] = kStart;
-        } else if (tid < RP) {
-            S.w[tid] = 0.f;
-        }
-        if (tid == 0) S.flag[1] = 0;
-        __syncthreads();
-        build<T, RP, CPL, THREADS, false>(S, R, x, z, a.d, r, a.scale);
-        bool bad = false;
-        u64 w[CPL / 2];
-        load_weights<RP, CPL>(L, w);
-        wnew = kStart;
-        for (++it; it < a.it1 && !bad; ++it)
-            bad = iterate<RP, CPL, THREADS, GROUP>(a, S, R, L, w, S.tgt[tid < RP ? tid : 0], group, c, seq, wold, wnew);
-        if (!bad) break;
-        --it;                                                // the iteration whose update has to be redone
-    }
-    finish<RP, CPL, THREADS>(a, S, R, P, c);
-    return seq;
-}
-
 template <typename T, int RP, int CPL, int THREADS, bool GROUP>
 __global__ void __launch_bounds__(THREADS, max_blocks(CPL, THREADS))
 sweep_kernel(const __grid_constant__ SweepArgs a)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    constexpr int STEP = (THREADS / 32) * Lay<RP, CPL>::RPW;
     const int tid = threadIdx.x, group = GROUP ? blockIdx.x / a.C : blockIdx.x, c = GROUP ? blockIdx.x % a.C : 0;
     const int NP = 2 * a.B * a.H, r = a.r;
     unsigned seq = a.seq0;
@@ -727,14 +67,8 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
             S.w[tid] = w0;
             S.tgt[tid] = tid < r ? __ldg(a.beta + P.h * r + tid) * (R.mass ? 1.f : (float)P.nv) : 0.f;
         }
-        for (int idx = tid; idx < R.steps * STEP * (RP / 4); idx += THREADS) {
-            const int i = idx / (RP / 4);
-            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(reinterpret_cast<float4 *>(S.K + (size_t)i * RP) + Lay<RP, CPL>::swz(i, idx % (RP / 4)));
-            // rows past the last are filled with zeros
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(reinterpret_cast<const float4 *>(R.g) + (i < R.ns ? idx : 0)),
-                         "r"(i < R.ns ? 16 : 0) : "memory");
-        }
-        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        load_rows<RP, CPL, THREADS>(S, R);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
         if (P.nv <= 0 && tid == 0 && a.first && c == 0) atomicOr(a.status, 2 /* LOT_DEV_EMPTY */);
         __syncthreads();
         float wold = 0.f, wnew = S.w[tid < RP ? tid : 0];
@@ -746,12 +80,17 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
             u64 w[CPL / 2];
             load_weights<RP, CPL>(L, w);
             for (; it < a.it1; ++it) {
+                if (a.hist != nullptr && c == 0 && tid < RP) a.hist[((size_t)it * NP + p) * RP + tid] = tid < r ? wnew : 0.f;
                 bad = iterate<RP, CPL, THREADS, GROUP>(a, S, R, L, w, tgt, group, c, seq, wold, wnew);
                 if (bad) break;
             }
+            if (!bad && a.hist != nullptr && c == 0) {
+                if (tid < RP) a.hist[((size_t)it * NP + p) * RP + tid] = tid < r ? wnew : 0.f;
+                if (tid == 0) a.wide[p] = 0;
+            }
         }
-        if (bad) seq = finish_slow<T, RP, CPL, THREADS, GROUP>(&a, p, group, c, it, seq, wold, wnew);
-        else finish<RP, CPL, THREADS>(a, S, R, P, c);
+        if (bad) seq = recover<T, RP, CPL, THREADS, GROUP>(&a, S, p, group, c, it, seq, wold, wnew);
+        finish<RP, CPL, THREADS>(a, S, R, P, c);
     }
 }
 

@@ -29,6 +29,10 @@ struct SweepArgs {
     float *g_out[2];         // [BH][r] potentials in natural units or nullptr
     unsigned long long *xbuf;   // exchange words of the groups (zero at the start of the first launch of a call)
     unsigned long long *ybuf;
+    float *hist;             // backward: [it1 + 1][problems][RP] weights before every iteration and after the last, relative to
+                             // the kernel as it is left, or nullptr
+    double *hist_g;          // ... and the potentials themselves, of the problems whose kernel was rebuilt
+    int *wide;               // ... [problems] 1: the kept weights leave float32's range, use hist_g
     int *status;
     int B, H, d, r;
     int n[2];                // tokens per slice
@@ -53,20 +57,42 @@ cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaS
 cudaError_t launch_sweep(const SweepPlan &P, const SweepArgs &a, int dtype, cudaStream_t st);
 
 struct SweepApplyArgs {
-    const float *kt[2], *inv[2], *w[2];
-    const float *beta;
+    const float *kt[2], *inv[2], *w[2];   // inv, w: nullptr means 1 (kt is used as it is)
+    const float *beta;       // nullptr: no scaling of W'
     const int32_t *key_len;
     const float *mass2;      // key weights or nullptr
     const void *v;
     void *out;
     float *wpart;            // [BH][chunks][r][d]
-    float *Wp;               // [BH][r][d]
+    float *Wp;               // [BH][r][d]; nullptr on the key side: the chunk partials are the result
+    const int32_t *out_len;  // query side: rows beyond this length are zero, or nullptr
     unsigned *counter;
     int B, H, nq, nk, d, r, RP;
     int skip;                // leading tokens that take no part
+    int per_head;            // query side: Wp is [H][r][d]
     int chunks, rows_per_chunk;
 };
 cudaError_t launch_sweep_apply_w(const SweepApplyArgs &a, int dtype, cudaStream_t st);
 cudaError_t launch_sweep_apply_out(const SweepApplyArgs &a, int dtype, cudaStream_t st);
+
+// ---- backward of bf16 tensors on the stored kernel (lot_sweep_bwd.cu); problem numbering as above ----
+struct SweepBwdArgs {
+    SweepArgs s;             // x, z, kt, inv, w, hist, hist_g, wide, groups as in the forward; seq0 continues its sequence
+    const void *g[2];        // [BH][n][d] bf16: dout (queries), v (keys)
+    const float *wmat[2];    // [BH][r][d]: W' (queries), dW (keys): the plan's gradient is g . wmat
+    float *dC[2];            // [BH][n][RP] gradient with respect to the similarities
+    float2 *coef;            // [problems][T][n] row coefficients of every reverse step
+    float *fk;               // [T][problems][RP] column coefficients
+    float *gpart;            // [problems][tiles][RP] column sums of the closing step
+    float *dbeta_acc;        // [problems][RP]
+    int T, tiles;
+    double eps;
+};
+cudaError_t launch_bwd_close(int RP, const SweepBwdArgs &a, cudaStream_t st);
+cudaError_t launch_bwd_reverse(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st);
+cudaError_t launch_bwd_assemble(int RP, const SweepBwdArgs &a, cudaStream_t st);
+// dz[h][t][c] = sum over batch, sides and chunks of the partials of dC^T x; dbeta as in launch_bwd_dz
+cudaError_t launch_bwd_merge(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz,
+                             float *dbeta, int B, int H, int d, int r, int RP, int chunks, cudaStream_t st);
 
 } // namespace lot

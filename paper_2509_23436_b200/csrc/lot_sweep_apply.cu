@@ -72,7 +72,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
     int nv = n;
     if (a.key_len != nullptr) nv = min(max(a.key_len[b], 0), n);
     const float *mass = a.mass2 ? a.mass2 + (size_t)bh * n : nullptr;
-    const float *K = a.kt[1] + (size_t)bh * n * RP + t0, *inv = a.inv[1] + (size_t)bh * n, *w = a.w[1] + (size_t)bh * RP + t0;
+    const float *K = a.kt[1] + (size_t)bh * n * RP + t0, *inv = a.inv[1] ? a.inv[1] + (size_t)bh * n : nullptr, *w = a.w[1] ? a.w[1] + (size_t)bh * RP + t0 : nullptr;
     const __nv_bfloat16 *V = static_cast<const __nv_bfloat16 *>(a.v) + (size_t)bh * n * d;
     const int row0 = chunk * a.rows_per_chunk + a.skip, row1 = min(min(row0 + a.rows_per_chunk, n), nv);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -89,7 +89,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
             sc[u] = 0.f;
             if (j < row1) {
                 kr[u] = __ldg(reinterpret_cast<const float4 *>(K + (size_t)j * RP + t));
-                sc[u] = __ldg(inv + j) * (mass ? __ldg(mass + j) : 1.f);
+                sc[u] = (inv ? __ldg(inv + j) : 1.f) * (mass ? __ldg(mass + j) : 1.f);
             }
         }
 #pragma unroll
@@ -101,7 +101,8 @@ apply_w_mma_kernel(SweepApplyArgs a)
     float acc[NTW][4] = {};
     float4 wt[NP];
 #pragma unroll
-    for (int u = 0; u < NP; ++u) wt[u] = __ldg(reinterpret_cast<const float4 *>(w + ((tid + u * kThreads) % (TP / 4)) * 4));
+    for (int u = 0; u < NP; ++u)
+        wt[u] = w ? __ldg(reinterpret_cast<const float4 *>(w + ((tid + u * kThreads) % (TP / 4)) * 4)) : make_float4(1.f, 1.f, 1.f, 1.f);
     if (row0 < row1) fetch(row0);
     const int mi = lane >> 3;
     for (int j0 = row0; j0 < row1; j0 += KT) {
@@ -172,7 +173,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
                 const int t = t0 + pt * 16 + g + 8 * hh, c = cg * NTW * 8 + nt * 8 + 2 * q;
                 if (t < r && c < d) {
                     const float2 v = make_float2(acc[nt][2 * hh], acc[nt][2 * hh + 1]);
-                    if (a.chunks > 1) {
+                    if (a.chunks > 1 || a.Wp == nullptr) {
                         __stcg(reinterpret_cast<float2 *>(wp + (size_t)t * d + c), v);
                     } else {
                         const float f = scale / a.beta[h * r + t];
@@ -181,7 +182,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
                 }
             }
     }
-    if (a.chunks == 1 || !last_of_tile(a.counter + (size_t)bh * gridDim.y + blockIdx.y, a.chunks)) return;
+    if (a.chunks == 1 || a.Wp == nullptr || !last_of_tile(a.counter + (size_t)bh * gridDim.y + blockIdx.y, a.chunks)) return;
     const int nt4 = min(TP, r - t0) * d / 4;
     for (int idx = tid; idx < nt4; idx += kThreads) {
         const size_t o = (size_t)t0 * d + idx * 4;
@@ -210,11 +211,13 @@ apply_out_mma_kernel(SweepApplyArgs a)
     const int bh = blockIdx.y, n = a.nq, r = a.r, d = a.d, RP = a.RP;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3, mi = lane >> 3;
     const int i0 = blockIdx.x * 128 + warp * 16 + a.skip;
-    const float *K = a.kt[0] + ((size_t)bh * n + i0) * RP, *w = a.w[0] + (size_t)bh * RP;
-    const float *W = a.Wp + (size_t)bh * r * d;
+    const int nrow = a.out_len ? min(max(__ldg(a.out_len + bh / a.H), 0), n) : n;     // rows beyond it are zero
+    const float *K = a.kt[0] + ((size_t)bh * n + i0) * RP, *w = a.w[0] ? a.w[0] + (size_t)bh * RP : nullptr;
+    const float *W = a.Wp + (size_t)(a.per_head ? bh % a.H : bh) * r * d;
     float s[2];
 #pragma unroll
-    for (int hh = 0; hh < 2; ++hh) s[hh] = i0 + g + 8 * hh < n ? __ldg(a.inv[0] + (size_t)bh * n + i0 + g + 8 * hh) : 0.f;
+    for (int hh = 0; hh < 2; ++hh)
+        s[hh] = i0 + g + 8 * hh < nrow ? (a.inv[0] ? __ldg(a.inv[0] + (size_t)bh * n + i0 + g + 8 * hh) : 1.f) : 0.f;
     float2 kr[TS / 16][4];
     float4 wr[NW];
     auto fetch = [&](int tb) {
@@ -223,7 +226,7 @@ apply_out_mma_kernel(SweepApplyArgs a)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int row = g + (e & 1) * 8, t = tb + k * 16 + (e >> 1) * 8 + 2 * q;
-                kr[k][e] = i0 + row < n ? __ldg(reinterpret_cast<const float2 *>(K + (size_t)row * RP + t)) : make_float2(0.f, 0.f);
+                kr[k][e] = i0 + row < nrow ? __ldg(reinterpret_cast<const float2 *>(K + (size_t)row * RP + t)) : make_float2(0.f, 0.f);
             }
 #pragma unroll
         for (int u = 0; u < NW; ++u) {
@@ -249,7 +252,7 @@ apply_out_mma_kernel(SweepApplyArgs a)
         for (int k = 0; k < TS / 16; ++k)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float2 ww = __ldg(reinterpret_cast<const float2 *>(w + tb + k * 16 + (e >> 1) * 8 + 2 * q));
+                const float2 ww = w ? __ldg(reinterpret_cast<const float2 *>(w + tb + k * 16 + (e >> 1) * 8 + 2 * q)) : make_float2(1.f, 1.f);
                 uint32_t o[3];
                 split3(kr[k][e].x * (ww.x * s[e & 1]), kr[k][e].y * (ww.y * s[e & 1]), o);
 #pragma unroll
@@ -307,7 +310,7 @@ apply_w_f32_kernel(SweepApplyArgs a)
     int nv = n;
     if (a.key_len != nullptr) nv = min(max(a.key_len[b], 0), n);
     const float *mass = a.mass2 ? a.mass2 + (size_t)bh * n : nullptr;
-    const float *K = a.kt[1] + (size_t)bh * n * RP + t0, *inv = a.inv[1] + (size_t)bh * n, *w = a.w[1] + (size_t)bh * RP + t0;
+    const float *K = a.kt[1] + (size_t)bh * n * RP + t0, *inv = a.inv[1] ? a.inv[1] + (size_t)bh * n : nullptr, *w = a.w[1] ? a.w[1] + (size_t)bh * RP + t0 : nullptr;
     const float *V = static_cast<const float *>(a.v) + (size_t)bh * n * d;
     const int row0 = chunk * a.rows_per_chunk + a.skip, row1 = min(min(row0 + a.rows_per_chunk, n), nv);
     const int grp = tid / GT, ty = (tid % GT) / 16, tx = tid % 16;
@@ -322,7 +325,7 @@ apply_w_f32_kernel(SweepApplyArgs a)
             sc[u] = 0.f;
             if (idx < kStep * TP / 4 && j < row1) {
                 kr[u] = __ldg(reinterpret_cast<const float4 *>(K + (size_t)j * RP + (idx % (TP / 4)) * 4));
-                sc[u] = __ldg(inv + j) * (mass ? __ldg(mass + j) : 1.f);
+                sc[u] = (inv ? __ldg(inv + j) : 1.f) * (mass ? __ldg(mass + j) : 1.f);
             }
         }
 #pragma unroll
