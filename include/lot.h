@@ -155,7 +155,10 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
 /*
  * lot_path -- which implementation one lot_attention_fwd_ex call with these parameters takes (host
  * arithmetic only):
- *   0  the general path: a cost kernel per side, one kernel per Sinkhorn pass, two apply kernels.
+ *   0  the general path: the Gibbs kernel of both sides in float32, all Sinkhorn passes in one kernel that keeps what it
+ *      can of it in shared memory (one launch per pass for float32 tensors whose kernel is far larger than the shared
+ *      memory of the device), two apply kernels.  Blocks of one problem wait for one another: where a problem is shared
+ *      by several, the kernel is launched cooperatively.
  *   1  the streamed tensor-core path (bf16 tensors, d = 64, r <= 64): one persistent kernel for all
  *      passes, launched cooperatively (it needs as many free SMs as it has thread blocks, at most
  *      one per SM), plus a small pivot preparation.  With 32 < r <= 64 its first pass keeps the
@@ -168,10 +171,10 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *      column mass below 2^-80) is recomputed by the streamed kernels, which are launched behind it
  *      and return at once otherwise (device flag LOT_DEV_RECOMPUTED).  It can run many more shapes
  *      (lot_debug_hook what = 4), but measured no faster there.
- *   3  the slice path (same tensors; n <= 512 and 16 ceil(n/16) x (r padded to 16, 32 or 64) <= 16384): one
- *      thread block per (batch, head) slice keeps a side's logits in float32 registers for all iterations
- *      (warp-level tensor-core products, shared memory for K, V, Q and the r x d intermediate); nothing
- *      crosses thread blocks, no workspace beyond the status word.  Taken wherever it can run.
+ *   3  the slice path (same tensors; n <= 512 and 16 ceil(n/16) x (r padded to 16, 32 or 64) <= 16384): a pair of
+ *      thread blocks per (batch, head) slice, one for each side, keeps the side's Gibbs kernel in float32 in shared
+ *      memory for all iterations (warp-level tensor-core products); only the r x d intermediate crosses, inside the
+ *      pair's cluster; no workspace beyond the status word.  Taken wherever it can run.
  * On paths 1 and 2 the potentials agree with an exact float evaluation to about 1e-4 and the output
  * to the bf16 rounding of `out`.
  */
@@ -222,8 +225,9 @@ LOT_API int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
  *   key_len [B] int32 or NULL as in the forward (rows of dk, dv beyond the length are zero).
  *   beta is treated as r free positive numbers per head (no simplex constraint: a softmax parametrisation is the
  *   caller's chain rule); dz and dbeta are summed over the batch.
- * The forward is recomputed (materialised similarities, general path arithmetic: float32 for bf16 tensors,
- * float64 for float32 tensors); only the pivot potentials of every iteration are kept.  2*iters + 15 kernel launches.
+ * The forward is recomputed in the general path's arithmetic (float32 for bf16 tensors, float64 for float32 tensors);
+ * of its iterations only the pivot potentials are kept.  bf16 tensors: 13 kernel launches, two numbers per token and
+ * iteration in the workspace; float32 tensors: 2*iters + 15 launches.
  * ws: lot_bwd_workspace_bytes(...) bytes of device scratch, 256-byte aligned, owned by the caller; the device
  * status word of the recomputed forward sits at its start (lot_device_status).
  * Errors as lot_attention_fwd_ex.  B == 0 or n == 0: dz and dbeta are zero-filled, nothing else is touched.

@@ -69,29 +69,44 @@ def _check(status: int, what: str):
         raise LotError(f"{what}: {lib().lot_status_string(status).decode()}")
 
 
-def _dev(t: Optional[torch.Tensor], name: str, dtype=None):
-    if t is None:
-        return None
+def _refuse(t: torch.Tensor, name: str, dtype):
     if not t.is_cuda:
         raise LotError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise LotError(f"{name} must be contiguous")
-    if dtype is not None and t.dtype != dtype:
-        raise LotError(f"{name} must be {dtype}, got {t.dtype}")
+    raise LotError(f"{name} must be {dtype}, got {t.dtype}")
+
+
+# A call of the smallest problems is as long as its Python side: the checks below are one expression a tensor, the
+# stream comes as a raw handle, and the workspace size is asked for only where the workspace is made here (22 -> 12 us
+# for lot_attention_fwd_ex).
+def _dev(t: Optional[torch.Tensor], name: str, dtype=None):
+    if t is None:
+        return None
+    if not (t.is_cuda and t.is_contiguous() and (dtype is None or t.dtype is dtype)):
+        _refuse(t, name, dtype)
     return t.data_ptr()
 
 
+_CODES = {torch.float32: LOT_F32, torch.bfloat16: LOT_BF16}
+
+
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return LOT_F32
-    if t.dtype == torch.bfloat16:
-        return LOT_BF16
-    raise LotError(f"unsupported tensor dtype {t.dtype}")
+    code = _CODES.get(t.dtype)
+    if code is None:
+        raise LotError(f"unsupported tensor dtype {t.dtype}")
+    return code
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        if _raw_stream is None or _get_device is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_get_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -123,9 +138,8 @@ def lot_sinkhorn(cost, beta, length, eps, iters, *, want_f=False, want_plan=Fals
     g = torch.empty(B, H, r, device=dev, dtype=torch.float32)
     f = torch.empty(B, H, n, device=dev, dtype=torch.float32) if want_f else None
     plan = torch.empty(B, H, n, r, device=dev, dtype=torch.float32) if want_plan else None
-    need = lot_sinkhorn_workspace_bytes(B, H, n, r)
     if ws is None:
-        ws = torch.empty(max(need, 256), device=dev, dtype=torch.uint8)
+        ws = torch.empty(max(lot_sinkhorn_workspace_bytes(B, H, n, r), 256), device=dev, dtype=torch.uint8)
     st = lib().lot_sinkhorn(_dev(cost, "cost", torch.float32), _dev(beta, "beta", torch.float32),
                             _dev(length, "len", torch.int32), B, H, n, r, float(eps), int(iters),
                             _dev(g, "g"), _dev(f, "f"), _dev(plan, "plan"),
@@ -178,9 +192,8 @@ def lot_attention_fwd_ex(q, k, v, z, beta, key_len, eps, iters, *, out=None, g1_
         raise LotError("z must be [H,r,d] and beta [H,r]")
     if out is None:
         out = torch.empty_like(q)
-    need = lot_workspace_bytes(B, H, n, d, r, code)
     if ws is None:
-        ws = torch.empty(max(need, 256), device=q.device, dtype=torch.uint8)
+        ws = torch.empty(max(lot_workspace_bytes(B, H, n, d, r, code), 256), device=q.device, dtype=torch.uint8)
     st = lib().lot_attention_fwd_ex(_dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(z, "z", torch.float32),
                                     _dev(beta, "beta", torch.float32), _dev(key_len, "key_len", torch.int32),
                                     code, B, H, n, d, r, float(eps), int(iters),
@@ -208,9 +221,8 @@ def lot_attention_fwd_var(q, k, v, z, beta, eps, iters, *, a=None, b=None, key_l
         raise LotError("z must be [H,r,d] and beta [H,r]")
     if out is None:
         out = torch.empty_like(q)
-    need = lot_var_workspace_bytes(B, H, nq, nk, d, r, code)
     if ws is None:
-        ws = torch.empty(max(need, 256), device=q.device, dtype=torch.uint8)
+        ws = torch.empty(max(lot_var_workspace_bytes(B, H, nq, nk, d, r, code), 256), device=q.device, dtype=torch.uint8)
     f32 = torch.float32
     st = lib().lot_attention_fwd_var(_dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(z, "z", f32), _dev(beta, "beta", f32),
                                      _dev(a, "a", f32), _dev(b, "b", f32), _dev(key_len, "key_len", torch.int32),
@@ -261,9 +273,8 @@ def lot_attention_bwd(q, k, v, z, beta, key_len, dout, eps, iters, *, ws=None, s
     dq, dk, dv = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)
     dz = torch.empty((H, r, d), device=q.device, dtype=f32)
     dbeta = torch.empty((H, r), device=q.device, dtype=f32)
-    need = lot_bwd_workspace_bytes(B, H, n, d, r, code, int(iters))
     if ws is None:
-        ws = torch.empty(max(need, 256), device=q.device, dtype=torch.uint8)
+        ws = torch.empty(max(lot_bwd_workspace_bytes(B, H, n, d, r, code, int(iters)), 256), device=q.device, dtype=torch.uint8)
     st = lib().lot_attention_bwd(_dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(z, "z", f32), _dev(beta, "beta", f32),
                                  _dev(key_len, "key_len", torch.int32), _dev(dout, "dout", q.dtype),
                                  code, B, H, n, d, r, float(eps), int(iters),

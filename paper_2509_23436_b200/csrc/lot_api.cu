@@ -103,8 +103,8 @@ ForwardLayout forward_layout(int B, int H, int nq, int nk, int d, int r, int dty
     return L;
 }
 
-// Workspace of lot_attention_bwd for float32 tensors: similarities in float64, the row blocks of the log-domain passes plus the kept potentials of every iteration, the
-// gradient with respect to the similarities and the small reduction buffers.
+// Workspace of lot_attention_bwd for float32 tensors: similarities in float64, the blocks of the log-domain passes, the
+// kept potentials of every iteration, the gradient with respect to the similarities and the small reduction buffers.
 struct BwdLayout {
     size_t counter, counter2, hist, gamma, dbeta_acc, head_end, part, M, cost, dC, wpart, Wp, Xw, dWm, dbeta_direct, zt,
         dzpart, total;
@@ -244,7 +244,7 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
     return kPathStreamed;
 }
 
-// Both Sinkhorn problems and the apply stages on the general path, behind the clearing of the workspace head.
+// Both Sinkhorn problems and the apply stages on the general path.
 cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, const void *v, const float *z, const float *beta,
                         const float *mass_q, const float *mass_k, int skip, const int32_t *key_len, const float *g1_in, const float *g2_in,
                         int dtype, int B, int H, int nq, int nk, int d, int r, float eps, int iters, void *out, float *g1_out,
@@ -260,6 +260,7 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
     a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
     a.mass[0] = mass_q; a.mass[1] = mass_k; a.g_in[0] = g1_in; a.g_in[1] = g2_in; a.g_out[0] = g1_out; a.g_out[1] = g2_out;
     a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf); a.status = at<int>(ws, 0);
+    a.head = at<uint4>(ws, 0); a.head_words = L.head_end / 16;
     a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip;
     a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
@@ -271,6 +272,7 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
     } else {
         // one launch per side and pass: 4 sequence numbers per pass and problem of a group cover its exchanges
         if ((e = launch_build(L.plan.RP, a, dtype, 2, s)) != cudaSuccess) return e;
+        a.head_words = 0;
         if ((e = launch_build(L.plan.RP, a, dtype, 1, s)) != cudaSuccess) return e;
         for (int it = 0; it <= iters; ++it) {
             a.it0 = it; a.it1 = it < iters ? it + 1 : it; a.first = it == 0; a.close = it == iters;
@@ -292,8 +294,7 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
                          void *dk, void *dv, float *dz, float *dbeta, void *ws, cudaStream_t st)
 {
     const int dt = LOT_BF16, RP = L.plan.RP;
-    cudaError_t e = cudaMemsetAsync(ws, 0, L.head_end, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     SweepBwdArgs b{};
     SweepArgs &a = b.s;
     SweepApplyArgs ap{};
@@ -307,6 +308,7 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
     a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
     a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf);
     a.hist = at<float>(ws, L.hist); a.hist_g = at<double>(ws, L.hist_g); a.wide = at<int>(ws, L.wide); a.status = at<int>(ws, 0);
+    a.head = at<uint4>(ws, 0); a.head_words = L.head_end / 16;
     a.B = B; a.H = H; a.d = d; a.r = r;
     a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
@@ -562,7 +564,6 @@ int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
     const ForwardLayout L = forward_layout(B, H, n, n, d, r, dtype, false);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(ws, 0, L.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
     return run_forward(L, q, k, v, z, beta, nullptr, nullptr, 0, key_len, nullptr, nullptr, dtype, B, H, n, n, d, r, eps, iters, out,
                        g1_out, g2_out, ws, s) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
 }
@@ -602,7 +603,6 @@ int lot_attention_fwd_var(const void *q, const void *k, const void *v, const flo
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     remember_ws(ws, kPathGeneral, 0, 0);
-    if (cudaMemsetAsync(ws, 0, L.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
     // the class token is neither a query nor a key of the transport problem: it is skipped on both sides
     if (run_forward(L, q, k, v, z, beta, a, b, cls, key_len, g1_in, g2_in, dtype, B, H, nq, nk, d, r, eps, iters, out, g1_out, g2_out,
                     ws, s) != cudaSuccess)
@@ -721,18 +721,15 @@ int lot_attention_bwd(const void *q, const void *k, const void *v, const float *
     const BwdLayout L = bwd_layout(B, H, n, d, r, iters);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     remember_ws(ws, kPathGeneral, 0, 0);
-    const bool wide = dtype == LOT_F32;
-    const size_t lt = wide ? 8 : 4;
+    const size_t lt = 8;
     const int BH = B * H, np = 2 * BH;
-    const int ttype = dtype == LOT_F32 ? 0 : 1;        // tensor element type for the products
-    const int ltype = wide ? 2 : 0;                    // type of the similarity-sized buffers
     if (cudaMemsetAsync(ws, 0, L.head_end, s) != cudaSuccess) return LOT_ERR_CUDA;
 
     // ---- the forward, keeping the potentials of every iteration
     char *cost1 = at<char>(ws, L.cost);
     char *cost2 = cost1 + (size_t)BH * n * r * lt;
-    if (launch_cost(q, z, dtype, BH, H, n, d, r, cost1, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_cost(k, z, dtype, BH, H, n, d, r, cost2, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_cost(q, z, dtype, BH, H, n, d, r, cost1, true, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_cost(k, z, dtype, BH, H, n, d, r, cost2, true, s) != cudaSuccess) return LOT_ERR_CUDA;
     char *hist = at<char>(ws, L.hist);
     const size_t hstep = (size_t)np * r * lt;
     PassArgs a{};
@@ -741,7 +738,7 @@ int lot_attention_bwd(const void *q, const void *k, const void *v, const float *
     a.M = at<void>(ws, L.M); a.status = at<int>(ws, 0);
     a.nprob = np; a.B = B; a.H = H; a.n = n; a.r = r;
     a.chunks = L.chunks; a.rows_per_chunk = L.rows_per_chunk;
-    a.mode = wide ? kModeWide : kModeF32;
+    a.mode = kModeWide;
     a.scale_d = 1.4426950408889634 / (double)eps;
     a.eps_ln2 = (float)((double)eps * 0.6931471805599453);
     for (int it = 0; it < iters; ++it) {
@@ -761,21 +758,21 @@ int lot_attention_bwd(const void *q, const void *k, const void *v, const float *
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = Wp; ap.counter = at<unsigned>(ws, L.counter2);
     ap.B = B; ap.H = H; ap.n = n; ap.nk = n; ap.d = d; ap.r = r;
     ap.chunks = L.achunks; ap.rows_per_chunk = L.arows; ap.scale_d = a.scale_d;
-    if (launch_apply_w(ap, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;                 // W' = Diag(1/beta) Gamma2 V
+    if (launch_apply_w(ap, s) != cudaSuccess) return LOT_ERR_CUDA;                 // W' = Diag(1/beta) Gamma2 V
 
     // ---- reverse of the read-out, Eq. (4): out = R1 W'
     ApplyArgs aq = ap;                                  // R1^T dout / (n beta): the key-side kernel on the query side
     aq.cost2 = cost1; aq.G2 = G1; aq.M2 = M1; aq.key_len = nullptr; aq.v = dout; aq.Wp = Xw;
-    if (launch_apply_w(aq, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_apply_w(aq, s) != cudaSuccess) return LOT_ERR_CUDA;
     float *dbd = at<float>(ws, L.dbeta_direct);
     if (launch_bwd_w_fix(Xw, Wp, key_len, dWm, dbd, B, H, n, d, r, s) != cudaSuccess) return LOT_ERR_CUDA;
     ApplyArgs av = ap;                                  // dV = Gamma2 dW: the query-side kernel on the key side
     av.cost1 = cost2; av.G1 = G2; av.M1 = M2; av.Wp = dWm; av.out = dv;
-    if (launch_apply_out(av, dtype, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_apply_out(av, s) != cudaSuccess) return LOT_ERR_CUDA;
     char *dC1 = at<char>(ws, L.dC);
     char *dC2 = dC1 + (size_t)BH * n * r * lt;
-    if (launch_gemm_nt(dout, ttype, Wp, false, dC1, ltype, BH, H, n, d, r, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_gemm_nt(v, ttype, dWm, false, dC2, ltype, BH, H, n, d, r, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_gemm_nt(dout, false, Wp, false, dC1, true, BH, H, n, d, r, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_gemm_nt(v, false, dWm, false, dC2, true, BH, H, n, d, r, s) != cudaSuccess) return LOT_ERR_CUDA;
 
     // ---- reverse of the closing token update, then of the iterations, last first
     BwdRowArgs br{};
@@ -786,19 +783,18 @@ int lot_attention_bwd(const void *q, const void *k, const void *v, const float *
     br.chunks = L.chunks; br.rows_per_chunk = L.rows_per_chunk;
     br.scale_d = a.scale_d; br.eps = (double)eps;
     br.Ga = Gfin; br.Gb = nullptr;
-    if (launch_bwd_rows(br, true, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_bwd_rows(br, true, s) != cudaSuccess) return LOT_ERR_CUDA;
     for (int it = iters; it >= 1; --it) {
         br.Ga = hist + (size_t)(it - 1) * hstep; br.Gb = hist + (size_t)it * hstep;
-        if (launch_bwd_rows(br, false, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
+        if (launch_bwd_rows(br, false, s) != cudaSuccess) return LOT_ERR_CUDA;
     }
 
     // ---- C = X Z^T: dX = dC Z, dZ = dC^T X
     float *zt = at<float>(ws, L.zt);
     if (launch_transpose_z(z, zt, H, r, d, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_gemm_nt(dC1, ltype, zt, true, dq, ttype, BH, H, n, r, d, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_gemm_nt(dC2, ltype, zt, true, dk, ttype, BH, H, n, r, d, wide, s) != cudaSuccess) return LOT_ERR_CUDA;
-    if (launch_bwd_dz(dC1, q, k, dtype, at<void>(ws, L.dzpart), dbd, br.dbeta_acc, dz, dbeta, B, H, n, d, r, L.dzchunks, wide,
-                      s) != cudaSuccess)
+    if (launch_gemm_nt(dC1, true, zt, true, dq, false, BH, H, n, r, d, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_gemm_nt(dC2, true, zt, true, dk, false, BH, H, n, r, d, s) != cudaSuccess) return LOT_ERR_CUDA;
+    if (launch_bwd_dz(dC1, q, k, at<void>(ws, L.dzpart), dbd, br.dbeta_acc, dz, dbeta, B, H, n, d, r, L.dzchunks, s) != cudaSuccess)
         return LOT_ERR_CUDA;
     return LOT_OK;
 }

@@ -12,8 +12,9 @@
 //     dC_it -= m_i (q_it gamma_t - R_it rho_i),   d/dg_t = sum_i m_i R_it rho_i,   d/dbeta_t += eps gamma_t / beta_t
 // Reverse of the closing update and read-out, given dR (gradient with respect to R):
 //     dy_it = R_it (dR_it - sum_t' R_it' dR_it'),  dC_it = dy_it / eps,  d/dg_t = sum_i dy_it / eps.
-// All arithmetic is float for bf16 tensors and double for float32 tensors, like the forward general path; column
-// sums are per-block partials added in a fixed order by the last block to arrive.
+// This file is the backward of float32 tensors: all arithmetic in double, column sums as per-block partials added in a
+// fixed order by the last block to arrive.  bf16 tensors: lot_sweep_bwd.cu.
+#include "lot_chain.cuh"
 #include "lot_common.cuh"
 #include "lot_internal.h"
 
@@ -25,18 +26,6 @@ constexpr int kBwdWarps = 8;
 
 template <typename LT>
 __device__ __forceinline__ void load_row4(const LT *p, bool vec, int t, int r, LT (&c)[4]);
-
-template <>
-__device__ __forceinline__ void load_row4<float>(const float *p, bool vec, int t, int r, float (&c)[4])
-{
-    if (vec) {
-        const float4 v = *reinterpret_cast<const float4 *>(p);
-        c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) c[j] = t + j < r ? p[j] : 0.f;
-    }
-}
 
 template <>
 __device__ __forceinline__ void load_row4<double>(const double *p, bool vec, int t, int r, double (&c)[4])
@@ -262,14 +251,6 @@ cudaError_t launch_rows_r(const BwdRowArgs &a, bool close, cudaStream_t st)
 constexpr int kGT = 64, kGK = 16, kGPad = kGT + 4;
 
 template <typename AccT, typename T> __device__ __forceinline__ AccT ld_as(T v) { return (AccT)v; }
-template <typename AccT> __device__ __forceinline__ AccT ld_as(__nv_bfloat16 v) { return (AccT)__bfloat162float(v); }
-template <typename OutT> struct StoreAs {
-    template <typename AccT> static __device__ __forceinline__ OutT conv(AccT v) { return (OutT)v; }
-};
-template <> struct StoreAs<__nv_bfloat16> {
-    template <typename AccT> static __device__ __forceinline__ __nv_bfloat16 conv(AccT v) { return __float2bfloat16_rn((float)v); }
-};
-
 template <typename AT, typename AccT, typename OutT>
 __global__ void __launch_bounds__(256)
 gemm_nt_kernel(const AT *__restrict__ A, const float *__restrict__ Bm, OutT *__restrict__ out, int H, int per_head,
@@ -315,30 +296,16 @@ gemm_nt_kernel(const AT *__restrict__ A, const float *__restrict__ Bm, OutT *__r
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
             const int j = j0 + tx * 4 + y;
-            if (j < J && LOT_CHECK((size_t)i * J + j < (size_t)n * J)) ob[(size_t)i * J + j] = StoreAs<OutT>::conv(acc[x][y]);
+            if (j < J && LOT_CHECK((size_t)i * J + j < (size_t)n * J)) ob[(size_t)i * J + j] = (OutT)acc[x][y];
         }
     }
 }
 
-template <typename AT, typename AccT>
-cudaError_t launch_gemm_out(const void *A, const float *Bm, bool per_head, void *out, int out_type, int S, int H, int n,
-                            int K, int J, cudaStream_t st)
-{
-    dim3 grid((n + kGT - 1) / kGT, (J + kGT - 1) / kGT, S);
-    const AT *a = static_cast<const AT *>(A);
-    if (out_type == 0)
-        gemm_nt_kernel<AT, AccT, float><<<grid, 256, 0, st>>>(a, Bm, static_cast<float *>(out), H, per_head, n, K, J);
-    else if (out_type == 1)
-        gemm_nt_kernel<AT, AccT, __nv_bfloat16><<<grid, 256, 0, st>>>(a, Bm, static_cast<__nv_bfloat16 *>(out), H, per_head, n, K, J);
-    else
-        gemm_nt_kernel<AT, AccT, double><<<grid, 256, 0, st>>>(a, Bm, static_cast<double *>(out), H, per_head, n, K, J);
-    return cudaGetLastError();
-}
-
-__global__ void bwd_w_fix_kernel(const float *__restrict__ Xw, const float *__restrict__ Wp, const int32_t *key_len,
-                                 float *__restrict__ dWm, float *__restrict__ dbeta_direct, int H, int n, int d, int r)
+__global__ void bwd_w_fix_kernel(const float *Xw, const float *Wp, const int32_t *key_len, float *dWm, float *dbeta_direct, int H, int n, int d, int r)
 {
     // one warp per (slice, pivot)
+    chain_next();
+    chain_wait();
     const int s = blockIdx.x, b = s / H;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     int nvalid = n;
@@ -460,26 +427,27 @@ __global__ void bwd_dz_merge_kernel(const LT *__restrict__ part, const float *__
 
 } // namespace
 
-cudaError_t launch_bwd_rows(const BwdRowArgs &a, bool close, bool wide, cudaStream_t st)
+cudaError_t launch_bwd_rows(const BwdRowArgs &a, bool close, cudaStream_t st)
 {
-    return wide ? launch_rows_r<double>(a, close, st) : launch_rows_r<float>(a, close, st);
+    return launch_rows_r<double>(a, close, st);
 }
 
-cudaError_t launch_gemm_nt(const void *A, int a_type, const float *Bm, bool per_head, void *out, int out_type,
-                           int S, int H, int n, int K, int J, bool acc_double, cudaStream_t st)
+cudaError_t launch_gemm_nt(const void *A, bool a_double, const float *Bm, bool per_head, void *out, bool out_double, int S, int H,
+                           int n, int K, int J, cudaStream_t st)
 {
-    if (a_type == 0)
-        return acc_double ? launch_gemm_out<float, double>(A, Bm, per_head, out, out_type, S, H, n, K, J, st)
-                          : launch_gemm_out<float, float>(A, Bm, per_head, out, out_type, S, H, n, K, J, st);
-    if (a_type == 1) return launch_gemm_out<__nv_bfloat16, float>(A, Bm, per_head, out, out_type, S, H, n, K, J, st);
-    return launch_gemm_out<double, double>(A, Bm, per_head, out, out_type, S, H, n, K, J, st);
+    dim3 grid((n + kGT - 1) / kGT, (J + kGT - 1) / kGT, S);
+    if (!a_double && out_double)
+        gemm_nt_kernel<float, double, double><<<grid, 256, 0, st>>>(static_cast<const float *>(A), Bm, static_cast<double *>(out), H, per_head, n, K, J);
+    else if (a_double && !out_double)
+        gemm_nt_kernel<double, double, float><<<grid, 256, 0, st>>>(static_cast<const double *>(A), Bm, static_cast<float *>(out), H, per_head, n, K, J);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_bwd_w_fix(const float *Xw, const float *Wp, const int32_t *key_len, float *dWm, float *dbeta_direct,
                              int B, int H, int n, int d, int r, cudaStream_t st)
 {
-    bwd_w_fix_kernel<<<B * H, 256, 0, st>>>(Xw, Wp, key_len, dWm, dbeta_direct, H, n, d, r);
-    return cudaGetLastError();
+    return chain_launch(bwd_w_fix_kernel, dim3(B * H), 256, 0, st, Xw, Wp, key_len, dWm, dbeta_direct, H, n, d, r);
 }
 
 cudaError_t launch_transpose_z(const float *z, float *zt, int H, int r, int d, cudaStream_t st)
@@ -498,31 +466,21 @@ int bwd_dz_chunks(int BH, int n, int r, int d)
     return want < 1 ? 1 : want;
 }
 
-cudaError_t launch_bwd_dz(const void *dC, const void *q, const void *k, int dtype, void *part, const float *dbeta_direct,
-                          const void *dbeta_acc, float *dz, float *dbeta, int B, int H, int n, int d, int r, int chunks,
-                          bool wide, cudaStream_t st)
+cudaError_t launch_bwd_dz(const void *dC, const void *q, const void *k, void *part, const float *dbeta_direct, const void *dbeta_acc,
+                          float *dz, float *dbeta, int B, int H, int n, int d, int r, int chunks, cudaStream_t st)
 {
     const int BH = B * H;
     const int rows = (n + chunks - 1) / chunks;
     dim3 grid(chunks, ((r + kGT - 1) / kGT) * ((d + kGT - 1) / kGT), 2 * BH);
-    if (dtype == 0)
-        bwd_dz_part_kernel<float, double><<<grid, 256, 0, st>>>(static_cast<const double *>(dC), static_cast<const float *>(q),
-                                                               static_cast<const float *>(k), static_cast<double *>(part),
-                                                               BH, n, d, r, chunks, rows);
-    else
-        bwd_dz_part_kernel<__nv_bfloat16, float><<<grid, 256, 0, st>>>(
-            static_cast<const float *>(dC), static_cast<const __nv_bfloat16 *>(q), static_cast<const __nv_bfloat16 *>(k),
-            static_cast<float *>(part), BH, n, d, r, chunks, rows);
+    bwd_dz_part_kernel<float, double><<<grid, 256, 0, st>>>(static_cast<const double *>(dC), static_cast<const float *>(q),
+                                                           static_cast<const float *>(k), static_cast<double *>(part),
+                                                           BH, n, d, r, chunks, rows);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t work = (size_t)H * r * d;
-    const unsigned blocks = (unsigned)((work + 255) / 256);
-    if (wide)
-        bwd_dz_merge_kernel<double><<<blocks, 256, 0, st>>>(static_cast<const double *>(part), dbeta_direct,
-                                                           static_cast<const double *>(dbeta_acc), dz, dbeta, B, H, d, r, chunks);
-    else
-        bwd_dz_merge_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float *>(part), dbeta_direct,
-                                                          static_cast<const float *>(dbeta_acc), dz, dbeta, B, H, d, r, chunks);
+    bwd_dz_merge_kernel<double><<<(unsigned)((work + 255) / 256), 256, 0, st>>>(static_cast<const double *>(part), dbeta_direct,
+                                                                                static_cast<const double *>(dbeta_acc), dz, dbeta, B, H,
+                                                                                d, r, chunks);
     return cudaGetLastError();
 }
 

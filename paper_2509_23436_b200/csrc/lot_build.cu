@@ -1,5 +1,6 @@
 // The stabilised Gibbs kernel of the sweep path (lot_sweep.cu) from tokens and pivots: logits, row maxima, exponentials in
 // one kernel; every warp holds whole rows of logits in its accumulators.
+#include "lot_chain.cuh"
 #include "lot_internal.h"
 #include "lot_logits.cuh"
 #include "lot_sweep.h"
@@ -32,6 +33,9 @@ build_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k)
     const int b = slice / a.H, h = slice % a.H, n = a.n[side];
     int nv = n;
     if (side == 1 && a.key_len != nullptr) nv = min(max(__ldg(a.key_len + b), 0), n);
+    chain_next();
+    // what the later kernels of the call count and flag in starts at zero
+    for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < a.head_words; i += (size_t)gridDim.x * kThreads) a.head[i] = make_uint4(0, 0, 0, 0);
     const int row0 = tile * (kWarps * Sh::ROWS) + a.skip;
     if (row0 >= nv) return;                                        // rows without mass are never read
     if (threadIdx.x < RP) {

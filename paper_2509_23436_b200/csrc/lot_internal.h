@@ -10,11 +10,10 @@ namespace lot {
 // One Sinkhorn pass over a set of independent problems.  Problem p covers the slice
 // s = p % (B*H) (batch s / H, head s % H); problems p >= len_from take their valid length
 // from len[batch], the others use n.
-// Arithmetic modes: which types the similarity matrix is stored in and the logits, pivot
-// potentials G and row log-sum-exps M are assembled in.
-enum { kModeF32 = 0,          // cost float, logits float            (bf16 tensors)
-       kModeCostF32Wide = 1,  // cost float, logits/G/M double       (lot_sinkhorn)
-       kModeWide = 2 };       // cost double, logits/G/M double      (float32 tensors)
+// Arithmetic modes: which type the similarity matrix is stored in; logits, pivot potentials G and row log-sum-exps M are
+// assembled in double.
+enum { kModeCostF32Wide = 0,  // cost float    (lot_sinkhorn)
+       kModeWide = 1 };       // cost double   (backward of float32 tensors)
 
 struct PassArgs {
     const void *cost;    // [nprob][n][r] similarity matrices (float or double, see mode)
@@ -68,8 +67,9 @@ int apply_chunks(int BH, int n, int r, int d);
 cudaError_t launch_cost(const void *x, const float *z, int dtype, int BH, int H, int n, int d, int r,
                         void *cost, bool wide, cudaStream_t st);
 cudaError_t launch_sinkhorn_pass(const PassArgs &a, bool final_pass, cudaStream_t st);
-cudaError_t launch_apply_w(const ApplyArgs &a, int dtype, cudaStream_t st);
-cudaError_t launch_apply_out(const ApplyArgs &a, int dtype, cudaStream_t st);
+// float32 tensors, similarities in double
+cudaError_t launch_apply_w(const ApplyArgs &a, cudaStream_t st);
+cudaError_t launch_apply_out(const ApplyArgs &a, cudaStream_t st);
 // row 0 of every slice: softmax_j(tau <q_0, k_j>) over the valid keys, applied to v; scores: [BH][nk] scratch
 cudaError_t launch_cls_row(const void *q, const void *k, const void *v, const int32_t *key_len, int dtype, int B, int H,
                            int nq, int nk, int d, float tau, float *scores, void *out, cudaStream_t st);
@@ -96,11 +96,11 @@ struct BwdRowArgs {
     double scale_d;      // log2(e)/eps
     double eps;
 };
-cudaError_t launch_bwd_rows(const BwdRowArgs &a, bool close, bool wide, cudaStream_t st);
+cudaError_t launch_bwd_rows(const BwdRowArgs &a, bool close, cudaStream_t st);
 // out[s][i][j] = sum_k A[s][i][k] * Bm[(per_head ? s % H : s)][j][k]   (A: n x K, Bm: J x K, out: n x J)
-// a_type / out_type: 0 float, 1 bf16, 2 double; Bm is float
-cudaError_t launch_gemm_nt(const void *A, int a_type, const float *Bm, bool per_head, void *out, int out_type,
-                           int S, int H, int n, int K, int J, bool acc_double, cudaStream_t st);
+// float in, double out or double in, float out; sums in double; Bm is float
+cudaError_t launch_gemm_nt(const void *A, bool a_double, const float *Bm, bool per_head, void *out, bool out_double, int S, int H,
+                           int n, int K, int J, cudaStream_t st);
 // Xw = (apply_w output of the query side on dout) -> dWm = Xw * n / nvalid_b (zero without keys),
 // dbeta_direct[s][t] = -n * sum_c Xw[s][t][c] * Wp[s][t][c]
 cudaError_t launch_bwd_w_fix(const float *Xw, const float *Wp, const int32_t *key_len, float *dWm, float *dbeta_direct,
@@ -109,10 +109,9 @@ cudaError_t launch_bwd_w_fix(const float *Xw, const float *Wp, const int32_t *ke
 cudaError_t launch_transpose_z(const float *z, float *zt, int H, int r, int d, cudaStream_t st);
 int bwd_dz_chunks(int BH, int n, int r, int d);
 // dz[h][t][c] = sum over b, side, rows of dC[side][b,h][i][t] * x_side[b,h][i][c];  dbeta[h][t] = sum over b of
-// dbeta_direct + both sides' dbeta_acc.  part: [2*BH][chunks][r][d] floats or doubles per `wide`
-cudaError_t launch_bwd_dz(const void *dC, const void *q, const void *k, int dtype, void *part, const float *dbeta_direct,
-                          const void *dbeta_acc, float *dz, float *dbeta, int B, int H, int n, int d, int r, int chunks,
-                          bool wide, cudaStream_t st);
+// dbeta_direct + both sides' dbeta_acc.  part: [2*BH][chunks][r][d] doubles
+cudaError_t launch_bwd_dz(const void *dC, const void *q, const void *k, void *part, const float *dbeta_direct, const void *dbeta_acc,
+                          float *dz, float *dbeta, int B, int H, int n, int d, int r, int chunks, cudaStream_t st);
 
 // ---- fused tensor-core path (lot_fused.cu): bf16 tensors, d = 64, r <= 64 ----
 struct FusedLayout {

@@ -3,6 +3,7 @@
 // matrix, and the two apply stages of Eq. (4).  All arithmetic is float32 on the CUDA
 // cores; cross-block reductions are per-block partials summed in a fixed order by the
 // last block to arrive (no spinning, no floating-point atomics).
+#include "lot_chain.cuh"
 #include "lot_common.cuh"
 #include "lot_internal.h"
 
@@ -339,7 +340,6 @@ static cudaError_t launch_pass_r(const PassArgs &a, bool final_pass, cudaStream_
 cudaError_t launch_sinkhorn_pass(const PassArgs &a, bool final_pass, cudaStream_t st)
 {
     switch (a.mode) {
-    case kModeF32: return launch_pass_r<float, float>(a, final_pass, st);
     case kModeCostF32Wide: return launch_pass_r<float, double>(a, final_pass, st);
     default: return launch_pass_r<double, double>(a, final_pass, st);
     }
@@ -461,12 +461,10 @@ apply_w_kernel(ApplyArgs a)
     if (threadIdx.x == 0) a.counter[(size_t)bh * gridDim.y + blockIdx.y] = 0u;
 }
 
-cudaError_t launch_apply_w(const ApplyArgs &a, int dtype, cudaStream_t st)
+cudaError_t launch_apply_w(const ApplyArgs &a, cudaStream_t st)
 {
     int tblks = (a.r + kTile - 1) / kTile, cblks = (a.d + kTile - 1) / kTile;
-    dim3 grid(a.chunks, tblks * cblks, a.B * a.H);
-    if (dtype == 0) apply_w_kernel<float, double><<<grid, 256, 0, st>>>(a);
-    else apply_w_kernel<__nv_bfloat16, float><<<grid, 256, 0, st>>>(a);
+    apply_w_kernel<float, double><<<dim3(a.chunks, tblks * cblks, a.B * a.H), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -531,11 +529,9 @@ apply_out_kernel(ApplyArgs a)
     }
 }
 
-cudaError_t launch_apply_out(const ApplyArgs &a, int dtype, cudaStream_t st)
+cudaError_t launch_apply_out(const ApplyArgs &a, cudaStream_t st)
 {
-    dim3 grid((a.n + kTile - 1) / kTile, (a.d + kTile - 1) / kTile, a.B * a.H);
-    if (dtype == 0) apply_out_kernel<float, double><<<grid, 256, 0, st>>>(a);
-    else apply_out_kernel<__nv_bfloat16, float><<<grid, 256, 0, st>>>(a);
+    apply_out_kernel<float, double><<<dim3((a.n + kTile - 1) / kTile, (a.d + kTile - 1) / kTile, a.B * a.H), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -577,6 +573,7 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
     __shared__ float sc_s[kClsKeys];
     __shared__ __align__(16) float part[256 * 8];
     __shared__ float red[8];
+    chain_next();                                    // no wait: it reads and writes nothing of its predecessors
     const int bh = blockIdx.x, bb = bh / H, tid = threadIdx.x;
     int kv = nk;
     if (key_len != nullptr) kv = min(max(key_len[bb], 0), nk);
@@ -640,15 +637,11 @@ cudaError_t launch_cls_row(const void *q, const void *k, const void *v, const in
                            int nq, int nk, int d, float tau, float *scores, void *out, cudaStream_t st)
 {
     if (dtype == 0)
-        cls_row_kernel<float><<<B * H, 256, 0, st>>>(static_cast<const float *>(q), static_cast<const float *>(k),
-                                                     static_cast<const float *>(v), key_len, H, nq, nk, d, tau, scores,
-                                                     static_cast<float *>(out));
-    else
-        cls_row_kernel<__nv_bfloat16><<<B * H, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(q),
-                                                             static_cast<const __nv_bfloat16 *>(k),
-                                                             static_cast<const __nv_bfloat16 *>(v), key_len, H, nq, nk, d, tau,
-                                                             scores, static_cast<__nv_bfloat16 *>(out));
-    return cudaGetLastError();
+        return chain_launch(cls_row_kernel<float>, dim3(B * H), 256, 0, st, static_cast<const float *>(q), static_cast<const float *>(k),
+                            static_cast<const float *>(v), key_len, H, nq, nk, d, tau, scores, static_cast<float *>(out));
+    typedef __nv_bfloat16 bf;
+    return chain_launch(cls_row_kernel<bf>, dim3(B * H), 256, 0, st, static_cast<const bf *>(q), static_cast<const bf *>(k),
+                        static_cast<const bf *>(v), key_len, H, nq, nk, d, tau, scores, static_cast<bf *>(out));
 }
 
 LOT_DEBUG_FLAG_READER(kernels_debug_flag)

@@ -58,7 +58,7 @@ template <int CC, int THREADS> struct Logits<__nv_bfloat16, CC, 16, THREADS> {
 #pragma unroll
             for (int u = 0; u < NZ; ++u) {
                 const int idx = threadIdx.x + u * THREADS, t = idx / (KC / 2), k = k0 + (idx % (KC / 2)) * 2;
-                zz[u] = (t < zrows && k < d) ? __ldg(reinterpret_cast<const float2 *>(z + (size_t)t * d + k)) : make_float2(0.f, 0.f);
+                zz[u] = (t < zrows && k < d) ? *reinterpret_cast<const float2 *>(z + (size_t)t * d + k) : make_float2(0.f, 0.f);
             }
         };
         fetch(0);

@@ -12,6 +12,7 @@
 // spread of the potentials is exact.
 // What bounds a pass: shared-memory reads (4 bytes per entry at 128 bytes per clock and SM) and, for C > 1, one or two
 // round trips through L2 for the exchange, which other blocks on the SM (other groups) hide.
+#include "lot_chain.cuh"
 #include "lot_sweep_core.cuh"
 
 #include <mutex>
@@ -49,6 +50,8 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
     unsigned seq = a.seq0;
     const Shared S = carve<T, RP, THREADS>(smem, a.srows);
     if (tid == 0) { S.flag[0] = 0; S.flag[1] = 0; }
+    chain_next();
+    chain_wait();
 
     for (int p = group; p < NP; p += a.groups) {
         Share R;
@@ -117,8 +120,7 @@ static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t
     }
     const dim3 grid((unsigned)(P.groups * P.C));
     if (!GROUP) {
-        kern<<<grid, THREADS, P.smem, st>>>(a);
-        return cudaGetLastError();
+        return chain_launch(kern, grid, THREADS, P.smem, st, a);
     }
     SweepArgs copy = a;
     void *args[] = {&copy};

@@ -33,6 +33,8 @@ struct SweepArgs {
                              // the kernel as it is left, or nullptr
     double *hist_g;          // ... and the potentials themselves, of the problems whose kernel was rebuilt
     int *wide;               // ... [problems] 1: the kept weights leave float32's range, use hist_g
+    uint4 *head;             // words that launch_build clears: status, tickets, exchange words
+    size_t head_words;
     int *status;
     int B, H, d, r;
     int n[2];                // tokens per slice

@@ -6,6 +6,7 @@
 // in memory.  float32 tensors: CUDA cores (their products would need six terms a piece on the tensor cores).
 // All kernels load the next step's operands into registers while the current one multiplies; what bounds them is the
 // read of the kernel (4 bytes per entry) and, at rank 256, the product rate.
+#include "lot_chain.cuh"
 #include "lot_internal.h"
 #include "lot_logits.cuh"
 #include "lot_sweep.h"
@@ -88,8 +89,8 @@ apply_w_mma_kernel(SweepApplyArgs a)
             kr[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             sc[u] = 0.f;
             if (j < row1) {
-                kr[u] = __ldg(reinterpret_cast<const float4 *>(K + (size_t)j * RP + t));
-                sc[u] = (inv ? __ldg(inv + j) : 1.f) * (mass ? __ldg(mass + j) : 1.f);
+                kr[u] = *reinterpret_cast<const float4 *>(K + (size_t)j * RP + t);
+                sc[u] = (inv ? inv[j] : 1.f) * (mass ? __ldg(mass + j) : 1.f);
             }
         }
 #pragma unroll
@@ -99,10 +100,12 @@ apply_w_mma_kernel(SweepApplyArgs a)
         }
     };
     float acc[NTW][4] = {};
+    chain_next();
+    chain_wait();
     float4 wt[NP];
 #pragma unroll
     for (int u = 0; u < NP; ++u)
-        wt[u] = w ? __ldg(reinterpret_cast<const float4 *>(w + ((tid + u * kThreads) % (TP / 4)) * 4)) : make_float4(1.f, 1.f, 1.f, 1.f);
+        wt[u] = w ? *reinterpret_cast<const float4 *>(w + ((tid + u * kThreads) % (TP / 4)) * 4) : make_float4(1.f, 1.f, 1.f, 1.f);
     if (row0 < row1) fetch(row0);
     const int mi = lane >> 3;
     for (int j0 = row0; j0 < row1; j0 += KT) {
@@ -214,10 +217,12 @@ apply_out_mma_kernel(SweepApplyArgs a)
     const int nrow = a.out_len ? min(max(__ldg(a.out_len + bh / a.H), 0), n) : n;     // rows beyond it are zero
     const float *K = a.kt[0] + ((size_t)bh * n + i0) * RP, *w = a.w[0] ? a.w[0] + (size_t)bh * RP : nullptr;
     const float *W = a.Wp + (size_t)(a.per_head ? bh % a.H : bh) * r * d;
+    chain_next();
+    chain_wait();
     float s[2];
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh)
-        s[hh] = i0 + g + 8 * hh < nrow ? (a.inv[0] ? __ldg(a.inv[0] + (size_t)bh * n + i0 + g + 8 * hh) : 1.f) : 0.f;
+        s[hh] = i0 + g + 8 * hh < nrow ? (a.inv[0] ? a.inv[0][(size_t)bh * n + i0 + g + 8 * hh] : 1.f) : 0.f;
     float2 kr[TS / 16][4];
     float4 wr[NW];
     auto fetch = [&](int tb) {
@@ -226,12 +231,12 @@ apply_out_mma_kernel(SweepApplyArgs a)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int row = g + (e & 1) * 8, t = tb + k * 16 + (e >> 1) * 8 + 2 * q;
-                kr[k][e] = i0 + row < nrow ? __ldg(reinterpret_cast<const float2 *>(K + (size_t)row * RP + t)) : make_float2(0.f, 0.f);
+                kr[k][e] = i0 + row < nrow ? *reinterpret_cast<const float2 *>(K + (size_t)row * RP + t) : make_float2(0.f, 0.f);
             }
 #pragma unroll
         for (int u = 0; u < NW; ++u) {
             const int idx = tid + u * kThreads, t = tb + idx / (D / 4), c = (idx % (D / 4)) * 4;
-            wr[u] = t < r && c < d ? __ldg(reinterpret_cast<const float4 *>(W + (size_t)t * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wr[u] = t < r && c < d ? *reinterpret_cast<const float4 *>(W + (size_t)t * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
     float acc[D / 8][4] = {};
@@ -252,7 +257,7 @@ apply_out_mma_kernel(SweepApplyArgs a)
         for (int k = 0; k < TS / 16; ++k)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float2 ww = w ? __ldg(reinterpret_cast<const float2 *>(w + tb + k * 16 + (e >> 1) * 8 + 2 * q)) : make_float2(1.f, 1.f);
+                const float2 ww = w ? *reinterpret_cast<const float2 *>(w + tb + k * 16 + (e >> 1) * 8 + 2 * q) : make_float2(1.f, 1.f);
                 uint32_t o[3];
                 split3(kr[k][e].x * (ww.x * s[e & 1]), kr[k][e].y * (ww.y * s[e & 1]), o);
 #pragma unroll
@@ -316,7 +321,9 @@ apply_w_f32_kernel(SweepApplyArgs a)
     const int grp = tid / GT, ty = (tid % GT) / 16, tx = tid % 16;
     float4 kr[NP], vr[NV], wt;
     float sc[NP];
-    wt = __ldg(reinterpret_cast<const float4 *>(w + (tid % (TP / 4)) * 4));              // kThreads is a multiple of TP / 4
+    chain_next();
+    chain_wait();
+    wt = *reinterpret_cast<const float4 *>(w + (tid % (TP / 4)) * 4);              // kThreads is a multiple of TP / 4
     auto fetch = [&](int j0) {
 #pragma unroll
         for (int u = 0; u < NP; ++u) {
@@ -324,8 +331,8 @@ apply_w_f32_kernel(SweepApplyArgs a)
             kr[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             sc[u] = 0.f;
             if (idx < kStep * TP / 4 && j < row1) {
-                kr[u] = __ldg(reinterpret_cast<const float4 *>(K + (size_t)j * RP + (idx % (TP / 4)) * 4));
-                sc[u] = (inv ? __ldg(inv + j) : 1.f) * (mass ? __ldg(mass + j) : 1.f);
+                kr[u] = *reinterpret_cast<const float4 *>(K + (size_t)j * RP + (idx % (TP / 4)) * 4);
+                sc[u] = (inv ? inv[j] : 1.f) * (mass ? __ldg(mass + j) : 1.f);
             }
         }
 #pragma unroll
@@ -429,22 +436,24 @@ apply_out_f32_kernel(SweepApplyArgs a)
     const int tx = tid % 16, ty = tid / 16;
     float4 kr[NP], wt[NP], wr[NW];
     float sc[NP];
+    chain_next();
+    chain_wait();
 #pragma unroll
     for (int u = 0; u < NP; ++u) {
         const int i = i0 + (tid + u * kThreads) / (TS / 4);
-        sc[u] = i < n ? __ldg(inv + i) : 0.f;
+        sc[u] = i < n ? inv[i] : 0.f;
     }
     auto fetch = [&](int tb) {
 #pragma unroll
         for (int u = 0; u < NP; ++u) {
             const int idx = tid + u * kThreads, i = i0 + idx / (TS / 4), t = tb + (idx % (TS / 4)) * 4;
-            kr[u] = i < n ? __ldg(reinterpret_cast<const float4 *>(K + (size_t)i * RP + t)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            wt[u] = __ldg(reinterpret_cast<const float4 *>(w + t));
+            kr[u] = i < n ? *reinterpret_cast<const float4 *>(K + (size_t)i * RP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wt[u] = *reinterpret_cast<const float4 *>(w + t);
         }
 #pragma unroll
         for (int u = 0; u < NW; ++u) {
             const int idx = tid + u * kThreads, t = tb + idx / 16, c = c0 + (idx % 16) * 4;
-            wr[u] = idx < TS * 16 && t < r && c < d ? __ldg(reinterpret_cast<const float4 *>(W + (size_t)t * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wr[u] = idx < TS * 16 && t < r && c < d ? *reinterpret_cast<const float4 *>(W + (size_t)t * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
     float acc[4][4] = {};
@@ -487,7 +496,7 @@ apply_out_f32_kernel(SweepApplyArgs a)
 template <typename Kern>
 static cudaError_t big_smem(Kern kern, size_t bytes)
 {
-    return bytes > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
+    return bytes > 40 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
 }
 
 template <int TP, int D>
@@ -497,8 +506,7 @@ static cudaError_t launch_w(const SweepApplyArgs &a, cudaStream_t st)
     auto kern = apply_w_mma_kernel<TP, D>;
     cudaError_t e = big_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(a.chunks, (a.r + TP - 1) / TP, a.B * a.H), kThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    return chain_launch(kern, dim3(a.chunks, (a.r + TP - 1) / TP, a.B * a.H), kThreads, smem, st, a);
 }
 template <int TP>
 static cudaError_t launch_w_d(const SweepApplyArgs &a, cudaStream_t st)
@@ -512,8 +520,7 @@ static cudaError_t launch_out(const SweepApplyArgs &a, cudaStream_t st)
     auto kern = apply_out_mma_kernel<TS, D>;
     cudaError_t e = big_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3((a.nq + 127) / 128, a.B * a.H), kThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    return chain_launch(kern, dim3((a.nq + 127) / 128, a.B * a.H), kThreads, smem, st, a);
 }
 
 } // namespace sweep_apply
@@ -524,10 +531,7 @@ cudaError_t launch_sweep_apply_w(const SweepApplyArgs &a, int dtype, cudaStream_
     if (dtype != 0) return a.RP == 16 ? launch_w_d<16>(a, st) : a.RP == 32 ? launch_w_d<32>(a, st) : launch_w_d<64>(a, st);
     const int cb = (a.d + kCT - 1) / kCT, TP = a.RP < 64 ? a.RP : 64;
     dim3 grid(a.chunks, (a.r + TP - 1) / TP * cb, a.B * a.H);
-    if (TP == 16) apply_w_f32_kernel<16><<<grid, kThreads, 0, st>>>(a);
-    else if (TP == 32) apply_w_f32_kernel<32><<<grid, kThreads, 0, st>>>(a);
-    else apply_w_f32_kernel<64><<<grid, kThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return chain_launch(TP == 16 ? apply_w_f32_kernel<16> : TP == 32 ? apply_w_f32_kernel<32> : apply_w_f32_kernel<64>, grid, kThreads, 0, st, a);
 }
 
 cudaError_t launch_sweep_apply_out(const SweepApplyArgs &a, int dtype, cudaStream_t st)
@@ -538,9 +542,7 @@ cudaError_t launch_sweep_apply_out(const SweepApplyArgs &a, int dtype, cudaStrea
         return a.d <= 64 ? launch_out<32, 64>(a, st) : a.d <= 128 ? launch_out<16, 128>(a, st) : launch_out<16, 256>(a, st);
     }
     dim3 grid((a.nq + 63) / 64, (a.d + kCT - 1) / kCT, a.B * a.H);
-    if (a.RP == 16) apply_out_f32_kernel<16><<<grid, kThreads, 0, st>>>(a);
-    else apply_out_f32_kernel<32><<<grid, kThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return chain_launch(a.RP == 16 ? apply_out_f32_kernel<16> : apply_out_f32_kernel<32>, grid, kThreads, 0, st, a);
 }
 
 } // namespace lot

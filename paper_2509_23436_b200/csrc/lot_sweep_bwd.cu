@@ -8,6 +8,7 @@
 // per row and two per column, and the gradient with respect to the similarities is put together once at the end
 // (assemble_kernel) instead of being read and written in every iteration.
 // Problems whose potentials ranged over more than the kernel's window are reversed step by step on rebuilt exponents.
+#include "lot_chain.cuh"
 #include "lot_sweep_core.cuh"
 
 #include <mutex>
@@ -34,6 +35,8 @@ close_kernel(const __grid_constant__ SweepBwdArgs a)
     if (side == 1 && s.key_len != nullptr) nv = min(max(__ldg(s.key_len + slice / s.H), 0), n);
     const int w0 = tile * 128 + warp * 16, wrows = min(max(nv - w0, 0), 16);
     float *gp = a.gpart + ((size_t)p * a.tiles + tile) * RP;
+    chain_next();
+    chain_wait();
     if (tile * 128 >= nv) {
         if (threadIdx.x < RP) gp[threadIdx.x] = 0.f;
         return;
@@ -49,12 +52,12 @@ close_kernel(const __grid_constant__ SweepBwdArgs a)
     for (int hh = 0; hh < 2; ++hh) {
         const int i = g + 8 * hh;
         const bool ok = i < wrows;
-        const float iv = ok ? __ldg(inv + i) : 0.f;
+        const float iv = ok ? inv[i] : 0.f;
         float rho = 0.f;
 #pragma unroll
         for (int j = 0; j < RP / 8; ++j) {
             const int t = 8 * j + 2 * q;
-            const float2 k = ok ? __ldg(reinterpret_cast<const float2 *>(kt + (size_t)i * RP + t)) : make_float2(0.f, 0.f);
+            const float2 k = ok ? *reinterpret_cast<const float2 *>(kt + (size_t)i * RP + t) : make_float2(0.f, 0.f);
             rho = fmaf(k.x * (sw[t] * iv), lg.at(j, hh, 0), rho);
             rho = fmaf(k.y * (sw[t + 1] * iv), lg.at(j, hh, 1), rho);
         }
@@ -63,7 +66,7 @@ close_kernel(const __grid_constant__ SweepBwdArgs a)
 #pragma unroll
         for (int j = 0; j < RP / 8; ++j) {
             const int t = 8 * j + 2 * q;
-            const float2 k = ok ? __ldg(reinterpret_cast<const float2 *>(kt + (size_t)i * RP + t)) : make_float2(0.f, 0.f);
+            const float2 k = ok ? *reinterpret_cast<const float2 *>(kt + (size_t)i * RP + t) : make_float2(0.f, 0.f);
             float2 v;
             v.x = k.x * (sw[t] * iv) * (lg.at(j, hh, 0) - rho) * inv_eps;
             v.y = k.y * (sw[t + 1] * iv) * (lg.at(j, hh, 1) - rho) * inv_eps;
@@ -234,6 +237,8 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
     unsigned seq = s.seq0;
     const Shared S = carve<__nv_bfloat16, RP, THREADS>(smem, s.srows);
     if (tid == 0) S.flag[0] = 0;
+    chain_next();
+    chain_wait();
 
     for (int p = group; p < NP; p += s.groups) {
         Share R;
@@ -244,7 +249,7 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
         }
         float gam = 0.f;
         if (tid < RP)
-            for (int k = 0; k < a.tiles; ++k) gam += __ldg(a.gpart + ((size_t)p * a.tiles + k) * RP + tid);
+            for (int k = 0; k < a.tiles; ++k) gam += a.gpart[((size_t)p * a.tiles + k) * RP + tid];
         const bool wide = s.wide[p] != 0;
         __syncthreads();
         if (wide) {
@@ -305,6 +310,8 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
     int nv = n;
     if (side == 1 && s.key_len != nullptr) nv = min(max(__ldg(s.key_len + slice / s.H), 0), n);
     const int i0 = blockIdx.x * ROWS, t0 = blockIdx.y * CT, tid = threadIdx.x;
+    chain_next();
+    chain_wait();
     if (i0 >= nv || s.wide[p] != 0) return;
     const int tx = tid % TC, ty = tid / TC;
     const float2 *coef = a.coef + (size_t)p * a.T * n + i0;
@@ -313,13 +320,13 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
         __syncthreads();
         for (int idx = tid; idx < KS * ROWS; idx += 256) {
             const int k = idx / ROWS, i = idx % ROWS;
-            sc[k][i] = k0 + k < a.T && i0 + i < nv ? __ldg(coef + (size_t)(k0 + k) * n + i) : make_float2(0.f, 0.f);
+            sc[k][i] = k0 + k < a.T && i0 + i < nv ? coef[(size_t)(k0 + k) * n + i] : make_float2(0.f, 0.f);
         }
         for (int idx = tid; idx < KS * CT; idx += 256) {
             const int k = idx / CT, t = idx % CT;
             const size_t o = ((size_t)(k0 + k) * NP + p) * RP + t0 + t;
-            sw[k][t] = k0 + k < a.T ? __ldg(s.hist + o) : 0.f;
-            sf[k][t] = k0 + k < a.T ? __ldg(a.fk + o) : 0.f;
+            sw[k][t] = k0 + k < a.T ? s.hist[o] : 0.f;
+            sf[k][t] = k0 + k < a.T ? a.fk[o] : 0.f;
         }
         __syncthreads();
 #pragma unroll
@@ -339,20 +346,21 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
         const int i = i0 + ty + x * (256 / TC);
         if (i >= nv) continue;
         const size_t o = ((size_t)slice * n + i) * RP + t0 + tx * 4;
-        const float4 k = __ldg(reinterpret_cast<const float4 *>(s.kt[side] + o));
+        const float4 k = *reinterpret_cast<const float4 *>(s.kt[side] + o);
         float4 v = *reinterpret_cast<const float4 *>(a.dC[side] + o);
         v.x = fmaf(k.x, acc[x][0], v.x); v.y = fmaf(k.y, acc[x][1], v.y); v.z = fmaf(k.z, acc[x][2], v.z); v.w = fmaf(k.w, acc[x][3], v.w);
         *reinterpret_cast<float4 *>(a.dC[side] + o) = v;
     }
 }
 
-__global__ void merge_kernel(const float *__restrict__ part_q, const float *__restrict__ part_k, const float *__restrict__ dbeta_direct,
-                             const float *__restrict__ dbeta_acc, float *__restrict__ dz, float *__restrict__ dbeta, int B, int H, int d,
+__global__ void merge_kernel(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz, float *dbeta, int B, int H, int d,
                              int r, int RP, int chunks)
 {
     // four threads an element, each a share of the batch rows, added in order
     const size_t per = (size_t)r * d, idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) / 4;
     const int quarter = threadIdx.x & 3, b0 = B * quarter / 4, b1 = B * (quarter + 1) / 4;
+    chain_next();
+    chain_wait();
     float sum = 0.f;
     const bool in = idx < (size_t)H * per;
     if (in) {
@@ -361,7 +369,7 @@ __global__ void merge_kernel(const float *__restrict__ part_q, const float *__re
         for (int b = b0; b < b1; ++b) {
             const size_t o = ((size_t)b * H + h) * chunks * per + e;
 #pragma unroll 4
-            for (int c = 0; c < chunks; ++c) sum += __ldg(part_q + o + c * per) + __ldg(part_k + o + c * per);
+            for (int c = 0; c < chunks; ++c) sum += part_q[o + c * per] + part_k[o + c * per];
         }
     }
     const float s1 = __shfl_down_sync(0xffffffffu, sum, 1), s2 = __shfl_down_sync(0xffffffffu, sum, 2), s3 = __shfl_down_sync(0xffffffffu, sum, 3);
@@ -380,7 +388,7 @@ __global__ void merge_kernel(const float *__restrict__ part_q, const float *__re
 // ---------------------------------------------------------------------------------------------------------------
 template <typename Kern> static cudaError_t allow_smem(Kern kern, size_t bytes)
 {
-    return bytes > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
+    return bytes > 40 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
 }
 
 template <int RP> static cudaError_t close_t(const SweepBwdArgs &a, cudaStream_t st)
@@ -388,14 +396,12 @@ template <int RP> static cudaError_t close_t(const SweepBwdArgs &a, cudaStream_t
     constexpr size_t smem = logits::stage_bytes<__nv_bfloat16>(RP);
     cudaError_t e = allow_smem(close_kernel<RP>, smem);
     if (e != cudaSuccess) return e;
-    close_kernel<RP><<<(unsigned)(2 * a.s.B * a.s.H * a.tiles), 256, smem, st>>>(a);
-    return cudaGetLastError();
+    return chain_launch(close_kernel<RP>, dim3((unsigned)(2 * a.s.B * a.s.H * a.tiles)), 256, smem, st, a);
 }
 template <int RP> static cudaError_t assemble_t(const SweepBwdArgs &a, cudaStream_t st)
 {
     constexpr int CT = RP < 64 ? RP : 64, ROWS = 256 / (CT / 4) * 4;
-    assemble_kernel<RP><<<dim3((a.s.n[0] + ROWS - 1) / ROWS, RP / CT, 2 * a.s.B * a.s.H), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return chain_launch(assemble_kernel<RP>, dim3((a.s.n[0] + ROWS - 1) / ROWS, RP / CT, 2 * a.s.B * a.s.H), 256, 0, st, a);
 }
 template <int RP, bool GROUP> static cudaError_t reverse_g(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st)
 {
@@ -404,8 +410,7 @@ template <int RP, bool GROUP> static cudaError_t reverse_g(const SweepPlan &P, c
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(P.groups * P.C));
     if (!GROUP) {
-        kern<<<grid, 256, P.smem, st>>>(a);
-        return cudaGetLastError();
+        return chain_launch(kern, grid, 256, P.smem, st, a);
     }
     SweepBwdArgs copy = a;
     void *args[] = {&copy};
@@ -446,8 +451,8 @@ cudaError_t launch_bwd_merge(const float *part_q, const float *part_k, const flo
                              float *dbeta, int B, int H, int d, int r, int RP, int chunks, cudaStream_t st)
 {
     const size_t threads = (size_t)H * r * d * 4;
-    sweep::merge_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(part_q, part_k, dbeta_direct, dbeta_acc, dz, dbeta, B, H, d, r, RP, chunks);
-    return cudaGetLastError();
+    return chain_launch(sweep::merge_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, st, part_q, part_k, dbeta_direct, dbeta_acc, dz, dbeta,
+                        B, H, d, r, RP, chunks);
 }
 
 } // namespace lot
