@@ -304,7 +304,6 @@ gemm_nt_kernel(const AT *__restrict__ A, const float *__restrict__ Bm, OutT *__r
 __global__ void bwd_w_fix_kernel(const float *Xw, const float *Wp, const int32_t *key_len, float *dWm, float *dbeta_direct, int H, int n, int d, int r)
 {
     // one warp per (slice, pivot)
-    chain_next();
     chain_wait();
     const int s = blockIdx.x, b = s / H;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;

@@ -33,7 +33,6 @@ build_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k)
     const int b = slice / a.H, h = slice % a.H, n = a.n[side];
     int nv = n;
     if (side == 1 && a.key_len != nullptr) nv = min(max(__ldg(a.key_len + b), 0), n);
-    chain_next();
     // what the later kernels of the call count and flag in starts at zero
     for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < a.head_words; i += (size_t)gridDim.x * kThreads) a.head[i] = make_uint4(0, 0, 0, 0);
     const int row0 = tile * (kWarps * Sh::ROWS) + a.skip;
@@ -46,6 +45,7 @@ build_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k)
     const int w0 = row0 + warp * Sh::ROWS, wrows = min(max(nv - w0, 0), Sh::ROWS);
     Lg lg;
     lg.run(static_cast<const T *>(a.x[side]) + ((size_t)slice * n + w0) * a.d, wrows, a.d, a.z + (size_t)h * r * a.d, r, stage, lane);
+    chain_next();
     float *kt = a.kt[side] + ((size_t)slice * n + w0) * RP;
 #pragma unroll
     for (int hh = 0; hh < Sh::ROWS / 8; ++hh) {

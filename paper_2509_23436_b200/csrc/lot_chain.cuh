@@ -1,6 +1,7 @@
 // Launches of a chain of kernels on one stream that overlap their starts: a kernel launched with chain_launch may begin
-// once every block of its predecessor has begun, and calls chain_wait before it touches anything the predecessors
-// write or read; every kernel of a chain calls chain_next first.  Hides most of the 2-3 us between dependent launches.
+// once every block of its predecessor has called chain_next or ended, and calls chain_wait before it touches anything
+// the predecessors write or read.  chain_next stands where a block's main work is done: called first thing, the waiting
+// blocks of the next kernel took a fifth of the sweep kernel's speed.  Hides most of the 2-3 us between dependent launches.
 // Loads of what a predecessor wrote must be plain ones: the compiler moves __ldg and loads through const __restrict__
 // pointers above the wait.
 // (Kernels whose blocks wait for one another are launched cooperatively instead and start the ordinary way.)
@@ -12,6 +13,26 @@ namespace lot {
 
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Loads that stay below the wait (and coherent ones: the read-only path may hold lines from before it).
+__device__ __forceinline__ float4 chain_ld4(const float *p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 chain_ld2(const float *p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float chain_ld(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 
 template <typename... P, typename... A>
 inline cudaError_t chain_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args)

@@ -573,7 +573,7 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
     __shared__ float sc_s[kClsKeys];
     __shared__ __align__(16) float part[256 * 8];
     __shared__ float red[8];
-    chain_next();                                    // no wait: it reads and writes nothing of its predecessors
+    // no chain_wait: it reads and writes nothing of its predecessors
     const int bh = blockIdx.x, bb = bh / H, tid = threadIdx.x;
     int kv = nk;
     if (key_len != nullptr) kv = min(max(key_len[bb], 0), nk);

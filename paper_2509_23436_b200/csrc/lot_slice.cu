@@ -224,7 +224,7 @@ slice_forward_kernel(const __grid_constant__ SliceParams P)
                 if (bad) break;
             }
         }
-        if (bad) recover<__nv_bfloat16, RP, CPL, kThreads, false>(&a, S, p, 0, 0, it, seq, wold, wnew);
+        if (bad) recover<__nv_bfloat16, RP, CPL, kThreads, false, Mem<RP>::work, Mem<RP>::ref>(&a, p, 0, 0, it, seq, wold, wnew);
         close_rows<RP, CPL>(S, R);
     } else {
         // no keys: nothing to transport; the output is zero (flagged), the key-side potentials stay at zero

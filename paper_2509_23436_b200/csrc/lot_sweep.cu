@@ -20,9 +20,16 @@
 namespace lot {
 namespace sweep {
 
-template <int RP, int CPL, int THREADS>
-__device__ __forceinline__ void finish(const SweepArgs &a, const Shared &S, const Share &R, const Problem &P, int c)
+// Closing update and results of problem p.  Out of line, and everything worked out again: nothing of the problem is live
+// across recover() and this call, which would cost the iteration loop its registers (spills in it: a fifth slower).
+template <typename T, int RP, int CPL, int THREADS>
+__device__ __noinline__ void finish(const SweepArgs *ap, int p, int c)
 {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const SweepArgs &a = *ap;
+    const Shared S = carve<T, RP, THREADS>(smem, a.srows);
+    Share R;
+    const Problem P = locate<RP, CPL, THREADS>(a, p, c, R);
     const int tid = threadIdx.x;
     if (a.close && P.nv > 0) {
         const Lane<RP, CPL> L = make_lane<RP, CPL>(S);
@@ -50,7 +57,6 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
     unsigned seq = a.seq0;
     const Shared S = carve<T, RP, THREADS>(smem, a.srows);
     if (tid == 0) { S.flag[0] = 0; S.flag[1] = 0; }
-    chain_next();
     chain_wait();
 
     for (int p = group; p < NP; p += a.groups) {
@@ -82,18 +88,22 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
             const float tgt = S.tgt[tid < RP ? tid : 0];
             u64 w[CPL / 2];
             load_weights<RP, CPL>(L, w);
+            // backward: the weights of every iteration are kept (thread t's column; nullptr: not kept here)
+            float *hp = a.hist != nullptr && c == 0 && tid < RP ? a.hist + (size_t)p * RP + tid : nullptr;
+            if (hp != nullptr) *hp = S.w[tid];
             for (; it < a.it1; ++it) {
-                if (a.hist != nullptr && c == 0 && tid < RP) a.hist[((size_t)it * NP + p) * RP + tid] = tid < r ? wnew : 0.f;
                 bad = iterate<RP, CPL, THREADS, GROUP>(a, S, R, L, w, tgt, group, c, seq, wold, wnew);
                 if (bad) break;
+                if (hp != nullptr) {
+                    hp += (size_t)NP * RP;
+                    *hp = tid < r ? wnew : 0.f;
+                }
             }
-            if (!bad && a.hist != nullptr && c == 0) {
-                if (tid < RP) a.hist[((size_t)it * NP + p) * RP + tid] = tid < r ? wnew : 0.f;
-                if (tid == 0) a.wide[p] = 0;
-            }
+            if (!bad && a.wide != nullptr && c == 0 && tid == 0) a.wide[p] = 0;
         }
-        if (bad) seq = recover<T, RP, CPL, THREADS, GROUP>(&a, S, p, group, c, it, seq, wold, wnew);
-        finish<RP, CPL, THREADS>(a, S, R, P, c);
+        if (bad) seq = recover<T, RP, CPL, THREADS, GROUP>(&a, p, group, c, it, seq, wold, wnew);
+        if (p + a.groups >= NP) chain_next();
+        finish<T, RP, CPL, THREADS>(&a, p, c);
     }
 }
 

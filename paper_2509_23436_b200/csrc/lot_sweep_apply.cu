@@ -89,8 +89,8 @@ apply_w_mma_kernel(SweepApplyArgs a)
             kr[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             sc[u] = 0.f;
             if (j < row1) {
-                kr[u] = *reinterpret_cast<const float4 *>(K + (size_t)j * RP + t);
-                sc[u] = (inv ? inv[j] : 1.f) * (mass ? __ldg(mass + j) : 1.f);
+                kr[u] = chain_ld4(K + (size_t)j * RP + t);
+                sc[u] = (inv ? chain_ld(inv + j) : 1.f) * (mass ? __ldg(mass + j) : 1.f);
             }
         }
 #pragma unroll
@@ -100,12 +100,11 @@ apply_w_mma_kernel(SweepApplyArgs a)
         }
     };
     float acc[NTW][4] = {};
-    chain_next();
     chain_wait();
     float4 wt[NP];
 #pragma unroll
     for (int u = 0; u < NP; ++u)
-        wt[u] = w ? *reinterpret_cast<const float4 *>(w + ((tid + u * kThreads) % (TP / 4)) * 4) : make_float4(1.f, 1.f, 1.f, 1.f);
+        wt[u] = w ? chain_ld4(w + ((tid + u * kThreads) % (TP / 4)) * 4) : make_float4(1.f, 1.f, 1.f, 1.f);
     if (row0 < row1) fetch(row0);
     const int mi = lane >> 3;
     for (int j0 = row0; j0 < row1; j0 += KT) {
@@ -146,6 +145,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
             }
         }
     }
+    chain_next();
     // halves of the keys, then the chunks
     const int g = lane >> 2, q = lane & 3;
     float *red = reinterpret_cast<float *>(sm);
@@ -217,12 +217,11 @@ apply_out_mma_kernel(SweepApplyArgs a)
     const int nrow = a.out_len ? min(max(__ldg(a.out_len + bh / a.H), 0), n) : n;     // rows beyond it are zero
     const float *K = a.kt[0] + ((size_t)bh * n + i0) * RP, *w = a.w[0] ? a.w[0] + (size_t)bh * RP : nullptr;
     const float *W = a.Wp + (size_t)(a.per_head ? bh % a.H : bh) * r * d;
-    chain_next();
     chain_wait();
     float s[2];
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh)
-        s[hh] = i0 + g + 8 * hh < nrow ? (a.inv[0] ? a.inv[0][(size_t)bh * n + i0 + g + 8 * hh] : 1.f) : 0.f;
+        s[hh] = i0 + g + 8 * hh < nrow ? (a.inv[0] ? chain_ld(a.inv[0] + (size_t)bh * n + i0 + g + 8 * hh) : 1.f) : 0.f;
     float2 kr[TS / 16][4];
     float4 wr[NW];
     auto fetch = [&](int tb) {
@@ -231,12 +230,12 @@ apply_out_mma_kernel(SweepApplyArgs a)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int row = g + (e & 1) * 8, t = tb + k * 16 + (e >> 1) * 8 + 2 * q;
-                kr[k][e] = i0 + row < nrow ? *reinterpret_cast<const float2 *>(K + (size_t)row * RP + t) : make_float2(0.f, 0.f);
+                kr[k][e] = i0 + row < nrow ? chain_ld2(K + (size_t)row * RP + t) : make_float2(0.f, 0.f);
             }
 #pragma unroll
         for (int u = 0; u < NW; ++u) {
             const int idx = tid + u * kThreads, t = tb + idx / (D / 4), c = (idx % (D / 4)) * 4;
-            wr[u] = t < r && c < d ? *reinterpret_cast<const float4 *>(W + (size_t)t * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wr[u] = t < r && c < d ? chain_ld4(W + (size_t)t * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
     float acc[D / 8][4] = {};
@@ -257,7 +256,7 @@ apply_out_mma_kernel(SweepApplyArgs a)
         for (int k = 0; k < TS / 16; ++k)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float2 ww = w ? *reinterpret_cast<const float2 *>(w + tb + k * 16 + (e >> 1) * 8 + 2 * q) : make_float2(1.f, 1.f);
+                const float2 ww = w ? chain_ld2(w + tb + k * 16 + (e >> 1) * 8 + 2 * q) : make_float2(1.f, 1.f);
                 uint32_t o[3];
                 split3(kr[k][e].x * (ww.x * s[e & 1]), kr[k][e].y * (ww.y * s[e & 1]), o);
 #pragma unroll
@@ -282,6 +281,7 @@ apply_out_mma_kernel(SweepApplyArgs a)
                     }
             }
     }
+    chain_next();
     __nv_bfloat16 *O = static_cast<__nv_bfloat16 *>(a.out) + ((size_t)bh * n + i0) * d;
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
@@ -321,9 +321,8 @@ apply_w_f32_kernel(SweepApplyArgs a)
     const int grp = tid / GT, ty = (tid % GT) / 16, tx = tid % 16;
     float4 kr[NP], vr[NV], wt;
     float sc[NP];
-    chain_next();
     chain_wait();
-    wt = *reinterpret_cast<const float4 *>(w + (tid % (TP / 4)) * 4);              // kThreads is a multiple of TP / 4
+    wt = chain_ld4(w + (tid % (TP / 4)) * 4);              // kThreads is a multiple of TP / 4
     auto fetch = [&](int j0) {
 #pragma unroll
         for (int u = 0; u < NP; ++u) {
@@ -331,8 +330,8 @@ apply_w_f32_kernel(SweepApplyArgs a)
             kr[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             sc[u] = 0.f;
             if (idx < kStep * TP / 4 && j < row1) {
-                kr[u] = *reinterpret_cast<const float4 *>(K + (size_t)j * RP + (idx % (TP / 4)) * 4);
-                sc[u] = (inv ? inv[j] : 1.f) * (mass ? __ldg(mass + j) : 1.f);
+                kr[u] = chain_ld4(K + (size_t)j * RP + (idx % (TP / 4)) * 4);
+                sc[u] = (inv ? chain_ld(inv + j) : 1.f) * (mass ? __ldg(mass + j) : 1.f);
             }
         }
 #pragma unroll
@@ -368,6 +367,7 @@ apply_w_f32_kernel(SweepApplyArgs a)
                 for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(pr[x], vv[y], acc[x][y]);
         }
     }
+    chain_next();
     if (G > 1) {
         for (int k = 1; k < G; ++k) {                              // key groups in order
             __syncthreads();
@@ -436,24 +436,23 @@ apply_out_f32_kernel(SweepApplyArgs a)
     const int tx = tid % 16, ty = tid / 16;
     float4 kr[NP], wt[NP], wr[NW];
     float sc[NP];
-    chain_next();
     chain_wait();
 #pragma unroll
     for (int u = 0; u < NP; ++u) {
         const int i = i0 + (tid + u * kThreads) / (TS / 4);
-        sc[u] = i < n ? inv[i] : 0.f;
+        sc[u] = i < n ? chain_ld(inv + i) : 0.f;
     }
     auto fetch = [&](int tb) {
 #pragma unroll
         for (int u = 0; u < NP; ++u) {
             const int idx = tid + u * kThreads, i = i0 + idx / (TS / 4), t = tb + (idx % (TS / 4)) * 4;
-            kr[u] = i < n ? *reinterpret_cast<const float4 *>(K + (size_t)i * RP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
-            wt[u] = *reinterpret_cast<const float4 *>(w + t);
+            kr[u] = i < n ? chain_ld4(K + (size_t)i * RP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wt[u] = chain_ld4(w + t);
         }
 #pragma unroll
         for (int u = 0; u < NW; ++u) {
             const int idx = tid + u * kThreads, t = tb + idx / 16, c = c0 + (idx % 16) * 4;
-            wr[u] = idx < TS * 16 && t < r && c < d ? *reinterpret_cast<const float4 *>(W + (size_t)t * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wr[u] = idx < TS * 16 && t < r && c < d ? chain_ld4(W + (size_t)t * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
     float acc[4][4] = {};
@@ -485,6 +484,7 @@ apply_out_f32_kernel(SweepApplyArgs a)
             }
         }
     }
+    chain_next();
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
         const int i = i0 + ty + 16 * x, c = c0 + tx * 4;

@@ -35,7 +35,6 @@ close_kernel(const __grid_constant__ SweepBwdArgs a)
     if (side == 1 && s.key_len != nullptr) nv = min(max(__ldg(s.key_len + slice / s.H), 0), n);
     const int w0 = tile * 128 + warp * 16, wrows = min(max(nv - w0, 0), 16);
     float *gp = a.gpart + ((size_t)p * a.tiles + tile) * RP;
-    chain_next();
     chain_wait();
     if (tile * 128 >= nv) {
         if (threadIdx.x < RP) gp[threadIdx.x] = 0.f;
@@ -75,6 +74,7 @@ close_kernel(const __grid_constant__ SweepBwdArgs a)
             lg.at(j, hh, 1) = ok ? v.y : 0.f;
         }
     }
+    chain_next();
 #pragma unroll
     for (int j = 0; j < RP / 8; ++j)
 #pragma unroll
@@ -237,7 +237,6 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
     unsigned seq = s.seq0;
     const Shared S = carve<__nv_bfloat16, RP, THREADS>(smem, s.srows);
     if (tid == 0) S.flag[0] = 0;
-    chain_next();
     chain_wait();
 
     for (int p = group; p < NP; p += s.groups) {
@@ -289,6 +288,7 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
             wb = wa;
             wa = wnext;
         }
+        if (p + s.groups >= NP) chain_next();
         if (c == 0 && tid < r) a.dbeta_acc[(size_t)p * RP + tid] = db;
         __syncthreads();
     }
@@ -310,7 +310,6 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
     int nv = n;
     if (side == 1 && s.key_len != nullptr) nv = min(max(__ldg(s.key_len + slice / s.H), 0), n);
     const int i0 = blockIdx.x * ROWS, t0 = blockIdx.y * CT, tid = threadIdx.x;
-    chain_next();
     chain_wait();
     if (i0 >= nv || s.wide[p] != 0) return;
     const int tx = tid % TC, ty = tid / TC;
@@ -341,6 +340,7 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
             }
         }
     }
+    chain_next();
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
         const int i = i0 + ty + x * (256 / TC);
@@ -359,7 +359,6 @@ __global__ void merge_kernel(const float *part_q, const float *part_k, const flo
     // four threads an element, each a share of the batch rows, added in order
     const size_t per = (size_t)r * d, idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) / 4;
     const int quarter = threadIdx.x & 3, b0 = B * quarter / 4, b1 = B * (quarter + 1) / 4;
-    chain_next();
     chain_wait();
     float sum = 0.f;
     const bool in = idx < (size_t)H * per;

@@ -633,10 +633,12 @@ __device__ __forceinline__ bool iterate(const SweepArgs &a, const Shared &S, con
 // The rest of a problem's iterations from `it` on, whose update left the kernel's range (wold, wnew: thread t < r's weight
 // before and after it): the kernel is rebuilt around the new potentials, after the update has been redone in the log
 // domain where a column sum was lost.  Out of line and behind the iteration loop, so that it costs the loop no registers.  Returns the sequence number.
-template <typename T, int RP, int CPL, int THREADS, bool GROUP>
-__device__ __noinline__ unsigned recover(const SweepArgs *ap, Shared S, int p, int group, int c, int it, unsigned seq, float wold, float wnew)
+template <typename T, int RP, int CPL, int THREADS, bool GROUP, size_t WORK = work_bytes<T>(RP, THREADS), size_t REF = ref_bytes(RP, THREADS)>
+__device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, int c, int it, unsigned seq, float wold, float wnew)
 {
+    extern __shared__ __align__(128) uint8_t smem[];
     const SweepArgs &a = *ap;
+    const Shared S = carve<T, RP, THREADS>(smem, a.srows, WORK, REF);
     Share R;
     const Problem P = locate<RP, CPL, THREADS>(a, p, c, R);
     const T *x = static_cast<const T *>(a.x[P.side]) + ((size_t)P.slice * P.n + P.row0) * a.d;
