@@ -52,7 +52,7 @@ def parse():
     ap.add_argument("--dtype", default=None, choices=["bf16", "f32"])
     ap.add_argument("--shard", default="batch", choices=["batch", "heads"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--path", default="auto", choices=["auto", "general", "streamed", "resident"],
+    ap.add_argument("--path", default="auto", choices=["auto", "general", "streamed", "resident", "long"],
                     help="kernel path the library takes where it can run (default: the library's own choice)")
     ap.add_argument("--op", default="fwd", choices=["fwd", "bwd"],
                     help="bwd: time lot_attention_bwd (gradients of q, k, v, z, beta; one GPU) instead of the forward")
@@ -222,14 +222,16 @@ def run_reference(args):
 
 
 # --------------------------------------------------------------------------- our arm
-PATH_NAMES = {0: "general path (cost, T+1 Sinkhorn passes, two apply kernels)",
+PATH_NAMES = {0: "general path (build_kernel, sweep_kernel for all Sinkhorn passes, two apply kernels)",
               1: "fused_forward_kernel (persistent, Gibbs kernel streamed from L2; plus the pivot preparation)",
               2: "resident_forward_kernel (persistent, Gibbs kernel resident in shared memory and TMEM)",
-              3: "slice_forward_kernel (one thread block per slice, logits and Gibbs kernel in float32 registers)"}
+              3: "slice_forward_kernel (two thread blocks per slice, float32 Gibbs kernel in shared memory)",
+              4: "stream_kernel (bf16 Gibbs kernel built and iterated on in one launch; plus two apply kernels)"}
 ARITH = {0: {"bfloat16": "f32", "float32": "f64"},
          1: {"bfloat16": "bf16 operands, f32 accumulate, bf16 stored Gibbs kernel"},
          2: {"bfloat16": "bf16 operands, f32 accumulate, bf16 resident Gibbs kernel"},
-         3: {"bfloat16": "bf16 operands, f32 accumulate, f32 Gibbs kernel in registers"}}
+         3: {"bfloat16": "bf16 operands, f32 accumulate, f32 Gibbs kernel"},
+         4: {"bfloat16": "bf16 operands, f32 accumulate, bf16 stored Gibbs kernel"}}
 
 
 def run_ours(args):
@@ -271,7 +273,7 @@ def run_ours(args):
     out = torch.empty_like(q)
     code = lot.LOT_BF16 if q.dtype == torch.bfloat16 else lot.LOT_F32
     if args.path != "auto":          # before the workspace is sized: its size follows the path
-        lot.lot_debug_hook(4, {"general": 0, "streamed": 1, "resident": 2}[args.path])
+        lot.lot_debug_hook(4, {"general": 0, "streamed": 1, "resident": 2, "long": 4}[args.path])
     ws = torch.empty(max(256, lot.lot_workspace_bytes(B, H, n, d, r, code)), device=dev, dtype=torch.uint8)
     flush = torch.empty(512 << 20, device=dev, dtype=torch.uint8)
     stream = torch.cuda.current_stream()
@@ -459,7 +461,7 @@ def run_backward(args):
             "vs_baseline": None, "dtype": ARITH[0][tdt], "data": "synthetic",
             "config": config_of(x, {"l2": "flushed between timed steps (512 MiB overwrite)",
                                     "op": "backward (forward recomputed inside, materialised similarities)"}),
-            "clocks": clocks, "gpu_launches": (2 * x.iters + 15) * args.steps,
+            "clocks": clocks, "gpu_launches": (2 * x.iters + 15 if tdt == "float32" else 13) * args.steps,
             "forward_ms_per_step": sum(tf) / len(tf), "backward_over_forward": ms / (sum(tf) / len(tf)),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": None, "peak_source": peak_src, "algorithmic_bytes": abytes,

@@ -171,11 +171,14 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *      column mass below 2^-80) is recomputed by the streamed kernels, which are launched behind it
  *      and return at once otherwise (device flag LOT_DEV_RECOMPUTED).  It can run many more shapes
  *      (lot_debug_hook what = 4), but measured no faster there.
+ *   4  the long path (same tensors, 32 < r <= 64): one cooperative launch builds that bf16 kernel and runs all passes
+ *      on it, a group of thread blocks per problem keeping what it can of it in shared memory; two apply kernels.
+ *      Taken for moderate row counts, n <= 1200 and few slices; path 0 takes smaller problems and r <= 16.
  *   3  the slice path (same tensors; n <= 512 and 16 ceil(n/16) x (r padded to 16, 32 or 64) <= 16384): a pair of
  *      thread blocks per (batch, head) slice, one for each side, keeps the side's Gibbs kernel in float32 in shared
  *      memory for all iterations (warp-level tensor-core products); only the r x d intermediate crosses, inside the
  *      pair's cluster; no workspace beyond the status word.  Taken wherever it can run.
- * On paths 1 and 2 the potentials agree with an exact float evaluation to about 1e-4 and the output
+ * On paths 1, 2 and 4 the potentials agree with an exact float evaluation to about 1e-4 and the output
  * to the bf16 rounding of `out`.
  */
 LOT_API int lot_path(int dtype, int B, int H, int n, int d, int r, int iters);
@@ -194,7 +197,7 @@ LOT_API int lot_launch_count(int dtype, int B, int H, int n, int d, int r, int i
  *   what = 2: limit of every device-side wait of the resident path in nanoseconds (0 = default, 1 s).
  *   what = 3: device address of a trace buffer (8002 64-bit words, zeroed by the caller) into which thread block 0 of
  *             the resident path logs (event code, global timer) pairs, or 0 to stop; for profiling.
- *   what = 4: 1 or 2 makes lot_attention_fwd_ex take tensor-core path 1 or 2 of lot_path wherever that path can run
+ *   what = 4: 1, 2 or 4 makes lot_attention_fwd_ex take tensor-core path 1, 2 or 4 of lot_path wherever that path can run
  *             at all (the default choice is by measured speed), 0 the general path; -1 restores the default.
  *             lot_path, lot_launch_count and lot_workspace_bytes follow the switch.
  * Returns LOT_ERR_INVALID_ARG for any other `what`.

@@ -221,7 +221,7 @@ void remember_ws(const void *ws, int path, unsigned tag, size_t fused_off)
     g_ws_records[ws] = WsRecord{path, tag, fused_off};
 }
 
-enum { kPathGeneral = 0, kPathStreamed = 1, kPathResident = 2, kPathSlice = 3 };
+enum { kPathGeneral = 0, kPathStreamed = 1, kPathResident = 2, kPathSlice = 3, kPathLong = 4 };
 std::atomic<int> g_force_path{-1};      // test hook: 0 picks the general path, 1 or 2 that tensor-core path wherever it can run
 int choose_path(int dtype, int B, int H, int n, int d, int r)
 {
@@ -231,9 +231,21 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
     const int force = g_force_path.load();
     if (force == kPathGeneral) return kPathGeneral;
     if (force == kPathStreamed) return kPathStreamed;
+    if (force == kPathLong && r > 32) return kPathLong;
     if (force == kPathResident) return res_ok ? kPathResident : kPathStreamed;
     // short sequences: one thread block per slice, everything on chip, exact float32 logits
     if (slice_ok) return kPathSlice;
+    // Measured at T = 10 against the streamed and the resident kernels (B200): the general path's float32 kernel wins with
+    // few pivots everywhere (r = 16: 1.05 to 4.5 times), else with few rows in all or short sequences (r = 32: 1.4 to 4
+    // times; r = 64, at most 50000 rows: 1.7 to 3), the bf16 kernel of the long path a little beyond (n = 4096, 16
+    // slices: 89 us against 100 and 116; n = 1000, 256 slices: 202 against 321) and where there are few slices.
+    if (B >= 1 && n >= 1) {
+        const long long slices = (long long)B * H, rows = slices * n;
+        if (r <= 16) return kPathGeneral;
+        if (r <= 32 && (n <= 1200 || rows <= 160000)) return kPathGeneral;
+        if (r > 32 && rows <= 50000) return kPathGeneral;
+        if (r > 32 && (n <= 1200 || rows <= 100000 || slices <= 6)) return kPathLong;
+    }
     // Measured on B200 (see the design notes): the resident kernel wins where the streamed one has no stored-kernel
     // passes (r <= 32, every pass recomputes logits and exponentials) and every thread block holds its whole share at
     // once (whole slices, one wave); elsewhere the streamed kernel is as fast or faster.
@@ -246,7 +258,7 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
 
 // Both Sinkhorn problems and the apply stages on the general path.
 cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, const void *v, const float *z, const float *beta,
-                        const float *mass_q, const float *mass_k, int skip, const int32_t *key_len, const float *g1_in, const float *g2_in,
+                        const float *mass_q, const float *mass_k, int skip, int terms, const int32_t *key_len, const float *g1_in, const float *g2_in,
                         int dtype, int B, int H, int nq, int nk, int d, int r, float eps, int iters, void *out, float *g1_out,
                         float *g2_out, void *ws, cudaStream_t s)
 {
@@ -261,7 +273,7 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
     a.mass[0] = mass_q; a.mass[1] = mass_k; a.g_in[0] = g1_in; a.g_in[1] = g2_in; a.g_out[0] = g1_out; a.g_out[1] = g2_out;
     a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf); a.status = at<int>(ws, 0);
     a.head = at<uint4>(ws, 0); a.head_words = L.head_end / 16;
-    a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip;
+    a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip; a.terms = terms;
     a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
     a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
@@ -282,7 +294,7 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
     }
     ap.beta = beta; ap.key_len = key_len; ap.mass2 = mass_k; ap.v = v; ap.out = out;
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
-    ap.B = B; ap.H = H; ap.nq = nq; ap.nk = nk; ap.d = d; ap.r = r; ap.RP = L.plan.RP; ap.skip = skip;
+    ap.B = B; ap.H = H; ap.nq = nq; ap.nk = nk; ap.d = d; ap.r = r; ap.RP = L.plan.RP; ap.skip = skip; ap.terms = terms;
     ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
     if ((e = launch_sweep_apply_w(ap, dtype, s)) != cudaSuccess) return e;
     return launch_sweep_apply_out(ap, dtype, s);
@@ -312,13 +324,13 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
     a.B = B; a.H = H; a.d = d; a.r = r;
     a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
-    a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
+    a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0; a.terms = 3;
     // ---- the forward, keeping the weights of every iteration
     if ((e = launch_build(RP, a, dt, 3, st)) != cudaSuccess) return e;
     if ((e = launch_sweep(L.plan, a, dt, st)) != cudaSuccess) return e;
     ap.beta = beta; ap.key_len = key_len; ap.v = v;
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
-    ap.B = B; ap.H = H; ap.nq = n; ap.nk = n; ap.d = d; ap.r = r; ap.RP = RP;
+    ap.B = B; ap.H = H; ap.nq = n; ap.nk = n; ap.d = d; ap.r = r; ap.RP = RP; ap.terms = 3;
     ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
     if ((e = launch_sweep_apply_w(ap, dt, st)) != cudaSuccess) return e;              // W' = Diag(1/beta) Gamma2 V
     // ---- reverse of the read-out, Eq. (4): out = R1 W'
@@ -482,6 +494,7 @@ size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
     const int path = choose_path(dtype, B, H, n, d, r);
     if (path == kPathResident) return up256(resident_layout(B, H, n, d, r).total) + fused_layout(B, H, n, d, r).total;
     if (path == kPathStreamed) return fused_layout(B, H, n, d, r).total;
+    if (path == kPathLong) return stream_plan(B * H, n).total;
     if (path == kPathSlice) return 256;                              // the status word
     return forward_layout(B, H, n, n, d, r, dtype, false).total;
 }
@@ -501,6 +514,7 @@ int lot_launch_count(int dtype, int B, int H, int n, int d, int r, int iters)
     if (path == kPathResident) return 1 + 2;                        // the two streamed kernels return at once unless asked to redo
     if (path == kPathStreamed) return fused_launches(B, H, n, r, iters);
     if (path == kPathSlice) return 1;
+    if (path == kPathLong) return 3;
     return sweep_plan(dtype, B * H > 0 ? B * H : 1, n, n, d, r).steps ? 2 + iters + 1 + 2 : 4;
 }
 
@@ -538,6 +552,12 @@ int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
                                         at<int>(ws, 0), (cudaStream_t)stream);
         return e == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
     }
+    if (path == kPathLong) {
+        if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < stream_plan(B * H, n).total) return LOT_ERR_WORKSPACE;
+        remember_ws(ws, kPathLong, 0, 0);
+        return stream_attention(q, k, v, z, beta, key_len, B, H, n, r, eps, iters, out, g1_out, g2_out, ws, (cudaStream_t)stream) == cudaSuccess
+                   ? LOT_OK : LOT_ERR_CUDA;
+    }
     if (path != kPathGeneral) {
         const size_t res_bytes = path == kPathResident ? up256(resident_layout(B, H, n, d, r).total) : 0;
         const size_t need = res_bytes + fused_layout(B, H, n, d, r).total;
@@ -564,7 +584,9 @@ int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
     const ForwardLayout L = forward_layout(B, H, n, n, d, r, dtype, false);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    return run_forward(L, q, k, v, z, beta, nullptr, nullptr, 0, key_len, nullptr, nullptr, dtype, B, H, n, n, d, r, eps, iters, out,
+    // sizes of the tensor-core paths keep their hi + lo operands here too; a forced general path is float32 throughout
+    const int terms = fused_supported(dtype, d, r) && g_force_path.load() != kPathGeneral ? 2 : 3;
+    return run_forward(L, q, k, v, z, beta, nullptr, nullptr, 0, terms, key_len, nullptr, nullptr, dtype, B, H, n, n, d, r, eps, iters, out,
                        g1_out, g2_out, ws, s) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
 }
 
@@ -604,7 +626,7 @@ int lot_attention_fwd_var(const void *q, const void *k, const void *v, const flo
     cudaStream_t s = (cudaStream_t)stream;
     remember_ws(ws, kPathGeneral, 0, 0);
     // the class token is neither a query nor a key of the transport problem: it is skipped on both sides
-    if (run_forward(L, q, k, v, z, beta, a, b, cls, key_len, g1_in, g2_in, dtype, B, H, nq, nk, d, r, eps, iters, out, g1_out, g2_out,
+    if (run_forward(L, q, k, v, z, beta, a, b, cls, 3, key_len, g1_in, g2_in, dtype, B, H, nq, nk, d, r, eps, iters, out, g1_out, g2_out,
                     ws, s) != cudaSuccess)
         return LOT_ERR_CUDA;
     if (cls && launch_cls_row(q, k, v, key_len, dtype, B, H, nq, nk, d, cls_tau, at<float>(ws, L.scores), out, s) != cudaSuccess)

@@ -18,13 +18,13 @@ template <typename T, int RP> struct Shape {
     static constexpr int MINB = ACC <= 32 ? 3 : ACC <= 64 ? 2 : 1;
 };
 
-template <typename T, int RP>
+template <typename T, int RP, int TERMS>
 __global__ void __launch_bounds__(kThreads, Shape<T, RP>::MINB)
 build_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k)
 {
     extern __shared__ __align__(128) uint8_t stage[];
     typedef Shape<T, RP> Sh;
-    typedef logits::Logits<T, RP, Sh::ROWS, kThreads> Lg;
+    typedef logits::Logits<T, RP, Sh::ROWS, kThreads, TERMS> Lg;
     typedef typename Lg::LT LT;
     __shared__ LT sG[RP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3, r = a.r;
@@ -73,11 +73,11 @@ build_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k)
     }
 }
 
-template <typename T, int RP>
+template <typename T, int RP, int TERMS = 3>
 static cudaError_t launch_t(const SweepArgs &a, int sides, cudaStream_t st)
 {
     typedef Shape<T, RP> Sh;
-    auto kern = build_kernel<T, RP>;
+    auto kern = build_kernel<T, RP, TERMS>;
     constexpr size_t smem = logits::stage_bytes<T>(RP);
     if (smem > 48 * 1024) {
         static std::mutex mu;
@@ -114,6 +114,11 @@ static cudaError_t launch_rp(int RP, const SweepArgs &a, int sides, cudaStream_t
 // sides: bit 0 the queries, bit 1 the keys
 cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st)
 {
+    if (dtype == 1 && a.terms == 2) {
+        if (RP == 16) return build::launch_t<__nv_bfloat16, 16, 2>(a, sides, st);
+        if (RP == 32) return build::launch_t<__nv_bfloat16, 32, 2>(a, sides, st);
+        if (RP == 64) return build::launch_t<__nv_bfloat16, 64, 2>(a, sides, st);
+    }
     return dtype == 0 ? build::launch_rp<float>(RP, a, sides, st) : build::launch_rp<__nv_bfloat16>(RP, a, sides, st);
 }
 

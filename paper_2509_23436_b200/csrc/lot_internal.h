@@ -151,6 +151,15 @@ cudaError_t slice_attention(const void *q, const void *k, const void *v, const f
                             const int32_t *key_len, int B, int H, int n, int r, float eps, int iters, void *out,
                             float *g1_out, float *g2_out, int *status, cudaStream_t st);
 
+// ---- long sequences on a stored bf16 kernel (lot_stream.cu): bf16 tensors, d = 64, 32 < r <= 64 ----
+struct StreamPlan {
+    int C, groups, srows, npad;
+    size_t xbuf, ybuf, head_end, G, decision, kt, wpart, total;
+};
+StreamPlan stream_plan(int BH, int n);
+cudaError_t stream_attention(const void *q, const void *k, const void *v, const float *z, const float *beta, const int32_t *key_len, int B,
+                             int H, int n, int r, float eps, int iters, void *out, float *g1_out, float *g2_out, void *ws, cudaStream_t st);
+
 // ---- apply stages from the stored Gibbs kernel (lot_apply.cu), behind the streamed Sinkhorn kernel ----
 size_t stored_apply_wpart_bytes(int B, int H, int n);
 cudaError_t stored_apply(const void *kt, int npad, const float *G, const float *beta, const int32_t *key_len, const int *decision,

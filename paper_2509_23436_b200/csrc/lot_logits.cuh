@@ -28,11 +28,12 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr)
 // Shared memory of one staged step of pivots.
 template <typename T> __host__ __device__ constexpr size_t stage_bytes(int cc) { return sizeof(T) == 2 ? (size_t)cc * 80 * 3 : (size_t)cc * 18 * 8; }
 
-template <typename T, int CC, int ROWS, int THREADS> struct Logits;
+// TERMS: bf16 terms a float32 pivot is taken as (bf16 tokens): 3 is exact, 2 is the precision of the tensor-core paths.
+template <typename T, int CC, int ROWS, int THREADS, int TERMS = 3> struct Logits;
 
 // bf16 tokens are exact operands; a float32 pivot is the exact sum of three bf16 terms, so the products are those of
 // the float32 evaluation, summed in float32.  The next step's operands are in flight while the current one multiplies.
-template <int CC, int THREADS> struct Logits<__nv_bfloat16, CC, 16, THREADS> {
+template <int CC, int THREADS, int TERMS> struct Logits<__nv_bfloat16, CC, 16, THREADS, TERMS> {
     typedef float LT;
     static constexpr int KC = 32, PITCH = 80, PLANE = CC * PITCH;     // 80-byte rows: conflict-free ldmatrix
     static constexpr int NZ = (CC * KC / 2 + THREADS - 1) / THREADS;  // pivot pairs a thread stages per step
@@ -71,7 +72,7 @@ template <int CC, int THREADS> struct Logits<__nv_bfloat16, CC, 16, THREADS> {
                 uint8_t *p = stage + t * PITCH + k * 2;
                 float2 v = zz[u];
 #pragma unroll
-                for (int term = 0; term < 3; ++term) {
+                for (int term = 0; term < TERMS; ++term) {
                     const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
                     *reinterpret_cast<__nv_bfloat162 *>(p + term * PLANE) = h;
                     v.x -= __low2float(h);
@@ -92,7 +93,7 @@ template <int CC, int THREADS> struct Logits<__nv_bfloat16, CC, 16, THREADS> {
                     for (int jp = 0; jp < CC / 16; ++jp) {
                         const uint32_t off = sb + (jp * 16 + (lane & 7) + (lane >> 4) * 8) * PITCH + (ks * 16 + ((lane >> 3) & 1) * 8) * 2;
 #pragma unroll
-                        for (int term = 2; term >= 0; --term) {       // small terms first
+                        for (int term = TERMS - 1; term >= 0; --term) {       // small terms first
                             uint32_t b[4];
                             ldsm4(b, off + term * PLANE);
                             mma_bf16(acc[2 * jp], ac[ks], b[0], b[1]);
@@ -107,7 +108,7 @@ template <int CC, int THREADS> struct Logits<__nv_bfloat16, CC, 16, THREADS> {
 
 // float32 tokens: products and sums in float64 (logits C/eps of magnitude 1e3 need an absolute accuracy far below
 // 1e-4).  Lane q of a quad reads four consecutive k of its row at once; product step s uses element s on both sides.
-template <int CC, int ROWS, int THREADS> struct Logits<float, CC, ROWS, THREADS> {
+template <int CC, int ROWS, int THREADS, int TERMS> struct Logits<float, CC, ROWS, THREADS, TERMS> {
     typedef double LT;
     static constexpr int MT = ROWS / 8, KC = 16, PITCH = 18;          // pitch of 18 doubles: conflict-free 16-byte reads
     static constexpr int NZ = (CC * KC / 4 + THREADS - 1) / THREADS;

@@ -1,0 +1,632 @@
+// Long sequences with 32 < r <= 64 pivots (bf16 tensors, d = 64): the Gibbs kernel as bf16, built and iterated on in one
+// launch, then applied by the tensor-core kernels of lot_apply.cu.
+//
+// As in lot_sweep.cu a problem (one side of one slice) is shared by a group of C blocks and every pass is two
+// multiply-adds per entry on the stored kernel, here K_it = 2^(L_it + Gref_t - ref_i) <= 2^67 in bf16 (the rounding the
+// streamed path has always had; potentials to about 1e-4): half the bytes, so a pass over n = 16384, H = 16 reads 67 MB, of
+// which the blocks keep the first rows of their share in shared memory and the rest comes from L2.  Each block
+// computes the logits of its own rows (warp-level products, Z as bf16 hi + lo), so building one group's kernel
+// overlaps another's passes.  When all problems together exceed the L2, groups are made larger and work through the problems
+// in rounds, so that what is iterated on stays in the L2.
+#include "lot_sweep_core.cuh"
+
+namespace lot {
+namespace stream {
+
+using namespace sweep;
+
+constexpr int kThreads = 256, kD = 64, RP = 64;
+constexpr int kRowsStep = 64;              // rows per step of a block: eight a warp, four lanes a row
+constexpr int kZPitch = 144;               // bytes per staged pivot row (conflict-free ldmatrix)
+constexpr int kWork = 2 * RP * kZPitch;    // staged pivots (hi, lo), later the column reduction
+constexpr int kFixed = kWork + kThreads * 4 + RP * 16 + 64;
+
+struct StreamArgs {
+    const __nv_bfloat16 *x[2];
+    const float *z, *beta;
+    const int32_t *key_len;
+    uint8_t *kt;               // [2][BH][npad][64] bf16, side 0 queries
+    float *G;                  // [2][BH][64] log2 of the final weights (relative to the kernel as stored)
+    int *decision;             // [2][BH], set to 1
+    float *g_out[2];
+    u64 *xbuf, *ybuf;
+    int *status;
+    int B, H, n, npad, r, T, C, groups, srows;
+    double scale, eps_ln2;
+};
+
+struct Mem {
+    uint8_t *K;                // [srows][128 bytes]
+    Shared s;
+};
+
+__device__ __forceinline__ Mem carve16(uint8_t *p, int srows)
+{
+    Mem m;
+    m.K = p; p += (size_t)srows * 128;
+    m.s.K = nullptr;
+    m.s.gref = reinterpret_cast<double *>(p); p += RP * 8;
+    m.s.work = p; p += kWork;
+    m.s.ref = reinterpret_cast<float *>(p); p += kThreads * 4;
+    m.s.w = reinterpret_cast<float *>(p); p += RP * 4;
+    m.s.tgt = reinterpret_cast<float *>(p); p += RP * 4;
+    m.s.flag = reinterpret_cast<volatile int *>(p);    // [0], [1] as in the sweep kernels; [2], [3]: see solve16
+    return m;
+}
+
+struct Part {                  // a block's share of a problem
+    int slice, side, h, nv, row0, nrows, ns, steps;
+    uint8_t *g;                // its rows in global memory
+    const __nv_bfloat16 *x;
+};
+
+__device__ __forceinline__ Part locate16(const StreamArgs &a, int p, int c)
+{
+    Part P;
+    P.slice = p >> 1;
+    P.side = (p & 1) ^ 1;
+    P.h = P.slice % a.H;
+    P.nv = a.n;
+    if (P.side == 1 && a.key_len != nullptr) P.nv = min(max(__ldg(a.key_len + P.slice / a.H), 0), a.n);
+    const int per = (P.nv + a.C - 1) / a.C;
+    P.row0 = min(c * per, P.nv);
+    P.nrows = min(per, P.nv - P.row0);
+    P.ns = min(P.nrows, a.srows);
+    P.steps = (P.ns + kRowsStep - 1) / kRowsStep;
+    P.g = a.kt + ((size_t)(P.side * a.B * a.H + P.slice) * a.npad + P.row0) * 128;
+    P.x = a.x[P.side] + ((size_t)P.slice * a.n + P.row0) * kD;
+    return P;
+}
+
+__device__ __forceinline__ uint32_t pack2(float lo, float hi)
+{
+    const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&t);
+}
+
+// Pivots of the head in base-2 logit units as bf16 hi + lo into the work area.
+__device__ __forceinline__ void stage_pivots(const StreamArgs &a, const Mem &m, const Part &P)
+{
+    const float *z = a.z + (size_t)P.h * a.r * kD;
+    const float scale = (float)a.scale;
+    float2 zz[RP * kD / 2 / kThreads];
+#pragma unroll
+    for (int u = 0; u < RP * kD / 2 / kThreads; ++u) {
+        const int idx = threadIdx.x + u * kThreads, t = idx / (kD / 2);
+        zz[u] = t < a.r ? __ldg(reinterpret_cast<const float2 *>(z + (size_t)t * kD + (idx % (kD / 2)) * 2)) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < RP * kD / 2 / kThreads; ++u) {
+        const int idx = threadIdx.x + u * kThreads, t = idx / (kD / 2), c2 = (idx % (kD / 2)) * 2;
+        const float x0 = zz[u].x * scale, x1 = zz[u].y * scale;
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+        *reinterpret_cast<__nv_bfloat162 *>(m.s.work + t * kZPitch + c2 * 2) = h;
+        *reinterpret_cast<uint32_t *>(m.s.work + (RP + t) * kZPitch + c2 * 2) = pack2(x0 - __low2float(h), x1 - __high2float(h));
+    }
+    __syncthreads();
+}
+
+// Logits of 16 rows a warp, all pivots: tokens straight from global memory, pivots from the work area.
+__device__ __forceinline__ void fetch_tokens(uint32_t (&a)[kD / 16][4], const Part &P, int rt)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+#pragma unroll
+    for (int ks = 0; ks < kD / 16; ++ks)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = rt + warp * 16 + g + (e & 1) * 8;
+            a[ks][e] = i < P.nrows ? __ldg(reinterpret_cast<const unsigned *>(P.x + (size_t)i * kD + ks * 16 + (e >> 1) * 8 + 2 * q)) : 0u;
+        }
+}
+__device__ __forceinline__ void tile_logits(float (&L)[RP / 8][4], const uint32_t (&a)[kD / 16][4], uint32_t zb)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < RP / 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) L[j][e] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < kD / 16; ++ks)
+#pragma unroll
+        for (int jp = 0; jp < RP / 16; ++jp) {
+            const uint32_t off = zb + (jp * 16 + (lane & 7) + (lane >> 4) * 8) * kZPitch + (ks * 16 + ((lane >> 3) & 1) * 8) * 2;
+            uint32_t bl[4], bh[4];
+            logits::ldsm4(bl, off + RP * kZPitch);
+            logits::ldsm4(bh, off);
+            logits::mma_bf16(L[2 * jp], a[ks], bl[0], bl[1]);
+            logits::mma_bf16(L[2 * jp + 1], a[ks], bl[2], bl[3]);
+            logits::mma_bf16(L[2 * jp], a[ks], bh[0], bh[1]);
+            logits::mma_bf16(L[2 * jp + 1], a[ks], bh[2], bh[3]);
+        }
+}
+
+// The block's kernel rows around the reference potentials: to global memory, and the first ns to shared memory too (rows up to
+// the next full step are zero there; the last block of the problem clears the global rows up to the next 128).
+// REF: reference potentials other than one constant.  Out of line: its registers are not the iteration loop's.
+template <bool REF>
+__device__ __noinline__ void build16(const StreamArgs *ap, int p, int c)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const StreamArgs &a = *ap;
+    const Mem m = carve16(smem, a.srows);
+    const Part P = locate16(a, p, c);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+    uint32_t tok[kD / 16][4];
+    fetch_tokens(tok, P, 0);
+    stage_pivots(a, m, P);
+    const uint32_t zb = smem_addr(m.s.work);
+    for (int rt = 0; rt < P.nrows; rt += 128) {
+        float L[RP / 8][4];
+        tile_logits(L, tok, zb);
+        if (rt + 128 < P.nrows) fetch_tokens(tok, P, rt + 128);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = rt + warp * 16 + g + 8 * h;
+            float mx = neg_inf();
+#pragma unroll
+            for (int j = 0; j < RP / 8; ++j)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int t = 8 * j + 2 * q + e;
+                    float l = L[j][2 * h + e];
+                    if (REF) l += (float)m.s.gref[t];
+                    if (t >= a.r) l = neg_inf();
+                    L[j][2 * h + e] = l;
+                    mx = fmaxf(mx, l);
+                }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2)) - kKernelTop;
+            // neighbouring lanes trade halves of neighbouring tiles: a lane stores 8 bytes, a quad 32 in a row
+#pragma unroll
+            for (int j = 0; j < RP / 8; j += 2) {
+                const uint32_t u0 = pack2(ex2(L[j][2 * h] - mx), ex2(L[j][2 * h + 1] - mx));
+                const uint32_t u1 = pack2(ex2(L[j + 1][2 * h] - mx), ex2(L[j + 1][2 * h + 1] - mx));
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, q & 1 ? u0 : u1, 1);
+                const uint2 o = q & 1 ? make_uint2(got, u1) : make_uint2(u0, got);
+                const int at = (8 * (j + (q & 1)) + 4 * (q >> 1)) * 2;
+                if (i < P.nrows) {
+                    *reinterpret_cast<uint2 *>(P.g + (size_t)i * 128 + at) = o;
+                    if (i < P.ns) *reinterpret_cast<uint2 *>(m.K + (size_t)i * 128 + at) = o;
+                }
+            }
+        }
+    }
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    for (int idx = threadIdx.x; idx < (P.steps * kRowsStep - P.ns) * 8; idx += kThreads)
+        *reinterpret_cast<uint4 *>(m.K + (size_t)P.ns * 128 + idx * 16) = zero;
+    if (c == a.C - 1) {
+        const int end = min((P.nv + 127) & ~127, a.npad) - P.nv;
+        uint8_t *o = a.kt + ((size_t)(P.side * a.B * a.H + P.slice) * a.npad + P.nv) * 128;
+        for (int idx = threadIdx.x; idx < end * 8; idx += kThreads) *reinterpret_cast<uint4 *>(o + (size_t)idx * 16) = zero;
+    }
+    __syncthreads();
+}
+
+// A lane's sixteen columns of a row: the 16-byte chunks cl and 4 + cl.  Lanes of odd rows read chunk 4 + cl first: the eight
+// lanes of a 128-byte phase, two rows, then cover all banks without a permuted layout, and the first halving of the
+// column sums is an exchange without selects.
+struct LaneMap {
+    uint32_t k[2], w[2], red, own;
+    int i0, cl, odd;
+};
+
+__device__ __forceinline__ LaneMap make_map16(const Mem &m)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 2;
+    LaneMap L;
+    L.cl = lane & 3;
+    L.odd = sub & 1;
+    L.i0 = warp * 8 + sub;
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        const int chunk = (v ^ L.odd) * 4 + L.cl;
+        L.k[v] = smem_addr(m.K) + L.i0 * 128 + chunk * 16;
+        L.w[v] = smem_addr(m.s.w) + chunk * 32;
+    }
+    // after the halvings: two columns of chunk (odd, cl)
+    const int col = (L.odd * 4 + L.cl) * 8 + ((lane & 8) ? 4 : 0) + ((lane & 16) ? 2 : 0);
+    L.red = smem_addr(m.s.work) + (warp * RP + col) * 4;
+    L.own = smem_addr(m.s.work) + threadIdx.x * 4;
+    return L;
+}
+
+__device__ __forceinline__ void load_weights16(const LaneMap &L, u64 (&w)[8])
+{
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        lds2(w[4 * v], w[4 * v + 1], L.w[v]);
+        lds2(w[4 * v + 2], w[4 * v + 3], L.w[v] + 16);
+    }
+}
+
+// pairs of bf16 as packed float pairs
+__device__ __forceinline__ u64 widen(uint32_t x) { return pack_f2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
+
+__device__ __forceinline__ void row16(const uint4 &a, const uint4 &b, const u64 (&w)[8], u64 (&acc)[8])
+{
+    const u64 k[8] = {widen(a.x), widen(a.y), widen(a.z), widen(a.w), widen(b.x), widen(b.y), widen(b.z), widen(b.w)};
+    u64 s0 = 0, s1 = 0;
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) { s0 = fma_f2(k[j], w[j], s0); s1 = fma_f2(k[j + 1], w[j + 1], s1); }
+    float x, y, u, v;
+    unpack_f2(s0, x, y);
+    unpack_f2(s1, u, v);
+    float s = (x + y) + (u + v);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    const float inv = rcp(fmaxf(s, 1e-37f));
+    const u64 ii = pack_f2(inv, inv);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = fma_f2(k[j], ii, acc[j]);
+}
+
+__device__ __forceinline__ uint4 lds4(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void pass16(const LaneMap &L, const Part &P, const u64 (&w)[8], u64 (&acc)[8])
+{
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = 0;
+    int st = 0;
+#pragma unroll 1
+    for (; st + 2 <= P.steps; st += 2) {
+        const uint4 a0 = lds4(L.k[0] + st * (kRowsStep * 128)), b0 = lds4(L.k[1] + st * (kRowsStep * 128));
+        const uint4 a1 = lds4(L.k[0] + (st + 1) * (kRowsStep * 128)), b1 = lds4(L.k[1] + (st + 1) * (kRowsStep * 128));
+        row16(a0, b0, w, acc);
+        row16(a1, b1, w, acc);
+    }
+    if (st < P.steps) row16(lds4(L.k[0] + st * (kRowsStep * 128)), lds4(L.k[1] + st * (kRowsStep * 128)), w, acc);
+    // rows that do not fit: kAhead steps requested together (a second set in flight spilled: 30 us a pass at n = 16384)
+    constexpr int kAhead = 4;
+    const uint8_t *g0 = P.g + (size_t)(P.ns + L.i0) * 128 + (L.odd * 4 + L.cl) * 16;
+    const int flip = (1 - 2 * L.odd) * 64;               // from the lane's first chunk to its second
+#pragma unroll 1
+    for (int left = P.nrows - P.ns - L.i0; left > -L.i0; left -= kAhead * kRowsStep, g0 += kAhead * kRowsStep * 128) {
+        uint4 ra[kAhead], rb[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const bool in = u * kRowsStep < left;
+            ra[u] = in ? __ldcg(reinterpret_cast<const uint4 *>(g0 + u * (kRowsStep * 128))) : make_uint4(0, 0, 0, 0);
+            rb[u] = in ? __ldcg(reinterpret_cast<const uint4 *>(g0 + u * (kRowsStep * 128) + flip)) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) row16(ra[u], rb[u], w, acc);
+    }
+}
+
+// One iteration, as in lot_sweep_core.cuh: thread t < r gets its column's weight before and after.
+template <bool GROUP>
+__device__ __forceinline__ bool iterate16(const StreamArgs &a, const Mem &m, const Part &P, const LaneMap &L, u64 (&w)[8], float tgt,
+                                          int group, int c, unsigned &seq, float &wold, float &wnew)
+{
+    u64 acc[8];
+    pass16(L, P, w, acc);
+    float v[16];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) unpack_f2(acc[j], v[2 * j], v[2 * j + 1]);
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[8 + i], 4);       // even rows keep chunk cl, odd ones 4 + cl
+#pragma unroll
+    for (int h = 4, bit = 8; h >= 2; h >>= 1, bit <<= 1) {
+        const bool up = (lane & bit) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+        }
+    }
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(L.red), "f"(v[0]), "f"(v[1]) : "memory");
+    __syncthreads();
+    float tot = 0.f;
+    if (threadIdx.x < RP) {
+        float o[kThreads / 32];
+#pragma unroll
+        for (int i = 0; i < kThreads / 32; ++i) o[i] = lds(L.own + i * (RP * 4));
+#pragma unroll
+        for (int h = kThreads / 64; h > 0; h >>= 1)
+#pragma unroll
+            for (int i = 0; i < h; ++i) o[i] += o[i + h];
+        tot = o[0];
+    }
+    if (GROUP) tot = group_columns<RP, kThreads, false>(a, m.s, tot, group, c, seq);
+    if ((int)threadIdx.x < a.r) {
+        wold = wnew;
+        wnew = tgt * rcp(tot);
+        if (out_of_range(wnew)) m.s.flag[1] = 1;
+        m.s.w[threadIdx.x] = wnew;
+    }
+    __syncthreads();
+    load_weights16(L, w);
+    return m.s.flag[1] != 0;
+}
+
+// Whether the weights spread over more than the 60 binades the apply kernels take (the same answer in every thread).
+__device__ __forceinline__ bool too_wide(const Mem &m, int r)
+{
+    float lo = 3e38f, hi = 0.f;
+    for (int t = threadIdx.x & 31; t < r; t += 32) {
+        const float w = m.s.w[t];
+        lo = fminf(lo, w);
+        hi = fmaxf(hi, w);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+    }
+    return hi * 8.6736174e-19f > lo;
+}
+
+// log2 of the column sums of the row-stochastic plan for the potentials in gref, in the log domain: logits once for the
+// column maxima and once more for the sums relative to them; nothing is stored.
+template <bool GROUP>
+__device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m, const Part &P, int group, int c, unsigned &seq)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+    float *red = reinterpret_cast<float *>(m.s.work);
+    float kap = 0.f, out = 0.f;
+#pragma unroll 1
+    for (int round = 0; round < 2; ++round) {
+        float col[RP / 8][2];
+#pragma unroll
+        for (int j = 0; j < RP / 8; ++j) { col[j][0] = round == 0 ? neg_inf() : 0.f; col[j][1] = col[j][0]; }
+        stage_pivots(a, m, P);
+        for (int rt = 0; rt < P.nrows; rt += 128) {
+            uint32_t tok[kD / 16][4];
+            fetch_tokens(tok, P, rt);
+            float L[RP / 8][4];
+            tile_logits(L, tok, smem_addr(m.s.work));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool ok = rt + warp * 16 + g + 8 * h < P.nrows;
+                float mx = neg_inf(), s = 0.f;
+#pragma unroll
+                for (int j = 0; j < RP / 8; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int t = 8 * j + 2 * q + e;
+                        L[j][2 * h + e] = t < a.r ? L[j][2 * h + e] + (float)m.s.gref[t] : neg_inf();
+                        mx = fmaxf(mx, L[j][2 * h + e]);
+                    }
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+#pragma unroll
+                for (int j = 0; j < RP / 8; ++j) s += ex2(L[j][2 * h] - mx) + ex2(L[j][2 * h + 1] - mx);
+                s += __shfl_xor_sync(0xffffffffu, s, 1);
+                s += __shfl_xor_sync(0xffffffffu, s, 2);
+                const float M = mx + lg2(s);
+                if (ok) {
+#pragma unroll
+                    for (int j = 0; j < RP / 8; ++j)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float x = L[j][2 * h + e] - M;
+                            if (round == 0) col[j][e] = fmaxf(col[j][e], x);
+                            else if (m.s.tgt[8 * j + 2 * q + e] > neg_inf()) col[j][e] += ex2(x - m.s.tgt[8 * j + 2 * q + e]);
+                        }
+                }
+            }
+        }
+        __syncthreads();                                           // the staged pivots are done with
+#pragma unroll
+        for (int j = 0; j < RP / 8; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float v = col[j][e];
+#pragma unroll
+                for (int off = 4; off < 32; off <<= 1) {
+                    const float o = __shfl_xor_sync(0xffffffffu, v, off);
+                    v = round == 0 ? fmaxf(v, o) : v + o;
+                }
+                if (g == 0) red[warp * RP + 8 * j + 2 * q + e] = v;
+            }
+        __syncthreads();
+        float tot = round == 0 ? neg_inf() : 0.f;
+        if (threadIdx.x < RP)
+            for (int w = 0; w < kThreads / 32; ++w) tot = round == 0 ? fmaxf(tot, red[w * RP + threadIdx.x]) : tot + red[w * RP + threadIdx.x];
+        if (GROUP) tot = round == 0 ? group_columns<RP, kThreads, true>(a, m.s, tot, group, c, seq)
+                                    : group_columns<RP, kThreads, false>(a, m.s, tot, group, c, seq);
+        __syncthreads();
+        if (round == 0) {
+            kap = tot;
+            if (threadIdx.x < RP) m.s.tgt[threadIdx.x] = kap;       // the maxima
+        } else {
+            out = kap + lg2(tot);
+        }
+        __syncthreads();
+    }
+    return out;
+}
+
+// The iterations of a problem on the kernel as built.  flag[2] = 1 where recover16 has to go on from iteration flag[3], with
+// the weights before and after that update in ref.  Returns the sequence number.
+template <bool GROUP>
+__device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const StreamArgs &a = *ap;
+    const Mem m = carve16(smem, a.srows);
+    const Part P = locate16(a, p, c);
+    const int tid = threadIdx.x, r = a.r;
+    const float tgt = tid < r ? __ldg(a.beta + P.h * r + tid) * (float)P.nv : 0.f;
+    float wold = 0.f, wnew = kStart;
+    bool bad = false;
+    int it = 0;
+    const LaneMap L = make_map16(m);
+    u64 w[8];
+    load_weights16(L, w);
+    for (; it < a.T; ++it) {
+        bad = iterate16<GROUP>(a, m, P, L, w, tgt, group, c, seq, wold, wnew);
+        if (bad) break;
+    }
+    bad = bad || too_wide(m, r);
+    __syncthreads();
+    if (tid < RP) { m.s.ref[tid] = wold; m.s.ref[RP + tid] = wnew; }
+    if (tid == 0) { m.s.flag[2] = bad; m.s.flag[3] = it; }
+    __syncthreads();
+    return seq;
+}
+
+// The rest of a problem's iterations behind an update that left the kernel's range, as recover() of the sweep kernels; and the
+// rebuilding around final potentials that spread too far for the apply kernels.
+template <bool GROUP>
+__device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const StreamArgs &a = *ap;
+    const Mem m = carve16(smem, a.srows);
+    const Part P = locate16(a, p, c);
+    const int tid = threadIdx.x, r = a.r;
+    const float tgt = tid < r ? __ldg(a.beta + P.h * r + tid) * (float)P.nv : 0.f;
+    int it = m.s.flag[3];
+    float wold = m.s.ref[tid < RP ? tid : 0], wnew = m.s.ref[RP + (tid < RP ? tid : 0)];
+    while (true) {
+        double gn = 0.0;
+        if (__syncthreads_or(tid < r && it < a.T && sum_lost(tgt, wnew))) {
+            if (tid < r) {
+                gn = m.s.gref[tid] + log2((double)wold);
+                m.s.gref[tid] = gn;
+            }
+            __syncthreads();
+            const float lam = log_columns16<GROUP>(a, m, P, group, c, seq);
+            if (tid < r) gn += log2((double)tgt) - (double)lam;
+        } else if (tid < r) {
+            gn = m.s.gref[tid] + log2((double)wnew);
+        }
+        __syncthreads();
+        if (tid < RP) {
+            if (tid < r && !isfinite(gn)) atomicOr(a.status, 1 /* LOT_DEV_NONFINITE */);
+            m.s.gref[tid] = gn - (double)kStartLog2;
+            m.s.w[tid] = tid < r ? kStart : 0.f;
+        }
+        if (tid == 0) m.s.flag[1] = 0;
+        __syncthreads();
+        build16<true>(ap, p, c);
+        bool bad = false;
+        const LaneMap L = make_map16(m);
+        u64 w[8];
+        load_weights16(L, w);
+        wnew = kStart;
+        if (it >= a.T) break;                                // rebuilt around the final potentials: equal weights
+        for (++it; it < a.T && !bad; ++it) bad = iterate16<GROUP>(a, m, P, L, w, tgt, group, c, seq, wold, wnew);
+        if (bad) --it;                                       // the iteration whose update has to be redone
+        else if (!too_wide(m, r)) break;
+        __syncthreads();
+    }
+    return seq;
+}
+
+template <bool GROUP>
+__global__ void __launch_bounds__(kThreads, 2)
+stream_kernel(const __grid_constant__ StreamArgs a)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int tid = threadIdx.x, group = GROUP ? blockIdx.x / a.C : blockIdx.x, c = GROUP ? blockIdx.x % a.C : 0;
+    unsigned seq = 0;
+    const Mem m = carve16(smem, a.srows);
+    if (tid < 4) m.s.flag[tid] = 0;
+
+    for (int p = group; p < 2 * a.B * a.H; p += a.groups) {
+        __syncthreads();                                            // the previous problem is done with shared memory
+        if (tid < RP) {
+            m.s.gref[tid] = -(double)kStartLog2;
+            m.s.w[tid] = tid < a.r ? kStart : 0.f;
+        }
+        if (tid == 0) m.s.flag[2] = 0;
+        if (locate16(a, p, c).nv > 0) {
+            build16<false>(&a, p, c);
+            seq = solve16<GROUP>(&a, p, group, c, seq);
+            if (m.s.flag[2]) seq = recover16<GROUP>(&a, p, group, c, seq);
+        } else {
+            if (tid == 0 && c == 0) atomicOr(a.status, 2 /* LOT_DEV_EMPTY */);
+            __syncthreads();
+        }
+        if (c == 0 && tid < RP) {
+            const Part F = locate16(a, p, c);
+            const size_t sp = (size_t)F.side * a.B * a.H + F.slice;
+            a.G[sp * RP + tid] = tid < a.r ? lg2(m.s.w[tid]) : 0.f;
+            if (tid == 0) a.decision[sp] = 1;
+            if (tid < a.r && a.g_out[F.side] != nullptr)
+                a.g_out[F.side][(size_t)F.slice * a.r + tid] = (float)((m.s.gref[tid] + log2((double)m.s.w[tid])) * a.eps_ln2);
+        }
+    }
+}
+
+} // namespace stream
+
+StreamPlan stream_plan(int BH, int n)
+{
+    using namespace stream;
+    StreamPlan L;
+    const int NP = 2 * BH, slots = 2 * device_sm_count();
+    const long long npad = ((long long)n + 127) / 128 * 128;
+    // problems in flight: all of them, or as many as keep what is iterated on in the L2
+    long long fly = 80000000ll / (npad * 128);
+    if (fly < 2) fly = 2;
+    if (fly > NP) fly = NP;
+    const int rounds = (int)((NP + fly - 1) / fly);
+    fly = (NP + rounds - 1) / rounds;
+    L.C = (int)(slots / fly) < 1 ? 1 : (int)(slots / fly);
+    const int most = (n + 2 * kRowsStep - 1) / (2 * kRowsStep);     // two steps a block at least
+    if (L.C > most) L.C = most;
+    if (L.C > 64) L.C = 64;
+    L.groups = L.C == 1 ? NP : (slots / L.C < NP ? slots / L.C : NP);
+    const int rows = (n + L.C - 1) / L.C, up = (rows + kRowsStep - 1) / kRowsStep * kRowsStep;
+    const int cap = (228 * 1024 / 2 - 1024 - kFixed) / 128 / kRowsStep * kRowsStep;
+    L.srows = up < cap ? up : cap;
+    L.npad = (int)npad;
+    size_t o = 256;
+    auto take = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~(size_t)255; return at; };
+    L.xbuf = take(L.C > 1 ? (size_t)L.groups * 2 * L.C * RP * 8 : 0);
+    L.ybuf = take(L.C > 1 ? (size_t)L.groups * 2 * kSweepCopies * RP * 8 : 0);
+    L.head_end = o;
+    L.G = take((size_t)NP * RP * 4);
+    L.decision = take((size_t)NP * 4);
+    L.kt = take((size_t)NP * npad * 128);
+    L.wpart = take(stored_apply_wpart_bytes(BH, 1, n));
+    L.total = o;
+    return L;
+}
+
+cudaError_t stream_attention(const void *q, const void *k, const void *v, const float *z, const float *beta, const int32_t *key_len, int B,
+                             int H, int n, int r, float eps, int iters, void *out, float *g1_out, float *g2_out, void *ws, cudaStream_t st)
+{
+    using namespace stream;
+    const StreamPlan L = stream_plan(B * H, n);
+    char *w = static_cast<char *>(ws);
+    cudaError_t e = cudaMemsetAsync(ws, 0, L.head_end, st);
+    if (e != cudaSuccess) return e;
+    StreamArgs a{};
+    a.x[0] = static_cast<const __nv_bfloat16 *>(q); a.x[1] = static_cast<const __nv_bfloat16 *>(k);
+    a.z = z; a.beta = beta; a.key_len = key_len;
+    a.kt = reinterpret_cast<uint8_t *>(w + L.kt);
+    a.G = reinterpret_cast<float *>(w + L.G); a.decision = reinterpret_cast<int *>(w + L.decision);
+    a.g_out[0] = g1_out; a.g_out[1] = g2_out;
+    a.xbuf = reinterpret_cast<u64 *>(w + L.xbuf); a.ybuf = reinterpret_cast<u64 *>(w + L.ybuf);
+    a.status = reinterpret_cast<int *>(ws);
+    a.B = B; a.H = H; a.n = n; a.npad = L.npad; a.r = r; a.T = iters; a.C = L.C; a.groups = L.groups; a.srows = L.srows;
+    a.scale = 1.4426950408889634 / (double)eps;
+    a.eps_ln2 = (double)eps * 0.6931471805599453;
+    const size_t smem = (size_t)L.srows * 128 + kFixed;
+    auto kern = L.C > 1 ? stream_kernel<true> : stream_kernel<false>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)(L.C * L.groups));
+    if (L.C > 1) {
+        // the blocks of a group wait for one another: all must be resident
+        void *args[] = {&a};
+        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), grid, dim3(kThreads), args, smem, st);
+    } else {
+        kern<<<grid, kThreads, smem, st>>>(a);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
+    return stored_apply(a.kt, L.npad, a.G, beta, key_len, a.decision, v, out, reinterpret_cast<float *>(w + L.wpart), a.status, B, H, n, r, st);
+}
+
+} // namespace lot

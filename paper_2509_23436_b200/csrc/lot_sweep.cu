@@ -184,7 +184,9 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
         size_t per_block = (size_t)kSmemPerSM / occ - kSmPerBlockReserve;
         if (per_block > (size_t)kSmemPerBlock) per_block = kSmemPerBlock;
         const int cap = (int)((per_block - fixed) / ((size_t)RP * 4)) / step * step;
-        for (int C = 1; C <= sms * occ && C <= (n + 15) / 16; C += C < 32 ? 1 : C / 16) {
+        const int all_slots = sms * occ;
+        // every group size up to 32 blocks, then those that divide the blocks into whole groups
+        for (int C = 1; C <= all_slots && C <= (n + 15) / 16; C = C < 32 ? C + 1 : all_slots / C > 1 ? all_slots / (all_slots / C - 1) : all_slots + 1) {
             const int rows = (n + C - 1) / C, up = (rows + step - 1) / step * step, srows = up < cap ? up : cap;
             const size_t smem = fixed + (size_t)srows * RP * 4;
             int fit = (int)((size_t)kSmemPerSM / (smem + kSmPerBlockReserve));
@@ -195,14 +197,17 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
             const int resident = C == 1 ? (P < slots ? P : slots) : groups * C;
             const int rounds = C == 1 ? (P + slots - 1) / slots : (P + groups - 1) / groups;
             const double per_sm = (double)((resident + sms - 1) / sms);       // blocks that share an SM
-            const double entry = 0.035 / 1900.0;
-            const double lat = C == 1 ? 0.4 : C * RP <= kDirectWords ? 0.8 + 0.1 * C : 4.5;
-            const double mine = (double)srows * RP * entry * 1.5;
-            const double glob = (double)(rows > srows ? rows - srows : 0) * RP * 4.0 * resident;
+            // us: SM time per entry (issue and shared-memory reads), twice that for a block alone on its SM; the exchange as
+            // measured (0.7 for two blocks at RP = 256, 2.1 for 16, 3.9-4.6 with owners at 74-148); streamed rows at the L2's
+            // rate, at the HBM's when all of them exceed the L2, and never faster than one SM reads
+            const double entry = (RP <= 32 ? 0.055 : 0.045) / 1900.0;
+            const double lat = C == 1 ? 0.45 : C * RP <= kDirectWords ? 0.9 + 0.4 * C * RP / 1024.0 : 2.8 + 0.018 * C;
+            const double mine = 2.0 * rows * RP * entry, sm_us = per_sm * rows * RP * entry;
+            const double glob = (double)(rows > srows ? rows - srows : 0) * RP * 4.0, all = glob * resident;
             double it = lat + mine;
-            const double sm_us = per_sm * srows * RP * entry;
             if (sm_us > it) it = sm_us;
-            it += glob / (glob > 90e6 ? 5.5e6 : 10e6);
+            const double gl_us = all / (all > 90e6 ? 5.5e6 : 10e6), gl_sm = per_sm * glob / 50e3;
+            it += gl_us > gl_sm ? gl_us : gl_sm;
             const double t = rounds * (12 * it + 3.0);
             if (t < best_t) {
                 best_t = t;

@@ -42,6 +42,7 @@ struct SweepArgs {
     int C, groups;           // thread blocks per problem, problems in flight
     int srows;               // rows of a block's share that stay in shared memory
     int it0, it1;            // iterations this launch runs
+    int terms;               // bf16 tokens: terms a pivot is taken as in the first build (3: exact, 2)
     int first, close;        // start from the given potentials (else from the state in w, gref) / closing update last
     unsigned seq0;           // exchange sequence number this launch starts from
     double scale;            // log2(e)/eps
@@ -71,6 +72,7 @@ struct SweepApplyArgs {
     unsigned *counter;
     int B, H, nq, nk, d, r, RP;
     int skip;                // leading tokens that take no part
+    int terms;               // bf16 tensors: terms of a plan entry and of W' (3: float32 products, 2: hi + lo)
     int per_head;            // query side: Wp is [H][r][d]
     int chunks, rows_per_chunk;
 };

@@ -22,11 +22,11 @@ __device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr)
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
-// two floats as three packed bf16 pairs
-__device__ __forceinline__ void split3(float x, float y, uint32_t (&o)[3])
+// two floats as N packed bf16 pairs
+template <int N> __device__ __forceinline__ void split(float x, float y, uint32_t (&o)[N])
 {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < N; ++i) {
         const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
         o[i] = *reinterpret_cast<const uint32_t *>(&h);
         x -= __low2float(h);
@@ -59,7 +59,7 @@ __device__ __forceinline__ bool last_of_tile(unsigned *counter, int chunks)
 // step: the plan tile goes to shared memory as three bf16 planes (transposed on the way to the tensor cores), the values
 // as they are.  Warps: TP / 16 pivot tiles x channel groups x (rank 16, narrow heads) halves of the keys.
 // ---------------------------------------------------------------------------------------------------------------
-template <int TP, int D>
+template <int TP, int D, int N>
 __global__ void __launch_bounds__(kThreads, 2)
 apply_w_mma_kernel(SweepApplyArgs a)
 {
@@ -67,7 +67,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
     constexpr int PT = TP / 16, CG = 8 / PT < D / 16 ? 8 / PT : D / 16, KS = 8 / (PT * CG), NTW = D / 8 / CG;
     constexpr int NP = KT * TP / 4 / kThreads, NV = KT * D / 8 / kThreads;
     extern __shared__ __align__(128) uint8_t sm[];
-    uint8_t *sP = sm, *sV = sm + 3 * PLANE;
+    uint8_t *sP = sm, *sV = sm + N * PLANE;
     const int bh = blockIdx.z, b = bh / a.H, h = bh % a.H, chunk = blockIdx.x, t0 = blockIdx.y * TP;
     const int n = a.nk, r = a.r, d = a.d, RP = a.RP;
     int nv = n;
@@ -113,11 +113,11 @@ apply_w_mma_kernel(SweepApplyArgs a)
         for (int u = 0; u < NP; ++u) {
             const int idx = tid + u * kThreads, j = idx / (TP / 4), t = (idx % (TP / 4)) * 4;
             const float4 p = scaled(kr[u], wt[u], sc[u]);
-            uint32_t x[3], y[3];
-            split3(p.x, p.y, x);
-            split3(p.z, p.w, y);
+            uint32_t x[N], y[N];
+            split<N>(p.x, p.y, x);
+            split<N>(p.z, p.w, y);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2 *>(sP + i * PLANE + j * PP + t * 2) = make_uint2(x[i], y[i]);
+            for (int i = 0; i < N; ++i) *reinterpret_cast<uint2 *>(sP + i * PLANE + j * PP + t * 2) = make_uint2(x[i], y[i]);
         }
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
@@ -129,16 +129,16 @@ apply_w_mma_kernel(SweepApplyArgs a)
 #pragma unroll
         for (int s = 0; s < KT / 16 / KS; ++s) {
             const int j = (ks * (KT / 16 / KS) + s) * 16;
-            uint32_t af[3][4];
+            uint32_t af[N][4];
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+            for (int i = 0; i < N; ++i)
                 ldsm4_t(af[i], smem_addr(sP) + i * PLANE + (j + (lane & 7) + (mi >> 1) * 8) * PP + (pt * 16 + (mi & 1) * 8) * 2);
 #pragma unroll
             for (int nt = 0; nt < NTW; nt += 2) {
                 uint32_t bf[4];
                 ldsm4_t(bf, smem_addr(sV) + (j + (lane & 7) + (mi & 1) * 8) * PV + (cg * NTW * 8 + nt * 8 + (mi >> 1) * 8) * 2);
 #pragma unroll
-                for (int i = 2; i >= 0; --i) {
+                for (int i = N - 1; i >= 0; --i) {
                     logits::mma_bf16(acc[nt], af[i], bf[0], bf[1]);
                     logits::mma_bf16(acc[nt + 1], af[i], bf[2], bf[3]);
                 }
@@ -205,7 +205,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
 // Query side, bf16 tensors: out[i][c] = sum_t R_it W'[t][c].  Block = 128 queries x D channels; a warp's 16 plan rows come
 // from global memory straight into operand fragments, W' in steps of TS pivots through shared memory as three planes.
 // ---------------------------------------------------------------------------------------------------------------
-template <int TS, int D>
+template <int TS, int D, int N>
 __global__ void __launch_bounds__(kThreads, D <= 128 ? 2 : 1)
 apply_out_mma_kernel(SweepApplyArgs a)
 {
@@ -245,22 +245,22 @@ apply_out_mma_kernel(SweepApplyArgs a)
 #pragma unroll
         for (int u = 0; u < NW; ++u) {
             const int idx = tid + u * kThreads, t = idx / (D / 4), c = (idx % (D / 4)) * 4;
-            uint32_t x[3], y[3];
-            split3(wr[u].x, wr[u].y, x);
-            split3(wr[u].z, wr[u].w, y);
+            uint32_t x[N], y[N];
+            split<N>(wr[u].x, wr[u].y, x);
+            split<N>(wr[u].z, wr[u].w, y);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) *reinterpret_cast<uint2 *>(sW + i * PLANE + t * PW + c * 2) = make_uint2(x[i], y[i]);
+            for (int i = 0; i < N; ++i) *reinterpret_cast<uint2 *>(sW + i * PLANE + t * PW + c * 2) = make_uint2(x[i], y[i]);
         }
-        uint32_t af[TS / 16][3][4];
+        uint32_t af[TS / 16][N][4];
 #pragma unroll
         for (int k = 0; k < TS / 16; ++k)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float2 ww = w ? chain_ld2(w + tb + k * 16 + (e >> 1) * 8 + 2 * q) : make_float2(1.f, 1.f);
-                uint32_t o[3];
-                split3(kr[k][e].x * (ww.x * s[e & 1]), kr[k][e].y * (ww.y * s[e & 1]), o);
+                uint32_t o[N];
+                split<N>(kr[k][e].x * (ww.x * s[e & 1]), kr[k][e].y * (ww.y * s[e & 1]), o);
 #pragma unroll
-                for (int i = 0; i < 3; ++i) af[k][i][e] = o[i];
+                for (int i = 0; i < N; ++i) af[k][i][e] = o[i];
             }
         __syncthreads();
         if (tb + TS < r) fetch(tb + TS);
@@ -268,12 +268,12 @@ apply_out_mma_kernel(SweepApplyArgs a)
         for (int k = 0; k < TS / 16; ++k)
 #pragma unroll
             for (int cp = 0; cp < D / 16; ++cp) {
-                uint32_t bf[3][4];
+                uint32_t bf[N][4];
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < N; ++i)
                     ldsm4_t(bf[i], smem_addr(sW) + i * PLANE + (k * 16 + (lane & 7) + (mi & 1) * 8) * PW + (cp * 16 + (mi >> 1) * 8) * 2);
 #pragma unroll
-                for (int o = 2; o >= 0; --o)                      // the products of total order o, small ones first
+                for (int o = N - 1; o >= 0; --o)                      // the products of total order o, small ones first
 #pragma unroll
                     for (int i = 0; i <= o; ++i) {
                         logits::mma_bf16(acc[2 * cp], af[k][i], bf[o - i][0], bf[o - i][1]);
@@ -499,11 +499,11 @@ static cudaError_t big_smem(Kern kern, size_t bytes)
     return bytes > 40 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
 }
 
-template <int TP, int D>
+template <int TP, int D, int N>
 static cudaError_t launch_w(const SweepApplyArgs &a, cudaStream_t st)
 {
-    constexpr size_t smem = 3 * 64 * (TP + 8) * 2 + 64 * (D + 8) * 2;
-    auto kern = apply_w_mma_kernel<TP, D>;
+    constexpr size_t smem = N * 64 * (TP + 8) * 2 + 64 * (D + 8) * 2;
+    auto kern = apply_w_mma_kernel<TP, D, N>;
     cudaError_t e = big_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return chain_launch(kern, dim3(a.chunks, (a.r + TP - 1) / TP, a.B * a.H), kThreads, smem, st, a);
@@ -511,16 +511,23 @@ static cudaError_t launch_w(const SweepApplyArgs &a, cudaStream_t st)
 template <int TP>
 static cudaError_t launch_w_d(const SweepApplyArgs &a, cudaStream_t st)
 {
-    return a.d <= 64 ? launch_w<TP, 64>(a, st) : a.d <= 128 ? launch_w<TP, 128>(a, st) : launch_w<TP, 256>(a, st);
+    if (a.d <= 64) return a.terms == 2 ? launch_w<TP, 64, 2>(a, st) : launch_w<TP, 64, 3>(a, st);
+    return a.d <= 128 ? launch_w<TP, 128, 3>(a, st) : launch_w<TP, 256, 3>(a, st);
 }
-template <int TS, int D>
+template <int TS, int D, int N>
 static cudaError_t launch_out(const SweepApplyArgs &a, cudaStream_t st)
 {
-    constexpr size_t smem = 3 * TS * (D + 8) * 2;
-    auto kern = apply_out_mma_kernel<TS, D>;
+    constexpr size_t smem = N * TS * (D + 8) * 2;
+    auto kern = apply_out_mma_kernel<TS, D, N>;
     cudaError_t e = big_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return chain_launch(kern, dim3((a.nq + 127) / 128, a.B * a.H), kThreads, smem, st, a);
+}
+template <int TS>
+static cudaError_t launch_out_d(const SweepApplyArgs &a, cudaStream_t st)
+{
+    if (a.d <= 64) return a.terms == 2 ? launch_out<TS, 64, 2>(a, st) : launch_out<TS, 64, 3>(a, st);
+    return a.d <= 128 ? launch_out<16, 128, 3>(a, st) : launch_out<16, 256, 3>(a, st);
 }
 
 } // namespace sweep_apply
@@ -538,8 +545,7 @@ cudaError_t launch_sweep_apply_out(const SweepApplyArgs &a, int dtype, cudaStrea
 {
     using namespace sweep_apply;
     if (dtype != 0) {
-        if (a.RP == 16) return a.d <= 64 ? launch_out<16, 64>(a, st) : a.d <= 128 ? launch_out<16, 128>(a, st) : launch_out<16, 256>(a, st);
-        return a.d <= 64 ? launch_out<32, 64>(a, st) : a.d <= 128 ? launch_out<16, 128>(a, st) : launch_out<16, 256>(a, st);
+        return a.RP == 16 ? launch_out_d<16>(a, st) : launch_out_d<32>(a, st);
     }
     dim3 grid((a.nq + 63) / 64, (a.d + kCT - 1) / kCT, a.B * a.H);
     return chain_launch(a.RP == 16 ? apply_out_f32_kernel<16> : apply_out_f32_kernel<32>, grid, kThreads, 0, st, a);

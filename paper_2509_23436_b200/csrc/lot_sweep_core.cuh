@@ -399,8 +399,8 @@ __device__ __forceinline__ float take_word(const u64 *p, u64 first, unsigned tag
 // and leaves the total in kCopies places, each read by a share of the blocks (one place for all of 148 blocks to poll
 // took 5.9 us per exchange at RP = 256, eight take 4.4; reading every block's words takes 12.9 there, but 2.1 for 16
 // blocks and 0.7 for two).  Two buffers by parity: a block can be at most one exchange ahead of the others.
-template <int RP, int THREADS, bool MAX>
-__device__ __forceinline__ float group_columns(const SweepArgs &a, const Shared &S, float part, int group, int c, unsigned &seq)
+template <int RP, int THREADS, bool MAX, typename Args>
+__device__ __forceinline__ float group_columns(const Args &a, const Shared &S, float part, int group, int c, unsigned &seq)
 {
     const int C = a.C, tid = threadIdx.x;
     if (C == 1) return part;

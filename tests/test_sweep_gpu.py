@@ -93,3 +93,38 @@ def test_backward_matches_oracle(case):
             check_slice(runs[0][i][h], ref[i][h], 2e-2, f"{name} head {h}")
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+# the long path: bf16 kernel, d = 64, 32 < r <= 64; B, H, n, r, iters, eps, key mask, clustered
+LONG = [
+    (1, 2, 1, 33, 2, 0.1, False, False),
+    (1, 2, 127, 40, 5, 0.1, True, False),
+    (1, 1, 1000, 64, 0, 0.1, False, False),
+    (2, 3, 1153, 33, 4, 0.05, True, False),
+    (1, 1, 20000, 64, 4, 0.1, False, False),               # rows streamed
+    (40, 8, 300, 64, 3, 0.1, True, False),                 # one block per problem
+    (1, 3, 65536, 50, 2, 0.1, False, False),
+    (1, 2, 3000, 64, 8, 0.02, False, True),                # rebuilt kernel
+    (1, 1, 1500, 50, 12, 0.01, True, True),                # lost column sums, final potentials far apart
+]
+
+
+@pytest.mark.parametrize("case", LONG, ids=lambda c: "B%d-H%d-n%d-r%d-T%d-eps%g%s%s" % (
+    c[:6] + ("-mask" if c[6] else "", "-peaked" if c[7] else "")))
+def test_long_path_matches_oracle(case):
+    B, H, n, r, iters, eps, masked, peaked = case
+    x = synth.make(B, H, n, 64, r, seed=9800 + n + r, dtype=BF16, eps=eps, iters=iters,
+                   key_len_range=(max(1, n // 2), n) if masked else None, qk="mixture" if peaked else "normal")
+    lot.lot_debug_hook(4, 4)
+    try:
+        assert lot.lot_path(lot.LOT_BF16, B, H, n, 64, r, iters) == 4
+        res, again = gpu_forward(x, want_g=True), gpu_forward(x)
+    finally:
+        lot.lot_debug_hook(4, -1)
+    assert res["status"] == 0 and np.array_equal(res["out"], again["out"])
+    slices = sorted({(0, 0), (B // 2, H // 2), (B - 1, H - 1)})
+    outs, g1s, g2s = oracle_slices(x, slices, return_potentials=True)
+    for (b, h), o, g1, g2 in zip(slices, outs, g1s, g2s):
+        check_slice(res["out"][b, h], o, 2e-2, f"slice {(b, h)}")
+        for got, ref in ((res["g1"][b, h], g1), (res["g2"][b, h], g2)):
+            assert np.abs(got - ref).max() <= 1e-3 * max(1.0, np.abs(ref).max())
