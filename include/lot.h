@@ -171,9 +171,10 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *      column mass below 2^-80) is recomputed by the streamed kernels, which are launched behind it
  *      and return at once otherwise (device flag LOT_DEV_RECOMPUTED).  It can run many more shapes
  *      (lot_debug_hook what = 4), but measured no faster there.
- *   4  the long path (same tensors, 32 < r <= 64): one cooperative launch builds that bf16 kernel and runs all passes
+ *   4  the long path (same tensors, 16 < r <= 64): one cooperative launch builds that bf16 kernel and runs all passes
  *      on it, a group of thread blocks per problem keeping what it can of it in shared memory; two apply kernels.
- *      Taken for moderate row counts, n <= 1200 and few slices; path 0 takes smaller problems and r <= 16.
+ *      Taken up to 300000 rows B H n (r <= 32: from 100000 to 200000) and for n <= 1200; path 0 takes r <= 16 and the smaller
+ *      problems of r <= 32.
  *   3  the slice path (same tensors; n <= 512 and 16 ceil(n/16) x (r padded to 16, 32 or 64) <= 16384): a pair of
  *      thread blocks per (batch, head) slice, one for each side, keeps the side's Gibbs kernel in float32 in shared
  *      memory for all iterations (warp-level tensor-core products); only the r x d intermediate crosses, inside the

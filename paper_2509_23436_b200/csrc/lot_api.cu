@@ -231,20 +231,20 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
     const int force = g_force_path.load();
     if (force == kPathGeneral) return kPathGeneral;
     if (force == kPathStreamed) return kPathStreamed;
-    if (force == kPathLong && r > 32) return kPathLong;
+    if (force == kPathLong && r > 16) return kPathLong;
     if (force == kPathResident) return res_ok ? kPathResident : kPathStreamed;
     // short sequences: one thread block per slice, everything on chip, exact float32 logits
     if (slice_ok) return kPathSlice;
-    // Measured at T = 10 against the streamed and the resident kernels (B200): the general path's float32 kernel wins with
-    // few pivots everywhere (r = 16: 1.05 to 4.5 times), else with few rows in all or short sequences (r = 32: 1.4 to 4
-    // times; r = 64, at most 50000 rows: 1.7 to 3), the bf16 kernel of the long path a little beyond (n = 4096, 16
-    // slices: 89 us against 100 and 116; n = 1000, 256 slices: 202 against 321) and where there are few slices.
+    // Measured at T = 10 (B200).  r <= 16: the general path's float32 kernel, 1.05 to 4.5 times the streamed kernel's speed
+    // everywhere.  r <= 32: it too with few rows in all or short sequences (65536 rows 71 us against 76 on the long path and
+    // 126 streamed), then the long path (131072 rows: 113 against 120 and 143) as long as its stored kernel, padded to 64
+    // pivots, stays in the L2 beside the rest.  Above that the long path takes everything up to 300000 rows (n = 2048, 16
+    // slices 64 us against 73 and 114; n = 16384, 16 slices 174 against 190; 24 slices 264 against 252) and all short
+    // sequences (n = 1024, 512 slices: 301 against 461).
     if (B >= 1 && n >= 1) {
-        const long long slices = (long long)B * H, rows = slices * n;
-        if (r <= 16) return kPathGeneral;
-        if (r <= 32 && (n <= 1200 || rows <= 160000)) return kPathGeneral;
-        if (r > 32 && rows <= 50000) return kPathGeneral;
-        if (r > 32 && (n <= 1200 || rows <= 100000 || slices <= 6)) return kPathLong;
+        const long long rows = (long long)B * H * n;
+        if (r <= 16 || (r <= 32 && (n <= 1200 || rows <= 100000))) return kPathGeneral;
+        if (r <= 32 ? rows <= 200000 : n <= 1200 || rows <= 300000) return kPathLong;
     }
     // Measured on B200 (see the design notes): the resident kernel wins where the streamed one has no stored-kernel
     // passes (r <= 32, every pass recomputes logits and exponentials) and every thread block holds its whole share at

@@ -12,6 +12,7 @@
 // grid barrier.  Slices whose stored kernel cannot carry the final potentials (decision word 2) were applied by the
 // Sinkhorn kernel itself and are skipped here.  Four tiles are in flight per block (TMA ring, one accumulator per ring
 // stage in the output kernel), so the tensor-core latency of one tile overlaps the CUDA-core work on its neighbours.
+#include "lot_chain.cuh"
 #include "lot_common.cuh"
 #include "lot_internal.h"
 #include "lot_sm100.cuh"
@@ -48,6 +49,26 @@ struct alignas(64) ApplyParams {
     int B, H, n, r, TPS, NT, ctas, maxslots;
 };
 
+// Loads of what the kernels before this one wrote: they stay behind chain_wait.
+__device__ __forceinline__ int ld_later(const int *p)
+{
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_later(const float *p)
+{
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_later2(const float *p)
+{
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ int range_lo(const ApplyParams &P, int cta) { return (int)(((long long)cta * P.NT) / P.ctas); }
 __device__ __forceinline__ int cta_of_tile(const ApplyParams &P, int u) { return (int)((((long long)u + 1) * P.ctas - 1) / P.NT); }
 __device__ __forceinline__ int key_count(const ApplyParams &P, int s)
@@ -57,7 +78,7 @@ __device__ __forceinline__ int key_count(const ApplyParams &P, int s)
 __device__ __forceinline__ bool slice_here(const ApplyParams &P, int s)
 {
     const int BH = P.B * P.H;
-    return __ldcg(P.decision + s) != 2 && __ldcg(P.decision + BH + s) != 2;
+    return ld_later(P.decision + s) != 2 && ld_later(P.decision + BH + s) != 2;
 }
 
 // Bounded mbarrier wait (cold part out of line, plain arguments).
@@ -104,7 +125,7 @@ struct Sync {
 // Weights w_t = 2^(G_t - max G) of one (slice, side) into shared memory (one warp; columns >= r get 0).
 __device__ __forceinline__ void weights_to_smem(const float *G, int r, float *sW, int lane)
 {
-    const float g0 = lane < r ? __ldcg(G + lane) : neg_inf(), g1 = lane + 32 < r ? __ldcg(G + lane + 32) : neg_inf();
+    const float g0 = lane < r ? ld_later(G + lane) : neg_inf(), g1 = lane + 32 < r ? ld_later(G + lane + 32) : neg_inf();
     float mx = fmaxf(g0, g1);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
@@ -173,6 +194,7 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *sTmem;
+    chain_wait();
     const int BH = P.B * P.H;
     const int u0 = range_lo(P, blockIdx.x), u1 = range_lo(P, blockIdx.x + 1);
     const int s_lo = u0 < u1 ? u0 / P.TPS : 0, s_hi = u0 < u1 ? (u1 - 1) / P.TPS : -1;
@@ -306,6 +328,7 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
             (void)wtid;
         }
     }
+    chain_next();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, 64); }
@@ -352,6 +375,7 @@ apply_out_kernel(const __grid_constant__ ApplyParams P)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *sTmem;
+    chain_wait();
     const int u0 = range_lo(P, blockIdx.x), u1 = range_lo(P, blockIdx.x + 1);
     const int s_lo = u0 < u1 ? u0 / P.TPS : 0, s_hi = u0 < u1 ? (u1 - 1) / P.TPS : -1;
     auto seg_range = [&](int s, int &t0, int &t1) {
@@ -433,14 +457,20 @@ apply_out_kernel(const __grid_constant__ ApplyParams P)
 #pragma unroll
                 for (int e = 0; e < 16; ++e) acc[e] = 0.f;
                 const float *src0 = P.wpart + (size_t)s * P.maxslots * (64 * kDK) + 32 * quad + 2 * cq;
-                for (int sl = 0; sl < wslots; ++sl) {
-                    const float *src = src0 + (size_t)sl * (64 * kDK);
+                // four slots requested together: one after the other, ten slots' L2 round trips were 4 us at n = 4096, H = 16
+                for (int s4 = 0; s4 < wslots; s4 += 4) {
+                    float2 x[4][8];
 #pragma unroll
-                    for (int rep = 0; rep < 4; ++rep) {
-                        const float2 a = __ldcg(reinterpret_cast<const float2 *>(src + tA * kDK + rep * 8));
-                        const float2 b = __ldcg(reinterpret_cast<const float2 *>(src + tB * kDK + rep * 8));
-                        acc[rep * 4 + 0] += a.x; acc[rep * 4 + 1] += a.y; acc[rep * 4 + 2] += b.x; acc[rep * 4 + 3] += b.y;
+                    for (int u = 0; u < 4; ++u) {
+                        const float *src = src0 + (size_t)(s4 + u) * (64 * kDK);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            x[u][e] = s4 + u < wslots ? ld_later2(src + (e & 1 ? tB : tA) * kDK + (e >> 1) * 8) : make_float2(0.f, 0.f);
                     }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) { acc[2 * e] += x[u][e].x; acc[2 * e + 1] += x[u][e].y; }
                 }
                 const float mass = kv > 0 ? 1.f / (float)kv : 0.f;
                 const float cA = tA < P.r ? sW[tA] * mass / __ldg(P.beta + h * P.r + tA) : 0.f;
@@ -588,11 +618,9 @@ cudaError_t stored_apply(const void *kt, int npad, const float *G, const float *
             attr[dev] = true;
         }
     }
-    apply_w_kernel<<<P.ctas, kThreads, PlanW::total, st>>>(P);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = chain_launch(apply_w_kernel, dim3(P.ctas), kThreads, PlanW::total, st, P);
     if (e != cudaSuccess) return e;
-    apply_out_kernel<<<P.ctas, kThreads, PlanO::total, st>>>(P);
-    return cudaGetLastError();
+    return chain_launch(apply_out_kernel, dim3(P.ctas), kThreads, PlanO::total, st, P);
 }
 
 } // namespace lot

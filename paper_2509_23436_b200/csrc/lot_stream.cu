@@ -1,4 +1,4 @@
-// Long sequences with 32 < r <= 64 pivots (bf16 tensors, d = 64): the Gibbs kernel as bf16, built and iterated on in one
+// Long sequences with 16 < r <= 64 pivots (bf16 tensors, d = 64): the Gibbs kernel as bf16, built and iterated on in one
 // launch, then applied by the tensor-core kernels of lot_apply.cu.
 //
 // As in lot_sweep.cu a problem (one side of one slice) is shared by a group of C blocks and every pass is two
@@ -6,8 +6,11 @@
 // streamed path has always had; potentials to about 1e-4): half the bytes, so a pass over n = 16384, H = 16 reads 67 MB, of
 // which the blocks keep the first rows of their share in shared memory and the rest comes from L2.  Each block
 // computes the logits of its own rows (warp-level products, Z as bf16 hi + lo), so building one group's kernel
-// overlaps another's passes.  When all problems together exceed the L2, groups are made larger and work through the problems
+// overlaps another's passes.  At n = 4096, H = 16, r = 64, T = 10: 47 us (15 of them building) and 26 for the apply kernels,
+// against 117 in all on the streamed path; at n = 16384 128 (46) + 42 against 190.  A pass is bound by latency: per
+// scheduler four warps, whose registers hold the weights, the column sums and two rows, issue in 40% of the cycles.  When all problems together exceed the L2, groups are made larger and work through the problems
 // in rounds, so that what is iterated on stays in the L2.
+#include "lot_chain.cuh"
 #include "lot_sweep_core.cuh"
 
 namespace lot {
@@ -18,8 +21,11 @@ using namespace sweep;
 constexpr int kThreads = 256, kD = 64, RP = 64;
 constexpr int kRowsStep = 64;              // rows per step of a block: eight a warp, four lanes a row
 constexpr int kZPitch = 144;               // bytes per staged pivot row (conflict-free ldmatrix)
-constexpr int kWork = 2 * RP * kZPitch;    // staged pivots (hi, lo), later the column reduction
-constexpr int kFixed = kWork + kThreads * 4 + RP * 16 + 64;
+constexpr int kStage = 2 * RP * kZPitch;   // staged pivots (hi, lo): in the kernel rows' area while building
+constexpr int kWork = kThreads / 32 * RP * 4;
+constexpr int kFixed = kWork + kThreads * 4 + RP * 20 + 64;
+
+__host__ __device__ constexpr int area_bytes(int srows) { return srows * 128 > kStage ? srows * 128 : kStage; }
 
 struct StreamArgs {
     const __nv_bfloat16 *x[2];
@@ -36,20 +42,23 @@ struct StreamArgs {
 };
 
 struct Mem {
-    uint8_t *K;                // [srows][128 bytes]
+    uint8_t *K, *z;            // [srows][128 bytes]; its last bytes hold the pivots while building
+    float *before;             // the weights before the last update
     Shared s;
 };
 
 __device__ __forceinline__ Mem carve16(uint8_t *p, int srows)
 {
     Mem m;
-    m.K = p; p += (size_t)srows * 128;
+    m.K = p; p += area_bytes(srows);
+    m.z = p - kStage;
     m.s.K = nullptr;
     m.s.gref = reinterpret_cast<double *>(p); p += RP * 8;
     m.s.work = p; p += kWork;
     m.s.ref = reinterpret_cast<float *>(p); p += kThreads * 4;
     m.s.w = reinterpret_cast<float *>(p); p += RP * 4;
     m.s.tgt = reinterpret_cast<float *>(p); p += RP * 4;
+    m.before = reinterpret_cast<float *>(p); p += RP * 4;
     m.s.flag = reinterpret_cast<volatile int *>(p);    // [0], [1] as in the sweep kernels; [2], [3]: see solve16
     return m;
 }
@@ -84,7 +93,13 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi)
     return *reinterpret_cast<const uint32_t *>(&t);
 }
 
-// Pivots of the head in base-2 logit units as bf16 hi + lo into the work area.
+// The order of the products' operands is free as long as both sides agree.  A lane's token values of two steps are eight
+// neighbours in memory, and its eight results of four tiles are eight neighbouring pivots: 16-byte loads and stores, a
+// quarter of the requests of the instruction's own layout (whose 4-byte loads and 8-byte stores held the load-store
+// unit for most of the 72 us that building took at n = 16384, H = 16).
+__device__ __forceinline__ int pivot_of(int j, int q, int e) { return 32 * (j >> 2) + 8 * q + 2 * (j & 3) + e; }
+
+// Pivots of the head in base-2 logit units as bf16 hi + lo.
 __device__ __forceinline__ void stage_pivots(const StreamArgs &a, const Mem &m, const Part &P)
 {
     const float *z = a.z + (size_t)P.h * a.r * kD;
@@ -97,25 +112,31 @@ __device__ __forceinline__ void stage_pivots(const StreamArgs &a, const Mem &m, 
     }
 #pragma unroll
     for (int u = 0; u < RP * kD / 2 / kThreads; ++u) {
-        const int idx = threadIdx.x + u * kThreads, t = idx / (kD / 2), c2 = (idx % (kD / 2)) * 2;
+        const int idx = threadIdx.x + u * kThreads, t = idx / (kD / 2), c = (idx % (kD / 2)) * 2;
+        const int row = (t & 32) | (t & 6) << 2 | (t >> 2 & 6) | (t & 1);                     // pivot_of(row / 8, ...) = t
+        const int col = (c & 32) | (c & 4) << 2 | (c & 2) << 2 | (c >> 2 & 6);                // as fetch_tokens
         const float x0 = zz[u].x * scale, x1 = zz[u].y * scale;
         const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-        *reinterpret_cast<__nv_bfloat162 *>(m.s.work + t * kZPitch + c2 * 2) = h;
-        *reinterpret_cast<uint32_t *>(m.s.work + (RP + t) * kZPitch + c2 * 2) = pack2(x0 - __low2float(h), x1 - __high2float(h));
+        *reinterpret_cast<__nv_bfloat162 *>(m.z + row * kZPitch + col * 2) = h;
+        *reinterpret_cast<uint32_t *>(m.z + (RP + row) * kZPitch + col * 2) = pack2(x0 - __low2float(h), x1 - __high2float(h));
     }
     __syncthreads();
 }
 
-// Logits of 16 rows a warp, all pivots: tokens straight from global memory, pivots from the work area.
+// Logits of 16 rows a warp, all pivots: tokens straight from global memory, pivots from shared memory.
 __device__ __forceinline__ void fetch_tokens(uint32_t (&a)[kD / 16][4], const Part &P, int rt)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
 #pragma unroll
-    for (int ks = 0; ks < kD / 16; ++ks)
+    for (int e = 0; e < 2; ++e)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int i = rt + warp * 16 + g + (e & 1) * 8;
-            a[ks][e] = i < P.nrows ? __ldg(reinterpret_cast<const unsigned *>(P.x + (size_t)i * kD + ks * 16 + (e >> 1) * 8 + 2 * q)) : 0u;
+        for (int kk = 0; kk < kD / 32; ++kk) {
+            const int i = rt + warp * 16 + g + e * 8;
+            const uint4 v = i < P.nrows ? __ldg(reinterpret_cast<const uint4 *>(P.x + (size_t)i * kD + kk * 32 + 8 * q)) : make_uint4(0, 0, 0, 0);
+            a[2 * kk][e] = v.x;
+            a[2 * kk][2 + e] = v.y;
+            a[2 * kk + 1][e] = v.z;
+            a[2 * kk + 1][2 + e] = v.w;
         }
 }
 __device__ __forceinline__ void tile_logits(float (&L)[RP / 8][4], const uint32_t (&a)[kD / 16][4], uint32_t zb)
@@ -154,50 +175,57 @@ __device__ __noinline__ void build16(const StreamArgs *ap, int p, int c)
     uint32_t tok[kD / 16][4];
     fetch_tokens(tok, P, 0);
     stage_pivots(a, m, P);
-    const uint32_t zb = smem_addr(m.s.work);
+    const uint32_t zb = smem_addr(m.z);
+    const int direct = min(P.ns, (int)(m.z - m.K) / 128);       // rows in front of the pivots
     for (int rt = 0; rt < P.nrows; rt += 128) {
         float L[RP / 8][4];
         tile_logits(L, tok, zb);
         if (rt + 128 < P.nrows) fetch_tokens(tok, P, rt + 128);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int i = rt + warp * 16 + g + 8 * h;
-            float mx = neg_inf();
+        if (REF) {
 #pragma unroll
             for (int j = 0; j < RP / 8; ++j)
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int t = 8 * j + 2 * q + e;
-                    float l = L[j][2 * h + e];
-                    if (REF) l += (float)m.s.gref[t];
-                    if (t >= a.r) l = neg_inf();
-                    L[j][2 * h + e] = l;
-                    mx = fmaxf(mx, l);
-                }
+                for (int e = 0; e < 4; ++e) L[j][e] += (float)m.s.gref[pivot_of(j, q, e & 1)];
+        }
+        if (a.r < RP) {
+#pragma unroll
+            for (int j = 0; j < RP / 8; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (pivot_of(j, q, e & 1) >= a.r) L[j][e] = neg_inf();
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = rt + warp * 16 + g + 8 * h;
+            float mx = fmaxf(L[0][2 * h], L[0][2 * h + 1]);
+#pragma unroll
+            for (int j = 1; j < RP / 8; ++j) mx = fmaxf(mx, fmaxf(L[j][2 * h], L[j][2 * h + 1]));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2)) - kKernelTop;
-            // neighbouring lanes trade halves of neighbouring tiles: a lane stores 8 bytes, a quad 32 in a row
+            uint32_t o[RP / 8];
 #pragma unroll
-            for (int j = 0; j < RP / 8; j += 2) {
-                const uint32_t u0 = pack2(ex2(L[j][2 * h] - mx), ex2(L[j][2 * h + 1] - mx));
-                const uint32_t u1 = pack2(ex2(L[j + 1][2 * h] - mx), ex2(L[j + 1][2 * h + 1] - mx));
-                const uint32_t got = __shfl_xor_sync(0xffffffffu, q & 1 ? u0 : u1, 1);
-                const uint2 o = q & 1 ? make_uint2(got, u1) : make_uint2(u0, got);
-                const int at = (8 * (j + (q & 1)) + 4 * (q >> 1)) * 2;
-                if (i < P.nrows) {
-                    *reinterpret_cast<uint2 *>(P.g + (size_t)i * 128 + at) = o;
-                    if (i < P.ns) *reinterpret_cast<uint2 *>(m.K + (size_t)i * 128 + at) = o;
-                }
+            for (int j = 0; j < RP / 8; ++j) o[j] = pack2(ex2(L[j][2 * h] - mx), ex2(L[j][2 * h + 1] - mx));
+            if (i >= P.nrows) continue;
+            // odd rows store their second half first: eight lanes then cover all banks
+            const bool odd = g & 1;
+            const uint4 o0 = odd ? make_uint4(o[4], o[5], o[6], o[7]) : make_uint4(o[0], o[1], o[2], o[3]);
+            const uint4 o1 = odd ? make_uint4(o[0], o[1], o[2], o[3]) : make_uint4(o[4], o[5], o[6], o[7]);
+            const int at = i * 128 + 16 * q + (odd ? 64 : 0), flip = odd ? -64 : 64;
+            *reinterpret_cast<uint4 *>(P.g + at) = o0;
+            *reinterpret_cast<uint4 *>(P.g + at + flip) = o1;
+            if (i < direct) {
+                *reinterpret_cast<uint4 *>(m.K + at) = o0;
+                *reinterpret_cast<uint4 *>(m.K + at + flip) = o1;
             }
         }
     }
-    const uint4 zero = make_uint4(0, 0, 0, 0);
-    for (int idx = threadIdx.x; idx < (P.steps * kRowsStep - P.ns) * 8; idx += kThreads)
-        *reinterpret_cast<uint4 *>(m.K + (size_t)P.ns * 128 + idx * 16) = zero;
+    __syncthreads();                                            // the pivots are done with
+    for (int idx = direct * 8 + threadIdx.x; idx < P.steps * kRowsStep * 8; idx += kThreads)
+        *reinterpret_cast<uint4 *>(m.K + idx * 16) = idx < P.ns * 8 ? __ldcg(reinterpret_cast<const uint4 *>(P.g + idx * 16)) : make_uint4(0, 0, 0, 0);
     if (c == a.C - 1) {
         const int end = min((P.nv + 127) & ~127, a.npad) - P.nv;
         uint8_t *o = a.kt + ((size_t)(P.side * a.B * a.H + P.slice) * a.npad + P.nv) * 128;
-        for (int idx = threadIdx.x; idx < end * 8; idx += kThreads) *reinterpret_cast<uint4 *>(o + (size_t)idx * 16) = zero;
+        for (int idx = threadIdx.x; idx < end * 8; idx += kThreads) *reinterpret_cast<uint4 *>(o + (size_t)idx * 16) = make_uint4(0, 0, 0, 0);
     }
     __syncthreads();
 }
@@ -206,25 +234,21 @@ __device__ __noinline__ void build16(const StreamArgs *ap, int p, int c)
 // lanes of a 128-byte phase, two rows, then cover all banks without a permuted layout, and the first halving of the
 // column sums is an exchange without selects.
 struct LaneMap {
-    uint32_t k[2], w[2], red, own;
-    int i0, cl, odd;
+    uint32_t k, w, red, own;             // the second chunk of a row is at k ^ 64, its weights at w ^ 128
+    int i0, at;
 };
 
 __device__ __forceinline__ LaneMap make_map16(const Mem &m)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 2;
     LaneMap L;
-    L.cl = lane & 3;
-    L.odd = sub & 1;
+    const int chunk = (sub & 1) * 4 + (lane & 3);
     L.i0 = warp * 8 + sub;
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        const int chunk = (v ^ L.odd) * 4 + L.cl;
-        L.k[v] = smem_addr(m.K) + L.i0 * 128 + chunk * 16;
-        L.w[v] = smem_addr(m.s.w) + chunk * 32;
-    }
+    L.at = L.i0 * 128 + chunk * 16;
+    L.k = smem_addr(m.K) + L.at;
+    L.w = smem_addr(m.s.w) + chunk * 32;
     // after the halvings: two columns of chunk (odd, cl)
-    const int col = (L.odd * 4 + L.cl) * 8 + ((lane & 8) ? 4 : 0) + ((lane & 16) ? 2 : 0);
+    const int col = chunk * 8 + ((lane & 8) ? 4 : 0) + ((lane & 16) ? 2 : 0);
     L.red = smem_addr(m.s.work) + (warp * RP + col) * 4;
     L.own = smem_addr(m.s.work) + threadIdx.x * 4;
     return L;
@@ -234,8 +258,8 @@ __device__ __forceinline__ void load_weights16(const LaneMap &L, u64 (&w)[8])
 {
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
-        lds2(w[4 * v], w[4 * v + 1], L.w[v]);
-        lds2(w[4 * v + 2], w[4 * v + 3], L.w[v] + 16);
+        lds2(w[4 * v], w[4 * v + 1], L.w ^ (v * 128));
+        lds2(w[4 * v + 2], w[4 * v + 3], (L.w ^ (v * 128)) + 16);
     }
 }
 
@@ -267,41 +291,54 @@ __device__ __forceinline__ uint4 lds4(uint32_t addr)
     return v;
 }
 
+__device__ __forceinline__ uint4 ldg_or_zero(bool in, const uint8_t *p)
+{
+    return in ? __ldcg(reinterpret_cast<const uint4 *>(p)) : make_uint4(0, 0, 0, 0);
+}
+
+// Column sums of the block's rows.  Rows that are not in shared memory come from L2, kAhead steps requested together, with
+// steps from shared memory between the request and the use.  Rows kept in registers, or the next request made before the
+// last is used, take registers that the loop has not got: 8.2 us a pass at n = 16384, H = 16 against 9.1 and 10.0.
 __device__ __forceinline__ void pass16(const LaneMap &L, const Part &P, const u64 (&w)[8], u64 (&acc)[8])
 {
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = 0;
-    int st = 0;
+    constexpr int kAhead = 2;
+    uint32_t k = L.k;
+    const uint32_t end = k + P.steps * (kRowsStep * 128);
+    int left = P.nrows - P.ns;
+    if (left > 0) {
+        const uint8_t *g = P.g + (size_t)(P.nrows - left) * 128 + L.at;
+        const int flip = 64 - 2 * (L.at & 64);
+        const uint32_t between = (P.steps / ((left + kAhead * kRowsStep - 1) / (kAhead * kRowsStep))) * (kRowsStep * 128);
 #pragma unroll 1
-    for (; st + 2 <= P.steps; st += 2) {
-        const uint4 a0 = lds4(L.k[0] + st * (kRowsStep * 128)), b0 = lds4(L.k[1] + st * (kRowsStep * 128));
-        const uint4 a1 = lds4(L.k[0] + (st + 1) * (kRowsStep * 128)), b1 = lds4(L.k[1] + (st + 1) * (kRowsStep * 128));
+        for (; left > 0; left -= kAhead * kRowsStep, g += kAhead * kRowsStep * 128) {
+            uint4 ra[kAhead], rb[kAhead];
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const bool in = u * kRowsStep + L.i0 < left;
+                ra[u] = ldg_or_zero(in, g + u * (kRowsStep * 128));
+                rb[u] = ldg_or_zero(in, g + u * (kRowsStep * 128) + flip);
+            }
+#pragma unroll 1
+            for (const uint32_t stop = k + between; k < stop; k += kRowsStep * 128) row16(lds4(k), lds4(k ^ 64), w, acc);
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) row16(ra[u], rb[u], w, acc);
+        }
+    }
+#pragma unroll 1
+    for (; k + kRowsStep * 128 < end; k += 2 * kRowsStep * 128) {
+        const uint4 a0 = lds4(k), b0 = lds4(k ^ 64), a1 = lds4(k + kRowsStep * 128), b1 = lds4((k ^ 64) + kRowsStep * 128);
         row16(a0, b0, w, acc);
         row16(a1, b1, w, acc);
     }
-    if (st < P.steps) row16(lds4(L.k[0] + st * (kRowsStep * 128)), lds4(L.k[1] + st * (kRowsStep * 128)), w, acc);
-    // rows that do not fit: kAhead steps requested together (a second set in flight spilled: 30 us a pass at n = 16384)
-    constexpr int kAhead = 4;
-    const uint8_t *g0 = P.g + (size_t)(P.ns + L.i0) * 128 + (L.odd * 4 + L.cl) * 16;
-    const int flip = (1 - 2 * L.odd) * 64;               // from the lane's first chunk to its second
-#pragma unroll 1
-    for (int left = P.nrows - P.ns - L.i0; left > -L.i0; left -= kAhead * kRowsStep, g0 += kAhead * kRowsStep * 128) {
-        uint4 ra[kAhead], rb[kAhead];
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            const bool in = u * kRowsStep < left;
-            ra[u] = in ? __ldcg(reinterpret_cast<const uint4 *>(g0 + u * (kRowsStep * 128))) : make_uint4(0, 0, 0, 0);
-            rb[u] = in ? __ldcg(reinterpret_cast<const uint4 *>(g0 + u * (kRowsStep * 128) + flip)) : make_uint4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) row16(ra[u], rb[u], w, acc);
-    }
+    if (k < end) row16(lds4(k), lds4(k ^ 64), w, acc);
 }
 
-// One iteration, as in lot_sweep_core.cuh: thread t < r gets its column's weight before and after.
+// One iteration, as in lot_sweep_core.cuh: the weights in shared memory and those before them.
 template <bool GROUP>
-__device__ __forceinline__ bool iterate16(const StreamArgs &a, const Mem &m, const Part &P, const LaneMap &L, u64 (&w)[8], float tgt,
-                                          int group, int c, unsigned &seq, float &wold, float &wnew)
+__device__ __forceinline__ bool iterate16(const StreamArgs &a, const Mem &m, const Part &P, const LaneMap &L, u64 (&w)[8], int group, int c,
+                                          unsigned &seq)
 {
     u64 acc[8];
     pass16(L, P, w, acc);
@@ -335,9 +372,9 @@ __device__ __forceinline__ bool iterate16(const StreamArgs &a, const Mem &m, con
     }
     if (GROUP) tot = group_columns<RP, kThreads, false>(a, m.s, tot, group, c, seq);
     if ((int)threadIdx.x < a.r) {
-        wold = wnew;
-        wnew = tgt * rcp(tot);
+        const float wnew = m.s.tgt[threadIdx.x] * rcp(tot);
         if (out_of_range(wnew)) m.s.flag[1] = 1;
+        m.before[threadIdx.x] = m.s.w[threadIdx.x];
         m.s.w[threadIdx.x] = wnew;
     }
     __syncthreads();
@@ -380,7 +417,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
             uint32_t tok[kD / 16][4];
             fetch_tokens(tok, P, rt);
             float L[RP / 8][4];
-            tile_logits(L, tok, smem_addr(m.s.work));
+            tile_logits(L, tok, smem_addr(m.z));
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const bool ok = rt + warp * 16 + g + 8 * h < P.nrows;
@@ -389,7 +426,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
                 for (int j = 0; j < RP / 8; ++j)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const int t = 8 * j + 2 * q + e;
+                        const int t = pivot_of(j, q, e);
                         L[j][2 * h + e] = t < a.r ? L[j][2 * h + e] + (float)m.s.gref[t] : neg_inf();
                         mx = fmaxf(mx, L[j][2 * h + e]);
                     }
@@ -407,12 +444,11 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
                         for (int e = 0; e < 2; ++e) {
                             const float x = L[j][2 * h + e] - M;
                             if (round == 0) col[j][e] = fmaxf(col[j][e], x);
-                            else if (m.s.tgt[8 * j + 2 * q + e] > neg_inf()) col[j][e] += ex2(x - m.s.tgt[8 * j + 2 * q + e]);
+                            else if (m.before[pivot_of(j, q, e)] > neg_inf()) col[j][e] += ex2(x - m.before[pivot_of(j, q, e)]);
                         }
                 }
             }
         }
-        __syncthreads();                                           // the staged pivots are done with
 #pragma unroll
         for (int j = 0; j < RP / 8; ++j)
 #pragma unroll
@@ -423,7 +459,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
                     const float o = __shfl_xor_sync(0xffffffffu, v, off);
                     v = round == 0 ? fmaxf(v, o) : v + o;
                 }
-                if (g == 0) red[warp * RP + 8 * j + 2 * q + e] = v;
+                if (g == 0) red[warp * RP + pivot_of(j, q, e)] = v;
             }
         __syncthreads();
         float tot = round == 0 ? neg_inf() : 0.f;
@@ -434,7 +470,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
         __syncthreads();
         if (round == 0) {
             kap = tot;
-            if (threadIdx.x < RP) m.s.tgt[threadIdx.x] = kap;       // the maxima
+            if (threadIdx.x < RP) m.before[threadIdx.x] = kap;      // the maxima
         } else {
             out = kap + lg2(tot);
         }
@@ -443,8 +479,8 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
     return out;
 }
 
-// The iterations of a problem on the kernel as built.  flag[2] = 1 where recover16 has to go on from iteration flag[3], with
-// the weights before and after that update in ref.  Returns the sequence number.
+// The iterations of a problem on the kernel as built.  flag[2] = 1 where recover16 has to go on from iteration flag[3].
+// Returns the sequence number.
 template <bool GROUP>
 __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
 {
@@ -452,22 +488,17 @@ __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group,
     const StreamArgs &a = *ap;
     const Mem m = carve16(smem, a.srows);
     const Part P = locate16(a, p, c);
-    const int tid = threadIdx.x, r = a.r;
-    const float tgt = tid < r ? __ldg(a.beta + P.h * r + tid) * (float)P.nv : 0.f;
-    float wold = 0.f, wnew = kStart;
     bool bad = false;
     int it = 0;
     const LaneMap L = make_map16(m);
     u64 w[8];
     load_weights16(L, w);
     for (; it < a.T; ++it) {
-        bad = iterate16<GROUP>(a, m, P, L, w, tgt, group, c, seq, wold, wnew);
+        bad = iterate16<GROUP>(a, m, P, L, w, group, c, seq);
         if (bad) break;
     }
-    bad = bad || too_wide(m, r);
-    __syncthreads();
-    if (tid < RP) { m.s.ref[tid] = wold; m.s.ref[RP + tid] = wnew; }
-    if (tid == 0) { m.s.flag[2] = bad; m.s.flag[3] = it; }
+    bad = bad || too_wide(m, a.r);
+    if (threadIdx.x == 0) { m.s.flag[2] = bad; m.s.flag[3] = it; }
     __syncthreads();
     return seq;
 }
@@ -482,11 +513,11 @@ __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int grou
     const Mem m = carve16(smem, a.srows);
     const Part P = locate16(a, p, c);
     const int tid = threadIdx.x, r = a.r;
-    const float tgt = tid < r ? __ldg(a.beta + P.h * r + tid) * (float)P.nv : 0.f;
+    const float tgt = m.s.tgt[tid < RP ? tid : 0];
     int it = m.s.flag[3];
-    float wold = m.s.ref[tid < RP ? tid : 0], wnew = m.s.ref[RP + (tid < RP ? tid : 0)];
     while (true) {
         double gn = 0.0;
+        const float wold = m.before[tid < RP ? tid : 0], wnew = m.s.w[tid < RP ? tid : 0];
         if (__syncthreads_or(tid < r && it < a.T && sum_lost(tgt, wnew))) {
             if (tid < r) {
                 gn = m.s.gref[tid] + log2((double)wold);
@@ -511,9 +542,8 @@ __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int grou
         const LaneMap L = make_map16(m);
         u64 w[8];
         load_weights16(L, w);
-        wnew = kStart;
         if (it >= a.T) break;                                // rebuilt around the final potentials: equal weights
-        for (++it; it < a.T && !bad; ++it) bad = iterate16<GROUP>(a, m, P, L, w, tgt, group, c, seq, wold, wnew);
+        for (++it; it < a.T && !bad; ++it) bad = iterate16<GROUP>(a, m, P, L, w, group, c, seq);
         if (bad) --it;                                       // the iteration whose update has to be redone
         else if (!too_wide(m, r)) break;
         __syncthreads();
@@ -534,8 +564,11 @@ stream_kernel(const __grid_constant__ StreamArgs a)
     for (int p = group; p < 2 * a.B * a.H; p += a.groups) {
         __syncthreads();                                            // the previous problem is done with shared memory
         if (tid < RP) {
+            const Part F = locate16(a, p, c);
             m.s.gref[tid] = -(double)kStartLog2;
             m.s.w[tid] = tid < a.r ? kStart : 0.f;
+            m.before[tid] = 0.f;
+            m.s.tgt[tid] = tid < a.r ? __ldg(a.beta + F.h * a.r + tid) * (float)F.nv : 0.f;
         }
         if (tid == 0) m.s.flag[2] = 0;
         if (locate16(a, p, c).nv > 0) {
@@ -546,6 +579,7 @@ stream_kernel(const __grid_constant__ StreamArgs a)
             if (tid == 0 && c == 0) atomicOr(a.status, 2 /* LOT_DEV_EMPTY */);
             __syncthreads();
         }
+        if (p + a.groups >= 2 * a.B * a.H) chain_next();
         if (c == 0 && tid < RP) {
             const Part F = locate16(a, p, c);
             const size_t sp = (size_t)F.side * a.B * a.H + F.slice;
@@ -612,7 +646,7 @@ cudaError_t stream_attention(const void *q, const void *k, const void *v, const 
     a.B = B; a.H = H; a.n = n; a.npad = L.npad; a.r = r; a.T = iters; a.C = L.C; a.groups = L.groups; a.srows = L.srows;
     a.scale = 1.4426950408889634 / (double)eps;
     a.eps_ln2 = (double)eps * 0.6931471805599453;
-    const size_t smem = (size_t)L.srows * 128 + kFixed;
+    const size_t smem = (size_t)area_bytes(L.srows) + kFixed;
     auto kern = L.C > 1 ? stream_kernel<true> : stream_kernel<false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
     if (e != cudaSuccess) return e;

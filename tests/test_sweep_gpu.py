@@ -101,6 +101,8 @@ LONG = [
     (1, 2, 127, 40, 5, 0.1, True, False),
     (1, 1, 1000, 64, 0, 0.1, False, False),
     (2, 3, 1153, 33, 4, 0.05, True, False),
+    (2, 3, 1153, 17, 4, 0.05, True, False),
+    (1, 2, 2048, 32, 6, 0.1, False, False),
     (1, 1, 20000, 64, 4, 0.1, False, False),               # rows streamed
     (40, 8, 300, 64, 3, 0.1, True, False),                 # one block per problem
     (1, 3, 65536, 50, 2, 0.1, False, False),
