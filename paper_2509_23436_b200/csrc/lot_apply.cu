@@ -580,12 +580,24 @@ static bool make_map(CUtensorMap *m, const void *base, long long outer, int rows
 
 } // namespace apply
 
+// Thread blocks of the apply kernels, each a contiguous range of the slices' tiles: one per SM, or as many fewer as make the
+// ranges end at slice boundaries, if that costs no block more than one tile.  A range that runs into another slice pays a
+// second set of weights, partials and (output kernel) operand.
+static int apply_blocks(long long BH, int TPS)
+{
+    const long long NT = BH * TPS;
+    const int sms = device_sm_count();
+    if (NT <= sms) return (int)NT;
+    const long long k = sms / BH;
+    if (k >= 1 && (TPS + k - 1) / k <= (NT + sms - 1) / sms + 1) return (int)(BH * k);
+    return sms;
+}
+
 size_t stored_apply_wpart_bytes(int B, int H, int n)
 {
     const int TPS = (n + 127) / 128;
     const long long NT = (long long)B * H * TPS;
-    const int sms = device_sm_count();
-    const int ctas = NT < sms ? (int)NT : sms;
+    const int ctas = apply_blocks((long long)B * H, TPS);
     const int maxslots = (int)(((long long)TPS * ctas) / NT) + 2;
     return (size_t)B * H * maxslots * 64 * 64 * 4;
 }
@@ -602,8 +614,7 @@ cudaError_t stored_apply(const void *kt, int npad, const float *G, const float *
     P.B = B; P.H = H; P.n = n; P.r = r;
     P.TPS = (n + 127) / 128;
     P.NT = (int)(BH * P.TPS);
-    const int sms = device_sm_count();
-    P.ctas = P.NT < sms ? P.NT : sms;
+    P.ctas = apply_blocks(BH, P.TPS);
     P.maxslots = (int)(((long long)P.TPS * P.ctas) / P.NT) + 2;
     static std::mutex mu;
     static bool attr[64] = {};
