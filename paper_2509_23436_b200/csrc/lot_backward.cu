@@ -303,25 +303,24 @@ gemm_nt_kernel(const AT *__restrict__ A, const float *__restrict__ Bm, OutT *__r
 
 __global__ void bwd_w_fix_kernel(const float *Xw, const float *Wp, const int32_t *key_len, float *dWm, float *dbeta_direct, int H, int n, int d, int r)
 {
-    // one warp per (slice, pivot)
+    // one warp per (slice, pivot), one pivot each: eight pivots a warp, one after the other, were 17 us at B H = 16, r = 64
     chain_wait();
     const int s = blockIdx.x, b = s / H;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, t = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int nvalid = n;
     if (key_len != nullptr) nvalid = min(max(key_len[b], 0), n);
     const float km = nvalid > 0 ? (float)n / (float)nvalid : 0.f;
-    for (int t = warp; t < r; t += warps) {
-        const size_t o = ((size_t)s * r + t) * d;
-        float dot = 0.f;
-        for (int c = lane; c < d; c += 32) {
-            const float x = Xw[o + c];
-            dot = fmaf(x, Wp[o + c], dot);
-            dWm[o + c] = x * km;
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-        if (lane == 0) dbeta_direct[(size_t)s * r + t] = -(float)n * dot;
+    if (t >= r) return;
+    const size_t o = ((size_t)s * r + t) * d;
+    float dot = 0.f;
+    for (int c = lane; c < d; c += 32) {
+        const float x = Xw[o + c];
+        dot = fmaf(x, Wp[o + c], dot);
+        dWm[o + c] = x * km;
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+    if (lane == 0) dbeta_direct[(size_t)s * r + t] = -(float)n * dot;
 }
 
 __global__ void transpose_z_kernel(const float *__restrict__ z, float *__restrict__ zt, int r, int d, size_t total)
@@ -446,7 +445,7 @@ cudaError_t launch_gemm_nt(const void *A, bool a_double, const float *Bm, bool p
 cudaError_t launch_bwd_w_fix(const float *Xw, const float *Wp, const int32_t *key_len, float *dWm, float *dbeta_direct,
                              int B, int H, int n, int d, int r, cudaStream_t st)
 {
-    return chain_launch(bwd_w_fix_kernel, dim3(B * H), 256, 0, st, Xw, Wp, key_len, dWm, dbeta_direct, H, n, d, r);
+    return chain_launch(bwd_w_fix_kernel, dim3(B * H, (r + 7) / 8), 256, 0, st, Xw, Wp, key_len, dWm, dbeta_direct, H, n, d, r);
 }
 
 cudaError_t launch_transpose_z(const float *z, float *zt, int H, int r, int d, cudaStream_t st)

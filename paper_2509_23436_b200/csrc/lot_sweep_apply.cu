@@ -39,6 +39,22 @@ __device__ __forceinline__ float4 scaled(float4 p, float4 w, float s)
     return make_float4(p.x * (w.x * s), p.y * (w.y * s), p.z * (w.z * s), p.w * (w.w * s));
 }
 
+// The partials of the chunks in order, eight requested together: the last block of a tile does this alone, one L2 round
+// trip after the other.
+__device__ __forceinline__ float4 add_partials(const float *src, size_t stride, int chunks)
+{
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c0 = 0; c0 < chunks; c0 += 8) {
+        float4 p[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            p[u] = c0 + u < chunks ? __ldcg(reinterpret_cast<const float4 *>(src + (size_t)(c0 + u) * stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { s.x += p[u].x; s.y += p[u].y; s.z += p[u].z; s.w += p[u].w; }
+    }
+    return s;
+}
+
 // The tickets of the blocks that share a tile: true in the last one to arrive, which adds the partials in chunk order.
 __device__ __forceinline__ bool last_of_tile(unsigned *counter, int chunks)
 {
@@ -60,7 +76,7 @@ __device__ __forceinline__ bool last_of_tile(unsigned *counter, int chunks)
 // as they are.  Warps: TP / 16 pivot tiles x channel groups x (rank 16, narrow heads) halves of the keys.
 // ---------------------------------------------------------------------------------------------------------------
 template <int TP, int D, int N>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, D <= 128 ? 2 : 1)
 apply_w_mma_kernel(SweepApplyArgs a)
 {
     constexpr int KT = 64, PP = (TP + 8) * 2, PV = (D + 8) * 2, PLANE = KT * PP;
@@ -190,12 +206,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
     for (int idx = tid; idx < nt4; idx += kThreads) {
         const size_t o = (size_t)t0 * d + idx * 4;
         const float *src = a.wpart + (size_t)bh * a.chunks * r * d + o;
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-        for (int ch = 0; ch < a.chunks; ++ch) {
-            const float4 p = __ldcg(reinterpret_cast<const float4 *>(src + (size_t)ch * r * d));
-            s.x += p.x; s.y += p.y; s.z += p.z; s.w += p.w;
-        }
+        const float4 s = add_partials(src, (size_t)r * d, a.chunks);
         const float f = scale / a.beta[h * r + t0 + idx * 4 / d];
         *reinterpret_cast<float4 *>(a.Wp + (size_t)bh * r * d + o) = make_float4(s.x * f, s.y * f, s.z * f, s.w * f);
     }
@@ -409,12 +420,7 @@ apply_w_f32_kernel(SweepApplyArgs a)
             const int t = t0 + ty * 4 + x;
             if (t >= r) continue;
             const float *src = a.wpart + ((size_t)bh * a.chunks * r + t) * d + c;
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-            for (int ch = 0; ch < a.chunks; ++ch) {
-                const float4 p = __ldcg(reinterpret_cast<const float4 *>(src + (size_t)ch * r * d));
-                s.x += p.x; s.y += p.y; s.z += p.z; s.w += p.w;
-            }
+            const float4 s = add_partials(src, (size_t)r * d, a.chunks);
             const float f = scale / a.beta[h * r + t];
             *reinterpret_cast<float4 *>(a.Wp + ((size_t)bh * r + t) * d + c) = make_float4(s.x * f, s.y * f, s.z * f, s.w * f);
         }

@@ -356,32 +356,38 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
 __global__ void merge_kernel(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz, float *dbeta, int B, int H, int d,
                              int r, int RP, int chunks)
 {
-    // four threads an element, each a share of the batch rows, added in order
-    const size_t per = (size_t)r * d, idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) / 4;
-    const int quarter = threadIdx.x & 3, b0 = B * quarter / 4, b1 = B * (quarter + 1) / 4;
+    // eight threads an element, each a share of the partials (of the batch rows for beta), requested eight at a time: bound by
+    // latency, 12 us at B = 32, H = 3, r = 16, d = 64 when one thread went through the batch rows of beta
+    constexpr int W = 8;
+    const size_t per = (size_t)r * d, idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
+    const int part = threadIdx.x % W;
     chain_wait();
-    float sum = 0.f;
-    const bool in = idx < (size_t)H * per;
-    if (in) {
-        const int h = (int)(idx / per);
+    float sum = 0.f, bsum = 0.f;
+    if (idx < (size_t)H * per) {
+        const int h = (int)(idx / per), all = B * chunks, j0 = (int)((long long)all * part / W), j1 = (int)((long long)all * (part + 1) / W);
         const size_t e = idx % per;
-        for (int b = b0; b < b1; ++b) {
-            const size_t o = ((size_t)b * H + h) * chunks * per + e;
+#pragma unroll 8
+        for (int j = j0; j < j1; ++j) {
+            const int b = j / chunks, c = j - b * chunks;
+            const size_t o = (((size_t)b * H + h) * chunks + c) * per + e;
+            sum += part_q[o] + part_k[o];
+        }
+    }
+    if (idx < (size_t)H * r) {
+        const int h = (int)(idx / r), t = (int)(idx % r), b1 = (int)((long long)B * (part + 1) / W);
 #pragma unroll 4
-            for (int c = 0; c < chunks; ++c) sum += part_q[o + c * per] + part_k[o + c * per];
-        }
-    }
-    const float s1 = __shfl_down_sync(0xffffffffu, sum, 1), s2 = __shfl_down_sync(0xffffffffu, sum, 2), s3 = __shfl_down_sync(0xffffffffu, sum, 3);
-    if (in && quarter == 0) dz[idx] = ((sum + s1) + s2) + s3;
-    if (idx < (size_t)H * r && quarter == 0) {
-        const int h = (int)(idx / r), t = (int)(idx % r);
-        float v = 0.f;
-        for (int b = 0; b < B; ++b) {
+        for (int b = (int)((long long)B * part / W); b < b1; ++b) {
             const size_t sl = (size_t)b * H + h;
-            v += dbeta_direct[sl * r + t] + dbeta_acc[(2 * sl) * RP + t] + dbeta_acc[(2 * sl + 1) * RP + t];
+            bsum += dbeta_direct[sl * r + t] + dbeta_acc[(2 * sl) * RP + t] + dbeta_acc[(2 * sl + 1) * RP + t];
         }
-        dbeta[idx] = v;
     }
+#pragma unroll
+    for (int off = 1; off < W; off <<= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        bsum += __shfl_xor_sync(0xffffffffu, bsum, off);
+    }
+    if (part == 0 && idx < (size_t)H * per) dz[idx] = sum;
+    if (part == 0 && idx < (size_t)H * r) dbeta[idx] = bsum;
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -449,7 +455,7 @@ cudaError_t launch_bwd_reverse(const SweepPlan &P, const SweepBwdArgs &a, cudaSt
 cudaError_t launch_bwd_merge(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz,
                              float *dbeta, int B, int H, int d, int r, int RP, int chunks, cudaStream_t st)
 {
-    const size_t threads = (size_t)H * r * d * 4;
+    const size_t threads = (size_t)H * r * d * 8;
     return chain_launch(sweep::merge_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, st, part_q, part_k, dbeta_direct, dbeta_acc, dz, dbeta,
                         B, H, d, r, RP, chunks);
 }
