@@ -246,7 +246,7 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
         if (r <= 16 || (r <= 32 && (n <= 1200 || rows <= 100000))) return kPathGeneral;
         if (r <= 32 ? rows <= 200000 : n <= 1200 || rows <= 300000) return kPathLong;
     }
-    // Measured on B200 (see the design notes): the resident kernel wins where the streamed one has no stored-kernel
+    // Measured on B200: the resident kernel wins where the streamed one has no stored-kernel
     // passes (r <= 32, every pass recomputes logits and exponentials) and every thread block holds its whole share at
     // once (whole slices, one wave); elsewhere the streamed kernel is as fast or faster.
     if (res_ok && r <= 32) {

@@ -108,6 +108,8 @@ LONG = [
     (1, 3, 65536, 50, 2, 0.1, False, False),
     (1, 2, 3000, 64, 8, 0.02, False, True),                # rebuilt kernel
     (1, 1, 1500, 50, 12, 0.01, True, True),                # lost column sums, final potentials far apart
+    (1, 2, 1000, 50, 12, 0.01, True, True),                # the same in a cluster of eight blocks
+    (3, 16, 1024, 64, 5, 0.05, True, False),
 ]
 
 
