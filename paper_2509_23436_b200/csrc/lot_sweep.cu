@@ -198,16 +198,16 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
             const int rounds = C == 1 ? (P + slots - 1) / slots : (P + groups - 1) / groups;
             const double per_sm = (double)((resident + sms - 1) / sms);       // blocks that share an SM
             // us: SM time per entry (issue and shared-memory reads), twice that for a block alone on its SM; the exchange as
-            // measured (0.7 for two blocks at RP = 256, 2.1 for 16; with owners 4.6-6.4 at 49-148, fitted with the rate one SM
+            // measured (0.7 for two blocks at RP = 256, 2.1 for 16; with owners 5.2-7.0 at 49-148, fitted with the rate one SM
             // reads at to config 5's times over C: 3771 us at 49, 3971 at 59, 4520 at 74, 6300 at 148); streamed rows at the L2's
             // rate, at the HBM's when all of them exceed the L2, and never faster than one SM reads
             const double entry = (RP <= 32 ? 0.055 : 0.045) / 1900.0;
-            const double lat = C == 1 ? 0.45 : C * RP <= kDirectWords ? 0.9 + 0.4 * C * RP / 1024.0 : 3.7 + 0.018 * C;
+            const double lat = C == 1 ? 0.45 : C * RP <= kDirectWords ? 0.9 + 0.4 * C * RP / 1024.0 : 4.3 + 0.018 * C;
             const double mine = 2.0 * rows * RP * entry, sm_us = per_sm * rows * RP * entry;
             const double glob = (double)(rows > srows ? rows - srows : 0) * RP * 4.0, all = glob * resident;
             double it = lat + mine;
             if (sm_us > it) it = sm_us;
-            const double gl_us = all / (all > 90e6 ? 5.5e6 : 10e6), gl_sm = per_sm * glob / 62e3;
+            const double gl_us = all / (all > 90e6 ? 5.5e6 : 10e6), gl_sm = per_sm * glob / 70e3;
             it += gl_us > gl_sm ? gl_us : gl_sm;
             const double t = rounds * (12 * it + 3.0);
             if (t < best_t) {
