@@ -181,7 +181,7 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
     uint32_t *sTmem = reinterpret_cast<uint32_t *>(smem + PlanW::offMisc + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Sync S{smem_u32(bars), sAbort, P.status, lane};
-    if ((sbase & 1023u) != 0) { if (threadIdx.x == 0) atomicOr(P.status, 4); return; }
+    if ((sbase & 1023u) != 0) { chain_wait(); if (threadIdx.x == 0) atomicOr(P.status, 4); return; }
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(S.bar(wFull + i), 1); mbar_init(S.bar(wEmpty + i), 1); mbar_init(S.bar(wScaled + i), 4); }
         mbar_init(S.bar(wAcc), 1); mbar_init(S.bar(wRead), 8);
@@ -360,7 +360,7 @@ apply_out_kernel(const __grid_constant__ ApplyParams P)
     uint32_t *sTmem = reinterpret_cast<uint32_t *>(smem + PlanO::offMisc + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Sync S{smem_u32(bars), sAbort, P.status, lane};
-    if ((sbase & 1023u) != 0) { if (threadIdx.x == 0) atomicOr(P.status, 4); return; }
+    if ((sbase & 1023u) != 0) { chain_wait(); if (threadIdx.x == 0) atomicOr(P.status, 4); return; }
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
             mbar_init(S.bar(oFull + i), 1); mbar_init(S.bar(oEmpty + i), 5); mbar_init(S.bar(oAcc + i), 1); mbar_init(S.bar(oRead + i), 4);

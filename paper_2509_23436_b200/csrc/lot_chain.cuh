@@ -1,6 +1,7 @@
 // Launches of a chain of kernels on one stream that overlap their starts: a kernel launched with chain_launch may begin
 // once every block of its predecessor has called chain_next or ended, and calls chain_wait before it touches anything
-// the predecessors write or read.  chain_next stands where a block's main work is done: called first thing, the waiting
+// the predecessors write or read.  Every path through such a kernel passes chain_wait, also of one that touches nothing of
+// theirs (it waits last): the end of the last kernel is taken for the end of the chain.  chain_next stands where a block's main work is done: called first thing, the waiting
 // blocks of the next kernel took a fifth of the sweep kernel's speed.  Hides most of the 2-3 us between dependent launches.
 // Loads of what a predecessor wrote must be plain ones: the compiler moves __ldg and loads through const __restrict__
 // pointers above the wait.

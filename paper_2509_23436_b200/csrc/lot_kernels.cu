@@ -573,7 +573,6 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
     __shared__ float sc_s[kClsKeys];
     __shared__ __align__(16) float part[256 * 8];
     __shared__ float red[8];
-    // no chain_wait: it reads and writes nothing of its predecessors
     const int bh = blockIdx.x, bb = bh / H, tid = threadIdx.x;
     int kv = nk;
     if (key_len != nullptr) kv = min(max(key_len[bb], 0), nk);
@@ -631,6 +630,9 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
         for (int i = 0; i < parts; ++i) s += part[i * d + cc];
         Elem<T>::store(out + (size_t)bh * nq * d + cc, kv > 0 ? s / den : 0.f);
     }
+    // It touches nothing of its predecessors, so it runs beside them; but what comes next on the stream (a reader of out, the
+    // next call's ordinary launch) waits for this kernel alone, so it must not end before they have.
+    chain_wait();
 }
 
 cudaError_t launch_cls_row(const void *q, const void *k, const void *v, const int32_t *key_len, int dtype, int B, int H,
