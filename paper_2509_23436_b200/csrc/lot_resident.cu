@@ -491,7 +491,8 @@ __device__ __noinline__ void mma_x(const Ctx c)
 // The value rows reach the tensor cores scaled by 1/s_j, as a bf16 hi part and a bf16 lo part (one rounding of the
 // product would cost the output three times its own bf16 rounding).  Both parts pass through the tile's one buffer:
 // the hi-part MMAs of position k, the hi-part MMAs of position k + 1 (the other quad's), then the lo-part MMAs of
-// position k, which its quad has written over the hi part meanwhile.
+// position k, which its quad has written over the hi part meanwhile; without position k + 1 in between where that one's
+// load needs a buffer that position k frees.
 __device__ __noinline__ void mma_w(const Ctx c)
 {
     const Misc *M = c.M;
@@ -503,6 +504,7 @@ __device__ __noinline__ void mma_w(const Ctx c)
     const int n1 = M->seg[1].t1 - M->seg[1].t0;       // positions [0, n1) belong to the first key segment
     bool ok = true;
     int pending = -1;                                 // position whose lo part is still to be issued
+    int li = 0;                                       // loads up to and with those of position k (as build_wave counts them)
     auto issue = [&](int k, bool lo_part) {
         const int kk = M->worder[k];
         const int kb = kk < nSp ? M->kbuf[kk] : kk - nSp, vb = M->wbuf[k];
@@ -529,6 +531,10 @@ __device__ __noinline__ void mma_w(const Ctx c)
             __syncwarp();
             if (ok) ok = warp_wait(c, bWRead + 0, 0);
         }
+        li += M->worder[k] < nSp ? 2 : 1;
+        // Where a tile of position k comes into a buffer that the waiting position frees (its key segment holds two tiles,
+        // both spilled), its lo part cannot wait for the hi part of position k: each would wait for the other.
+        if (pending >= 0 && M->wdep[li - 1] >= pending) { issue(pending, true); pending = -1; }
         issue(k, false);
         if (pending >= 0) issue(pending, true);
         pending = k;

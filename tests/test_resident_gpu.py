@@ -65,6 +65,8 @@ CASES = [
     (2, 8, 3000, 33, 6, 0.1, True),
     (1, 16, 4096, 64, 10, 0.1, False),
     (1, 16, 16384, 64, 10, 0.1, False),    # 14 + 14 tiles per block: the capacity of the path
+    (4, 16, 4096, 24, 4, 0.1, False),      # blocks whose first key segment is two tiles, both spilled
+    (4, 16, 4096, 64, 2, 0.1, True),
     (16, 12, 512, 32, 20, 0.05, True),
     (32, 3, 197, 16, 10, 0.1, False),
 ]
