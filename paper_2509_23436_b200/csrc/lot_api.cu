@@ -223,7 +223,7 @@ void remember_ws(const void *ws, int path, unsigned tag, size_t fused_off)
 
 enum { kPathGeneral = 0, kPathStreamed = 1, kPathResident = 2, kPathSlice = 3, kPathLong = 4 };
 std::atomic<int> g_force_path{-1};      // test hook: 0 picks the general path, 1 or 2 that tensor-core path wherever it can run
-int choose_path(int dtype, int B, int H, int n, int d, int r)
+int choose_path(int dtype, int B, int H, int n, int d, int r, int iters)
 {
     if (!fused_supported(dtype, d, r)) return kPathGeneral;
     const bool res_ok = B >= 1 && n >= 1 && resident_geometry(dtype, B, H, n, d, r).ok;
@@ -244,7 +244,10 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
     if (B >= 1 && n >= 1) {
         const long long rows = (long long)B * H * n;
         if (r <= 16 || (r <= 32 && (n <= 1200 || rows <= 100000))) return kPathGeneral;
-        if (r <= 32 ? rows <= 200000 : n <= 1200 || rows <= 300000) return kPathLong;
+        // ... of calls with three iterations and more: one or two show that the streamed path's first pass is on float32 values
+        // (errors of the potentials at n = 4096 in units of eps: 5e-6 against 1.3e-4 after one, 1.1e-4 against 1.3e-4 after
+        // two, 1.6e-4 on both after three)
+        if (iters >= 3 && (r <= 32 ? rows <= 200000 : n <= 1200 || rows <= 300000)) return kPathLong;
     }
     // Measured on B200: the resident kernel wins where the streamed one has no stored-kernel
     // passes (r <= 32, every pass recomputes logits and exponentials) and every thread block holds its whole share at
@@ -254,6 +257,22 @@ int choose_path(int dtype, int B, int H, int n, int d, int r)
         if (G.whole && (long long)B * H <= (long long)G.ctas * G.wave_slices) return kPathResident;
     }
     return kPathStreamed;
+}
+
+size_t path_bytes(int path, int dtype, int B, int H, int n, int d, int r)
+{
+    if (path == kPathResident) return up256(resident_layout(B, H, n, d, r).total) + fused_layout(B, H, n, d, r).total;
+    if (path == kPathStreamed) return fused_layout(B, H, n, d, r).total;
+    if (path == kPathLong) return stream_plan(B * H, n).total;
+    if (path == kPathSlice) return 256;                              // the status word
+    return forward_layout(B, H, n, n, d, r, dtype, false).total;
+}
+
+// Whether the first `bytes` of two tensors share memory.
+bool overlap(const void *a, const void *b, size_t bytes)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y ? y - x < bytes : x - y < bytes;
 }
 
 // Both Sinkhorn problems and the apply stages on the general path.
@@ -491,20 +510,17 @@ size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
 {
     if (dtype != LOT_F32 && dtype != LOT_BF16) return 0;
     if (check_dims(B, H, n, r) != LOT_OK || check_d(n, d) != LOT_OK) return 0;
-    const int path = choose_path(dtype, B, H, n, d, r);
-    if (path == kPathResident) return up256(resident_layout(B, H, n, d, r).total) + fused_layout(B, H, n, d, r).total;
-    if (path == kPathStreamed) return fused_layout(B, H, n, d, r).total;
-    if (path == kPathLong) return stream_plan(B * H, n).total;
-    if (path == kPathSlice) return 256;                              // the status word
-    return forward_layout(B, H, n, n, d, r, dtype, false).total;
+    // the most of any number of iterations
+    const size_t few = path_bytes(choose_path(dtype, B, H, n, d, r, 0), dtype, B, H, n, d, r);
+    const size_t many = path_bytes(choose_path(dtype, B, H, n, d, r, 1 << 20), dtype, B, H, n, d, r);
+    return few > many ? few : many;
 }
 
 int lot_path(int dtype, int B, int H, int n, int d, int r, int iters)
 {
-    (void)iters;
     if (dtype != LOT_F32 && dtype != LOT_BF16) return 0;
     if (check_dims(B, H, n, r) != LOT_OK || check_d(n, d) != LOT_OK) return 0;
-    return choose_path(dtype, B, H, n, d, r);
+    return choose_path(dtype, B, H, n, d, r, iters);
 }
 
 int lot_launch_count(int dtype, int B, int H, int n, int d, int r, int iters)
@@ -544,7 +560,10 @@ int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
         !aligned16(out) || !aligned16(g1_out) || !aligned16(g2_out) ||
         (key_len && (reinterpret_cast<uintptr_t>(key_len) & 3u)))
         return LOT_ERR_INVALID_ARG;
-    const int path = choose_path(dtype, B, H, n, d, r);
+    int path = choose_path(dtype, B, H, n, d, r, iters);
+    // the long path keeps part of the kernel in out until it is written; the streamed one takes an output over an input
+    const size_t bytes = (size_t)B * H * n * d * 2;
+    if (path == kPathLong && (overlap(out, q, bytes) || overlap(out, k, bytes) || overlap(out, v, bytes))) path = kPathStreamed;
     if (path == kPathSlice) {
         if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < 256) return LOT_ERR_WORKSPACE;
         remember_ws(ws, kPathSlice, 0, 0);

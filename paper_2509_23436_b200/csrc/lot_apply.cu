@@ -1,10 +1,12 @@
-// The two apply stages of Eq. (4) from the stored Gibbs kernel (bf16 tensors, d = 64, 32 < r <= 64), as two
-// kernels launched behind the persistent Sinkhorn kernel (lot_fused.cu) on the same stream:
+// The two apply stages of Eq. (4) from the stored Gibbs kernel (bf16 tensors, d = 64, r <= 64), as two kernels
+// launched on the same stream behind the kernel that iterated on it (lot_stream.cu, lot_fused.cu):
 //
 //   apply_w_kernel    W = Gamma2 V per slice.  With K~2_jt = 2^(L_jt - max_t L_jt) stored as bf16 (workspace, L2) and
 //                     w_t = 2^(G2_t - max G2):  W_t = w_t sum_j K~2_jt (v_j / s_j) / kv,  s_j = sum_t K~2_jt w_t.  The
 //                     stored tile is the A operand as it is (MN-major, no rewrite); the value rows are scaled by 1/s_j
 //                     and split into bf16 hi + lo in shared memory.  Every block writes the partial of its tile range.
+//                     With the low half (LO, the long path): K~2 to twice bf16's precision, its rows scaled by 1/s_j in
+//                     float32 and split into bf16 hi + lo in place, both against the value rows as they are.
 //   apply_out_kernel  out_i = sum_t K~1_it (w1_t W'_t) / s_i,  W' = W / beta.  The stored query tile is the A operand
 //                     straight from TMA; W'' = Diag(w1) W' (partials added in slot order) is the B operand, hi + lo.
 //
@@ -155,13 +157,61 @@ __device__ __forceinline__ void tile_row_sums(const uint8_t *tileptr, int w4, in
     for (int j = 0; j < 4; ++j) sr[j] += __shfl_xor_sync(0xffffffffu, sr[j], 2);
 }
 
+// The thread's four rows of a stored tile (as tile_row_sums) and of its low half, in place: the float32 value K~ / s, s its
+// row's sum against the weights, as bf16 hi + lo; rows from `valid` on are zero.
+__device__ __forceinline__ void scale_kernel_rows(uint8_t *hi, uint8_t *lo, int w4, int rq, int cq, const float2 (&w2)[8], int valid)
+{
+    uint4 x[4][2], y[4][2];
+    float sr[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int rin = w4 * 32 + j * 8 + rq;
+        float2 sa = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int off = rin * 128 + (((2 * cq + h) ^ (rin & 7)) * 16);
+            x[j][h] = *reinterpret_cast<const uint4 *>(hi + off);
+            y[j][h] = *reinterpret_cast<const uint4 *>(lo + off);
+            const uint32_t *xw = reinterpret_cast<const uint32_t *>(&x[j][h]), *yw = reinterpret_cast<const uint32_t *>(&y[j][h]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sa = __ffma2_rn(__fadd2_rn(unpack_bf16(xw[e]), unpack_bf16(yw[e])), w2[4 * h + e], sa);
+        }
+        sr[j] = sa.x + sa.y;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sr[j] += __shfl_xor_sync(0xffffffffu, sr[j], 1);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sr[j] += __shfl_xor_sync(0xffffffffu, sr[j], 2);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int rin = w4 * 32 + j * 8 + rq;
+        const float u = __fdividef(1.f, sr[j]);
+        const float2 uu = make_float2(u, u);
+        const bool in = rin < valid;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int off = rin * 128 + (((2 * cq + h) ^ (rin & 7)) * 16);
+            uint32_t *xw = reinterpret_cast<uint32_t *>(&x[j][h]), *yw = reinterpret_cast<uint32_t *>(&y[j][h]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 f = __fmul2_rn(__fadd2_rn(unpack_bf16(xw[e]), unpack_bf16(yw[e])), uu);
+                const __nv_bfloat162 hh = __floats2bfloat162_rn(f.x, f.y);
+                xw[e] = in ? *reinterpret_cast<const uint32_t *>(&hh) : 0u;
+                yw[e] = in ? pack_bf16(f.x - __low2float(hh), f.y - __high2float(hh)) : 0u;
+            }
+            *reinterpret_cast<uint4 *>(hi + off) = x[j][h];
+            *reinterpret_cast<uint4 *>(lo + off) = y[j][h];
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------------------
 // W = Gamma2 V
 // ---------------------------------------------------------------------------------------
 struct PlanW {
-    static constexpr int offK = 0;                              // stored key tiles
-    static constexpr int offV = offK + kStages * kTileBytes;    // value tiles, rewritten as the hi part of V / s
-    static constexpr int offL = offV + kStages * kTileBytes;    // lo part
+    static constexpr int offK = 0;                              // stored key tiles (LO: rewritten as the hi part of K~ / s)
+    static constexpr int offV = offK + kStages * kTileBytes;    // value tiles, rewritten as the hi part of V / s (LO: as they are)
+    static constexpr int offL = offV + kStages * kTileBytes;    // lo part (LO: loaded as the kernel's low half)
     static constexpr int offBar = offL + kStages * kTileBytes;  // 32 mbarriers
     static constexpr int offW = offBar + 32 * 8;                // float sW[64]
     static constexpr int offMisc = offW + 64 * 4;
@@ -170,6 +220,8 @@ struct PlanW {
 enum BarW { wFull = 0 /* [4] */, wEmpty = 4 /* [4] */, wScaled = 8 /* [4] count 4 */, wAcc = 12 /* accumulator of a segment complete */,
             wRead = 13 /* count 8: read out */ };
 
+// LO: the low half of the stored key-side kernel (K~ minus its bf16 rounding, in bf16) lies where the output rows will be.
+template <bool LO>
 __global__ void __launch_bounds__(kThreads, 1)
 apply_w_kernel(const __grid_constant__ ApplyParams P)
 {
@@ -188,6 +240,7 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
         *sAbort = 0;
         fence_barrier_init();
         prefetch_tensormap(&P.tmKt); prefetch_tensormap(&P.tmV);
+        if (LO) prefetch_tensormap(&P.tmO);
     }
     if (warp == 1) { tmem_alloc(smem_u32(sTmem), 64); tmem_relinquish(); }
     tc_fence_before();
@@ -219,9 +272,10 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
                     const int st = cnt % kStages;
                     if (cnt >= kStages) ok = S.wait(wEmpty + st, ((cnt / kStages) - 1) & 1);
                     if (!ok) break;
-                    mbar_arrive_expect_tx(S.bar(wFull + st), 2 * kTileBytes);
+                    mbar_arrive_expect_tx(S.bar(wFull + st), (LO ? 3 : 2) * kTileBytes);
                     tma_load_3d(sbase + PlanW::offK + st * kTileBytes, &P.tmKt, S.bar(wFull + st), 0, t * kTileRows, BH + s);
                     tma_load_3d(sbase + PlanW::offV + st * kTileBytes, &P.tmV, S.bar(wFull + st), 0, t * kTileRows, s);
+                    if (LO) tma_load_3d(sbase + PlanW::offL + st * kTileBytes, &P.tmO, S.bar(wFull + st), 0, t * kTileRows, s);
                 }
             }
         }
@@ -247,7 +301,8 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
                     for (int part = 0; part < 2; ++part)
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            umma_bf16(tmem, ((uint64_t)d_hi << 32) | (ka + ks * 128), ((uint64_t)d_hi << 32) | ((part ? la : va) + ks * 128),
+                            umma_bf16(tmem, ((uint64_t)d_hi << 32) | ((LO && part ? la : ka) + ks * 128),
+                                      ((uint64_t)d_hi << 32) | ((!LO && part ? la : va) + ks * 128),
                                       idesc, (t == t0 && part == 0 && ks == 0) ? 0u : 1u);
                     umma_commit(S.bar(wEmpty + st));
                     if (t == t1 - 1) umma_commit(S.bar(wAcc));
@@ -275,6 +330,12 @@ apply_w_kernel(const __grid_constant__ ApplyParams P)
                 const int st = cnt % kStages;
                 if (ok) ok = S.warp_wait(wFull + st, (cnt / kStages) & 1);
                 if (!ok) continue;
+                if (LO) {
+                    scale_kernel_rows(smem + PlanW::offK + st * kTileBytes, smem + PlanW::offL + st * kTileBytes, w4, rq, cq, w2, kv - t * kTileRows);
+                    fence_proxy_async_smem();
+                    S.warp_arrive(wScaled + st);
+                    continue;
+                }
                 float sr[4];
                 tile_row_sums(smem + PlanW::offK + st * kTileBytes, w4, rq, cq, w2, sr);
                 uint8_t *vt = smem + PlanW::offV + st * kTileBytes, *lt = smem + PlanW::offL + st * kTileBytes;
@@ -603,7 +664,7 @@ size_t stored_apply_wpart_bytes(int B, int H, int n)
 }
 
 cudaError_t stored_apply(const void *kt, int npad, const float *G, const float *beta, const int32_t *key_len, const int *decision,
-                         const void *v, void *out, float *wpart, int *status, int B, int H, int n, int r, cudaStream_t st)
+                         const void *v, void *out, bool low_half, float *wpart, int *status, int B, int H, int n, int r, cudaStream_t st)
 {
     using namespace apply;
     ApplyParams P;
@@ -623,13 +684,14 @@ cudaError_t stored_apply(const void *kt, int npad, const float *G, const float *
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!attr[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(apply_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PlanW::total);
+            cudaError_t e = cudaFuncSetAttribute(apply_w_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PlanW::total);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(apply_w_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PlanW::total);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(apply_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PlanO::total);
             if (e != cudaSuccess) return e;
             attr[dev] = true;
         }
     }
-    cudaError_t e = chain_launch(apply_w_kernel, dim3(P.ctas), kThreads, PlanW::total, st, P);
+    cudaError_t e = chain_launch(low_half ? apply_w_kernel<true> : apply_w_kernel<false>, dim3(P.ctas), kThreads, PlanW::total, st, P);
     if (e != cudaSuccess) return e;
     return chain_launch(apply_out_kernel, dim3(P.ctas), kThreads, PlanO::total, st, P);
 }

@@ -1678,7 +1678,7 @@ cudaError_t fused_attention(const void *q, const void *k, const void *v, const f
     else e = launch_forward<64, false>(P, ctas, st);
     if (e != cudaSuccess || !P.ext_apply) return e;
     // the apply stages from the stored kernel, for every slice the Sinkhorn kernel left to them
-    return stored_apply(P.Kt, P.npad, P.G, beta, key_len, P.decision, v, out, reinterpret_cast<float *>(w + L.wpart2), P.status,
+    return stored_apply(P.Kt, P.npad, P.G, beta, key_len, P.decision, v, out, false, reinterpret_cast<float *>(w + L.wpart2), P.status,
                         B, H, n, r, st);
 }
 

@@ -143,7 +143,7 @@ ResidentLayout resident_layout(int B, int H, int n, int d, int r);
 cudaError_t resident_attention(const void *q, const void *k, const void *v, const float *z, const float *beta,
                                const int32_t *key_len, int B, int H, int n, int d, int r, float eps, int iters,
                                void *out, float *g1_out, float *g2_out, void *ws, unsigned *tag_out, cudaStream_t st);
-void resident_debug(int what, long long value);
+void resident_debug(int what, long long value);   // test hooks: 1 = block that skips its first publish (one call), 2 = wait limit in ns
 
 // ---- slice path (lot_slice.cu): bf16 tensors, d = 64, r <= 64, short sequences; one thread block per slice ----
 bool slice_supported(int dtype, int n, int d, int r);
@@ -151,18 +151,20 @@ cudaError_t slice_attention(const void *q, const void *k, const void *v, const f
                             const int32_t *key_len, int B, int H, int n, int r, float eps, int iters, void *out,
                             float *g1_out, float *g2_out, int *status, cudaStream_t st);
 
-// ---- long sequences on a stored bf16 kernel (lot_stream.cu): bf16 tensors, d = 64, 32 < r <= 64 ----
+// ---- long sequences on a stored bf16 kernel (lot_stream.cu): bf16 tensors, d = 64, 16 < r <= 64 ----
 struct StreamPlan {
     int C, groups, srows, npad;
     size_t xbuf, ybuf, head_end, G, decision, kt, wpart, total;
 };
 StreamPlan stream_plan(int BH, int n);
+// out must not overlap the other tensors: it holds part of the kernel until it is written
 cudaError_t stream_attention(const void *q, const void *k, const void *v, const float *z, const float *beta, const int32_t *key_len, int B,
                              int H, int n, int r, float eps, int iters, void *out, float *g1_out, float *g2_out, void *ws, cudaStream_t st);
 
-// ---- apply stages from the stored Gibbs kernel (lot_apply.cu), behind the streamed Sinkhorn kernel ----
+// ---- apply stages from the stored Gibbs kernel (lot_apply.cu), behind the long path's kernel or the streamed one ----
 size_t stored_apply_wpart_bytes(int B, int H, int n);
+// low_half: out holds the key side's kernel minus its bf16 rounding on entry
 cudaError_t stored_apply(const void *kt, int npad, const float *G, const float *beta, const int32_t *key_len, const int *decision,
-                         const void *v, void *out, float *wpart, int *status, int B, int H, int n, int r, cudaStream_t st);   // test hooks: 1 = block that skips its first publish (one call), 2 = wait limit in ns
+                         const void *v, void *out, bool low_half, float *wpart, int *status, int B, int H, int n, int r, cudaStream_t st);
 
 } // namespace lot

@@ -35,6 +35,7 @@ struct StreamArgs {
     const float *z, *beta;
     const int32_t *key_len;
     uint8_t *kt;               // [2][BH][npad][64] bf16, side 0 queries
+    uint8_t *low;              // [BH][n][64] bf16: the key side's kernel minus its bf16 rounding, or nullptr
     float *G;                  // [2][BH][64] log2 of the final weights (relative to the kernel as stored)
     int *decision;             // [2][BH], set to 1
     float *g_out[2];
@@ -70,7 +71,7 @@ __device__ __forceinline__ Mem carve16(uint8_t *p, int srows)
 
 struct Part {                  // a block's share of a problem
     int slice, side, h, nv, row0, nrows, ns, steps;
-    uint8_t *g;                // its rows in global memory
+    uint8_t *g, *low;          // its rows in global memory, and those of the low half or nullptr
     const __nv_bfloat16 *x;
 };
 
@@ -88,6 +89,7 @@ __device__ __forceinline__ Part locate16(const StreamArgs &a, int p, int c)
     P.ns = min(P.nrows, a.srows);
     P.steps = (P.ns + kRowsStep - 1) / kRowsStep;
     P.g = a.kt + ((size_t)(P.side * a.B * a.H + P.slice) * a.npad + P.row0) * 128;
+    P.low = P.side == 1 && a.low != nullptr ? a.low + ((size_t)P.slice * a.n + P.row0) * 128 : nullptr;
     P.x = a.x[P.side] + ((size_t)P.slice * a.n + P.row0) * kD;
     return P;
 }
@@ -207,9 +209,13 @@ __device__ __noinline__ void build16(const StreamArgs *ap, int p, int c)
             for (int j = 1; j < RP / 8; ++j) mx = fmaxf(mx, fmaxf(L[j][2 * h], L[j][2 * h + 1]));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2)) - kKernelTop;
-            uint32_t o[RP / 8];
+            uint32_t o[RP / 8], l[RP / 8];
 #pragma unroll
-            for (int j = 0; j < RP / 8; ++j) o[j] = pack2(ex2(L[j][2 * h] - mx), ex2(L[j][2 * h + 1] - mx));
+            for (int j = 0; j < RP / 8; ++j) {
+                const float x = ex2(L[j][2 * h] - mx), y = ex2(L[j][2 * h + 1] - mx);
+                o[j] = pack2(x, y);
+                l[j] = pack2(x - __uint_as_float(o[j] << 16), y - __uint_as_float(o[j] & 0xffff0000u));
+            }
             if (i >= P.nrows) continue;
             // odd rows store their second half first: eight lanes then cover all banks
             const bool odd = g & 1;
@@ -221,6 +227,10 @@ __device__ __noinline__ void build16(const StreamArgs *ap, int p, int c)
             if (i < direct) {
                 *reinterpret_cast<uint4 *>(m.K + at) = o0;
                 *reinterpret_cast<uint4 *>(m.K + at + flip) = o1;
+            }
+            if (P.low != nullptr) {                                 // read once, by the apply kernel: not to be kept in the L2
+                __stcs(reinterpret_cast<uint4 *>(P.low + at), odd ? make_uint4(l[4], l[5], l[6], l[7]) : make_uint4(l[0], l[1], l[2], l[3]));
+                __stcs(reinterpret_cast<uint4 *>(P.low + at + flip), odd ? make_uint4(l[0], l[1], l[2], l[3]) : make_uint4(l[4], l[5], l[6], l[7]));
             }
         }
     }
@@ -729,6 +739,10 @@ cudaError_t stream_attention(const void *q, const void *k, const void *v, const 
     a.x[0] = static_cast<const __nv_bfloat16 *>(q); a.x[1] = static_cast<const __nv_bfloat16 *>(k);
     a.z = z; a.beta = beta; a.key_len = key_len;
     a.kt = reinterpret_cast<uint8_t *>(w + L.kt);
+    // Where the streamed path would apply from the logits, the key side is applied from twice bf16's precision.  The low
+    // half waits in the output's own memory: the last kernel, which writes the output, starts behind its only reader.
+    const bool low_half = !fused_ext_apply(B, H, n, r, iters);
+    a.low = low_half ? static_cast<uint8_t *>(out) : nullptr;
     a.G = reinterpret_cast<float *>(w + L.G); a.decision = reinterpret_cast<int *>(w + L.decision);
     a.g_out[0] = g1_out; a.g_out[1] = g2_out;
     a.xbuf = reinterpret_cast<u64 *>(w + L.xbuf); a.ybuf = reinterpret_cast<u64 *>(w + L.ybuf);
@@ -754,7 +768,7 @@ cudaError_t stream_attention(const void *q, const void *k, const void *v, const 
         }
     }
     if (e != cudaSuccess) return e;
-    return stored_apply(a.kt, L.npad, a.G, beta, key_len, a.decision, v, out, reinterpret_cast<float *>(w + L.wpart), a.status, B, H, n, r, st);
+    return stored_apply(a.kt, L.npad, a.G, beta, key_len, a.decision, v, out, low_half, reinterpret_cast<float *>(w + L.wpart), a.status, B, H, n, r, st);
 }
 
 } // namespace lot
