@@ -164,23 +164,25 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *      one per SM), plus a small pivot preparation.  With 32 < r <= 64 its first pass keeps the
  *      stabilised Gibbs kernel exp(C/eps - rowmax) of the scaling form of Eq. (1)-(2) as bf16 in the
  *      workspace and the later passes stream that copy back.
- *   2  the resident tensor-core path (same tensors; taken for r <= 32 when every thread block can
- *      hold whole sequences, up to 1792 tokens, and all of its share at once): one persistent kernel in
- *      which that bf16 kernel never leaves the SM (tensor memory and shared memory) between the
- *      iterations.  A problem it cannot represent (potentials spread over more than 96 binades, a
- *      column mass below 2^-80) is recomputed by the streamed kernels, which are launched behind it
- *      and return at once otherwise (device flag LOT_DEV_RECOMPUTED).  It can run many more shapes
- *      (lot_debug_hook what = 4), but measured no faster there.
- *   4  the long path (same tensors, 16 < r <= 64): one cooperative launch builds that bf16 kernel and runs all passes
+ *   2  the resident tensor-core path (same tensors): one persistent kernel in which that bf16 kernel never
+ *      leaves the SM (tensor memory and shared memory) between the iterations.  A problem it cannot
+ *      represent (potentials spread over more than 96 binades, a column mass below 2^-80) is
+ *      recomputed by the streamed kernels, which are launched behind it and return at once otherwise
+ *      (device flag LOT_DEV_RECOMPUTED).  Nowhere the fastest, so only taken by lot_debug_hook what = 4.
+ *   4  the long path (same tensors, 16 < r <= 64, three iterations and more): one launch (cooperative, or clusters
+ *      of thread blocks, or plain where a block has a problem to itself) builds that bf16 kernel and runs all passes
  *      on it, a group of thread blocks per problem keeping what it can of it in shared memory; two apply kernels.
- *      Taken up to 300000 rows B H n (r <= 32: from 100000 to 200000) and for n <= 1200; path 0 takes r <= 16 and the smaller
- *      problems of r <= 32.
+ *      Taken for r > 32 up to 300000 rows B H n and for n <= 1200, for r <= 32 at about one slice per SM of up to 1792
+ *      tokens; path 0 takes r <= 16 and the other problems of r <= 32 up to 160000 rows or n <= 1200.  A call whose
+ *      out overlaps q, k or v takes path 1 instead: the low half of the key side's kernel waits in out.
  *   3  the slice path (same tensors; n <= 512 and 16 ceil(n/16) x (r padded to 16, 32 or 64) <= 16384): a pair of
  *      thread blocks per (batch, head) slice, one for each side, keeps the side's Gibbs kernel in float32 in shared
  *      memory for all iterations (warp-level tensor-core products); only the r x d intermediate crosses, inside the
  *      pair's cluster; no workspace beyond the status word.  Taken wherever it can run.
- * On paths 1, 2 and 4 the potentials agree with an exact float evaluation to about 1e-4 and the output
- * to the bf16 rounding of `out`.
+ * On paths 1, 2 and 4 with 32 < r (1), any r (2, 4) the potentials of calls of two iterations and more agree with an exact
+ * float evaluation to about 1e-4 (the iterations read a bf16 kernel); elsewhere to float32.  Beside its own bf16 rounding
+ * `out` has an error of a quarter to four tenths of that rounding's: the plan's query side is read in bf16 (paths 1, 2, 4),
+ * and on path 2, and path 1 from 4096 tiles of 128 tokens on, its key side too.
  */
 LOT_API int lot_path(int dtype, int B, int H, int n, int d, int r, int iters);
 

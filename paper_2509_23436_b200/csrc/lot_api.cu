@@ -222,41 +222,38 @@ void remember_ws(const void *ws, int path, unsigned tag, size_t fused_off)
 }
 
 enum { kPathGeneral = 0, kPathStreamed = 1, kPathResident = 2, kPathSlice = 3, kPathLong = 4 };
-std::atomic<int> g_force_path{-1};      // test hook: 0 picks the general path, 1 or 2 that tensor-core path wherever it can run
+std::atomic<int> g_force_path{-1};      // test hook: 0 picks the general path, 1, 2 or 4 that tensor-core path wherever it can run
 int choose_path(int dtype, int B, int H, int n, int d, int r, int iters)
 {
-    if (!fused_supported(dtype, d, r)) return kPathGeneral;
-    const bool res_ok = B >= 1 && n >= 1 && resident_geometry(dtype, B, H, n, d, r).ok;
-    const bool slice_ok = B >= 1 && slice_supported(dtype, n, d, r);
+    if (!fused_supported(dtype, d, r) || B < 1 || n < 1) return kPathGeneral;
+    const bool res_ok = resident_geometry(dtype, B, H, n, d, r).ok;
+    const bool slice_ok = slice_supported(dtype, n, d, r);
     const int force = g_force_path.load();
     if (force == kPathGeneral) return kPathGeneral;
     if (force == kPathStreamed) return kPathStreamed;
     if (force == kPathLong && r > 16) return kPathLong;
     if (force == kPathResident) return res_ok ? kPathResident : kPathStreamed;
-    // short sequences: one thread block per slice, everything on chip, exact float32 logits
+    // short sequences: a pair of thread blocks per slice, everything on chip
     if (slice_ok) return kPathSlice;
-    // Measured at T = 10 (B200).  r <= 16: the general path's float32 kernel, 1.05 to 4.5 times the streamed kernel's speed
-    // everywhere.  r <= 32: it too with few rows in all or short sequences (65536 rows 71 us against 76 on the long path and
-    // 126 streamed), then the long path (131072 rows: 113 against 120 and 143) as long as its stored kernel, padded to 64
-    // pivots, stays in the L2 beside the rest.  Above that the long path takes everything up to 300000 rows (n = 2048, 16
-    // slices 64 us against 73 and 114; n = 16384, 16 slices 174 against 190; 24 slices 264 against 252) and all short
-    // sequences (n = 1024, 512 slices: 301 against 461).
-    if (B >= 1 && n >= 1) {
-        const long long rows = (long long)B * H * n;
-        if (r <= 16 || (r <= 32 && (n <= 1200 || rows <= 100000))) return kPathGeneral;
-        // ... of calls with three iterations and more: one or two show that the streamed path's first pass is on float32 values
-        // (errors of the potentials at n = 4096 in units of eps: 5e-6 against 1.3e-4 after one, 1.1e-4 against 1.3e-4 after
-        // two, 1.6e-4 on both after three)
-        if (iters >= 3 && (r <= 32 ? rows <= 200000 : n <= 1200 || rows <= 300000)) return kPathLong;
+    // Everything below measured on B200 at T = 10 unless said otherwise; us, in the order general / streamed / resident / long.
+    // r <= 16: the general path's float32 kernel, 1.05 to 4.5 times the streamed kernel's speed everywhere.
+    const long long rows = (long long)B * H * n, slices = (long long)B * H, sms = device_sm_count();
+    if (r <= 16) return kPathGeneral;
+    // r <= 32: it too with few rows or short sequences (16 slices of 8192 tokens 118 / 152, 192 of 1024 157 / 328), then the
+    // streamed path, which does not wait for memory there (16 of 11000 177 / 167, 16 of 16384 230 / 210).  Both keep
+    // float32 between the passes, which the long path's bf16 kernel does not (potentials to 8e-5 of eps instead of 2e-6), so
+    // it is taken only where a bf16 kernel always has been: about one slice per SM, of up to 14 tiles, whose kernel the
+    // resident path would keep on the SM (128 slices of 1400 tokens 159 / 165 / 159 / 122, of 1700 189 / 196 / 179 / 144).
+    if (r <= 32) {
+        if (n <= 1200 || rows <= 100000) return kPathGeneral;
+        if (iters >= 3 && n <= 1792 && slices <= sms && 2 * slices >= sms) return kPathLong;
+        return rows <= 160000 ? kPathGeneral : kPathStreamed;
     }
-    // Measured on B200: the resident kernel wins where the streamed one has no stored-kernel
-    // passes (r <= 32, every pass recomputes logits and exponentials) and every thread block holds its whole share at
-    // once (whole slices, one wave); elsewhere the streamed kernel is as fast or faster.
-    if (res_ok && r <= 32) {
-        const ResidentGeom G = resident_geometry(dtype, B, H, n, d, r);
-        if (G.whole && (long long)B * H <= (long long)G.ctas * G.wave_slices) return kPathResident;
-    }
-    return kPathStreamed;
+    // Above that the long path takes everything up to 300000 rows (n = 2048, 16 slices 73 / 114 / - / 64; n = 16384, 16 slices
+    // streamed 190, long 180) and all short sequences (n = 1024, 512 slices: 461 / - / - / 301), in calls of three iterations and
+    // more: one or two show that the streamed path's first pass is on float32 values (errors of the potentials at n = 4096 in
+    // units of eps: 5e-6 against 1.3e-4 after one, 1.1e-4 against 1.3e-4 after two, 1.6e-4 on both after three).
+    return iters >= 3 && (n <= 1200 || rows <= 300000) ? kPathLong : kPathStreamed;
 }
 
 size_t path_bytes(int path, int dtype, int B, int H, int n, int d, int r)
