@@ -47,7 +47,8 @@ __device__ __noinline__ void finish(const SweepArgs *ap, int p, int c)
     }
 }
 
-template <typename T, int RP, int CPL, int THREADS, bool GROUP>
+// KEEP: the weights of every iteration go to a.hist (backward).
+template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool KEEP>
 __global__ void __launch_bounds__(THREADS, max_blocks(CPL, THREADS))
 sweep_kernel(const __grid_constant__ SweepArgs a)
 {
@@ -88,18 +89,17 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
             const float tgt = S.tgt[tid < RP ? tid : 0];
             u64 w[CPL / 2];
             load_weights<RP, CPL>(L, w);
-            // backward: the weights of every iteration are kept (thread t's column; nullptr: not kept here)
-            float *hp = a.hist != nullptr && c == 0 && tid < RP ? a.hist + (size_t)p * RP + tid : nullptr;
-            if (hp != nullptr) *hp = S.w[tid];
+            float *hp = KEEP && c == 0 && tid < RP ? a.hist + (size_t)p * RP + tid : nullptr;      // thread t's column
+            if (KEEP && hp != nullptr) *hp = S.w[tid];
             for (; it < a.it1; ++it) {
                 bad = iterate<RP, CPL, THREADS, GROUP>(a, S, R, L, w, tgt, group, c, seq, wold, wnew);
                 if (bad) break;
-                if (hp != nullptr) {
+                if (KEEP && hp != nullptr) {
                     hp += (size_t)NP * RP;
                     *hp = tid < r ? wnew : 0.f;
                 }
             }
-            if (!bad && a.wide != nullptr && c == 0 && tid == 0) a.wide[p] = 0;
+            if (KEEP && !bad && c == 0 && tid == 0) a.wide[p] = 0;
         }
         if (bad) seq = recover<T, RP, CPL, THREADS, GROUP>(&a, p, group, c, it, seq, wold, wnew);
         if (p + a.groups >= NP) chain_next();
@@ -112,10 +112,10 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
 // ---------------------------------------------------------------------------------------------------------------
 constexpr int kSmPerBlockReserve = 1024, kSmemPerSM = 228 * 1024, kSmemPerBlock = 227 * 1024;
 
-template <typename T, int RP, int CPL, int THREADS, bool GROUP>
+template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool KEEP>
 static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t st)
 {
-    auto kern = sweep_kernel<T, RP, CPL, THREADS, GROUP>;
+    auto kern = sweep_kernel<T, RP, CPL, THREADS, GROUP, KEEP>;
     static std::mutex mu;
     static bool attr_set[64] = {};
     int dev = 0;
@@ -140,7 +140,11 @@ static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t
 template <typename T, int RP>
 static cudaError_t launch_t(const SweepPlan &P, const SweepArgs &a, cudaStream_t st)
 {
-    return P.C > 1 ? launch_g<T, RP, wide_cols(RP), 256, true>(P, a, st) : launch_g<T, RP, wide_cols(RP), 256, false>(P, a, st);
+    if constexpr (sizeof(T) == 2) {                          // the backward of float32 tensors keeps its own history
+        if (a.hist != nullptr)
+            return P.C > 1 ? launch_g<T, RP, wide_cols(RP), 256, true, true>(P, a, st) : launch_g<T, RP, wide_cols(RP), 256, false, true>(P, a, st);
+    }
+    return P.C > 1 ? launch_g<T, RP, wide_cols(RP), 256, true, false>(P, a, st) : launch_g<T, RP, wide_cols(RP), 256, false, false>(P, a, st);
 }
 
 template <typename T>
