@@ -149,7 +149,11 @@ LOT_API int lot_sinkhorn_static(const float *cost, const float *beta, const int3
                         float *g, float *f, float *plan, int32_t *status_out,
                         lot_stream_t stream);
 
-/* Scratch bytes lot_attention_fwd_ex needs for these sizes. */
+/*
+ * Scratch bytes lot_attention_fwd_ex needs for these sizes, whatever the number of iterations.  Path 0 of lot_path: one
+ * float32 number per token, side and pivot (r padded to a power of two from 16 on), but for bf16 tensors at most 8 GiB, the
+ * slices of larger calls running in parts (a slice is never split); float32 tensors: never less than 8 bytes per similarity.
+ */
 LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype);
 
 /*
@@ -181,7 +185,7 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *      pair's cluster; no workspace beyond the status word.  Taken wherever it can run.
  * On paths 1, 2 and 4 with 32 < r (1), any r (2, 4) the potentials of calls of two iterations and more agree with an exact
  * float evaluation to about 1e-4 (the iterations read a bf16 kernel); elsewhere to float32.  Beside its own bf16 rounding
- * `out` has an error of a quarter to four tenths of that rounding's: the plan's query side is read in bf16 (paths 1, 2, 4),
+ * `out` has an error of a quarter to a half of that rounding's: the plan's query side is read in bf16 (paths 1, 2, 4),
  * and on path 2, and path 1 from 4096 tiles of 128 tokens on, its key side too.
  */
 LOT_API int lot_path(int dtype, int B, int H, int n, int d, int r, int iters);
@@ -232,8 +236,10 @@ LOT_API int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
  *   beta is treated as r free positive numbers per head (no simplex constraint: a softmax parametrisation is the
  *   caller's chain rule); dz and dbeta are summed over the batch.
  * The forward is recomputed in the general path's arithmetic (float32 for bf16 tensors, float64 for float32 tensors);
- * of its iterations only the pivot potentials are kept.  bf16 tensors: 13 kernel launches, two numbers per token and
- * iteration in the workspace; float32 tensors: 2*iters + 15 launches.
+ * of its iterations only the pivot potentials are kept.  bf16 tensors: 13 kernel launches; the workspace holds, per token
+ * and side, two float32 numbers for each of the r pivots (r padded to a power of two from 16 on) and two for each iteration;
+ * calls that would need more than 8 GiB run their slices in parts of at most that, 13 launches each (a slice is never split).
+ * float32 tensors: 2*iters + 15 launches.
  * ws: lot_bwd_workspace_bytes(...) bytes of device scratch, 256-byte aligned, owned by the caller; the device
  * status word of the recomputed forward sits at its start (lot_device_status).
  * Errors as lot_attention_fwd_ex.  B == 0 or n == 0: dz and dbeta are zero-filled, nothing else is touched.
@@ -245,7 +251,7 @@ LOT_API int lot_attention_bwd(const void *q, const void *k, const void *v, const
                       void *dq, void *dk, void *dv, float *dz, float *dbeta,
                       void *ws, size_t ws_bytes, lot_stream_t stream);
 
-/* Scratch bytes lot_attention_fwd_var needs for these sizes. */
+/* Scratch bytes lot_attention_fwd_var needs for these sizes (as lot_workspace_bytes on path 0). */
 LOT_API size_t lot_var_workspace_bytes(int B, int H, int nq, int nk, int d, int r, int dtype);
 
 /*

@@ -196,7 +196,65 @@ BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
     return L;
 }
 
+// A call on the stored kernel whose workspace would pass kPartBytes runs its slices in parts one after the other: batch rows,
+// or heads of one row.  Below that nothing is gained, a part of that size keeps the device busy for milliseconds.
+constexpr size_t kPartBytes = (size_t)8 << 30;
+struct Parts {
+    int rows, heads;         // of a part; heads < H only with rows == 1
+};
+// bytes(rows, heads): workspace of such a part
+template <typename F> Parts split_parts(int B, int H, F bytes)
+{
+    auto most = [](int n, auto fits) {                        // the largest k <= n that fits, then as even as the parts allow
+        int lo = 1, hi = n;
+        while (lo < hi) {
+            const int mid = lo + (hi - lo + 1) / 2;
+            if (fits(mid)) lo = mid; else hi = mid - 1;
+        }
+        const int parts = (n + lo - 1) / lo;
+        return (n + parts - 1) / parts;
+    };
+    if (B < 1 || bytes(B, H) <= kPartBytes) return Parts{B, H};
+    if (bytes(1, H) <= kPartBytes) return Parts{most(B, [&](int k) { return bytes(k, H) <= kPartBytes; }), H};
+    return Parts{1, most(H, [&](int k) { return bytes(1, k) <= kPartBytes; })};
+}
+// Workspace of the whole call: that of a part or of the smaller last one.
+template <typename F> size_t parts_bytes(int B, int H, F bytes)
+{
+    const Parts P = split_parts(B, H, bytes);
+    size_t most = bytes(P.rows, P.heads);
+    if (P.rows > 0 && B % P.rows != 0 && bytes(B % P.rows, H) > most) most = bytes(B % P.rows, H);
+    if (H % P.heads != 0 && bytes(P.rows, H % P.heads) > most) most = bytes(P.rows, H % P.heads);
+    return most;
+}
+// run(b0, rows, h0, heads) for every part, until one fails
+template <typename F> cudaError_t for_parts(int B, int H, Parts P, F run)
+{
+    for (int b = 0; b < B; b += P.rows)
+        for (int h = 0; h < H; h += P.heads) {
+            const cudaError_t e = run(b, B - b < P.rows ? B - b : P.rows, h, H - h < P.heads ? H - h : P.heads);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
 template <typename T> inline T *at(void *ws, size_t off) { return reinterpret_cast<T *>(static_cast<char *>(ws) + off); }
+
+// bf16 tensors only: for float32 ones the interface has always asked for more than the kernel takes
+Parts forward_parts(int B, int H, int nq, int nk, int d, int r, int dtype, bool variant)
+{
+    if (dtype == LOT_F32) return Parts{B, H};
+    return split_parts(B, H, [&](int rows, int heads) { return forward_layout(rows, heads, nq, nk, d, r, dtype, variant).total; });
+}
+size_t forward_bytes(int B, int H, int nq, int nk, int d, int r, int dtype, bool variant)
+{
+    auto bytes = [&](int rows, int heads) { return forward_layout(rows, heads, nq, nk, d, r, dtype, variant).total; };
+    return dtype == LOT_F32 ? bytes(B, H) : parts_bytes(B, H, bytes);
+}
+size_t bwd_bytes(int B, int H, int n, int d, int r, int iters)
+{
+    return parts_bytes(B, H, [&](int rows, int heads) { return bwd_sweep_layout(rows, heads, n, d, r, iters).total; });
+}
 
 struct Managed {
     void *ptr = nullptr;
@@ -262,7 +320,7 @@ size_t path_bytes(int path, int dtype, int B, int H, int n, int d, int r)
     if (path == kPathStreamed) return fused_layout(B, H, n, d, r).total;
     if (path == kPathLong) return stream_plan(B * H, n).total;
     if (path == kPathSlice) return 256;                              // the status word
-    return forward_layout(B, H, n, n, d, r, dtype, false).total;
+    return forward_bytes(B, H, n, n, d, r, dtype, false);
 }
 
 // Whether the first `bytes` of two tensors share memory.
@@ -272,12 +330,43 @@ bool overlap(const void *a, const void *b, size_t bytes)
     return x < y ? y - x < bytes : x - y < bytes;
 }
 
-// Both Sinkhorn problems and the apply stages on the general path.
-cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, const void *v, const float *z, const float *beta,
-                        const float *mass_q, const float *mass_k, int skip, int terms, const int32_t *key_len, const float *g1_in, const float *g2_in,
-                        int dtype, int B, int H, int nq, int nk, int d, int r, float eps, int iters, void *out, float *g1_out,
-                        float *g2_out, void *ws, cudaStream_t s)
+// A forward on the general path.
+struct ForwardCall {
+    const void *q, *k, *v;
+    const float *z, *beta, *mass_q, *mass_k;
+    int skip, terms;
+    const int32_t *key_len;
+    const float *g1_in, *g2_in;
+    int dtype, B, H, nq, nk, d, r;
+    float eps;
+    int iters;
+    void *out;
+    float *g1_out, *g2_out;
+
+    // heads h0 .. h0 + heads - 1 of batch rows b0 .. b0 + rows - 1, which are neighbours in memory
+    ForwardCall part(int b0, int rows, int h0, int heads) const
+    {
+        ForwardCall c = *this;
+        const size_t s = (size_t)b0 * H + h0, es = dtype == LOT_F32 ? 4 : 2;
+        c.q = static_cast<const char *>(q) + s * nq * d * es; c.k = static_cast<const char *>(k) + s * nk * d * es;
+        c.v = static_cast<const char *>(v) + s * nk * d * es; c.out = static_cast<char *>(out) + s * nq * d * es;
+        c.z = z + (size_t)h0 * r * d; c.beta = beta + (size_t)h0 * r;
+        if (mass_q) c.mass_q = mass_q + s * nq;
+        if (mass_k) c.mass_k = mass_k + s * nk;
+        if (key_len) c.key_len = key_len + b0;
+        if (g1_in) c.g1_in = g1_in + s * r;
+        if (g2_in) c.g2_in = g2_in + s * r;
+        if (g1_out) c.g1_out = g1_out + s * r;
+        if (g2_out) c.g2_out = g2_out + s * r;
+        c.B = rows; c.H = heads;
+        return c;
+    }
+};
+
+// Both Sinkhorn problems and the apply stages.  first: of the call's parts (the status word is cleared once).
+cudaError_t run_forward(const ForwardLayout &L, const ForwardCall &f, bool first, void *ws, cudaStream_t s)
 {
+    const int dtype = f.dtype, B = f.B, H = f.H, nq = f.nq, nk = f.nk, d = f.d, r = f.r, skip = f.skip, terms = f.terms, iters = f.iters;
     SweepArgs a{};
     SweepApplyArgs ap{};
     for (int side = 0; side < 2; ++side) {
@@ -285,13 +374,13 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
         a.w[side] = at<float>(ws, L.w[side]); a.gref[side] = at<double>(ws, L.gref[side]);
         ap.kt[side] = a.kt[side]; ap.inv[side] = a.inv[side]; ap.w[side] = a.w[side];
     }
-    a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
-    a.mass[0] = mass_q; a.mass[1] = mass_k; a.g_in[0] = g1_in; a.g_in[1] = g2_in; a.g_out[0] = g1_out; a.g_out[1] = g2_out;
+    a.x[0] = f.q; a.x[1] = f.k; a.z = f.z; a.beta = f.beta; a.key_len = f.key_len;
+    a.mass[0] = f.mass_q; a.mass[1] = f.mass_k; a.g_in[0] = f.g1_in; a.g_in[1] = f.g2_in; a.g_out[0] = f.g1_out; a.g_out[1] = f.g2_out;
     a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf); a.status = at<int>(ws, 0);
-    a.head = at<uint4>(ws, 0); a.head_words = L.head_end / 16;
+    a.head = at<uint4>(ws, first ? 0 : 256); a.head_words = (L.head_end - (first ? 0 : 256)) / 16;
     a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip; a.terms = terms;
     a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
-    a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
+    a.scale = 1.4426950408889634 / (double)f.eps; a.eps_ln2 = (double)f.eps * 0.6931471805599453;
     a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
     cudaError_t e;
     if (!L.plan.steps) {
@@ -308,7 +397,7 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
             if ((e = launch_sweep(L.plan, a, dtype, s)) != cudaSuccess) return e;
         }
     }
-    ap.beta = beta; ap.key_len = key_len; ap.mass2 = mass_k; ap.v = v; ap.out = out;
+    ap.beta = f.beta; ap.key_len = f.key_len; ap.mass2 = f.mass_k; ap.v = f.v; ap.out = f.out;
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
     ap.B = B; ap.H = H; ap.nq = nq; ap.nk = nk; ap.d = d; ap.r = r; ap.RP = L.plan.RP; ap.skip = skip; ap.terms = terms;
     ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
@@ -316,10 +405,23 @@ cudaError_t run_forward(const ForwardLayout &L, const void *q, const void *k, co
     return launch_sweep_apply_out(ap, dtype, s);
 }
 
-// lot_attention_bwd for bf16 tensors, behind the argument checks.
+// ... of all parts, the class-token row of each behind it.
+cudaError_t run_forward_parts(const ForwardCall &f, bool variant, float cls_tau, void *ws, cudaStream_t s)
+{
+    return for_parts(f.B, f.H, forward_parts(f.B, f.H, f.nq, f.nk, f.d, f.r, f.dtype, variant), [&](int b0, int rows, int h0, int heads) {
+        const ForwardCall c = f.part(b0, rows, h0, heads);
+        const ForwardLayout L = forward_layout(rows, heads, f.nq, f.nk, f.d, f.r, f.dtype, variant);
+        const cudaError_t e = run_forward(L, c, b0 == 0 && h0 == 0, ws, s);
+        if (e != cudaSuccess || !f.skip) return e;
+        return launch_cls_row(c.q, c.k, c.v, c.key_len, f.dtype, rows, heads, f.nq, f.nk, f.d, cls_tau, at<float>(ws, L.scores), c.out, s);
+    });
+}
+
+// lot_attention_bwd for bf16 tensors, behind the argument checks.  first: of the call's parts; add: dz and dbeta hold the
+// sums of earlier parts.
 cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, const void *v, const float *z, const float *beta,
                          const int32_t *key_len, const void *dout, int B, int H, int n, int d, int r, float eps, int iters, void *dq,
-                         void *dk, void *dv, float *dz, float *dbeta, void *ws, cudaStream_t st)
+                         void *dk, void *dv, float *dz, float *dbeta, bool first, bool add, void *ws, cudaStream_t st)
 {
     const int dt = LOT_BF16, RP = L.plan.RP;
     cudaError_t e;
@@ -336,7 +438,7 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
     a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
     a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf);
     a.hist = at<float>(ws, L.hist); a.hist_g = at<double>(ws, L.hist_g); a.wide = at<int>(ws, L.wide); a.status = at<int>(ws, 0);
-    a.head = at<uint4>(ws, 0); a.head_words = L.head_end / 16;
+    a.head = at<uint4>(ws, first ? 0 : 256); a.head_words = (L.head_end - (first ? 0 : 256)) / 16;
     a.B = B; a.H = H; a.d = d; a.r = r;
     a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
@@ -377,7 +479,7 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
         y.v = side ? k : q; y.Wp = nullptr; y.wpart = at<float>(ws, L.zpart[side]);
         if ((e = launch_sweep_apply_w(y, dt, st)) != cudaSuccess) return e;
     }
-    return launch_bwd_merge(at<float>(ws, L.zpart[0]), at<float>(ws, L.zpart[1]), dbd, b.dbeta_acc, dz, dbeta, B, H, d, r, RP, L.achunks, st);
+    return launch_bwd_merge(at<float>(ws, L.zpart[0]), at<float>(ws, L.zpart[1]), dbd, b.dbeta_acc, dz, dbeta, B, H, d, r, RP, L.achunks, add, st);
 }
 
 // Scratch of lot_sinkhorn_static: part of the library image, present on every device that loads
@@ -528,7 +630,9 @@ int lot_launch_count(int dtype, int B, int H, int n, int d, int r, int iters)
     if (path == kPathStreamed) return fused_launches(B, H, n, r, iters);
     if (path == kPathSlice) return 1;
     if (path == kPathLong) return 3;
-    return sweep_plan(dtype, B * H > 0 ? B * H : 1, n, n, d, r).steps ? 2 + iters + 1 + 2 : 4;
+    if (B < 1 || n < 1) return 0;
+    const Parts P = forward_parts(B, H, n, n, d, r, dtype, false);
+    return sweep_plan(dtype, B * H, n, n, d, r).steps ? 2 + iters + 1 + 2 : 4 * ((B + P.rows - 1) / P.rows) * ((H + P.heads - 1) / P.heads);
 }
 
 int lot_debug_hook(int what, long long value)
@@ -597,13 +701,12 @@ int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
         return e == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
     }
     remember_ws(ws, kPathGeneral, 0, 0);
-    const ForwardLayout L = forward_layout(B, H, n, n, d, r, dtype, false);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
-    cudaStream_t s = (cudaStream_t)stream;
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < forward_bytes(B, H, n, n, d, r, dtype, false)) return LOT_ERR_WORKSPACE;
     // sizes of the tensor-core paths keep their hi + lo operands here too; a forced general path is float32 throughout
     const int terms = fused_supported(dtype, d, r) && g_force_path.load() != kPathGeneral ? 2 : 3;
-    return run_forward(L, q, k, v, z, beta, nullptr, nullptr, 0, terms, key_len, nullptr, nullptr, dtype, B, H, n, n, d, r, eps, iters, out,
-                       g1_out, g2_out, ws, s) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
+    const ForwardCall f{q, k, v, z, beta, nullptr, nullptr, 0, terms, key_len, nullptr, nullptr, dtype, B, H, n, n, d, r, eps, iters, out,
+                        g1_out, g2_out};
+    return run_forward_parts(f, false, 0.f, ws, (cudaStream_t)stream) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
 }
 
 size_t lot_var_workspace_bytes(int B, int H, int nq, int nk, int d, int r, int dtype)
@@ -611,7 +714,7 @@ size_t lot_var_workspace_bytes(int B, int H, int nq, int nk, int d, int r, int d
     if (dtype != LOT_F32 && dtype != LOT_BF16) return 0;
     if (check_dims(B, H, nq, r) != LOT_OK || check_dims(B, H, nk, r) != LOT_OK) return 0;
     if (check_d(nq, d) != LOT_OK || check_d(nk, d) != LOT_OK) return 0;
-    return forward_layout(B, H, nq, nk, d, r, dtype, true).total;
+    return forward_bytes(B, H, nq, nk, d, r, dtype, true);
 }
 
 int lot_attention_fwd_var(const void *q, const void *k, const void *v, const float *z, const float *beta,
@@ -637,17 +740,11 @@ int lot_attention_fwd_var(const void *q, const void *k, const void *v, const flo
         !aligned16(g1_out) || !aligned16(g2_out) || !aligned16(g1_in) || !aligned16(g2_in) || !aligned16(a) ||
         !aligned16(b) || (key_len && (reinterpret_cast<uintptr_t>(key_len) & 3u)))
         return LOT_ERR_INVALID_ARG;
-    const ForwardLayout L = forward_layout(B, H, nq, nk, d, r, dtype, true);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
-    cudaStream_t s = (cudaStream_t)stream;
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < forward_bytes(B, H, nq, nk, d, r, dtype, true)) return LOT_ERR_WORKSPACE;
     remember_ws(ws, kPathGeneral, 0, 0);
     // the class token is neither a query nor a key of the transport problem: it is skipped on both sides
-    if (run_forward(L, q, k, v, z, beta, a, b, cls, 3, key_len, g1_in, g2_in, dtype, B, H, nq, nk, d, r, eps, iters, out, g1_out, g2_out,
-                    ws, s) != cudaSuccess)
-        return LOT_ERR_CUDA;
-    if (cls && launch_cls_row(q, k, v, key_len, dtype, B, H, nq, nk, d, cls_tau, at<float>(ws, L.scores), out, s) != cudaSuccess)
-        return LOT_ERR_CUDA;
-    return LOT_OK;
+    const ForwardCall f{q, k, v, z, beta, a, b, cls, 3, key_len, g1_in, g2_in, dtype, B, H, nq, nk, d, r, eps, iters, out, g1_out, g2_out};
+    return run_forward_parts(f, true, cls_tau, ws, (cudaStream_t)stream) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
 }
 
 int lot_attention_fwd(const float *q, const float *k, const float *v,
@@ -721,7 +818,7 @@ size_t lot_bwd_workspace_bytes(int B, int H, int n, int d, int r, int dtype, int
 {
     if (dtype != LOT_F32 && dtype != LOT_BF16) return 0;
     if (check_dims(B, H, n, r) != LOT_OK || check_d(n, d) != LOT_OK || iters < 0) return 0;
-    return dtype == LOT_BF16 ? bwd_sweep_layout(B, H, n, d, r, iters).total : bwd_layout(B, H, n, d, r, iters).total;
+    return dtype == LOT_BF16 ? bwd_bytes(B, H, n, d, r, iters) : bwd_layout(B, H, n, d, r, iters).total;
 }
 
 int lot_attention_bwd(const void *q, const void *k, const void *v, const float *z, const float *beta,
@@ -750,11 +847,17 @@ int lot_attention_bwd(const void *q, const void *k, const void *v, const float *
         !aligned16(dv) || (key_len && (reinterpret_cast<uintptr_t>(key_len) & 3u)))
         return LOT_ERR_INVALID_ARG;
     if (dtype == LOT_BF16) {
-        const BwdSweepLayout L = bwd_sweep_layout(B, H, n, d, r, iters);
-        if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;
+        if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < bwd_bytes(B, H, n, d, r, iters)) return LOT_ERR_WORKSPACE;
         remember_ws(ws, kPathGeneral, 0, 0);
-        return run_backward(L, q, k, v, z, beta, key_len, dout, B, H, n, d, r, eps, iters, dq, dk, dv, dz, dbeta, ws, s) == cudaSuccess
-                   ? LOT_OK : LOT_ERR_CUDA;
+        const Parts P = split_parts(B, H, [&](int rows, int heads) { return bwd_sweep_layout(rows, heads, n, d, r, iters).total; });
+        return for_parts(B, H, P, [&](int b0, int rows, int h0, int heads) {
+            const size_t o = ((size_t)b0 * H + h0) * n * d * 2, oz = (size_t)h0 * r * d, ob = (size_t)h0 * r;
+            auto in = [&](const void *p) { return static_cast<const void *>(static_cast<const char *>(p) + o); };
+            auto res = [&](void *p) { return static_cast<void *>(static_cast<char *>(p) + o); };
+            return run_backward(bwd_sweep_layout(rows, heads, n, d, r, iters), in(q), in(k), in(v), z + oz, beta + ob,
+                                key_len ? key_len + b0 : nullptr, in(dout), rows, heads, n, d, r, eps, iters, res(dq), res(dk), res(dv),
+                                dz + oz, dbeta + ob, b0 == 0 && h0 == 0, b0 > 0, ws, s);
+        }) == cudaSuccess ? LOT_OK : LOT_ERR_CUDA;
     }
     const BwdLayout L = bwd_layout(B, H, n, d, r, iters);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < L.total) return LOT_ERR_WORKSPACE;

@@ -95,8 +95,8 @@ struct SweepBwdArgs {
 cudaError_t launch_bwd_close(int RP, const SweepBwdArgs &a, cudaStream_t st);
 cudaError_t launch_bwd_reverse(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st);
 cudaError_t launch_bwd_assemble(int RP, const SweepBwdArgs &a, cudaStream_t st);
-// dz[h][t][c] = sum over batch, sides and chunks of the partials of dC^T x; dbeta as in launch_bwd_dz
+// dz[h][t][c] = sum over batch, sides and chunks of the partials of dC^T x; dbeta as in launch_bwd_dz; add: on top of what they hold
 cudaError_t launch_bwd_merge(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz,
-                             float *dbeta, int B, int H, int d, int r, int RP, int chunks, cudaStream_t st);
+                             float *dbeta, int B, int H, int d, int r, int RP, int chunks, bool add, cudaStream_t st);
 
 } // namespace lot

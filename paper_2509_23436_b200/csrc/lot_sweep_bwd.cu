@@ -354,7 +354,7 @@ assemble_kernel(const __grid_constant__ SweepBwdArgs a)
 }
 
 __global__ void merge_kernel(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz, float *dbeta, int B, int H, int d,
-                             int r, int RP, int chunks)
+                             int r, int RP, int chunks, bool add)
 {
     // eight threads an element, each a share of the partials (of the batch rows for beta), requested eight at a time: bound by
     // latency, 12 us at B = 32, H = 3, r = 16, d = 64 when one thread went through the batch rows of beta
@@ -386,8 +386,8 @@ __global__ void merge_kernel(const float *part_q, const float *part_k, const flo
         sum += __shfl_xor_sync(0xffffffffu, sum, off);
         bsum += __shfl_xor_sync(0xffffffffu, bsum, off);
     }
-    if (part == 0 && idx < (size_t)H * per) dz[idx] = sum;
-    if (part == 0 && idx < (size_t)H * r) dbeta[idx] = bsum;
+    if (part == 0 && idx < (size_t)H * per) dz[idx] = add ? dz[idx] + sum : sum;
+    if (part == 0 && idx < (size_t)H * r) dbeta[idx] = add ? dbeta[idx] + bsum : bsum;
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -453,11 +453,11 @@ cudaError_t launch_bwd_reverse(const SweepPlan &P, const SweepBwdArgs &a, cudaSt
 }
 
 cudaError_t launch_bwd_merge(const float *part_q, const float *part_k, const float *dbeta_direct, const float *dbeta_acc, float *dz,
-                             float *dbeta, int B, int H, int d, int r, int RP, int chunks, cudaStream_t st)
+                             float *dbeta, int B, int H, int d, int r, int RP, int chunks, bool add, cudaStream_t st)
 {
     const size_t threads = (size_t)H * r * d * 8;
     return chain_launch(sweep::merge_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, st, part_q, part_k, dbeta_direct, dbeta_acc, dz, dbeta,
-                        B, H, d, r, RP, chunks);
+                        B, H, d, r, RP, chunks, add);
 }
 
 } // namespace lot

@@ -47,3 +47,19 @@ def test_empty_problems_have_a_path(L):
     for B, n in ((0, 1000), (2, 0), (0, 0)):
         assert L.lot_path(lot.LOT_BF16, B, 4, n, 64, 64, 10) == GENERAL
         assert L.lot_workspace_bytes(B, 4, n, 64, 64, lot.LOT_BF16) > 0
+
+
+def test_workspace_of_large_calls_is_bounded(L):
+    """Slices beyond 8 GiB of workspace go in parts; a slice by itself is never split, and float32 tensors keep the size they
+    always asked for."""
+    limit = 8 << 30
+    assert L.lot_bwd_workspace_bytes(64, 128, 4096, 8, 16, lot.LOT_BF16, 10) <= limit
+    assert L.lot_bwd_workspace_bytes(2, 8192, 4096, 8, 16, lot.LOT_BF16, 50) <= limit
+    assert L.lot_bwd_workspace_bytes(1, 7, 1 << 22, 64, 256, lot.LOT_BF16, 50) == L.lot_bwd_workspace_bytes(1, 1, 1 << 22, 64, 256, lot.LOT_BF16, 50) > limit
+    assert L.lot_workspace_bytes(512, 64, 8000, 32, 129, lot.LOT_BF16) <= limit
+    assert L.lot_var_workspace_bytes(512, 63, 8000, 777, 32, 129, lot.LOT_BF16) <= limit
+    assert L.lot_workspace_bytes(512, 63, 8000, 32, 129, lot.LOT_F32) >= 512 * 63 * 16000 * 129 * 8
+    assert L.lot_launch_count(lot.LOT_BF16, 128, 128, 4096, 8, 16, 10) == 8 and L.lot_launch_count(lot.LOT_BF16, 12, 128, 4096, 8, 16, 10) == 4
+    # below the limit it is that of one part
+    one = L.lot_bwd_workspace_bytes(1, 16, 4096, 64, 64, lot.LOT_BF16, 10)
+    assert one < 3 * 2 * 16 * 4096 * 64 * 4
