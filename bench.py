@@ -460,7 +460,7 @@ def run_backward(args):
             "steps": args.steps, "warmup": warm, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": ARITH[0][tdt], "data": "synthetic",
             "config": config_of(x, {"l2": "flushed between timed steps (512 MiB overwrite)",
-                                    "op": "backward (forward recomputed inside, materialised similarities)"}),
+                                    "op": "backward (forward recomputed inside: on the stored kernel for bf16 tensors, on materialised similarities for float32)"}),
             "clocks": clocks, "gpu_launches": (2 * x.iters + 15 if tdt == "float32" else 13) * args.steps,
             "forward_ms_per_step": sum(tf) / len(tf), "backward_over_forward": ms / (sum(tf) / len(tf)),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,

@@ -6,10 +6,14 @@
 // streamed path has always had; potentials to about 1e-4): half the bytes, so a pass over n = 16384, H = 16 reads 67 MB, of
 // which the blocks keep the first rows of their share in shared memory and the rest comes from L2.  Each block
 // computes the logits of its own rows (warp-level products, Z as bf16 hi + lo), so building one group's kernel
-// overlaps another's passes.  At n = 4096, H = 16, r = 64, T = 10: 46 us (15 of them building) and 23 for the apply kernels,
-// against 117 in all on the streamed path; at n = 16384 128 (46) + 42 against 190.  A pass is bound by latency: per
-// scheduler four warps, whose registers hold the weights, the column sums and two rows, issue in 40% of the cycles.  When all problems together exceed the L2, groups are made larger and work through the problems
-// in rounds, so that what is iterated on stays in the L2.
+// overlaps another's passes.  At n = 4096, H = 16, r = 64, T = 10: 47 us (17 of them building) of a call of 71, which took 117 on
+// the streamed path; at n = 16384 135 (52) of 180, against 190.  A pass is bound by latency: per
+// scheduler four warps, whose registers hold the weights, the column sums and two rows, issue in 40% of the cycles.
+//
+// The key side is applied from twice bf16's precision, as the streamed path's apply passes do with recomputed logits: the
+// building also leaves K minus its rounding, which only apply_w reads (1.4 us of a call at n = 4096; 12 at n = 16384: 34 MB
+// written, 6 us, read again, 5, and in the L2 in place of other rows).  When all problems together exceed the L2, groups are
+// made larger and work through the problems in rounds, so that what is iterated on stays in the L2.
 #include "lot_chain.cuh"
 #include "lot_sweep_core.cuh"
 

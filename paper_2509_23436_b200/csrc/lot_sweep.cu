@@ -168,7 +168,7 @@ cudaError_t launch_sweep(const SweepPlan &P, const SweepArgs &a, int dtype, cuda
 
 // Blocks per problem and where the rows live: the split with the least modelled time.  A round (all resident groups
 // finish one problem each) costs its build plus, per iteration, the larger of one block's latency chain and the SM's
-// shared-memory and issue time; see the comments at the constants for what was measured.
+// shared-memory and issue time; see the comment at the constants for what they come from.
 SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
 {
     using namespace sweep;
@@ -201,10 +201,13 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
             const int resident = C == 1 ? (P < slots ? P : slots) : groups * C;
             const int rounds = C == 1 ? (P + slots - 1) / slots : (P + groups - 1) / groups;
             const double per_sm = (double)((resident + sms - 1) / sms);       // blocks that share an SM
-            // us: SM time per entry (issue and shared-memory reads), twice that for a block alone on its SM; the exchange as
-            // measured (0.7 for two blocks at RP = 256, 2.1 for 16; with owners 5.2-7.0 at 49-148, fitted with the rate one SM
-            // reads at to config 5's times over C: 3771 us at 49, 3971 at 59, 4520 at 74, 6300 at 148); streamed rows at the L2's
-            // rate, at the HBM's when all of them exceed the L2, and never faster than one SM reads
+            // us: SM time per entry (issue and shared-memory reads), twice that for a block alone on its SM; the latency of an
+            // iteration with its exchange; streamed rows at the L2's rate, at the HBM's when all of them exceed the L2, and
+            // never faster than one SM reads.  The constants are fitted to the times of whole calls, the last two lines of
+            // latency and the rate of one SM to those of 64 problems of 16384 rows at RP = 256 over C (sweep kernel, 20
+            // iterations: 4152 us at 42, 3833 at 49, 3957 at 59, 4312 at 74, 4877 at 98, 5947 at 148).  Measured by itself
+            // (group_columns) the latency is 4.9 at 49 blocks, 5.6 at 74, 7.7 at 148 with owners, where the line says 5.2,
+            // 5.6, 7.0; without them the line is too low from 8 blocks on (16 blocks at RP = 256: 3.7, line 2.5).
             const double entry = (RP <= 32 ? 0.055 : 0.045) / 1900.0;
             const double lat = C == 1 ? 0.45 : C * RP <= kDirectWords ? 0.9 + 0.4 * C * RP / 1024.0 : 4.3 + 0.018 * C;
             const double mine = 2.0 * rows * RP * entry, sm_us = per_sm * rows * RP * entry;

@@ -1,9 +1,9 @@
 // Apply stages behind the sweep kernel (Eq. (4)): W' = Diag(1/beta) Gamma2 V and out = R1 W', with the plan rows read
 // off the stored Gibbs kernel: R_it = kt_it w_t inv_i.
 //
-// bf16 tensors: tensor cores, warp-level products.  A float32 factor is the exact sum of three bf16 terms, so the products
-// are those of the float32 evaluation up to terms below 2^-24 and sums accumulate in float32; the plan entries never exist
-// in memory.  float32 tensors: CUDA cores (their products would need six terms a piece on the tensor cores).
+// bf16 tensors: tensor cores, warp-level products.  A float32 factor is the exact sum of three bf16 terms, so with N = 3 the
+// products are those of the float32 evaluation up to terms below 2^-24 (N = 2, hi + lo: 2^-17) and sums accumulate in
+// float32; the plan entries never exist in memory.  float32 tensors: CUDA cores (their products would need six terms a piece on the tensor cores).
 // All kernels load the next step's operands into registers while the current one multiplies; what bounds them is the
 // read of the kernel (4 bytes per entry) and, at rank 256, the product rate.
 #include "lot_chain.cuh"
@@ -72,7 +72,7 @@ __device__ __forceinline__ bool last_of_tile(unsigned *counter, int chunks)
 
 // ---------------------------------------------------------------------------------------------------------------
 // Key side, bf16 tensors: W[t][c] = sum_j R_jt m_j v_jc.  Block = TP pivots x D channels over one chunk of keys, 64 keys per
-// step: the plan tile goes to shared memory as three bf16 planes (transposed on the way to the tensor cores), the values
+// step: the plan tile goes to shared memory as N bf16 planes (transposed on the way to the tensor cores), the values
 // as they are.  Warps: TP / 16 pivot tiles x channel groups x (rank 16, narrow heads) halves of the keys.
 // ---------------------------------------------------------------------------------------------------------------
 template <int TP, int D, int N>
@@ -214,7 +214,7 @@ apply_w_mma_kernel(SweepApplyArgs a)
 
 // ---------------------------------------------------------------------------------------------------------------
 // Query side, bf16 tensors: out[i][c] = sum_t R_it W'[t][c].  Block = 128 queries x D channels; a warp's 16 plan rows come
-// from global memory straight into operand fragments, W' in steps of TS pivots through shared memory as three planes.
+// from global memory straight into operand fragments, W' in steps of TS pivots through shared memory as N planes.
 // ---------------------------------------------------------------------------------------------------------------
 template <int TS, int D, int N>
 __global__ void __launch_bounds__(kThreads, D <= 128 ? 2 : 1)

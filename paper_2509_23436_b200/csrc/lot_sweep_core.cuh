@@ -397,8 +397,10 @@ __device__ __forceinline__ float take_word(const u64 *p, u64 first, unsigned tag
 // Totals of the group's column values: thread t < RP gives its block's value of column t and gets the group's.
 // Small groups: every block reads every block's words.  Large ones (C * RP > kDirectWords): block t % C adds up column t
 // and leaves the total in kCopies places, each read by a share of the blocks (one place for all of 148 blocks to poll
-// took 5.9 us per exchange at RP = 256, eight take 4.4; reading every block's words takes 12.9 there, but 2.1 for 16
-// blocks and 0.7 for two).  Two buffers by parity: a block can be at most one exchange ahead of the others.
+// took a third more per exchange than eight at RP = 256, and reading every block's words there three times as long).  A
+// whole iteration with 16 rows a block takes 0.6 us alone; at RP = 256 1.2 with two blocks, 2.1 with 8, 3.7 with 16 (every
+// word read), 4.9 with 49, 5.6 with 74, 7.7 with 148 (owners); at RP = 32 1.1, 1.4, 1.8, 2.5, 3.0, 5.8.  Two buffers by
+// parity: a block can be at most one exchange ahead of the others.
 template <int RP, int THREADS, bool MAX, typename Args>
 __device__ __forceinline__ float group_columns(const Args &a, const Shared &S, float part, int group, int c, unsigned &seq)
 {

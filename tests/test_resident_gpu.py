@@ -3,7 +3,7 @@ memory across the Sinkhorn iterations) against the float64 oracle, over the laun
 (one contiguous tile range per thread block, column partials exchanged through global memory), whole mode (whole
 sequences per block, one or two at a time, several waves), spilled key tiles (a block with more than 12 key tiles),
 key masks that leave blocks without key tiles, every padded pivot width, zero and one iteration.  The library
-takes this path by default only where it measured faster; here the test hook selects it everywhere it can run.
+takes it nowhere by default (other paths measured faster); the test hook selects it everywhere it can run.
 Also: a problem the stored kernel cannot represent is recomputed by the streamed kernels, and a wait that cannot
 end runs out, is reported, and leaves the workspace usable."""
 import numpy as np
