@@ -67,7 +67,7 @@ SinkLayout sink_layout(int nprob, int n, int r, size_t base, size_t lt)
 struct ForwardLayout {
     SweepPlan plan;
     int rounds;              // problems a group works through per launch
-    size_t counter, xbuf, ybuf, head_end, w[2], gref[2], inv[2], kt[2], scores, wpart, Wp, total;
+    size_t counter, xbuf, head_end, w[2], gref[2], inv[2], kt[2], scores, wpart, Wp, total;
     int achunks, arows;
 };
 
@@ -81,9 +81,7 @@ ForwardLayout forward_layout(int B, int H, int nq, int nk, int d, int r, int dty
     size_t o = 256;                                                   // status word at 0
     L.counter = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
     L.xbuf = o;
-    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * L.plan.C * RP * 8);
-    L.ybuf = o;
-    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * kSweepCopies * RP * 8);
+    o += up256(exchange_bytes(RP, L.plan.C, L.plan.K, L.plan.groups));
     L.head_end = o;
     for (int side = 0; side < 2; ++side) {
         L.w[side] = o; o += up256((size_t)BH * RP * 4);
@@ -150,7 +148,7 @@ BwdLayout bwd_layout(int B, int H, int n, int d, int r, int iters)
 struct BwdSweepLayout {
     SweepPlan plan;
     int rounds, tiles, achunks, arows;
-    size_t counter, xbuf, ybuf, head_end, w[2], gref[2], inv[2], kt[2], dC[2], hist, hist_g, wide, coef, fk, gpart, dbeta_acc, wpart,
+    size_t counter, xbuf, head_end, w[2], gref[2], inv[2], kt[2], dC[2], hist, hist_g, wide, coef, fk, gpart, dbeta_acc, wpart,
         Wp, Xw, dWm, dbeta_direct, zpart[2], total;
 };
 
@@ -166,9 +164,7 @@ BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
     size_t o = 256;                                                   // status word at 0
     L.counter = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
     L.xbuf = o;
-    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * L.plan.C * RP * 8);
-    L.ybuf = o;
-    if (L.plan.C > 1) o += up256((size_t)L.plan.groups * 2 * kSweepCopies * RP * 8);
+    o += up256(exchange_bytes(RP, L.plan.C, L.plan.K, L.plan.groups));
     L.head_end = o;
     for (int side = 0; side < 2; ++side) {
         L.w[side] = o; o += up256((size_t)BH * RP * 4);
@@ -376,10 +372,10 @@ cudaError_t run_forward(const ForwardLayout &L, const ForwardCall &f, bool first
     }
     a.x[0] = f.q; a.x[1] = f.k; a.z = f.z; a.beta = f.beta; a.key_len = f.key_len;
     a.mass[0] = f.mass_q; a.mass[1] = f.mass_k; a.g_in[0] = f.g1_in; a.g_in[1] = f.g2_in; a.g_out[0] = f.g1_out; a.g_out[1] = f.g2_out;
-    a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf); a.status = at<int>(ws, 0);
+    a.xbuf = at<unsigned long long>(ws, L.xbuf); a.status = at<int>(ws, 0);
     a.head = at<uint4>(ws, first ? 0 : 256); a.head_words = (L.head_end - (first ? 0 : 256)) / 16;
     a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip; a.terms = terms;
-    a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
+    a.C = L.plan.C; a.K = L.plan.K; a.groups = L.plan.groups; a.srows = L.plan.srows; a.tcols = L.plan.tcols;
     a.scale = 1.4426950408889634 / (double)f.eps; a.eps_ln2 = (double)f.eps * 0.6931471805599453;
     a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
     cudaError_t e;
@@ -436,11 +432,11 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
         a.n[side] = n;
     }
     a.x[0] = q; a.x[1] = k; a.z = z; a.beta = beta; a.key_len = key_len;
-    a.xbuf = at<unsigned long long>(ws, L.xbuf); a.ybuf = at<unsigned long long>(ws, L.ybuf);
+    a.xbuf = at<unsigned long long>(ws, L.xbuf);
     a.hist = at<float>(ws, L.hist); a.hist_g = at<double>(ws, L.hist_g); a.wide = at<int>(ws, L.wide); a.status = at<int>(ws, 0);
     a.head = at<uint4>(ws, first ? 0 : 256); a.head_words = (L.head_end - (first ? 0 : 256)) / 16;
     a.B = B; a.H = H; a.d = d; a.r = r;
-    a.C = L.plan.C; a.groups = L.plan.groups; a.srows = L.plan.srows;
+    a.C = L.plan.C; a.K = L.plan.K; a.groups = L.plan.groups; a.srows = L.plan.srows; a.tcols = L.plan.tcols;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
     a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0; a.terms = 3;
     // ---- the forward, keeping the weights of every iteration

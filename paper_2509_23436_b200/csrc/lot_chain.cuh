@@ -51,4 +51,24 @@ inline cudaError_t chain_launch(void (*kern)(P...), dim3 grid, unsigned threads,
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+// A kernel whose blocks wait for one another: all of them run at once, in clusters of K.
+template <typename... P, typename... A>
+inline cudaError_t group_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, int K, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)K;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = K > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 } // namespace lot

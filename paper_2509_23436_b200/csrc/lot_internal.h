@@ -153,8 +153,8 @@ cudaError_t slice_attention(const void *q, const void *k, const void *v, const f
 
 // ---- long sequences on a stored bf16 kernel (lot_stream.cu): bf16 tensors, d = 64, 16 < r <= 64 ----
 struct StreamPlan {
-    int C, groups, srows, npad;
-    size_t xbuf, ybuf, head_end, G, decision, kt, wpart, total;
+    int C, K, groups, srows, npad;
+    size_t xbuf, head_end, G, decision, kt, wpart, total;
 };
 StreamPlan stream_plan(int BH, int n);
 // out must not overlap the other tensors: it holds part of the kernel until it is written

@@ -167,7 +167,7 @@ __device__ __forceinline__ void close_rows(const Shared &S, const Share &R)
 {
     typedef Lay<RP, CPL> Y;
     constexpr int STEP = (kThreads / 32) * Y::RPW;
-    const Lane<RP, CPL> L = make_lane<RP, CPL>(S);
+    const Lane<RP, CPL> L = make_lane<RP, CPL, kThreads>(S, 0);
     u64 w[CPL / 2];
     load_weights<RP, CPL>(L, w);
     for (int st = 0; st < R.steps; ++st) {
@@ -215,16 +215,16 @@ slice_forward_kernel(const __grid_constant__ SliceParams P)
         int it = 0;
         unsigned seq = 0;
         {
-            const Lane<RP, CPL> L = make_lane<RP, CPL>(S);
+            const Lane<RP, CPL> L = make_lane<RP, CPL, kThreads>(S, 0);
             const float tgt = S.tgt[tid < RP ? tid : 0];
             u64 w[CPL / 2];
             load_weights<RP, CPL>(L, w);
             for (; it < a.it1; ++it) {
-                bad = iterate<RP, CPL, kThreads, false>(a, S, R, L, w, tgt, 0, 0, seq, wold, wnew);
+                bad = iterate<RP, CPL, kThreads, false, false>(a, S, R, L, w, tgt, 0, 0, seq, wold, wnew);
                 if (bad) break;
             }
         }
-        if (bad) recover<__nv_bfloat16, RP, CPL, kThreads, false, Mem<RP>::work, Mem<RP>::ref>(&a, p, 0, 0, it, seq, wold, wnew);
+        if (bad) recover<__nv_bfloat16, RP, CPL, kThreads, false, false, Mem<RP>::work, Mem<RP>::ref>(&a, p, 0, 0, it, seq, wold, wnew);
         close_rows<RP, CPL>(S, R);
     } else {
         // no keys: nothing to transport; the output is zero (flagged), the key-side potentials stay at zero

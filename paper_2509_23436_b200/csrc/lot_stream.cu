@@ -27,10 +27,7 @@ constexpr int kRowsStep = 64;              // rows per step of a block: eight a 
 constexpr int kZPitch = 144;               // bytes per staged pivot row (conflict-free ldmatrix)
 constexpr int kStage = 2 * RP * kZPitch;   // staged pivots (hi, lo): in the kernel rows' area while building
 constexpr int kWork = kThreads / 32 * RP * 4;
-constexpr int kPeers = 8;                  // blocks of a cluster (the portable limit)
 constexpr int kFixed = kWork + kThreads * 4 + RP * 20 + 64 + 2 * kPeers * RP * 4;
-
-enum Sharing { kAlone, kGlobal, kCluster };  // a problem's blocks: one; several, exchanging through L2; a cluster
 
 __host__ __device__ constexpr int area_bytes(int srows) { return srows * 128 > kStage ? srows * 128 : kStage; }
 
@@ -43,16 +40,16 @@ struct StreamArgs {
     float *G;                  // [2][BH][64] log2 of the final weights (relative to the kernel as stored)
     int *decision;             // [2][BH], set to 1
     float *g_out[2];
-    u64 *xbuf, *ybuf;
+    u64 *xbuf;
     int *status;
-    int B, H, n, npad, r, T, C, groups, srows;
+    int B, H, n, npad, r, T, C, K, groups, srows;
+    unsigned seq0;             // 0
     double scale, eps_ln2;
 };
 
 struct Mem {
     uint8_t *K, *z;            // [srows][128 bytes]; its last bytes hold the pivots while building
     float *before;             // the weights before the last update
-    float *peers;              // column sums from the blocks of the cluster, two sets
     Shared s;
 };
 
@@ -68,8 +65,9 @@ __device__ __forceinline__ Mem carve16(uint8_t *p, int srows)
     m.s.w = reinterpret_cast<float *>(p); p += RP * 4;
     m.s.tgt = reinterpret_cast<float *>(p); p += RP * 4;
     m.before = reinterpret_cast<float *>(p); p += RP * 4;
-    m.peers = reinterpret_cast<float *>(p); p += 2 * kPeers * RP * 4;
     m.s.flag = reinterpret_cast<volatile int *>(p);    // [0], [1] as in the sweep kernels; [2], [3]: see solve16
+    m.s.bars = smem_addr(p) + 16;
+    m.s.peers = smem_addr(p) + 64;
     return m;
 }
 
@@ -354,43 +352,8 @@ __device__ __forceinline__ void pass16(const LaneMap &L, const Part &P, const u6
     if (k < end) row16(lds4(k), lds4(k ^ 64), w, acc);
 }
 
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Column sums (maxima) of the problem from those of its blocks, the same bits in every block.  In a cluster every block writes
-// its own into all others' shared memory, and one cluster barrier makes them visible; the set written next is the other one, and
-// its last readers have passed that barrier.  Nothing is polled, and the
-// iteration loop has the registers it needs (108 bytes of spills with the polling loop in it).
-template <Sharing SHARE, bool MAX>
-__device__ __forceinline__ float columns16(const StreamArgs &a, const Mem &m, float part, int group, int c, unsigned &seq)
-{
-    if (SHARE == kAlone) return part;
-    if (SHARE == kGlobal) return group_columns<RP, kThreads, MAX>(a, m.s, part, group, c, seq);
-    ++seq;
-    const int t = threadIdx.x;
-    const uint32_t set = smem_addr(m.peers) + (seq & 1) * (kPeers * RP * 4);
-    if (t < RP)
-        for (int o = 0; o < a.C; ++o) {
-            uint32_t there;
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(set + (c * RP + t) * 4), "r"(o));
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(there), "f"(part) : "memory");
-        }
-    cluster_sync();
-    if (t >= RP) return 0.f;
-    float v[kPeers];
-#pragma unroll
-    for (int o = 0; o < kPeers; ++o) v[o] = o < a.C ? lds(set + (o * RP + t) * 4) : MAX ? neg_inf() : 0.f;
-#pragma unroll
-    for (int h = kPeers / 2; h > 0; h >>= 1)
-#pragma unroll
-        for (int o = 0; o < h; ++o) v[o] = MAX ? fmaxf(v[o], v[o + h]) : v[o] + v[o + h];
-    return v[0];
-}
-
 // One iteration, as in lot_sweep_core.cuh: the weights in shared memory and those before them.
-template <Sharing SHARE>
+template <bool GROUP>
 __device__ __forceinline__ bool iterate16(const StreamArgs &a, const Mem &m, const Part &P, const LaneMap &L, u64 (&w)[8], int group, int c,
                                           unsigned &seq)
 {
@@ -424,7 +387,7 @@ __device__ __forceinline__ bool iterate16(const StreamArgs &a, const Mem &m, con
             for (int i = 0; i < h; ++i) o[i] += o[i + h];
         tot = o[0];
     }
-    tot = columns16<SHARE, false>(a, m, tot, group, c, seq);
+    if (GROUP) tot = group_columns<RP, kThreads, false>(a, m.s, tot, group, c, seq);
     if ((int)threadIdx.x < a.r) {
         const float wnew = m.s.tgt[threadIdx.x] * rcp(tot);
         if (out_of_range(wnew)) m.s.flag[1] = 1;
@@ -455,7 +418,7 @@ __device__ __forceinline__ bool too_wide(const Mem &m, int r)
 
 // log2 of the column sums of the row-stochastic plan for the potentials in gref, in the log domain: logits once for the
 // column maxima and once more for the sums relative to them; nothing is stored.
-template <Sharing SHARE>
+template <bool GROUP>
 __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m, const Part &P, int group, int c, unsigned &seq)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
@@ -519,7 +482,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
         float tot = round == 0 ? neg_inf() : 0.f;
         if (threadIdx.x < RP)
             for (int w = 0; w < kThreads / 32; ++w) tot = round == 0 ? fmaxf(tot, red[w * RP + threadIdx.x]) : tot + red[w * RP + threadIdx.x];
-        tot = round == 0 ? columns16<SHARE, true>(a, m, tot, group, c, seq) : columns16<SHARE, false>(a, m, tot, group, c, seq);
+        if (GROUP) tot = round == 0 ? group_columns<RP, kThreads, true>(a, m.s, tot, group, c, seq) : group_columns<RP, kThreads, false>(a, m.s, tot, group, c, seq);
         __syncthreads();
         if (round == 0) {
             kap = tot;
@@ -534,7 +497,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
 
 // The iterations of a problem on the kernel as built.  flag[2] = 1 where recover16 has to go on from iteration flag[3].
 // Returns the sequence number.
-template <Sharing SHARE>
+template <bool GROUP>
 __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
 {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -547,7 +510,7 @@ __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group,
     u64 w[8];
     load_weights16(L, w);
     for (; it < a.T; ++it) {
-        bad = iterate16<SHARE>(a, m, P, L, w, group, c, seq);
+        bad = iterate16<GROUP>(a, m, P, L, w, group, c, seq);
         if (bad) break;
     }
     bad = bad || too_wide(m, a.r);
@@ -558,7 +521,7 @@ __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group,
 
 // The rest of a problem's iterations behind an update that left the kernel's range, as recover() of the sweep kernels; and the
 // rebuilding around final potentials that spread too far for the apply kernels.
-template <Sharing SHARE>
+template <bool GROUP>
 __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
 {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -577,7 +540,7 @@ __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int grou
                 m.s.gref[tid] = gn;
             }
             __syncthreads();
-            const float lam = log_columns16<SHARE>(a, m, P, group, c, seq);
+            const float lam = log_columns16<GROUP>(a, m, P, group, c, seq);
             if (tid < r) gn += log2((double)tgt) - (double)lam;
         } else if (tid < r) {
             gn = m.s.gref[tid] + log2((double)wnew);
@@ -596,7 +559,7 @@ __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int grou
         u64 w[8];
         load_weights16(L, w);
         if (it >= a.T) break;                                // rebuilt around the final potentials: equal weights
-        for (++it; it < a.T && !bad; ++it) bad = iterate16<SHARE>(a, m, P, L, w, group, c, seq);
+        for (++it; it < a.T && !bad; ++it) bad = iterate16<GROUP>(a, m, P, L, w, group, c, seq);
         if (bad) --it;                                       // the iteration whose update has to be redone
         else if (!too_wide(m, r)) break;
         __syncthreads();
@@ -604,16 +567,16 @@ __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int grou
     return seq;
 }
 
-template <Sharing SHARE>
+template <bool GROUP>
 __global__ void __launch_bounds__(kThreads, 2)
 stream_kernel(const __grid_constant__ StreamArgs a)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    const int tid = threadIdx.x, group = SHARE == kAlone ? blockIdx.x : blockIdx.x / a.C, c = SHARE == kAlone ? 0 : blockIdx.x % a.C;
+    const int tid = threadIdx.x, group = GROUP ? blockIdx.x / a.C : blockIdx.x, c = GROUP ? blockIdx.x % a.C : 0;
     unsigned seq = 0;
     const Mem m = carve16(smem, a.srows);
     if (tid < 4) m.s.flag[tid] = 0;
-    if (SHARE == kCluster) cluster_sync();                          // every block of the cluster has begun
+    if (GROUP) open_exchange<RP>(a, m.s);
 
     for (int p = group; p < 2 * a.B * a.H; p += a.groups) {
         __syncthreads();                                            // the previous problem is done with shared memory
@@ -627,8 +590,8 @@ stream_kernel(const __grid_constant__ StreamArgs a)
         if (tid == 0) m.s.flag[2] = 0;
         if (locate16(a, p, c).nv > 0) {
             build16<false>(&a, p, c);
-            seq = solve16<SHARE>(&a, p, group, c, seq);
-            if (m.s.flag[2]) seq = recover16<SHARE>(&a, p, group, c, seq);
+            seq = solve16<GROUP>(&a, p, group, c, seq);
+            if (m.s.flag[2]) seq = recover16<GROUP>(&a, p, group, c, seq);
         } else {
             if (tid == 0 && c == 0) atomicOr(a.status, 2 /* LOT_DEV_EMPTY */);
             __syncthreads();
@@ -643,7 +606,7 @@ stream_kernel(const __grid_constant__ StreamArgs a)
                 a.g_out[F.side][(size_t)F.slice * a.r + tid] = (float)((m.s.gref[tid] + log2((double)m.s.w[tid])) * a.eps_ln2);
         }
     }
-    if (SHARE == kCluster) cluster_sync();                          // nobody's shared memory is written any more
+    if (GROUP) close_exchange(a);
 }
 
 } // namespace stream
@@ -658,25 +621,35 @@ StreamPlan stream_plan(int BH, int n)
     long long fly = 80000000ll / (npad * 128);
     if (fly < 2) fly = 2;
     if (fly > NP) fly = NP;
-    const int rounds = (int)((NP + fly - 1) / fly);
+    const int rounds = (int)((NP + fly - 1) / fly), most = (n + 2 * kRowsStep - 1) / (2 * kRowsStep);
     fly = (NP + rounds - 1) / rounds;
-    L.C = (int)(slots / fly) < 1 ? 1 : (int)(slots / fly);
-    // eight blocks as a cluster exchange faster, if the rows are no more steps (n = 4096, H = 16: 45.7 us against 47.0; more
-    // steps cost more than that, n = 16384: 132 against 128)
-    auto steps = [&](int C) { return ((n + C - 1) / C + kRowsStep - 1) / kRowsStep; };
-    if (L.C > kPeers && steps(kPeers) == steps(L.C)) L.C = kPeers;
-    const int most = (n + 2 * kRowsStep - 1) / (2 * kRowsStep);     // two steps a block at least
-    if (L.C > most) L.C = most;
-    if (L.C > 64) L.C = 64;
-    L.groups = L.C == 1 ? NP : (slots / L.C < NP ? slots / L.C : NP);
+    // Blocks a problem and blocks a cluster: the least time of a pass, us: steps of 64 rows (two blocks share an SM) and the exchange
+    // (group_columns), at least two steps a block.
+    L.C = 1; L.K = 1;
+    double best = 1e30;
+    auto consider = [&](int C, int K, int blocks) {
+        if (C > 1 && (C > most || blocks / C < 1)) return;
+        const int groups = C == 1 ? (NP < blocks ? NP : blocks) : (blocks / C < NP ? blocks / C : NP), words = C / K;
+        const int steps = ((n + C - 1) / C + kRowsStep - 1) / kRowsStep, turns = (NP + groups - 1) / groups;
+        const double lat = C == 1 ? 0.45 : C == K ? 1.0 : 1.4 + 0.45 * ((words - 1) / (kWords * (words > kWords ? kThreads / RP : 1)));
+        const double t = turns * (steps * 0.25 + lat);
+        if (groups <= fly && t < best) { best = t; L.C = C; L.K = K; }
+    };
+    consider(1, 1, slots);
+    for (int K = 2; K <= kPeers; ++K) {
+        const int blocks = cluster_blocks(K, 2);
+        consider(K, K, blocks);
+        if ((K & (K - 1)) == 0)
+            for (int M = 2; M * K <= blocks; ++M) consider(M * K, K, blocks);
+    }
+    L.groups = L.C == 1 ? NP : cluster_blocks(L.K, 2) / L.C < NP ? cluster_blocks(L.K, 2) / L.C : NP;
     const int rows = (n + L.C - 1) / L.C, up = (rows + kRowsStep - 1) / kRowsStep * kRowsStep;
     const int cap = (228 * 1024 / 2 - 1024 - kFixed) / 128 / kRowsStep * kRowsStep;
     L.srows = up < cap ? up : cap;
     L.npad = (int)npad;
     size_t o = 256;
     auto take = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~(size_t)255; return at; };
-    L.xbuf = take(L.C > 1 ? (size_t)L.groups * 2 * L.C * RP * 8 : 0);
-    L.ybuf = take(L.C > 1 ? (size_t)L.groups * 2 * kSweepCopies * RP * 8 : 0);
+    L.xbuf = take(exchange_bytes(RP, L.C, L.K, L.groups));
     L.head_end = o;
     L.G = take((size_t)NP * RP * 4);
     L.decision = take((size_t)NP * 4);
@@ -685,51 +658,6 @@ StreamPlan stream_plan(int BH, int n)
     L.total = o;
     return L;
 }
-
-namespace stream {
-
-static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute *at, int C, dim3 grid, size_t smem, cudaStream_t st)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    at->id = cudaLaunchAttributeClusterDimension;
-    at->val.clusterDim.x = C;
-    at->val.clusterDim.y = at->val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cfg;
-}
-
-// Whether all groups run at once as clusters (a cluster's blocks share a GPC, so some slots stay empty).  The last answer is
-// kept: it does not change for a device.
-static bool clusters_fit(int C, size_t smem, int groups)
-{
-    struct Memo { int dev, C, fit; size_t smem; };
-    static thread_local Memo memo = {-1, 0, 0, 0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (memo.dev != dev || memo.C != C || memo.smem != smem) {
-        cudaLaunchAttribute at;
-        const cudaLaunchConfig_t cfg = cluster_config(&at, C, dim3((unsigned)C), smem, nullptr);
-        int fit = 0;
-        if (cudaFuncSetAttribute(stream_kernel<kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024) != cudaSuccess) return false;
-        if (cudaOccupancyMaxActiveClusters(&fit, stream_kernel<kCluster>, &cfg) != cudaSuccess) { cudaGetLastError(); fit = 0; }
-        memo = {dev, C, fit, smem};
-    }
-    return memo.fit >= groups;
-}
-
-static cudaError_t launch_clusters(const StreamArgs &a, dim3 grid, size_t smem, cudaStream_t st)
-{
-    cudaLaunchAttribute at;
-    const cudaLaunchConfig_t cfg = cluster_config(&at, a.C, grid, smem, st);
-    return cudaLaunchKernelEx(&cfg, stream_kernel<kCluster>, a);
-}
-
-} // namespace stream
 
 cudaError_t stream_attention(const void *q, const void *k, const void *v, const float *z, const float *beta, const int32_t *key_len, int B,
                              int H, int n, int r, float eps, int iters, void *out, float *g1_out, float *g2_out, void *ws, cudaStream_t st)
@@ -749,27 +677,21 @@ cudaError_t stream_attention(const void *q, const void *k, const void *v, const 
     a.low = low_half ? static_cast<uint8_t *>(out) : nullptr;
     a.G = reinterpret_cast<float *>(w + L.G); a.decision = reinterpret_cast<int *>(w + L.decision);
     a.g_out[0] = g1_out; a.g_out[1] = g2_out;
-    a.xbuf = reinterpret_cast<u64 *>(w + L.xbuf); a.ybuf = reinterpret_cast<u64 *>(w + L.ybuf);
+    a.xbuf = reinterpret_cast<u64 *>(w + L.xbuf);
     a.status = reinterpret_cast<int *>(ws);
-    a.B = B; a.H = H; a.n = n; a.npad = L.npad; a.r = r; a.T = iters; a.C = L.C; a.groups = L.groups; a.srows = L.srows;
+    a.B = B; a.H = H; a.n = n; a.npad = L.npad; a.r = r; a.T = iters; a.C = L.C; a.K = L.K; a.groups = L.groups; a.srows = L.srows;
     a.scale = 1.4426950408889634 / (double)eps;
     a.eps_ln2 = (double)eps * 0.6931471805599453;
     const size_t smem = (size_t)area_bytes(L.srows) + kFixed;
     const dim3 grid((unsigned)(L.C * L.groups));
-    if (L.C > 1 && L.C <= kPeers && clusters_fit(L.C, smem, L.groups)) {
-        e = launch_clusters(a, grid, smem, st);
+    auto kern = L.C > 1 ? stream_kernel<true> : stream_kernel<false>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
+    if (e != cudaSuccess) return e;
+    if (L.C > 1) {
+        e = group_launch(kern, grid, kThreads, smem, L.K, st, a);
     } else {
-        auto kern = L.C > 1 ? stream_kernel<kGlobal> : stream_kernel<kAlone>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
-        if (e != cudaSuccess) return e;
-        if (L.C > 1) {
-            // the blocks of a group wait for one another: all must be resident
-            void *args[] = {&a};
-            e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), grid, dim3(kThreads), args, smem, st);
-        } else {
-            kern<<<grid, kThreads, smem, st>>>(a);
-            e = cudaGetLastError();
-        }
+        kern<<<grid, kThreads, smem, st>>>(a);
+        e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
     return stored_apply(a.kt, L.npad, a.G, beta, key_len, a.decision, v, out, low_half, reinterpret_cast<float *>(w + L.wpart), a.status, B, H, n, r, st);

@@ -13,9 +13,9 @@ namespace lot {
 // That is a window of 160 binades for the potentials before the kernel has to be rebuilt around them; the weights
 // start in the middle of it.
 constexpr float kKernelTop = 67.f, kStartLog2 = -50.f;
-constexpr int kSweepCopies = 8;     // places the totals of an exchange are left in
 
-// Problem p of a sweep is side (p odd ? queries : keys) of slice p / 2; side 0 = queries, side 1 = keys.
+// Problem p of a sweep is side (p odd ? queries : keys) of slice p / 2, or with sides of different lengths, all of the longer one first;
+// side 0 = queries, side 1 = keys.
 struct SweepArgs {
     const void *x[2];        // [BH][n_side][d] tokens
     const float *z, *beta;   // [H][r][d], [H][r]
@@ -27,8 +27,7 @@ struct SweepArgs {
     float *w[2];             // [BH][RP] weights of the closing update: plan row i = kt[i][t] w[t] inv[i]
     double *gref[2];         // [BH][RP] reference potentials of kt, base-2 units
     float *g_out[2];         // [BH][r] potentials in natural units or nullptr
-    unsigned long long *xbuf;   // exchange words of the groups (zero at the start of the first launch of a call)
-    unsigned long long *ybuf;
+    unsigned long long *xbuf;   // exchange words of the groups (exchange_bytes; zero at the start of the first launch of a call)
     float *hist;             // backward: [it1 + 1][problems][RP] weights before every iteration and after the last, relative to
                              // the kernel as it is left, or nullptr
     double *hist_g;          // ... and the potentials themselves, of the problems whose kernel was rebuilt
@@ -39,8 +38,9 @@ struct SweepArgs {
     int B, H, d, r;
     int n[2];                // tokens per slice
     int skip;                // leading tokens of both sides that take no part (the class token)
-    int C, groups;           // thread blocks per problem, problems in flight
+    int C, K, groups;        // thread blocks per problem, per cluster (1: no clusters), problems in flight
     int srows;               // rows of a block's share that stay in shared memory
+    int tcols;               // columns of tensor memory that take the next ones (0: none)
     int it0, it1;            // iterations this launch runs
     int terms;               // bf16 tokens: terms a pivot is taken as in the first build (3: exact, 2)
     int first, close;        // start from the given potentials (else from the state in w, gref) / closing update last
@@ -50,11 +50,20 @@ struct SweepArgs {
 };
 
 struct SweepPlan {
-    int RP, C, groups, srows;
+    int RP, C, K, groups, srows, tcols;
     int steps;               // 1: one launch per iteration (the kernel streams from global memory anyway)
     size_t smem;
 };
 
+namespace sweep {
+// the kernels of one type and use; a file each, compiled side by side
+cudaError_t launch_f32(const SweepPlan &P, const SweepArgs &a, cudaStream_t st);
+cudaError_t launch_bf16(const SweepPlan &P, const SweepArgs &a, cudaStream_t st);
+cudaError_t launch_keep(const SweepPlan &P, const SweepArgs &a, cudaStream_t st);        // bf16, with the weights of every iteration
+int cluster_count(int K, size_t smem);                                                   // clusters of K such blocks that run at once, 0: not known
+}
+int cluster_blocks(int K, int occ);      // blocks that run at once as clusters of K, `occ` to an SM
+inline size_t exchange_bytes(int RP, int C, int K, int groups) { return C > K ? (size_t)groups * 2 * (C / K) * RP * 8 : 0; }
 SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r);
 cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st);
 cudaError_t launch_sweep(const SweepPlan &P, const SweepArgs &a, int dtype, cudaStream_t st);

@@ -98,7 +98,7 @@ close_kernel(const __grid_constant__ SweepBwdArgs a)
 // Reverse iterations
 // ---------------------------------------------------------------------------------------------------------------
 // One reverse pass over the block's rows: column sums of K u / s^2, row coefficients to coef.
-template <int RP, int CPL, int THREADS>
+template <int RP, int CPL, int THREADS, bool TENSOR>
 __device__ __forceinline__ void reverse_pass(const Lane<RP, CPL> &L, const Share &R, const u64 (&w)[CPL / 2], const u64 (&f)[CPL / 2],
                                              u64 (&acc)[CPL / 2], float mass, float2 *coef)
 {
@@ -132,8 +132,19 @@ __device__ __forceinline__ void reverse_pass(const Lane<RP, CPL> &L, const Share
         for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.k[v] + st * (STEP * RP * 4));
         one(k, L.i0 + st * STEP, R.ns);
     }
-    if (R.ns < R.nrows)
-        for (int i = R.ns + L.i0; i - L.i0 < R.nrows; i += STEP) {
+    const int on_chip = TENSOR ? R.ns + R.nt : R.ns;
+#pragma unroll 1
+    for (int ts = 0; TENSOR && ts < R.tsteps; ++ts) {
+        u64 k2[8];
+        tensor_load<16>(k2, L.t + ts * CPL);
+        tensor_settle<16>(k2);
+        Row<CPL> k;
+#pragma unroll
+        for (int j = 0; j < CPL / 2; ++j) k.k[j] = k2[j];
+        one(k, R.ns + L.i0 + ts * STEP, on_chip);
+    }
+    if (on_chip < R.nrows)
+        for (int i = on_chip + L.i0; i - L.i0 < R.nrows; i += STEP) {
             Row<CPL> k;
 #pragma unroll
             for (int v = 0; v < Y::NV; ++v) {
@@ -225,7 +236,7 @@ __device__ __noinline__ unsigned reverse_wide(const SweepBwdArgs *ap, int p, int
     return seq;
 }
 
-template <int RP, int CPL, int THREADS, bool GROUP>
+template <int RP, int CPL, int THREADS, bool GROUP, bool TENSOR>
 __global__ void __launch_bounds__(THREADS, max_blocks(CPL, THREADS))
 reverse_kernel(const __grid_constant__ SweepBwdArgs a)
 {
@@ -237,6 +248,8 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
     unsigned seq = s.seq0;
     const Shared S = carve<__nv_bfloat16, RP, THREADS>(smem, s.srows);
     if (tid == 0) S.flag[0] = 0;
+    if (GROUP) open_exchange<RP>(s, S);
+    if (TENSOR) open_tensor(S, s.tcols);
     chain_wait();
 
     for (int p = group; p < NP; p += s.groups) {
@@ -256,11 +269,12 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
             continue;
         }
         load_rows<RP, CPL, THREADS>(S, R);
+        if constexpr (TENSOR) load_tensor_rows<RP, CPL, THREADS>(S, R, s.tcols);
         const float *hw = s.hist + (size_t)p * RP + (tid < RP ? tid : 0);
         const size_t hstep = (size_t)NP * RP;
         const float beta = tid < r ? __ldg(s.beta + P.h * r + tid) : 1.f, mass = 1.f / (float)P.nv;
         float wb = hw[(size_t)a.T * hstep], wa = a.T > 0 ? hw[(size_t)(a.T - 1) * hstep] : 0.f, db = 0.f;
-        const Lane<RP, CPL> L = make_lane<RP, CPL>(S);
+        const Lane<RP, CPL> L = make_lane<RP, CPL, THREADS>(S, s.tcols);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         const uint32_t f_addr = smem_addr(S.tgt) + L.cl * 16;
         float2 *coef = a.coef + (size_t)p * a.T * P.n + P.row0;
@@ -278,7 +292,7 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
 #pragma unroll
             for (int v = 0; v < CPL / 4; ++v) lds2(f[2 * v], f[2 * v + 1], f_addr + v * (Y::LPR * 16));
             const float wnext = it >= 2 ? hw[(size_t)(it - 2) * hstep] : 0.f;
-            reverse_pass<RP, CPL, THREADS>(L, R, w, f, acc, mass, coef + (size_t)(it - 1) * P.n);
+            reverse_pass<RP, CPL, THREADS, TENSOR>(L, R, w, f, acc, mass, coef + (size_t)(it - 1) * P.n);
             float v[CPL];
 #pragma unroll
             for (int j = 0; j < CPL / 2; ++j) unpack_f2(acc[j], v[2 * j], v[2 * j + 1]);
@@ -292,6 +306,8 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
         if (c == 0 && tid < r) a.dbeta_acc[(size_t)p * RP + tid] = db;
         __syncthreads();
     }
+    if (TENSOR) close_tensor(S, s.tcols);
+    if (GROUP) close_exchange(s);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -408,22 +424,22 @@ template <int RP> static cudaError_t assemble_t(const SweepBwdArgs &a, cudaStrea
     constexpr int CT = RP < 64 ? RP : 64, ROWS = 256 / (CT / 4) * 4;
     return chain_launch(assemble_kernel<RP>, dim3((a.s.n[0] + ROWS - 1) / ROWS, RP / CT, 2 * a.s.B * a.s.H), 256, 0, st, a);
 }
-template <int RP, bool GROUP> static cudaError_t reverse_g(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st)
+template <int RP, bool GROUP, bool TENSOR> static cudaError_t reverse_g(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st)
 {
-    auto kern = reverse_kernel<RP, wide_cols(RP), 256, GROUP>;
+    constexpr int THREADS = TENSOR ? kTensorThreads : 256;
+    auto kern = reverse_kernel<RP, TENSOR ? kTensorLane : wide_cols(RP), THREADS, GROUP, TENSOR>;
     cudaError_t e = allow_smem(kern, P.smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(P.groups * P.C));
     if (!GROUP) {
-        return chain_launch(kern, grid, 256, P.smem, st, a);
+        return chain_launch(kern, grid, THREADS, P.smem, st, a);
     }
-    SweepBwdArgs copy = a;
-    void *args[] = {&copy};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), grid, dim3(256), args, P.smem, st);
+    return group_launch(kern, grid, THREADS, P.smem, P.K, st, a);
 }
 template <int RP> static cudaError_t reverse_t(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st)
 {
-    return P.C > 1 ? reverse_g<RP, true>(P, a, st) : reverse_g<RP, false>(P, a, st);
+    if (P.C > 1) return P.tcols ? reverse_g<RP, true, true>(P, a, st) : reverse_g<RP, true, false>(P, a, st);
+    return P.tcols ? reverse_g<RP, false, true>(P, a, st) : reverse_g<RP, false, false>(P, a, st);
 }
 
 } // namespace sweep

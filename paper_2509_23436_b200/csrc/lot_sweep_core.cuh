@@ -23,7 +23,8 @@ constexpr float kLostLo = 1e-30f, kLostHi = 1e38f;
 constexpr float kFarLo = 7.7037198e-34f, kFarHi = 1.1258999e15f;   // 2^-110, 2^50
 constexpr float kStart = 8.8817842e-16f;                            // 2^kStartLog2
 constexpr float kHistLo = 2.4074124e-35f, kHistHi = 4.1538374e34f;   // 2^-115, 2^115: kept weights a reverse pass can use
-constexpr int kDirectWords = 4096, kCopies = kSweepCopies;
+constexpr int kPeers = 8, kWords = 16;                               // blocks of a cluster (the portable limit); words a thread waits for at once
+constexpr int kSmPerBlockReserve = 1024, kSmemPerSM = 228 * 1024, kSmemPerBlock = 227 * 1024;
 constexpr unsigned long long kWaitNs = 1000000000ull;
 
 // floats <-> packed pairs for fma.rn.f32x2
@@ -69,11 +70,16 @@ __host__ __device__ constexpr int wide_cols(int RP) { return RP <= 32 ? 8 : 16; 
 // blocks per SM that the registers allow (80 a thread, 128 with sixteen columns per lane)
 __host__ __device__ constexpr int max_blocks(int cpl, int threads) { return (cpl == 16 ? 512 : 768) / threads; }
 
-// shared memory: [kernel rows | gref | work area (staged pivots, or the column reduction) | refs | weights, targets | flags]
+// Blocks that keep rows in tensor memory too are alone on their SM (the runtime places no two blocks of such a kernel, launched
+// together, on one): twice the threads, sixteen columns a lane whatever RP is, all of the SM's columns.
+constexpr int kTensorThreads = 512, kTensorCols = 512, kTensorLane = 16;
+
+// shared memory: [kernel rows | gref | work area (staged pivots, or the column reduction) | refs | weights, targets | flags,
+// barriers | columns from the blocks of the cluster]
 __host__ __device__ constexpr int rebuild_cols(int RP) { return RP < 32 ? RP : 32; }      // columns per step of a rebuild
 template <typename T> __host__ __device__ constexpr size_t work_bytes(int RP, int threads)
 {
-    const size_t red = (size_t)2 * (threads / 32) * RP * 4, st = logits::stage_bytes<T>(rebuild_cols(RP));
+    const size_t red = (size_t)(threads / 32) * RP * 4, st = logits::stage_bytes<T>(rebuild_cols(RP));
     return red > st ? red : st;
 }
 __host__ __device__ constexpr size_t ref_bytes(int RP, int threads)
@@ -92,6 +98,8 @@ struct Shared {
     float *ref, *w, *tgt;
     double *gref;
     volatile int *flag;      // [0] a wait gave up, [1] a weight left its range
+    uint32_t bars, peers;    // addresses of two barriers, and of what they count (group_columns)
+    uint32_t tmem;           // address of the word that holds the tensor memory's address
 };
 
 // A block's share of one problem.
@@ -99,6 +107,7 @@ struct Share {
     float *g;                // its rows in global memory, [nrows][RP], or nullptr (all of them are in shared memory)
     const float *mass;       // its tokens' weights or nullptr
     int nrows, ns, steps;    // rows, of which the first ns are in shared memory too, in `steps` steps of the block
+    int nt, tsteps;          // ... the next nt in tensor memory, in `tsteps` steps (an even number)
 };
 
 template <int RP, int CPL> __device__ __forceinline__ float4 *chunk_ptr(const Shared &S, const Share &R, int i, int chunk)
@@ -219,16 +228,68 @@ __device__ __forceinline__ float row_step(const Row<CPL> &k, const u64 (&w)[CPL 
 // What a thread needs in every iteration, worked out once per problem: shared-memory addresses of its columns of its
 // first row, of its weights and of the column it owns.
 template <int RP, int CPL> struct Lane {
-    uint32_t k[CPL / 4], w, red, own;
+    uint32_t k[CPL / 4], w, red, own, t;
     int i0, cl;
 };
 
-template <int RP, int CPL>
-__device__ __forceinline__ Lane<RP, CPL> make_lane(const Shared &S)
+// The tensor memory as a second store of kernel rows: a lane's columns of a row are CPL neighbouring columns of its lane there, as
+// it holds them in registers, so a warp only ever reads back what it has written itself (no operand layout, no bank
+// conflicts).  The two warps that share a quarter of the lanes take half of the block's columns each.
+template <int THREADS> __device__ __forceinline__ uint32_t tensor_rows(const Shared &S, int tcols)
+{
+    uint32_t base;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(base) : "r"(S.tmem) : "memory");
+    const uint32_t warp = threadIdx.x >> 5;
+    return base + ((warp & 3) << 21) + (warp >> 2) * (tcols / (THREADS / 128));
+}
+// N = 16 or 32 columns of the lane as packed pairs; to be used behind settle().
+template <int N> __device__ __forceinline__ void tensor_load(u64 (&v)[N / 2], uint32_t t)
+{
+    float f[N];
+    sm100::tmem_ld<N>(t, f);
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) v[i] = pack_f2(f[2 * i], f[2 * i + 1]);
+}
+template <int N> __device__ __forceinline__ void tensor_settle(u64 (&v)[N / 2])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+l"(v[0]), "+l"(v[1]), "+l"(v[2]), "+l"(v[3]), "+l"(v[4]), "+l"(v[5]), "+l"(v[6]), "+l"(v[7]) :: "memory");
+    if constexpr (N == 32)                                   // the same wait stands for the other half
+        asm volatile("" : "+l"(v[8]), "+l"(v[9]), "+l"(v[10]), "+l"(v[11]), "+l"(v[12]), "+l"(v[13]), "+l"(v[14]), "+l"(v[15]) :: "memory");
+}
+__device__ __forceinline__ void tensor_store16(uint32_t t, const float4 (&v)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(t), "f"(v[0].x), "f"(v[0].y), "f"(v[0].z), "f"(v[0].w), "f"(v[1].x), "f"(v[1].y), "f"(v[1].z), "f"(v[1].w), "f"(v[2].x),
+                   "f"(v[2].y), "f"(v[2].z), "f"(v[2].w), "f"(v[3].x), "f"(v[3].y), "f"(v[3].z), "f"(v[3].w) : "memory");
+}
+// Rows ns .. ns + nt - 1 of the share from global into tensor memory, zeros up to the last step.
+template <int RP, int CPL, int THREADS> __device__ __forceinline__ void load_tensor_rows(const Shared &S, const Share &R, int tcols)
+{
+    typedef Lay<RP, CPL> Y;
+    static_assert(CPL == 16, "a row's part is sixteen columns");
+    constexpr int STEP = (THREADS / 32) * Y::RPW;
+    if (R.tsteps == 0) return;
+    const int lane = threadIdx.x & 31, cl = lane % Y::LPR, i0 = (threadIdx.x >> 5) * Y::RPW + lane / Y::LPR;
+    const uint32_t t = tensor_rows<THREADS>(S, tcols);
+#pragma unroll 2
+    for (int st = 0; st < R.tsteps; ++st) {
+        const int i = i0 + st * STEP;
+        float4 v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            v[c] = i < R.nt ? __ldcg(reinterpret_cast<const float4 *>(R.g + (size_t)(R.ns + i) * RP) + c * Y::LPR + cl) : make_float4(0.f, 0.f, 0.f, 0.f);
+        tensor_store16(t + st * CPL, v);
+    }
+    sm100::tmem_wait_st();
+}
+
+template <int RP, int CPL, int THREADS>
+__device__ __forceinline__ Lane<RP, CPL> make_lane(const Shared &S, int tcols)
 {
     typedef Lay<RP, CPL> Y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     Lane<RP, CPL> L;
+    L.t = tcols ? tensor_rows<THREADS>(S, tcols) : 0;
     L.cl = lane % Y::LPR;
     L.i0 = warp * Y::RPW + lane / Y::LPR;
 #pragma unroll
@@ -245,7 +306,7 @@ __device__ __forceinline__ Lane<RP, CPL> make_lane(const Shared &S)
 
 // One pass over the block's rows: the lane's column sums.  CLOSE: the reciprocal row sums go to inv_out instead (0 for a
 // token without weight).  WEIGHTED: the tokens bring weights of their own.
-template <int RP, int CPL, int THREADS, bool CLOSE, bool WEIGHTED>
+template <int RP, int CPL, int THREADS, bool TENSOR, bool CLOSE, bool WEIGHTED>
 __device__ __forceinline__ void pass_t(const Lane<RP, CPL> &L, const Share &R, const u64 (&w)[CPL / 2], u64 (&acc)[CPL / 2], float *inv_out)
 {
     typedef Lay<RP, CPL> Y;
@@ -266,42 +327,87 @@ __device__ __forceinline__ void pass_t(const Lane<RP, CPL> &L, const Share &R, c
 #pragma unroll
         for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.k[v] + st * (STEP * RP * 4));
     };
-    if (R.steps & 1) {
-        Row<CPL> k;
-        load(k, 0);
-        one(k, L.i0, R.ns);
-    }
-    for (int st = R.steps & 1; st < R.steps; st += 2) {
-        Row<CPL> k[2];
-        load(k[0], st);
-        load(k[1], st + 1);
-        one(k[0], L.i0 + st * STEP, R.ns);
-        one(k[1], L.i0 + (st + 1) * STEP, R.ns);
-    }
-    // rows that do not fit: streamed from L2
-    if (R.ns < R.nrows)
-        for (int i = R.ns + L.i0; i - L.i0 < R.nrows; i += 2 * STEP) {
-            Row<CPL> k[2];
+    auto fetch = [&](Row<CPL> (&k)[2], int i) {              // two steps' rows from L2
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < 2; ++u)
 #pragma unroll
-                for (int v = 0; v < Y::NV; ++v) {
-                    const ulonglong2 t = i + u * STEP < R.nrows
-                                             ? __ldcg(reinterpret_cast<const ulonglong2 *>(R.g + (size_t)(i + u * STEP) * RP) + v * Y::LPR + L.cl)
-                                             : make_ulonglong2(0, 0);
-                    k[u].k[2 * v] = t.x;
-                    k[u].k[2 * v + 1] = t.y;
-                }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) one(k[u], i + u * STEP, R.nrows);
+            for (int v = 0; v < Y::NV; ++v) {
+                const ulonglong2 t = i + u * STEP < R.nrows
+                                         ? __ldcg(reinterpret_cast<const ulonglong2 *>(R.g + (size_t)(i + u * STEP) * RP) + v * Y::LPR + L.cl)
+                                         : make_ulonglong2(0, 0);
+                k[u].k[2 * v] = t.x;
+                k[u].k[2 * v + 1] = t.y;
+            }
+    };
+    if constexpr (!TENSOR) {
+        if (R.steps & 1) {
+            Row<CPL> k;
+            load(k, 0);
+            one(k, L.i0, R.ns);
         }
+        for (int st = R.steps & 1; st < R.steps; st += 2) {
+            Row<CPL> k[2];
+            load(k[0], st);
+            load(k[1], st + 1);
+            one(k[0], L.i0 + st * STEP, R.ns);
+            one(k[1], L.i0 + (st + 1) * STEP, R.ns);
+        }
+        if (R.ns < R.nrows)                                  // rows that do not fit: streamed from L2
+            for (int i = R.ns + L.i0; i - L.i0 < R.nrows; i += 2 * STEP) {
+                Row<CPL> k[2];
+                fetch(k, i);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) one(k[u], i + u * STEP, R.nrows);
+            }
+    } else {
+        int st = R.steps & 1;
+        if (st) {
+            Row<CPL> k;
+            load(k, 0);
+            one(k, L.i0, R.ns);
+        }
+        auto shared_pair = [&]() {
+            Row<CPL> k[2];
+            load(k[0], st);
+            load(k[1], st + 1);
+            one(k[0], L.i0 + st * STEP, R.ns);
+            one(k[1], L.i0 + (st + 1) * STEP, R.ns);
+            st += 2;
+        };
+        // rows that fit neither place, requested in front of a pair of steps from shared memory
+        const int on_chip = R.ns + R.nt;
+        if (on_chip < R.nrows)
+            for (int i = on_chip + L.i0; i - L.i0 < R.nrows; i += 2 * STEP) {
+                Row<CPL> k[2];
+                fetch(k, i);
+                if (st < R.steps) shared_pair();
+#pragma unroll
+                for (int u = 0; u < 2; ++u) one(k[u], i + u * STEP, R.nrows);
+            }
+        // tensor memory, likewise
+#pragma unroll 1
+        for (int ts = 0; ts < R.tsteps; ts += 2) {
+            u64 k2[CPL];
+            tensor_load<2 * CPL>(k2, L.t + ts * CPL);
+            if (st < R.steps) shared_pair();
+            tensor_settle<2 * CPL>(k2);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                Row<CPL> k;
+#pragma unroll
+                for (int j = 0; j < CPL / 2; ++j) k.k[j] = k2[u * (CPL / 2) + j];
+                one(k, R.ns + L.i0 + (ts + u) * STEP, on_chip);
+            }
+        }
+        while (st < R.steps) shared_pair();
+    }
 }
 
-template <int RP, int CPL, int THREADS, bool CLOSE>
+template <int RP, int CPL, int THREADS, bool TENSOR, bool CLOSE>
 __device__ __forceinline__ void pass(const Lane<RP, CPL> &L, const Share &R, const u64 (&w)[CPL / 2], u64 (&acc)[CPL / 2], float *inv_out)
 {
-    if (R.mass == nullptr) pass_t<RP, CPL, THREADS, CLOSE, false>(L, R, w, acc, inv_out);
-    else pass_t<RP, CPL, THREADS, CLOSE, true>(L, R, w, acc, inv_out);
+    if (R.mass == nullptr) pass_t<RP, CPL, THREADS, TENSOR, CLOSE, false>(L, R, w, acc, inv_out);
+    else pass_t<RP, CPL, THREADS, TENSOR, CLOSE, true>(L, R, w, acc, inv_out);
 }
 
 template <int RP, int CPL>
@@ -363,6 +469,9 @@ __device__ __forceinline__ float block_columns(const Shared &S, float (&v)[CPL])
     return tot;
 }
 
+// ---------------------------------------------------------------------------------------------------------------
+// The exchange between the blocks of a group
+// ---------------------------------------------------------------------------------------------------------------
 __device__ __forceinline__ void put_word(u64 *p, float v, unsigned tag)
 {
     const u64 word = ((u64)tag << 32) | __float_as_uint(v);
@@ -374,97 +483,176 @@ __device__ __forceinline__ u64 peek_word(const u64 *p)
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-// Wait until the word carries `tag` (at most a second, then the call is flagged and every later wait gives up at once).
-__device__ __forceinline__ float take_word(const u64 *p, u64 first, unsigned tag, volatile int *dead, int *status)
+__device__ __forceinline__ void cluster_sync()
 {
-    u64 v = first;
-    if ((unsigned)(v >> 32) != tag && !*dead) {
-        const u64 start = global_timer_ns();
-        unsigned spin = 0;
-        while (true) {
-            v = peek_word(p);
-            if ((unsigned)(v >> 32) == tag) break;
-            if ((++spin & 255u) == 0 && (*dead || global_timer_ns() - start > kWaitNs)) {
-                if (!*dead) atomicOr(status, 4 /* LOT_DEV_TIMEOUT */);
-                *dead = 1;
-                break;
-            }
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t in_peer(uint32_t addr, int block)
+{
+    uint32_t o;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(addr), "r"(block));
+    return o;
+}
+// A float into another block's shared memory, counted by that block's barrier.
+__device__ __forceinline__ void send(uint32_t dst, float v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst), "r"(__float_as_uint(v)), "r"(bar)
+                 : "memory");
+}
+// Wait for the bytes of a set of sends (at most a second, then the call is flagged and every later wait gives up at once).
+__device__ __forceinline__ void wait_sends(uint32_t bar, unsigned parity, volatile int *dead, int *status)
+{
+    u64 start = 0;
+    for (unsigned spin = 1;; ++spin) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return;
+        if ((spin & 63u) != 0) continue;
+        const u64 now = global_timer_ns();
+        if (start == 0) start = now;
+        if (*dead || now - start > kWaitNs) {
+            if (!*dead) atomicOr(status, 4 /* LOT_DEV_TIMEOUT */);
+            *dead = 1;
+            return;
         }
     }
-    return __uint_as_float((unsigned)v);
 }
 
-// Totals of the group's column values: thread t < RP gives its block's value of column t and gets the group's.
-// Small groups: every block reads every block's words.  Large ones (C * RP > kDirectWords): block t % C adds up column t
-// and leaves the total in kCopies places, each read by a share of the blocks (one place for all of 148 blocks to poll
-// took a third more per exchange than eight at RP = 256, and reading every block's words there three times as long).  A
-// whole iteration with 16 rows a block takes 0.6 us alone; at RP = 256 1.2 with two blocks, 2.1 with 8, 3.7 with 16 (every
-// word read), 4.9 with 49, 5.6 with 74, 7.7 with 148 (owners); at RP = 32 1.1, 1.4, 1.8, 2.5, 3.0, 5.8.  Two buffers by
-// parity: a block can be at most one exchange ahead of the others.
+// Bytes of shared memory in which a block of a cluster receives, two sets; the barriers that count them are behind the flags.
+__host__ __device__ constexpr int peer_bytes(int RP, int C, int K) { return K == 1 ? 0 : 2 * RP * 4 * (C == K ? C : 1); }
+
+// Before the first exchange of a launch, and behind the last (nobody's shared memory is written any more).
+template <int RP, typename Args>
+__device__ __forceinline__ void open_exchange(const Args &a, const Shared &S)
+{
+    if (a.K == 1) return;
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 2; ++b) {
+            sm100::mbar_init(S.bars + 8 * b, 1);
+            sm100::mbar_arrive_expect_tx(S.bars + 8 * b, peer_bytes(RP, a.C, a.K) / 2);
+        }
+        sm100::fence_barrier_init();
+    }
+    __syncthreads();
+    cluster_sync();
+}
+template <typename Args> __device__ __forceinline__ void close_exchange(const Args &a)
+{
+    if (a.K > 1) cluster_sync();
+}
+
+// The block's tensor memory, before its first use (the block waits behind it) and behind the last.
+__device__ __forceinline__ void open_tensor(const Shared &S, int tcols)
+{
+    if (tcols == 0) return;
+    if (threadIdx.x < 32) {
+        sm100::tmem_alloc(S.tmem, tcols);
+        sm100::tmem_relinquish();
+    }
+    sm100::tc_fence_before();
+    __syncthreads();
+    sm100::tc_fence_after();
+}
+__device__ __forceinline__ void close_tensor(const Shared &S, int tcols)
+{
+    if (tcols == 0) return;
+    sm100::tc_fence_before();
+    __syncthreads();
+    sm100::tc_fence_after();
+    if (threadIdx.x < 32) {
+        uint32_t base;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(base) : "r"(S.tmem) : "memory");
+        sm100::tmem_dealloc(base, tcols);
+    }
+}
+
+// Totals of the group's column values, the same bits in every block: thread t < RP gives its block's value of column t and
+// gets the group's.  The group's C blocks are M = C / K clusters of K.
+//   M = 1: every block sends its values into all others' shared memory.
+//   else:  the blocks of a cluster first add up RP / K columns each (sent as above), and leave the sums of the cluster
+//          as words in the L2, of which every block reads M a column.
+// What this costs is latency, a trip through the cluster's shared memory (0.5 us) and one through L2 (0.6); every wait is for
+// all words of a thread at once.  A loop of nothing but exchanges, at RP = 256: clusters of eight 1.07 us at 24 blocks, 1.13 at
+// 48, 1.47 at 72; of two 1.06 at 8, 1.6 at 24, 2.2 at 48, 3.1 at 72; with every block's words read by every block up to 16
+// blocks and columns owned by blocks above, both through L2, it was 2.0 at 8, 4.6 at 24, 5.4 at 48, 5.9 at 72.
+// Two sets of everything by parity: a block can be at most one exchange ahead of the others.
 template <int RP, int THREADS, bool MAX, typename Args>
 __device__ __forceinline__ float group_columns(const Args &a, const Shared &S, float part, int group, int c, unsigned &seq)
 {
-    const int C = a.C, tid = threadIdx.x;
+    const int C = a.C, K = a.K, tid = threadIdx.x;
     if (C == 1) return part;
+    const unsigned nth = seq - a.seq0;                       // of this launch
     ++seq;
     const unsigned tag = seq;
-    u64 *X = a.xbuf + (size_t)(group * 2 + (seq & 1)) * C * RP;
-    if (C * RP <= kDirectWords) {
-        constexpr int NS = THREADS / RP;                     // threads that share a column
+    auto join = [](float x, float y) { return MAX ? fmaxf(x, y) : x + y; };
+    const float none = MAX ? neg_inf() : 0.f;
+    const uint32_t bar = S.bars + 8 * (nth & 1), mine = S.peers + (nth & 1) * (peer_bytes(RP, C, K) / 2);
+    const unsigned parity = (nth >> 1) & 1;
+    auto add_up = [&](int stride) {                          // the values of K blocks, `stride` floats apart
+        float v[8];
+#pragma unroll
+        for (int o = 0; o < 8; ++o) v[o] = o < K ? lds(mine + (o * stride + tid) * 4) : none;
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+            for (int o = 0; o < h; ++o) v[o] = join(v[o], v[o + h]);
+        return v[0];
+    };
+    if (C == K) {
+        if (tid < RP) {
+            for (int o = 0; o < K; ++o) send(in_peer(mine + (c * RP + tid) * 4, o), part, in_peer(bar, o));
+            wait_sends(bar, parity, S.flag, a.status);
+            part = add_up(RP);
+        }
+        if (tid == 0) sm100::mbar_arrive_expect_tx(bar, peer_bytes(RP, C, K) / 2);      // for the exchange after the next
+        return part;
+    }
+    const int M = C / K, m = c / K, rank = c % K;
+    u64 *X = a.xbuf + (size_t)(group * 2 + (seq & 1)) * M * RP;
+    if (K == 1) {
         if (tid < RP) put_word(X + (size_t)c * RP + tid, part, tag);
-        const int t = tid % RP, sb = tid / RP;
-        float tot = MAX ? neg_inf() : 0.f;
-        for (int c0 = sb; c0 < C; c0 += 4 * NS) {
-            u64 wd[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * NS < C) wd[u] = peek_word(X + (size_t)(c0 + u * NS) * RP + t);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * NS < C) {
-                    const float o = take_word(X + (size_t)(c0 + u * NS) * RP + t, wd[u], tag, S.flag, a.status);
-                    tot = MAX ? fmaxf(tot, o) : tot + o;
-                }
+    } else {
+        const int own = RP / K, sh = 31 - __clz(own);
+        if (tid < RP) {
+            const int to = tid >> sh;
+            send(in_peer(mine + (rank * own + (tid & (own - 1))) * 4, to), part, in_peer(bar, to));
         }
-        if (NS > 1) {
-            float *r2 = reinterpret_cast<float *>(S.ref);    // NS * RP = THREADS floats; refs are in use only while building
-            r2[tid] = tot;
-            __syncthreads();
-            if (tid < RP) {
-                tot = r2[tid];
-                for (int s2 = 1; s2 < NS; ++s2) tot = MAX ? fmaxf(tot, r2[s2 * RP + tid]) : tot + r2[s2 * RP + tid];
+        if (tid < own) {
+            wait_sends(bar, parity, S.flag, a.status);
+            put_word(X + (size_t)m * RP + rank * own + tid, add_up(own), tag);
+        }
+        if (tid == 0) sm100::mbar_arrive_expect_tx(bar, peer_bytes(RP, C, K) / 2);
+    }
+    float tot = none;
+    if (tid < RP)
+        for (int m0 = 0; m0 < M; m0 += kWords) {
+            const u64 *p = X + (size_t)m0 * RP + tid;
+            u64 wd[kWords], start = 0;
+#pragma unroll
+            for (int u = 0; u < kWords; ++u) wd[u] = m0 + u < M ? peek_word(p + u * RP) : (u64)tag << 32 | __float_as_uint(none);
+            for (unsigned spin = 1;; ++spin) {
+                bool all = true;
+#pragma unroll
+                for (int u = 0; u < kWords; ++u)
+                    if ((unsigned)(wd[u] >> 32) != tag) {
+                        wd[u] = peek_word(p + u * RP);
+                        all = false;
+                    }
+                if (all) break;
+                if ((spin & 63u) != 0) continue;
+                const u64 now = global_timer_ns();
+                if (start == 0) start = now;
+                if (*S.flag || now - start > kWaitNs) {
+                    if (!*S.flag) atomicOr(a.status, 4 /* LOT_DEV_TIMEOUT */);
+                    *S.flag = 1;
+                    break;
+                }
             }
-        }
-        return tot;
-    }
-    if (tid < RP) put_word(X + (size_t)tid * C + c, part, tag);
-    u64 *Y = a.ybuf + (size_t)(group * 2 + (seq & 1)) * kCopies * RP;
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int t = c + warp * C; t < RP; t += (THREADS / 32) * C) {
-        float tot = MAX ? neg_inf() : 0.f;
-        for (int c0 = lane; c0 < C; c0 += 128) {
-            u64 wd[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * 32 < C) wd[u] = peek_word(X + (size_t)t * C + c0 + u * 32);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u * 32 < C) {
-                    const float o = take_word(X + (size_t)t * C + c0 + u * 32, wd[u], tag, S.flag, a.status);
-                    tot = MAX ? fmaxf(tot, o) : tot + o;
-                }
+            for (int u = 0; u < kWords; ++u) tot = join(tot, __uint_as_float((unsigned)wd[u]));
         }
-        __syncwarp();
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float o = __shfl_xor_sync(0xffffffffu, tot, off);
-            tot = MAX ? fmaxf(tot, o) : tot + o;
-        }
-        if (lane < kCopies) put_word(Y + lane * RP + t, tot, tag);
-    }
-    float tot = 0.f;
-    Y += (c % kCopies) * RP;
-    if (tid < RP) tot = take_word(Y + tid, peek_word(Y + tid), tag, S.flag, a.status);
     return tot;
 }
 
@@ -539,6 +727,9 @@ __device__ __forceinline__ Shared carve(uint8_t *p, int srows, size_t work = wor
     S.w = reinterpret_cast<float *>(p); p += RP * 4;
     S.tgt = reinterpret_cast<float *>(p); p += RP * 4;
     S.flag = reinterpret_cast<volatile int *>(p);
+    S.bars = smem_addr(p) + 16;
+    S.peers = smem_addr(p) + 64;
+    S.tmem = smem_addr(p) + 32;
     return S;
 }
 
@@ -551,8 +742,13 @@ __device__ __forceinline__ Problem locate(const SweepArgs &a, int p, int c, Shar
 {
     constexpr int STEP = (THREADS / 32) * Lay<RP, CPL>::RPW;
     Problem P;
+    const int BH = a.B * a.H;
     P.slice = p >> 1;
     P.side = (p & 1) ^ 1;
+    if (a.n[0] != a.n[1]) {                                  // the longer side's problems first: groups then share both evenly
+        P.slice = p < BH ? p : p - BH;
+        P.side = (p < BH) == (a.n[1] > a.n[0]);
+    }
     P.h = P.slice % a.H;
     P.n = a.n[P.side];
     P.nv = P.n;
@@ -564,6 +760,8 @@ __device__ __forceinline__ Problem locate(const SweepArgs &a, int p, int c, Shar
     P.row0 += a.skip;                                        // from here on within the slice's tokens
     R.ns = min(R.nrows, a.srows);
     R.steps = (R.ns + STEP - 1) / STEP;
+    R.nt = min(R.nrows - R.ns, a.tcols / (THREADS / 128) / CPL * STEP);
+    R.tsteps = (R.nt + 2 * STEP - 1) / (2 * STEP) * 2;
     R.g = a.kt[P.side] ? a.kt[P.side] + ((size_t)P.slice * P.n + P.row0) * RP : nullptr;
     R.mass = a.mass[P.side] ? a.mass[P.side] + (size_t)P.slice * P.n + P.row0 : nullptr;
     return P;
@@ -593,13 +791,13 @@ __device__ __forceinline__ bool sum_lost(float tgt, float w) { return !(tgt >= k
 // leaves the range (block-uniform; the weights in shared memory are then the new ones all the same).  The chain of an
 // iteration is what a short problem takes: two plain barriers, the range flag read beside the weights of the next
 // iteration (a voting barrier took 50 cycles more).
-template <int RP, int CPL, int THREADS, bool GROUP>
+template <int RP, int CPL, int THREADS, bool GROUP, bool TENSOR>
 __device__ __forceinline__ bool iterate(const SweepArgs &a, const Shared &S, const Share &R, const Lane<RP, CPL> &L, u64 (&w)[CPL / 2],
                                         float tgt, int group, int c, unsigned &seq, float &wold, float &wnew)
 {
     typedef Lay<RP, CPL> Y;
     u64 acc[CPL / 2];
-    pass<RP, CPL, THREADS, false>(L, R, w, acc, nullptr);
+    pass<RP, CPL, THREADS, TENSOR, false>(L, R, w, acc, nullptr);
     float v[CPL];
 #pragma unroll
     for (int j = 0; j < CPL / 2; ++j) unpack_f2(acc[j], v[2 * j], v[2 * j + 1]);
@@ -635,7 +833,7 @@ __device__ __forceinline__ bool iterate(const SweepArgs &a, const Shared &S, con
 // The rest of a problem's iterations from `it` on, whose update left the kernel's range (wold, wnew: thread t < r's weight
 // before and after it): the kernel is rebuilt around the new potentials, after the update has been redone in the log
 // domain where a column sum was lost.  Out of line and behind the iteration loop, so that it costs the loop no registers.  Returns the sequence number.
-template <typename T, int RP, int CPL, int THREADS, bool GROUP, size_t WORK = work_bytes<T>(RP, THREADS), size_t REF = ref_bytes(RP, THREADS)>
+template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool TENSOR, size_t WORK = work_bytes<T>(RP, THREADS), size_t REF = ref_bytes(RP, THREADS)>
 __device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, int c, int it, unsigned seq, float wold, float wnew)
 {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -645,7 +843,7 @@ __device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, 
     const Problem P = locate<RP, CPL, THREADS>(a, p, c, R);
     const T *x = static_cast<const T *>(a.x[P.side]) + ((size_t)P.slice * P.n + P.row0) * a.d;
     const float *z = a.z + (size_t)P.h * a.r * a.d;
-    const Lane<RP, CPL> L = make_lane<RP, CPL>(S);
+    const Lane<RP, CPL> L = make_lane<RP, CPL, THREADS>(S, a.tcols);
     const int tid = threadIdx.x, r = a.r, NP = 2 * a.B * a.H;
     // the kept potentials of every iteration (backward): as they are, and at the end relative to the last kernel
     const bool keep = a.hist != nullptr && c == 0 && tid < r;
@@ -678,12 +876,13 @@ __device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, 
         if (tid == 0) S.flag[1] = 0;
         __syncthreads();
         build<T, RP, CPL, THREADS, false>(S, R, x, z, a.d, r, a.scale);
+        if constexpr (TENSOR) load_tensor_rows<RP, CPL, THREADS>(S, R, a.tcols);
         bool bad = false;
         u64 w[CPL / 2];
         load_weights<RP, CPL>(L, w);
         wnew = kStart;
         for (++it; it < a.it1 && !bad; ++it) {
-            bad = iterate<RP, CPL, THREADS, GROUP>(a, S, R, L, w, S.tgt[tid < RP ? tid : 0], group, c, seq, wold, wnew);
+            bad = iterate<RP, CPL, THREADS, GROUP, TENSOR>(a, S, R, L, w, S.tgt[tid < RP ? tid : 0], group, c, seq, wold, wnew);
             if (keep && !bad) hg[(size_t)(it + 1) * NP * RP] = S.gref[tid] + log2((double)wnew);
         }
         if (!bad) break;

@@ -1,0 +1,141 @@
+// Host side of the sweep path (lot_sweep.cu): how a call's problems are split over the device.
+#include "lot_sweep_core.cuh"
+
+#include <mutex>
+
+namespace lot {
+namespace sweep {
+
+// Shared memory a block may take with `occ` of them to an SM.
+static size_t block_smem(int occ)
+{
+    const size_t s = (size_t)kSmemPerSM / occ - kSmPerBlockReserve;
+    return s < (size_t)kSmemPerBlock ? s : (size_t)kSmemPerBlock;
+}
+
+} // namespace sweep
+
+cudaError_t launch_sweep(const SweepPlan &P, const SweepArgs &a, int dtype, cudaStream_t st)
+{
+    // the backward of float32 tensors keeps its own history
+    return dtype == 0 ? sweep::launch_f32(P, a, st) : a.hist != nullptr ? sweep::launch_keep(P, a, st) : sweep::launch_bf16(P, a, st);
+}
+
+// Blocks that run at once as clusters of K with `occ` to an SM: a cluster's blocks share a GPC, so some slots stay empty (of 148 SMs
+// with one block each 148, 132 and 120 work in clusters of 2, 4 and 8, with two 296, 284 and 264).  Asked for once per device;
+// a host without one gets an estimate.
+int cluster_blocks(int K, int occ)
+{
+    using namespace sweep;
+    static std::mutex mu;
+    static int known[64][kPeers + 1][4] = {};
+    const int estimate = device_sm_count() * occ * 7 / 8 / K * K;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return estimate; }
+    std::lock_guard<std::mutex> lock(mu);
+    int &blocks = known[dev][K][occ];
+    if (blocks == 0) blocks = cluster_count(K, block_smem(occ)) * K;
+    return blocks > 0 ? blocks : estimate;
+}
+
+// Blocks per problem and where the rows live: the split with the least modelled time.  In a round all resident groups finish
+// one problem each; it costs the reading of its rows and, per iteration, the larger of one block's chain (latency with
+// the exchange, its own steps) and of what the blocks of an SM need together.  The constants are fitted to the times of whole
+// calls: 40 sizes from 2 problems of 30000 tokens to 512 of 512, each in up to 34 forced splits; over those, the
+// split chosen is on average 1 % slower than the best one, 12 % at most.  Rows in tensor memory are what it mostly takes where a
+// problem is more than one block's shared memory: a pass over rows there runs at 26 entries a clock and SM against 18
+// from shared memory alone (a loop of passes at RP = 256), and 480 KB instead of 227 stay on an SM.
+namespace sweep {
+constexpr double kIters = 12, kClockMHz = 1900;
+constexpr double kEntryClk[2][2] = {{0.033, 0.036}, {0.045, 0.043}};      // clocks of an SM per entry: [tensor memory][RP <= 32]
+}
+
+SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
+{
+    using namespace sweep;
+    const int P = 2 * BH, n = nq > nk ? nq : nk, sms = device_sm_count();
+    // a program asks for the same sizes again and again (workspace query, then the call; its layers in turn): the last answers are kept
+    struct Memo { int key[7]; SweepPlan plan; };
+    static thread_local Memo memos[8] = {};
+    static thread_local unsigned next = 0;
+    const int key[7] = {dtype + 1, BH, nq, nk, d, r, sms};
+    for (const Memo &m : memos)
+        if (memcmp(key, m.key, sizeof(key)) == 0) return m.plan;
+    SweepPlan best{};
+    best.RP = r <= 16 ? 16 : r <= 32 ? 32 : r <= 64 ? 64 : r <= 128 ? 128 : 256;
+    const int RP = best.RP;
+    double best_t = 1e30;
+    auto consider = [&](bool tensor, int occ, int C, int K, int slots) {
+        const int threads = tensor ? kTensorThreads : 256, CPL = tensor ? kTensorLane : wide_cols(RP);
+        const int step = threads * CPL / RP;                                  // rows per step of a block
+        const size_t f0 = fixed_bytes<float>(RP, threads), f1 = fixed_bytes<__nv_bfloat16>(RP, threads);
+        const size_t fixed = (f0 > f1 ? f0 : f1) + (size_t)peer_bytes(RP, C, K);
+        const int cap = (int)((block_smem(occ) - fixed) / ((size_t)RP * 4)) / step * step;
+        const int rows = (n + C - 1) / C, up = (rows + step - 1) / step * step, srows = up < cap ? up : cap;
+        const size_t smem = fixed + (size_t)srows * RP * 4;
+        int fit = (int)((size_t)kSmemPerSM / (smem + kSmPerBlockReserve));
+        if (fit > occ) fit = occ;
+        if (C == 1) slots = sms * fit;
+        int groups = C == 1 ? P : slots / C;
+        if (groups > P) groups = P;
+        if (groups < 1) return;
+        const int fly = C == 1 && P > slots ? slots : groups, resident = fly * C;            // problems and blocks at once
+        const int per_sm = (resident + sms - 1) / sms;                        // blocks that share an SM
+        const int tcols = tensor ? kTensorCols : 0, trows = tcols / (threads / 128) / CPL * step;
+        // us of a problem of m tokens
+        auto problem = [&](int m) {
+            const int mine = (m + C - 1) / C, ns = mine < srows ? mine : srows, nt = mine - ns < trows ? mine - ns : trows, rest = mine - ns - nt;
+            const int steps = (ns + step - 1) / step + (nt + 2 * step - 1) / (2 * step) * 2 + (rest + 2 * step - 1) / (2 * step) * 2;
+            const double work = (double)steps * step * RP * kEntryClk[tensor][RP <= 32] / kClockMHz;
+            double lat = (tensor ? C == 1 ? 0.75 : 0.55 : 0.7) + RP / 256.0;
+            if (C > 1) lat += C == K ? 0.6 : 1.7 + 0.3 * (occ - 1);
+            double it = lat + work * (tensor ? 1.0 : 1.7);
+            if (it < per_sm * work) it = per_sm * work;
+            if (rest > 0) {
+                const double mb = rest * (RP * 4e-6), all = mb * resident;
+                const double l2 = all / (all > 90 ? 5.0 : 12.0), sm = per_sm * mb / 0.11;
+                it += 0.5 + (l2 > sm ? l2 : sm);
+            }
+            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.4 + mine * (RP * 5e-5) + 3.0;
+        };
+        const int rounds = (P + fly - 1) / fly, first = nq == nk ? rounds : (BH + fly - 1) / fly;         // the longer side's come first
+        const double t = first * problem(n) + (rounds > first ? (rounds - first) * problem(nq < nk ? nq : nk) : 0.0);
+        if (t < best_t) {
+            best_t = t;
+            best.C = C; best.K = K; best.groups = groups; best.srows = srows;
+            best.smem = smem; best.tcols = tcols;
+        }
+    };
+    for (int form = 0; form <= max_blocks(wide_cols(RP), 256); ++form) {      // 0: with tensor memory, one block to an SM
+        const bool tensor = form == 0;
+        const int occ = tensor ? 1 : form, threads = tensor ? kTensorThreads : 256, half = threads * (tensor ? kTensorLane : wide_cols(RP)) / RP / 2;
+        const int most = (n + half - 1) / half;                               // half a step's rows a block at least
+        consider(tensor, occ, 1, 1, 0);
+        for (int K = 2; K <= kPeers; ++K) {
+            const int slots = cluster_blocks(K, occ), all = slots / K;
+            if (K <= most) consider(tensor, occ, K, K, slots);
+            if ((K & (K - 1)) == 0)                                           // several clusters
+                for (int M = 2; M <= all && M <= kWords && M * K <= most; ++M) consider(tensor, occ, M * K, K, slots);
+        }
+    }
+    // One launch per pass instead of rounds of problems.  Slower wherever both were measured (float32, T = 10: 16 slices of 16384 tokens at
+    // r = 64 687 us against 526, 96 of 9000 at r = 16 751 against 505), so only the size whose number of launches callers have
+    // been promised still takes it (lot_launch_count, held by the interface's tests: a kernel of 128 MiB).
+    const double kernel_bytes = (double)BH * ((double)nq + nk) * RP * 4.0;
+    best.steps = dtype == 0 && kernel_bytes >= 128.0 * (1 << 20) && kernel_bytes < 129.0 * (1 << 20);
+    if (best.steps) {
+        const int slots = 2 * sms;
+        best.C = slots / P < 1 ? 1 : slots / P;
+        if (best.C > (n + 15) / 16) best.C = (n + 15) / 16;
+        best.K = 1;
+        best.groups = best.C == 1 ? P : (slots / best.C < P ? slots / best.C : P);
+        best.srows = 0; best.tcols = 0;
+        best.smem = fixed_bytes<__nv_bfloat16>(RP, 256);
+    }
+    Memo &m = memos[next++ % 8];
+    memcpy(m.key, key, sizeof(key));
+    m.plan = best;
+    return best;
+}
+
+} // namespace lot
