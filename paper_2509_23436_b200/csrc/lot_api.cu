@@ -147,9 +147,9 @@ BwdLayout bwd_layout(int B, int H, int n, int d, int r, int iters)
 // similarities.
 struct BwdSweepLayout {
     SweepPlan plan;
-    int rounds, tiles, achunks, arows;
+    int rounds, tiles, achunks, arows, gchunks, grows;
     size_t counter, xbuf, head_end, w[2], gref[2], inv[2], kt[2], dC[2], hist, hist_g, wide, coef, fk, gpart, dbeta_acc, wpart,
-        Wp, Xw, dWm, dbeta_direct, zpart[2], total;
+        wpart2, counter2, Wp, Xw, dWm, dbeta_direct, zpart[2], total;
 };
 
 BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
@@ -163,6 +163,7 @@ BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
     L.tiles = (n + 127) / 128;
     size_t o = 256;                                                   // status word at 0
     L.counter = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
+    L.counter2 = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
     L.xbuf = o;
     o += up256(exchange_bytes(RP, L.plan.C, L.plan.K, L.plan.groups));
     L.head_end = o;
@@ -182,12 +183,15 @@ BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
     L.dbeta_acc = o; o += up256((size_t)NP * RP * 4);
     L.achunks = apply_chunks(BH, n, r, 64);
     L.arows = (n + L.achunks - 1) / L.achunks;
+    L.gchunks = sweep_grad_chunks(BH, n);
+    L.grows = ((n + 63) / 64 + L.gchunks - 1) / L.gchunks * 64;
     L.wpart = o; o += up256((size_t)BH * L.achunks * r * d * 4);
+    L.wpart2 = o; o += up256((size_t)BH * L.achunks * r * d * 4);
     L.Wp = o; o += up256((size_t)BH * r * d * 4);
     L.Xw = o; o += up256((size_t)BH * r * d * 4);
     L.dWm = o; o += up256((size_t)BH * r * d * 4);
     L.dbeta_direct = o; o += up256((size_t)BH * r * 4);
-    for (int side = 0; side < 2; ++side) { L.zpart[side] = o; o += up256((size_t)BH * L.achunks * r * d * 4); }
+    for (int side = 0; side < 2; ++side) { L.zpart[side] = o; o += up256((size_t)BH * (L.achunks > L.gchunks ? L.achunks : L.gchunks) * r * d * 4); }
     L.total = o;
     return L;
 }
@@ -446,11 +450,12 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
     ap.B = B; ap.H = H; ap.nq = n; ap.nk = n; ap.d = d; ap.r = r; ap.RP = RP; ap.terms = 3;
     ap.chunks = L.achunks; ap.rows_per_chunk = L.arows;
-    if ((e = launch_sweep_apply_w(ap, dt, st)) != cudaSuccess) return e;              // W' = Diag(1/beta) Gamma2 V
-    // ---- reverse of the read-out, Eq. (4): out = R1 W'
-    SweepApplyArgs aq = ap;                                                             // R1^T dout / (n beta): the key-side product on the query side
+    // W' = Diag(1/beta) Gamma2 V, and with it the reverse of the read-out, Eq. (4), out = R1 W': R1^T dout / (n beta) is the key-side
+    // product on the query side
+    SweepApplyArgs aq = ap;
     aq.kt[1] = ap.kt[0]; aq.inv[1] = ap.inv[0]; aq.w[1] = ap.w[0]; aq.key_len = nullptr; aq.v = dout; aq.Wp = at<float>(ws, L.Xw);
-    if ((e = launch_sweep_apply_w(aq, dt, st)) != cudaSuccess) return e;
+    aq.wpart = at<float>(ws, L.wpart2); aq.counter = at<unsigned>(ws, L.counter2);
+    if ((e = launch_sweep_apply_w(ap, dt, st, &aq)) != cudaSuccess) return e;
     float *dbd = at<float>(ws, L.dbeta_direct), *dWm = at<float>(ws, L.dWm);
     if ((e = launch_bwd_w_fix(at<float>(ws, L.Xw), ap.Wp, key_len, dWm, dbd, B, H, n, d, r, st)) != cudaSuccess) return e;
     SweepApplyArgs av = ap;                                                             // dV = Gamma2 dW: the query-side product on the key side
@@ -463,6 +468,13 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
     // ---- the iterations, last first
     a.seq0 = 4u * (unsigned)(iters + 1) * (unsigned)L.rounds;
     if ((e = launch_bwd_reverse(L.plan, b, st)) != cudaSuccess) return e;
+    if (sweep_grad_supported(r, d)) {
+        SweepGradArgs g{};
+        g.b = b; g.dx[0] = dq; g.dx[1] = dk; g.chunks = L.gchunks; g.rows = L.grows;
+        for (int side = 0; side < 2; ++side) g.part[side] = at<float>(ws, L.zpart[side]);
+        if ((e = launch_sweep_grad(RP, g, st)) != cudaSuccess) return e;
+        return launch_bwd_merge(g.part[0], g.part[1], dbd, b.dbeta_acc, dz, dbeta, B, H, d, r, RP, L.gchunks, add, st);
+    }
     if (iters > 0 && (e = launch_bwd_assemble(RP, b, st)) != cudaSuccess) return e;
     // ---- C = X Z^T: dX = dC Z, dZ = dC^T X, the same two products with the gradient in place of the plan
     for (int side = 0; side < 2; ++side) {

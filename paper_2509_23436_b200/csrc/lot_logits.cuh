@@ -25,6 +25,24 @@ __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr)
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
 
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+// two floats as N packed bf16 pairs
+template <int N> __device__ __forceinline__ void split(float x, float y, uint32_t (&o)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+        o[i] = *reinterpret_cast<const uint32_t *>(&h);
+        x -= __low2float(h);
+        y -= __high2float(h);
+    }
+}
+
 // Shared memory of one staged step of pivots.
 template <typename T> __host__ __device__ constexpr size_t stage_bytes(int cc) { return sizeof(T) == 2 ? (size_t)cc * 80 * 3 : (size_t)cc * 18 * 8; }
 

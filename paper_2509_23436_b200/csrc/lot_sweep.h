@@ -85,7 +85,8 @@ struct SweepApplyArgs {
     int per_head;            // query side: Wp is [H][r][d]
     int chunks, rows_per_chunk;
 };
-cudaError_t launch_sweep_apply_w(const SweepApplyArgs &a, int dtype, cudaStream_t st);
+// second: another product of the same sizes, buffers of its own, in the same launch (bf16 tensors)
+cudaError_t launch_sweep_apply_w(const SweepApplyArgs &a, int dtype, cudaStream_t st, const SweepApplyArgs *second = nullptr);
 cudaError_t launch_sweep_apply_out(const SweepApplyArgs &a, int dtype, cudaStream_t st);
 
 // ---- backward of bf16 tensors on the stored kernel (lot_sweep_bwd.cu); problem numbering as above ----
@@ -101,6 +102,16 @@ struct SweepBwdArgs {
     int T, tiles;
     double eps;
 };
+// Everything behind the reverse steps: dx = dC Z, part = chunk partials of dC^T x (lot_sweep_grad.cu)
+struct SweepGradArgs {
+    SweepBwdArgs b;
+    void *dx[2];             // [BH][n][d] bf16
+    float *part[2];          // [BH][chunks][r][d]
+    int chunks, rows;
+};
+bool sweep_grad_supported(int r, int d);
+int sweep_grad_chunks(int BH, int n);                // of whole steps of 64 rows
+cudaError_t launch_sweep_grad(int RP, const SweepGradArgs &a, cudaStream_t st);
 cudaError_t launch_bwd_close(int RP, const SweepBwdArgs &a, cudaStream_t st);
 cudaError_t launch_bwd_reverse(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st);
 cudaError_t launch_bwd_assemble(int RP, const SweepBwdArgs &a, cudaStream_t st);

@@ -16,23 +16,9 @@ namespace sweep_apply {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-// two floats as N packed bf16 pairs
-template <int N> __device__ __forceinline__ void split(float x, float y, uint32_t (&o)[N])
-{
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-        o[i] = *reinterpret_cast<const uint32_t *>(&h);
-        x -= __low2float(h);
-        y -= __high2float(h);
-    }
-}
+using logits::ldsm4_t;
+using logits::smem_addr;
+using logits::split;
 
 __device__ __forceinline__ float4 scaled(float4 p, float4 w, float s)
 {
@@ -77,14 +63,16 @@ __device__ __forceinline__ bool last_of_tile(unsigned *counter, int chunks)
 // ---------------------------------------------------------------------------------------------------------------
 template <int TP, int D, int N>
 __global__ void __launch_bounds__(kThreads, D <= 128 ? 2 : 1)
-apply_w_mma_kernel(SweepApplyArgs a)
+apply_w_mma_kernel(const __grid_constant__ SweepApplyArgs a0, const __grid_constant__ SweepApplyArgs a1)
 {
+    const bool second = (int)blockIdx.z >= a0.B * a0.H;            // two products of the same sizes in one launch
+    const SweepApplyArgs &a = second ? a1 : a0;
     constexpr int KT = 64, PP = (TP + 8) * 2, PV = (D + 8) * 2, PLANE = KT * PP;
     constexpr int PT = TP / 16, CG = 8 / PT < D / 16 ? 8 / PT : D / 16, KS = 8 / (PT * CG), NTW = D / 8 / CG;
     constexpr int NP = KT * TP / 4 / kThreads, NV = KT * D / 8 / kThreads;
     extern __shared__ __align__(128) uint8_t sm[];
     uint8_t *sP = sm, *sV = sm + N * PLANE;
-    const int bh = blockIdx.z, b = bh / a.H, h = bh % a.H, chunk = blockIdx.x, t0 = blockIdx.y * TP;
+    const int bh = blockIdx.z - (second ? a0.B * a0.H : 0), b = bh / a.H, h = bh % a.H, chunk = blockIdx.x, t0 = blockIdx.y * TP;
     const int n = a.nk, r = a.r, d = a.d, RP = a.RP;
     int nv = n;
     if (a.key_len != nullptr) nv = min(max(a.key_len[b], 0), n);
@@ -506,19 +494,19 @@ static cudaError_t big_smem(Kern kern, size_t bytes)
 }
 
 template <int TP, int D, int N>
-static cudaError_t launch_w(const SweepApplyArgs &a, cudaStream_t st)
+static cudaError_t launch_w(const SweepApplyArgs &a, const SweepApplyArgs *b, cudaStream_t st)
 {
     constexpr size_t smem = N * 64 * (TP + 8) * 2 + 64 * (D + 8) * 2;
     auto kern = apply_w_mma_kernel<TP, D, N>;
     cudaError_t e = big_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    return chain_launch(kern, dim3(a.chunks, (a.r + TP - 1) / TP, a.B * a.H), kThreads, smem, st, a);
+    return chain_launch(kern, dim3(a.chunks, (a.r + TP - 1) / TP, a.B * a.H * (b ? 2 : 1)), kThreads, smem, st, a, b ? *b : a);
 }
 template <int TP>
-static cudaError_t launch_w_d(const SweepApplyArgs &a, cudaStream_t st)
+static cudaError_t launch_w_d(const SweepApplyArgs &a, const SweepApplyArgs *b, cudaStream_t st)
 {
-    if (a.d <= 64) return a.terms == 2 ? launch_w<TP, 64, 2>(a, st) : launch_w<TP, 64, 3>(a, st);
-    return a.d <= 128 ? launch_w<TP, 128, 3>(a, st) : launch_w<TP, 256, 3>(a, st);
+    if (a.d <= 64) return a.terms == 2 ? launch_w<TP, 64, 2>(a, b, st) : launch_w<TP, 64, 3>(a, b, st);
+    return a.d <= 128 ? launch_w<TP, 128, 3>(a, b, st) : launch_w<TP, 256, 3>(a, b, st);
 }
 template <int TS, int D, int N>
 static cudaError_t launch_out(const SweepApplyArgs &a, cudaStream_t st)
@@ -538,10 +526,10 @@ static cudaError_t launch_out_d(const SweepApplyArgs &a, cudaStream_t st)
 
 } // namespace sweep_apply
 
-cudaError_t launch_sweep_apply_w(const SweepApplyArgs &a, int dtype, cudaStream_t st)
+cudaError_t launch_sweep_apply_w(const SweepApplyArgs &a, int dtype, cudaStream_t st, const SweepApplyArgs *second)
 {
     using namespace sweep_apply;
-    if (dtype != 0) return a.RP == 16 ? launch_w_d<16>(a, st) : a.RP == 32 ? launch_w_d<32>(a, st) : launch_w_d<64>(a, st);
+    if (dtype != 0) return a.RP == 16 ? launch_w_d<16>(a, second, st) : a.RP == 32 ? launch_w_d<32>(a, second, st) : launch_w_d<64>(a, second, st);
     const int cb = (a.d + kCT - 1) / kCT, TP = a.RP < 64 ? a.RP : 64;
     dim3 grid(a.chunks, (a.r + TP - 1) / TP * cb, a.B * a.H);
     return chain_launch(TP == 16 ? apply_w_f32_kernel<16> : TP == 32 ? apply_w_f32_kernel<32> : apply_w_f32_kernel<64>, grid, kThreads, 0, st, a);
