@@ -535,7 +535,8 @@ cudaError_t launch_apply_out(const ApplyArgs &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Eq. (5): row 0 of every slice is the plain softmax over the valid keys.  One block per slice: eight lanes a key for the
+// Eq. (5): row 0 of every slice is the plain softmax over the valid keys.  A cluster of up to eight blocks shares a slice's keys; the
+// blocks' parts are joined relative to the largest score.  A block: eight lanes a key for the
 // scores (kept in shared memory while they fit, else in global scratch), their maximum, the exponentials and their sum,
 // then d / 8 threads a key for the weighted values, the threads' parts added in a fixed order.
 constexpr int kClsKeys = 4096;
@@ -565,6 +566,16 @@ template <bool MAX> __device__ __forceinline__ float cls_block(float v, float *r
     return v;
 }
 
+// Element i of an array at `base` in another block's shared memory.
+__device__ __forceinline__ float peer_float(uint32_t base, int i, int block)
+{
+    uint32_t there;
+    float x;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(base + i * 4), "r"(block));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(there) : "memory");
+    return x;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, const int32_t *key_len, int H,
@@ -573,11 +584,13 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
     __shared__ float sc_s[kClsKeys];
     __shared__ __align__(16) float part[256 * 8];
     __shared__ float red[8];
-    const int bh = blockIdx.x, bb = bh / H, tid = threadIdx.x;
-    int kv = nk;
-    if (key_len != nullptr) kv = min(max(key_len[bb], 0), nk);
-    const T *qb = q + (size_t)bh * nq * d, *kb = k + (size_t)bh * nk * d, *vb = v + (size_t)bh * nk * d;
-    float *sc = kv <= kClsKeys ? sc_s : scores + (size_t)bh * nk;
+    // the slice's keys are shared evenly by the blocks of its cluster
+    const int bh = blockIdx.y, bb = bh / H, tid = threadIdx.x, rank = blockIdx.x, blocks = gridDim.x;
+    int all = nk;
+    if (key_len != nullptr) all = min(max(key_len[bb], 0), nk);
+    const int first = (int)((long long)all * rank / blocks), kv = (int)((long long)all * (rank + 1) / blocks) - first;
+    const T *qb = q + (size_t)bh * nq * d, *kb = k + ((size_t)bh * nk + first) * d, *vb = v + ((size_t)bh * nk + first) * d;
+    float *sc = kv <= kClsKeys ? sc_s : scores + (size_t)bh * nk + first;
     const int l8 = tid & 7;
     float mx = neg_inf();
 #pragma unroll 4
@@ -625,10 +638,34 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
         for (int i = 0; i < 8; ++i) part[p * d + c + i] = acc[i];
     }
     __syncthreads();
-    for (int cc = tid; cc < d; cc += 256) {
-        float s = 0.f;
-        for (int i = 0; i < parts; ++i) s += part[i * d + cc];
-        Elem<T>::store(out + (size_t)bh * nq * d + cc, kv > 0 ? s / den : 0.f);
+    float own = 0.f;                                               // d <= 256: a channel a thread
+    if (tid < d)
+        for (int i = 0; i < parts; ++i) own += part[i * d + tid];
+    if (blocks == 1) {
+        if (tid < d) Elem<T>::store(out + (size_t)bh * nq * d + tid, kv > 0 ? own / den : 0.f);
+    } else {
+        __syncthreads();
+        if (tid < d) part[tid] = own;
+        if (tid == 0) { part[256] = mx; part[257] = den; }
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank == 0 && tid < d) {
+            const uint32_t base = (uint32_t)__cvta_generic_to_shared(part);
+            float m[8], top = neg_inf(), sum = 0.f, sden = 0.f;
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                m[o] = o < blocks ? peer_float(base, 256, o) : neg_inf();       // a block without keys: -infinity, nothing of it below
+                top = fmaxf(top, m[o]);
+            }
+#pragma unroll
+            for (int o = 0; o < 8; ++o)
+                if (o < blocks && m[o] > neg_inf()) {
+                    const float f = __expf(m[o] - top);
+                    sum = fmaf(f, peer_float(base, tid, o), sum);
+                    sden = fmaf(f, peer_float(base, 257, o), sden);
+                }
+            Elem<T>::store(out + (size_t)bh * nq * d + tid, all > 0 ? sum / sden : 0.f);
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");       // read by now
     }
     // It touches nothing of its predecessors, so it runs beside them; but what comes next on the stream (a reader of out, the
     // next call's ordinary launch) waits for this kernel alone, so it must not end before they have.
@@ -638,12 +675,16 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
 cudaError_t launch_cls_row(const void *q, const void *k, const void *v, const int32_t *key_len, int dtype, int B, int H,
                            int nq, int nk, int d, float tau, float *scores, void *out, cudaStream_t st)
 {
+    // Blocks a slice: about two an SM over all slices, 128 keys each at least.  12 slices of 832 float32 keys 28 us with one block each,
+    // 6.4 with six; 96 of 197 run beside the kernels in front of this one, and three blocks each made the call 30.7 -> 32.6.
+    const int most = nk / 128 < 8 ? nk / 128 : 8, want = 2 * device_sm_count() / (B * H), per = want < 1 ? 1 : want < most ? want : most < 1 ? 1 : most;
+    const dim3 grid((unsigned)per, (unsigned)(B * H));
     if (dtype == 0)
-        return chain_launch(cls_row_kernel<float>, dim3(B * H), 256, 0, st, static_cast<const float *>(q), static_cast<const float *>(k),
+        return chain_launch(cls_row_kernel<float>, grid, 256, 0, per, st, static_cast<const float *>(q), static_cast<const float *>(k),
                             static_cast<const float *>(v), key_len, H, nq, nk, d, tau, scores, static_cast<float *>(out));
     typedef __nv_bfloat16 bf;
-    return chain_launch(cls_row_kernel<bf>, dim3(B * H), 256, 0, st, static_cast<const bf *>(q), static_cast<const bf *>(k),
-                        static_cast<const bf *>(v), key_len, H, nq, nk, d, tau, scores, static_cast<bf *>(out));
+    return chain_launch(cls_row_kernel<bf>, grid, 256, 0, per, st, static_cast<const bf *>(q), static_cast<const bf *>(k),
+                            static_cast<const bf *>(v), key_len, H, nq, nk, d, tau, scores, static_cast<bf *>(out));
 }
 
 LOT_DEBUG_FLAG_READER(kernels_debug_flag)
