@@ -114,6 +114,7 @@ static cudaError_t launch_rp(int RP, const SweepArgs &a, int sides, cudaStream_t
 // sides: bit 0 the queries, bit 1 the keys
 cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st)
 {
+    if (dtype == 1 && build_tc_supported(RP, a.d)) return launch_build_tc(RP, a, sides, st);
     if (dtype == 1 && a.terms == 2) {
         if (RP == 16) return build::launch_t<__nv_bfloat16, 16, 2>(a, sides, st);
         if (RP == 32) return build::launch_t<__nv_bfloat16, 32, 2>(a, sides, st);

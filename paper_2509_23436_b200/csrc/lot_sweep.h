@@ -66,6 +66,8 @@ int cluster_blocks(int K, int occ);      // blocks that run at once as clusters 
 inline size_t exchange_bytes(int RP, int C, int K, int groups) { return C > K ? (size_t)groups * 2 * (C / K) * RP * 8 : 0; }
 SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r);
 cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st);
+bool build_tc_supported(int RP, int d);  // bf16 tokens on tcgen05 (lot_build_tc.cu)
+cudaError_t launch_build_tc(int RP, const SweepArgs &a, int sides, cudaStream_t st);
 cudaError_t launch_sweep(const SweepPlan &P, const SweepArgs &a, int dtype, cudaStream_t st);
 
 struct SweepApplyArgs {
