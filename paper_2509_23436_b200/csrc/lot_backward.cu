@@ -63,7 +63,7 @@ template <int LPR, int NV, bool CLOSE, typename LT>
 __global__ void __launch_bounds__(kBwdWarps * 32)
 bwd_row_kernel(BwdRowArgs a)
 {
-    __shared__ LT sm_c[kBwdWarps][256];
+    __shared__ LT sm_c[kBwdWarps][256], sm_h[256];
     __shared__ int sm_last;
     constexpr int CPL = 4 * NV;
     constexpr int RPW = 32 / LPR;
@@ -83,6 +83,15 @@ bwd_row_kernel(BwdRowArgs a)
     const LT inv_eps = (LT)(1.0 / a.eps);
     const LT mass = nvalid > 0 ? (LT)1 / (LT)nvalid : (LT)0;
 
+    // the exponent offset of q_it = 2^(L_it + G+_t - log2 beta_t - M_i), worked out once a column: sixteen float64 logarithms a thread took
+    // most of a launch on short problems
+    if (!CLOSE) {
+        if ((int)threadIdx.x < r) {
+            const int t = threadIdx.x;
+            sm_h[t] = static_cast<const LT *>(a.Gb)[(size_t)p * r + t] - (LT)log2((double)a.beta[h * r + t]);
+        }
+        __syncthreads();
+    }
     LT Gk[CPL], Hk[CPL], gk[CPL], col[CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
@@ -91,8 +100,7 @@ bwd_row_kernel(BwdRowArgs a)
         Hk[k] = (LT)0;
         gk[k] = (LT)0;
         if (!CLOSE && t < r) {
-            // exponent offset of q_it = 2^(L_it + G+_t - log2 beta_t - M_i)
-            Hk[k] = static_cast<const LT *>(a.Gb)[(size_t)p * r + t] - (LT)log2((double)a.beta[h * r + t]);
+            Hk[k] = sm_h[t];
             gk[k] = gam[t];
         }
         col[k] = (LT)0;
