@@ -157,7 +157,7 @@ BwdSweepLayout bwd_sweep_layout(int B, int H, int n, int d, int r, int iters)
     BwdSweepLayout L;
     const int BH = B * H > 0 ? B * H : 1, NP = 2 * BH;
     if (n < 1) n = 1;
-    L.plan = sweep_plan(LOT_BF16, BH, n, n, d, r);
+    L.plan = sweep_plan(LOT_BF16, BH, n, n, d, r, true);
     const int RP = L.plan.RP;
     L.rounds = (NP + L.plan.groups - 1) / L.plan.groups;
     L.tiles = (n + 127) / 128;

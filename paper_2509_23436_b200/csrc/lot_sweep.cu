@@ -138,6 +138,9 @@ static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t
 template <typename T, int RP, bool KEEP>
 static cudaError_t launch_k(const SweepPlan &P, const SweepArgs &a, cudaStream_t st)
 {
+    if constexpr (RP <= 32 && !KEEP) {
+        if (P.threads == 32) return launch_g<T, RP, wide_cols(RP), 32, false, false, false>(P, a, st);
+    }
     if (P.tcols)
         return P.C > 1 ? launch_g<T, RP, kTensorLane, kTensorThreads, true, true, KEEP>(P, a, st)
                        : launch_g<T, RP, kTensorLane, kTensorThreads, false, true, KEEP>(P, a, st);

@@ -51,6 +51,7 @@ struct SweepArgs {
 
 struct SweepPlan {
     int RP, C, K, groups, srows, tcols;
+    int threads;             // of a block
     int steps;               // 1: one launch per iteration (the kernel streams from global memory anyway)
     size_t smem;
 };
@@ -64,7 +65,8 @@ int cluster_count(int K, size_t smem);                                          
 }
 int cluster_blocks(int K, int occ);      // blocks that run at once as clusters of K, `occ` to an SM
 inline size_t exchange_bytes(int RP, int C, int K, int groups) { return C > K ? (size_t)groups * 2 * (C / K) * RP * 8 : 0; }
-SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r);
+SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep = false);      // keep: for the backward
+constexpr int kWarpEntries = 4096;       // the most entries of a problem that one warp takes by itself
 cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st);
 bool build_tc_supported(int RP, int d);  // bf16 tokens on tcgen05 (lot_build_tc.cu)
 cudaError_t launch_build_tc(int RP, const SweepArgs &a, int sides, cudaStream_t st);

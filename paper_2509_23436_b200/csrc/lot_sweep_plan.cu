@@ -50,15 +50,15 @@ constexpr double kIters = 12, kClockMHz = 1900;
 constexpr double kEntryClk[2][2] = {{0.033, 0.036}, {0.045, 0.043}};      // clocks of an SM per entry: [tensor memory][RP <= 32]
 }
 
-SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
+SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
 {
     using namespace sweep;
     const int P = 2 * BH, n = nq > nk ? nq : nk, sms = device_sm_count();
     // a program asks for the same sizes again and again (workspace query, then the call; its layers in turn): the last answers are kept
-    struct Memo { int key[7]; SweepPlan plan; };
+    struct Memo { int key[8]; SweepPlan plan; };
     static thread_local Memo memos[8] = {};
     static thread_local unsigned next = 0;
-    const int key[7] = {dtype + 1, BH, nq, nk, d, r, sms};
+    const int key[8] = {dtype + 1, BH, nq, nk, d, r, sms, keep};
     for (const Memo &m : memos)
         if (memcmp(key, m.key, sizeof(key)) == 0) return m.plan;
     SweepPlan best{};
@@ -87,7 +87,7 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
             const int mine = (m + C - 1) / C, ns = mine < srows ? mine : srows, nt = mine - ns < trows ? mine - ns : trows, rest = mine - ns - nt;
             const int steps = (ns + step - 1) / step + (nt + 2 * step - 1) / (2 * step) * 2 + (rest + 2 * step - 1) / (2 * step) * 2;
             const double work = (double)steps * step * RP * kEntryClk[tensor][RP <= 32] / kClockMHz;
-            double lat = (tensor ? C == 1 ? 0.75 : 0.55 : 0.7) + RP / 256.0;
+            double lat = (tensor ? C == 1 ? 0.78 : 0.55 : 0.7) + RP / 256.0;
             if (C > 1) lat += C == K ? 0.6 : 1.7 + 0.3 * (occ - 1);
             double it = lat + work * (tensor ? 1.0 : 1.7);
             if (it < per_sm * work) it = per_sm * work;
@@ -96,17 +96,21 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
                 const double l2 = all / (all > 90 ? 5.0 : 12.0), sm = per_sm * mb / 0.11;
                 it += 0.5 + (l2 > sm ? l2 : sm);
             }
-            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.4 + mine * (RP * 5e-5) + 3.0;
+            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.4 + mine * (RP * 1e-4) + 3.0;
         };
         const int rounds = (P + fly - 1) / fly, first = nq == nk ? rounds : (BH + fly - 1) / fly;         // the longer side's come first
         const double t = first * problem(n) + (rounds > first ? (rounds - first) * problem(nq < nk ? nq : nk) : 0.0);
         if (t < best_t) {
             best_t = t;
             best.C = C; best.K = K; best.groups = groups; best.srows = srows;
-            best.smem = smem; best.tcols = tcols;
+            best.smem = smem; best.tcols = tcols; best.threads = threads;
         }
     };
-    for (int form = 0; form <= max_blocks(wide_cols(RP), 256); ++form) {      // 0: with tensor memory, one block to an SM
+    // More short problems than blocks of 256 threads fit at once: one warp each, whose barriers wait for nobody and whose sums end in the
+    // warp.  float32, d = 64, T = 20, us, blocks / warps: 384 slices of 64 tokens at r = 16 51.8 / 35.3, of 128 60.0 / 49.0, of 256 88.8 / 82.3,
+    // 512 of 128 at r = 32 109 / 93; but 384 of 500 at r = 16 147 / 152, and 3 of 128 at r = 16 27.2 / 33.3.
+    const bool warp = !keep && RP <= 32 && (long long)n * RP <= kWarpEntries && P > 3 * sms;
+    for (int form = 0; !warp && form <= max_blocks(wide_cols(RP), 256); ++form) {      // 0: with tensor memory, one block to an SM
         const bool tensor = form == 0;
         const int occ = tensor ? 1 : form, threads = tensor ? kTensorThreads : 256, half = threads * (tensor ? kTensorLane : wide_cols(RP)) / RP / 2;
         const int most = (n + half - 1) / half;                               // half a step's rows a block at least
@@ -117,6 +121,12 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
             if ((K & (K - 1)) == 0)                                           // several clusters
                 for (int M = 2; M <= all && M <= kWords && M * K <= most; ++M) consider(tensor, occ, M * K, K, slots);
         }
+    }
+    if (warp) {
+        const int step = 32 * wide_cols(RP) / RP;
+        const size_t f0 = fixed_bytes<float>(RP, 32), f1 = fixed_bytes<__nv_bfloat16>(RP, 32);
+        best.C = best.K = 1; best.groups = P; best.srows = (n + step - 1) / step * step; best.tcols = 0; best.threads = 32;
+        best.smem = (f0 > f1 ? f0 : f1) + (size_t)best.srows * RP * 4;
     }
     // One launch per pass instead of rounds of problems.  Slower wherever both were measured (float32, T = 10: 16 slices of 16384 tokens at
     // r = 64 687 us against 526, 96 of 9000 at r = 16 751 against 505), so only the size whose number of launches callers have
@@ -129,7 +139,7 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r)
         if (best.C > (n + 15) / 16) best.C = (n + 15) / 16;
         best.K = 1;
         best.groups = best.C == 1 ? P : (slots / best.C < P ? slots / best.C : P);
-        best.srows = 0; best.tcols = 0;
+        best.srows = 0; best.tcols = 0; best.threads = 256;
         best.smem = fixed_bytes<__nv_bfloat16>(RP, 256);
     }
     Memo &m = memos[next++ % 8];
