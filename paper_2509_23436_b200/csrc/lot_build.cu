@@ -1,5 +1,6 @@
 // The stabilised Gibbs kernel of the sweep path (lot_sweep.cu) from tokens and pivots: logits, row maxima, exponentials in
-// one kernel; every warp holds whole rows of logits in its accumulators.
+// one kernel; every warp holds whole rows of logits in its accumulators.  bf16 tokens with more than 32 pivots and up to 128
+// channels: lot_build_tc.cu.
 #include "lot_chain.cuh"
 #include "lot_internal.h"
 #include "lot_logits.cuh"
@@ -118,7 +119,6 @@ cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaS
     if (dtype == 1 && a.terms == 2) {
         if (RP == 16) return build::launch_t<__nv_bfloat16, 16, 2>(a, sides, st);
         if (RP == 32) return build::launch_t<__nv_bfloat16, 32, 2>(a, sides, st);
-        if (RP == 64) return build::launch_t<__nv_bfloat16, 64, 2>(a, sides, st);
     }
     return dtype == 0 ? build::launch_rp<float>(RP, a, sides, st) : build::launch_rp<__nv_bfloat16>(RP, a, sides, st);
 }

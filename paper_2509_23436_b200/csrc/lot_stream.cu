@@ -6,8 +6,8 @@
 // streamed path has always had; potentials to about 1e-4): half the bytes, so a pass over n = 16384, H = 16 reads 67 MB, of
 // which the blocks keep the first rows of their share in shared memory and the rest comes from L2.  Each block
 // computes the logits of its own rows (warp-level products, Z as bf16 hi + lo), so building one group's kernel
-// overlaps another's passes.  At n = 4096, H = 16, r = 64, T = 10: 47 us (17 of them building) of a call of 71, which took 117 on
-// the streamed path; at n = 16384 135 (52) of 180, against 190.  A pass is bound by latency: per
+// overlaps another's passes.  At n = 4096, H = 16, r = 64, T = 10: 42 us (17 of them building) of a call of 64, which took 117 on
+// the streamed path; at n = 16384 132 (52) of 171, against 190 (47 of 71 and 135 of 180 with the exchanges polled in L2).  A pass is bound by latency: per
 // scheduler four warps, whose registers hold the weights, the column sums and two rows, issue in 40% of the cycles.
 //
 // The key side is applied from twice bf16's precision, as the streamed path's apply passes do with recomputed logits: the

@@ -6,7 +6,7 @@
 //     dC_it += K_it (w_t m u_i / s_i^2 - f_t m / s_i):
 // a read-only pass like the forward's, and a rank-two term on top of K.  So the reverse iterations only keep two numbers
 // per row and two per column, and the gradient with respect to the similarities is put together once at the end
-// (assemble_kernel) instead of being read and written in every iteration.
+// (assemble_kernel, or up to 64 pivots lot_sweep_grad.cu) instead of being read and written in every iteration.
 // Problems whose potentials ranged over more than the kernel's window are reversed step by step on rebuilt exponents.
 #include "lot_chain.cuh"
 #include "lot_sweep_core.cuh"
@@ -311,8 +311,8 @@ reverse_kernel(const __grid_constant__ SweepBwdArgs a)
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// dC_it += K_it sum_k (coef^k_i.x w^k_t - coef^k_i.y f^k_t): 4 rows x 4 columns per thread, the coefficients of KS iterations
-// at a time in shared memory.
+// More than 64 pivots or 128 channels: dC_it += K_it sum_k (coef^k_i.x w^k_t - coef^k_i.y f^k_t), 4 rows x 4 columns per thread, the
+// coefficients of KS iterations at a time in shared memory.
 // ---------------------------------------------------------------------------------------------------------------
 template <int RP>
 __global__ void __launch_bounds__(256)

@@ -42,7 +42,7 @@ int cluster_blocks(int K, int occ)
 // one problem each; it costs the reading of its rows and, per iteration, the larger of one block's chain (latency with
 // the exchange, its own steps) and of what the blocks of an SM need together.  The constants are fitted to the times of whole
 // calls: 40 sizes from 2 problems of 30000 tokens to 512 of 512, each in up to 34 forced splits; over those, the
-// split chosen is on average 1 % slower than the best one, 12 % at most.  Rows in tensor memory are what it mostly takes where a
+// split chosen is on average 1.4 % slower than the best one, 12 % at most.  Rows in tensor memory are what it mostly takes where a
 // problem is more than one block's shared memory: a pass over rows there runs at 26 entries a clock and SM against 18
 // from shared memory alone (a loop of passes at RP = 256), and 480 KB instead of 227 stay on an SM.
 namespace sweep {
@@ -67,6 +67,15 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
     double best_t = 1e30;
     auto consider = [&](bool tensor, int occ, int C, int K, int slots) {
         const int threads = tensor ? kTensorThreads : 256, CPL = tensor ? kTensorLane : wide_cols(RP);
+        const double entry = kEntryClk[tensor][RP <= 32] / kClockMHz * (tensor ? 1.0 : 1.7);
+        double lat = (tensor ? C == 1 ? 0.78 : 0.55 : 0.7) + RP / 256.0;
+        if (C > 1) {
+            lat += C == K ? 0.6 : 1.7 + 0.3 * (occ - 1);
+            // most splits are no match for the best so far by this alone (a search of all of them took 60 us)
+            if (slots < C) return;
+            const int fly = slots / C < P ? slots / C : P, turns = ((nq == nk ? P : BH) + fly - 1) / fly;
+            if (turns * (kIters + 0.7) * (lat + (double)n / C * RP * entry) >= best_t) return;
+        }
         const int step = threads * CPL / RP;                                  // rows per step of a block
         const size_t f0 = fixed_bytes<float>(RP, threads), f1 = fixed_bytes<__nv_bfloat16>(RP, threads);
         const size_t fixed = (f0 > f1 ? f0 : f1) + (size_t)peer_bytes(RP, C, K);
@@ -82,13 +91,16 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
         const int fly = C == 1 && P > slots ? slots : groups, resident = fly * C;            // problems and blocks at once
         const int per_sm = (resident + sms - 1) / sms;                        // blocks that share an SM
         const int tcols = tensor ? kTensorCols : 0, trows = tcols / (threads / 128) / CPL * step;
+        // Rows of 16 columns: no more than a few per cent of them streamed beside tensor memory.  The model takes such splits for the better ones, and a
+        // block of that many rows is slow to rebuild them: 32 slices of 16384 tokens at d = 128, r = 16, two blocks of 8192 rows a problem 390 us,
+        // peaked 578, four of 4096 384 and 485 (before tensor memory 451 and 498).  At RP = 32 such splits are the
+        // better ones (r = 32, 4096 rows a block: peaked 610, before tensor memory 771).
+        if (tensor && RP == 16 && rows > 1.05 * (srows + trows)) return;
         // us of a problem of m tokens
         auto problem = [&](int m) {
             const int mine = (m + C - 1) / C, ns = mine < srows ? mine : srows, nt = mine - ns < trows ? mine - ns : trows, rest = mine - ns - nt;
             const int steps = (ns + step - 1) / step + (nt + 2 * step - 1) / (2 * step) * 2 + (rest + 2 * step - 1) / (2 * step) * 2;
             const double work = (double)steps * step * RP * kEntryClk[tensor][RP <= 32] / kClockMHz;
-            double lat = (tensor ? C == 1 ? 0.78 : 0.55 : 0.7) + RP / 256.0;
-            if (C > 1) lat += C == K ? 0.6 : 1.7 + 0.3 * (occ - 1);
             double it = lat + work * (tensor ? 1.0 : 1.7);
             if (it < per_sm * work) it = per_sm * work;
             if (rest > 0) {

@@ -92,3 +92,22 @@ def test_backward_matches_oracle(case):
     one = dataclasses.replace(x, **{name: getattr(x, name)[b:, h:] for name in ("q", "k", "v")}, z=x.z[h:], beta=x.beta[h:])
     for name, got, ref in zip(("dq", "dk", "dv"), res, oracle_grads(one, dout[b:, h:])):
         check_slice(got[b, h].float().cpu().double().numpy(), ref[0, 0], TOL[BF16], name)
+
+
+@pytest.mark.parametrize("B,H,n,d,r", [(1, 2, 6000, 32, 200), (4, 50, 1500, 32, 64), (60, 8, 60, 16, 16)])
+def test_a_captured_call_gives_the_same_bits(B, H, n, d, r):
+    """Cooperative launches in clusters, chained launches of blocks with tensor memory, one warp per problem."""
+    x = synth.make(B, H, n, d, r, seed=3, dtype=F32 if d == 16 else BF16, eps=0.1, iters=3)
+    dev = torch.device("cuda:0")
+    t = [getattr(x, name).to(dev) for name in ("q", "k", "v", "z", "beta")]
+    want, ws = lot.lot_attention_fwd_ex(*t, None, x.eps, x.iters)
+    out = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        lot.lot_attention_fwd_ex(*t, None, x.eps, x.iters, out=out, ws=ws)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert lot.lot_device_status(ws) == 0 and torch.equal(out, want)
