@@ -461,7 +461,7 @@ def run_backward(args):
             "vs_baseline": None, "dtype": ARITH[0][tdt], "data": "synthetic",
             "config": config_of(x, {"l2": "flushed between timed steps (512 MiB overwrite)",
                                     "op": "backward (forward recomputed inside: on the stored kernel for bf16 tensors, on materialised similarities for float32)"}),
-            "clocks": clocks, "gpu_launches": (2 * x.iters + 15 if tdt == "float32" else 13) * args.steps,
+            "clocks": clocks, "gpu_launches": (2 * x.iters + 15 if tdt == "float32" else 9 if r <= 64 and d <= 128 else 12) * args.steps,
             "forward_ms_per_step": sum(tf) / len(tf), "backward_over_forward": ms / (sum(tf) / len(tf)),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": None, "peak_source": peak_src, "algorithmic_bytes": abytes,
