@@ -614,9 +614,12 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
         }
     }
     mx = cls_block<true>(mx, red);
+    // A maximum of -infinity: no keys here, keys that all score it, or keys that score NaN, which the maximum passes over.  Taken
+    // relative to 0 they come out as nothing, nothing and NaN.
+    const float ref = mx > neg_inf() ? mx : 0.f;
     float den = 0.f;
     for (int j = tid; j < kv; j += 256) {
-        const float e = __expf(sc[j] - mx);
+        const float e = __expf(sc[j] - ref);
         sc[j] = e;
         den += e;
     }
@@ -653,13 +656,13 @@ cls_row_kernel(const T *__restrict__ q, const T *__restrict__ k, const T *__rest
             float m[8], top = neg_inf(), sum = 0.f, sden = 0.f;
 #pragma unroll
             for (int o = 0; o < 8; ++o) {
-                m[o] = o < blocks ? peer_float(base, 256, o) : neg_inf();       // a block without keys: -infinity, nothing of it below
+                m[o] = o < blocks ? peer_float(base, 256, o) : neg_inf();
                 top = fmaxf(top, m[o]);
             }
 #pragma unroll
             for (int o = 0; o < 8; ++o)
-                if (o < blocks && m[o] > neg_inf()) {
-                    const float f = __expf(m[o] - top);
+                if (o < blocks) {
+                    const float f = m[o] > neg_inf() ? __expf(m[o] - top) : 1.f;       // its sums are 0 or NaN
                     sum = fmaf(f, peer_float(base, tid, o), sum);
                     sden = fmaf(f, peer_float(base, 257, o), sden);
                 }
