@@ -116,6 +116,7 @@ template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool TENSOR, boo
 static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t st)
 {
     auto kern = sweep_kernel<T, RP, CPL, THREADS, GROUP, TENSOR, KEEP>;
+    if (TENSOR && P.smem < kAloneSmem) return cudaErrorInvalidConfiguration;
     static std::mutex mu;
     static bool attr_set[64] = {};
     int dev = 0;

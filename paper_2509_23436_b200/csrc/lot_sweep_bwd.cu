@@ -428,6 +428,7 @@ template <int RP, bool GROUP, bool TENSOR> static cudaError_t reverse_g(const Sw
 {
     constexpr int THREADS = TENSOR ? kTensorThreads : 256;
     auto kern = reverse_kernel<RP, TENSOR ? kTensorLane : wide_cols(RP), THREADS, GROUP, TENSOR>;
+    if (TENSOR && P.smem < kAloneSmem) return cudaErrorInvalidConfiguration;
     cudaError_t e = allow_smem(kern, P.smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(P.groups * P.C));

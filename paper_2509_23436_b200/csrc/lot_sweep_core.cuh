@@ -70,9 +70,13 @@ __host__ __device__ constexpr int wide_cols(int RP) { return RP <= 32 ? 8 : 16; 
 // blocks per SM that the registers allow (80 a thread, 128 with sixteen columns per lane)
 __host__ __device__ constexpr int max_blocks(int cpl, int threads) { return (cpl == 16 ? 512 : 768) / threads; }
 
-// Blocks that keep rows in tensor memory too are alone on their SM (the runtime places no two blocks of such a kernel, launched
-// together, on one): twice the threads, sixteen columns a lane whatever RP is, all of the SM's columns.
+// Blocks that keep rows in tensor memory too: twice the threads, sixteen columns a lane whatever RP is, all of the SM's columns.  Two of
+// them on one SM would wait for each other, one in tcgen05.alloc, which no limit ends, the other for its column sums.  So such a
+// block takes more than half of the SM's shared memory, whatever it needs (plans and launches hold to it).  Registers would not do: 512
+// threads have all of them only as long as the compiler uses more than 64 a thread.
 constexpr int kTensorThreads = 512, kTensorCols = 512, kTensorLane = 16;
+constexpr size_t kAloneSmem = kSmemPerSM / 2;
+static_assert(2 * (kAloneSmem + kSmPerBlockReserve) > (size_t)kSmemPerSM && kAloneSmem <= (size_t)kSmemPerBlock, "one such block an SM");
 
 // shared memory: [kernel rows | gref | work area (staged pivots, or the column reduction) | refs | weights, targets | flags,
 // barriers | columns from the blocks of the cluster]

@@ -81,7 +81,8 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
         const size_t fixed = (f0 > f1 ? f0 : f1) + (size_t)peer_bytes(RP, C, K);
         const int cap = (int)((block_smem(occ) - fixed) / ((size_t)RP * 4)) / step * step;
         const int rows = (n + C - 1) / C, up = (rows + step - 1) / step * step, srows = up < cap ? up : cap;
-        const size_t smem = fixed + (size_t)srows * RP * 4;
+        size_t smem = fixed + (size_t)srows * RP * 4;
+        if (tensor && smem < kAloneSmem) smem = kAloneSmem;
         int fit = (int)((size_t)kSmemPerSM / (smem + kSmPerBlockReserve));
         if (fit > occ) fit = occ;
         if (C == 1) slots = sms * fit;
