@@ -162,7 +162,7 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *   0  the general path: the Gibbs kernel of both sides in float32, all Sinkhorn passes in one kernel that keeps what it
  *      can of it in shared and tensor memory (one launch per pass for float32 tensors whose kernel is 128 MiB), two apply
  *      kernels.  Blocks of one problem wait for one another: where a problem is shared by several, the kernel is
- *      launched cooperatively, in clusters.
+ *      launched in clusters, and cooperatively where a problem is more than one cluster's.
  *   1  the streamed tensor-core path (bf16 tensors, d = 64, r <= 64): one persistent kernel for all
  *      passes, launched cooperatively (it needs as many free SMs as it has thread blocks, at most
  *      one per SM), plus a small pivot preparation.  With 32 < r <= 64 its first pass keeps the
@@ -173,8 +173,8 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  *      represent (potentials spread over more than 96 binades, a column mass below 2^-80) is
  *      recomputed by the streamed kernels, which are launched behind it and return at once otherwise
  *      (device flag LOT_DEV_RECOMPUTED).  Nowhere the fastest, so only taken by lot_debug_hook what = 4.
- *   4  the long path (same tensors, 16 < r <= 64, three iterations and more): one launch (cooperative, in clusters
- *      of thread blocks, or plain where a block has a problem to itself) builds that bf16 kernel and runs all passes
+ *   4  the long path (same tensors, 16 < r <= 64, three iterations and more): one launch (in clusters of
+ *      thread blocks, cooperative where a problem is more than one cluster's) builds that bf16 kernel and runs all passes
  *      on it, a group of thread blocks per problem keeping what it can of it in shared memory; two apply kernels.
  *      Taken for r > 32 up to 300000 rows B H n and for n <= 1200, for r <= 32 at about one slice per SM of up to 1792
  *      tokens; path 0 takes r <= 16 and the other problems of r <= 32 up to 160000 rows or n <= 1200.  A call whose

@@ -5,7 +5,7 @@
 // blocks of the next kernel took a fifth of the sweep kernel's speed.  Hides most of the 2-3 us between dependent launches.
 // Loads of what a predecessor wrote must be plain ones: the compiler moves __ldg and loads through const __restrict__
 // pointers above the wait.
-// (Kernels whose blocks wait for one another are launched cooperatively instead and start the ordinary way.)
+// (Kernels whose blocks wait for blocks of other clusters are launched cooperatively instead and start the ordinary way.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -35,24 +35,31 @@ __device__ __forceinline__ float chain_ld(const float *p)
     return v;
 }
 
-// ... in clusters of K blocks
+// A launch in clusters of K blocks with one more attribute, or none (attr.id == cudaLaunchAttributeIgnore).
 template <typename... P, typename... A>
-inline cudaError_t chain_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, int K, cudaStream_t st, A... args)
+inline cudaError_t launch_with(cudaLaunchAttribute attr, void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, int K, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[2] = {};
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2] = {attr, {}};
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = (unsigned)K;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = K > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... A>
+inline cudaError_t chain_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, int K, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    return launch_with(at, kern, grid, threads, smem, K, st, args...);
 }
 template <typename... P, typename... A>
 inline cudaError_t chain_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args)
@@ -60,24 +67,24 @@ inline cudaError_t chain_launch(void (*kern)(P...), dim3 grid, unsigned threads,
     return chain_launch(kern, grid, threads, smem, 1, st, args...);
 }
 
-// A kernel whose blocks wait for one another: all of them run at once, in clusters of K.
+// The ordinary start, in clusters of K.
+template <typename... P, typename... A>
+inline cudaError_t cluster_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, int K, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeIgnore;
+    return launch_with(at, kern, grid, threads, smem, K, st, args...);
+}
+
+// A kernel whose blocks wait for one another across clusters: all of them run at once.  Blocks that wait only within their cluster do not need
+// it, the hardware starts a cluster whole; a cooperative launch starts the ordinary way, and ncu gives no time for one in clusters.
 template <typename... P, typename... A>
 inline cudaError_t group_launch(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, int K, cudaStream_t st, A... args)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2] = {};
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = (unsigned)K;
-    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = K > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    return launch_with(at, kern, grid, threads, smem, K, st, args...);
 }
 
 } // namespace lot

@@ -687,12 +687,7 @@ cudaError_t stream_attention(const void *q, const void *k, const void *v, const 
     auto kern = L.C > 1 ? stream_kernel<true> : stream_kernel<false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
     if (e != cudaSuccess) return e;
-    if (L.C > 1) {
-        e = group_launch(kern, grid, kThreads, smem, L.K, st, a);
-    } else {
-        kern<<<grid, kThreads, smem, st>>>(a);
-        e = cudaGetLastError();
-    }
+    e = L.C == L.K ? cluster_launch(kern, grid, kThreads, smem, L.K, st, a) : group_launch(kern, grid, kThreads, smem, L.K, st, a);
     if (e != cudaSuccess) return e;
     return stored_apply(a.kt, L.npad, a.G, beta, key_len, a.decision, v, out, low_half, reinterpret_cast<float *>(w + L.wpart), a.status, B, H, n, r, st);
 }

@@ -130,9 +130,7 @@ static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t
         }
     }
     const dim3 grid((unsigned)(P.groups * P.C));
-    if (!GROUP) {
-        return chain_launch(kern, grid, THREADS, P.smem, st, a);
-    }
+    if (P.C == P.K) return chain_launch(kern, grid, THREADS, P.smem, P.K, st, a);
     return group_launch(kern, grid, THREADS, P.smem, P.K, st, a);
 }
 
