@@ -160,9 +160,8 @@ LOT_API size_t lot_workspace_bytes(int B, int H, int n, int d, int r, int dtype)
  * lot_path -- which implementation one lot_attention_fwd_ex call with these parameters takes (host
  * arithmetic only):
  *   0  the general path: the Gibbs kernel of both sides in float32, all Sinkhorn passes in one kernel that keeps what it
- *      can of it in shared and tensor memory (one launch per pass for float32 tensors whose kernel is 128 MiB), two apply
- *      kernels.  Blocks of one problem wait for one another: where a problem is shared by several, the kernel is
- *      launched in clusters, and cooperatively where a problem is more than one cluster's.
+ *      can of it in shared and tensor memory, two apply kernels.  Blocks of one problem wait for one another: where a
+ *      problem is shared by several, the kernel is launched in clusters, and cooperatively where it is more than one cluster's.
  *   1  the streamed tensor-core path (bf16 tensors, d = 64, r <= 64): one persistent kernel for all
  *      passes, launched cooperatively (it needs as many free SMs as it has thread blocks, at most
  *      one per SM), plus a small pivot preparation.  With 32 < r <= 64 its first pass keeps the

@@ -66,7 +66,6 @@ SinkLayout sink_layout(int nprob, int n, int r, size_t base, size_t lt)
 // the apply stage, exchange words of the sweep) is one region cleared at the start of every call.
 struct ForwardLayout {
     SweepPlan plan;
-    int rounds;              // problems a group works through per launch
     size_t counter, xbuf, head_end, w[2], gref[2], inv[2], kt[2], scores, wpart, Wp, total;
     int achunks, arows;
 };
@@ -77,7 +76,6 @@ ForwardLayout forward_layout(int B, int H, int nq, int nk, int d, int r, int dty
     const int BH = B * H, n[2] = {nq, nk};
     L.plan = sweep_plan(dtype, BH > 0 ? BH : 1, nq > 0 ? nq : 1, nk > 0 ? nk : 1, d, r);
     const int RP = L.plan.RP;
-    L.rounds = (2 * BH + L.plan.groups - 1) / L.plan.groups;
     size_t o = 256;                                                   // status word at 0
     L.counter = o; o += up256((size_t)((r + 63) / 64) * ((d + 63) / 64) * BH * 4);
     L.xbuf = o;
@@ -381,22 +379,10 @@ cudaError_t run_forward(const ForwardLayout &L, const ForwardCall &f, bool first
     a.B = B; a.H = H; a.d = d; a.r = r; a.n[0] = nq; a.n[1] = nk; a.skip = skip; a.terms = terms;
     a.C = L.plan.C; a.K = L.plan.K; a.groups = L.plan.groups; a.srows = L.plan.srows; a.tcols = L.plan.tcols;
     a.scale = 1.4426950408889634 / (double)f.eps; a.eps_ln2 = (double)f.eps * 0.6931471805599453;
-    a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0;
+    a.iters = iters;
     cudaError_t e;
-    if (!L.plan.steps) {
-        if ((e = launch_build(L.plan.RP, a, dtype, 3, s)) != cudaSuccess) return e;
-        if ((e = launch_sweep(L.plan, a, dtype, s)) != cudaSuccess) return e;
-    } else {
-        // one launch per side and pass: 4 sequence numbers per pass and problem of a group cover its exchanges
-        if ((e = launch_build(L.plan.RP, a, dtype, 2, s)) != cudaSuccess) return e;
-        a.head_words = 0;
-        if ((e = launch_build(L.plan.RP, a, dtype, 1, s)) != cudaSuccess) return e;
-        for (int it = 0; it <= iters; ++it) {
-            a.it0 = it; a.it1 = it < iters ? it + 1 : it; a.first = it == 0; a.close = it == iters;
-            a.seq0 = 4u * (unsigned)it * (unsigned)L.rounds;
-            if ((e = launch_sweep(L.plan, a, dtype, s)) != cudaSuccess) return e;
-        }
-    }
+    if ((e = launch_build(L.plan.RP, a, dtype, s)) != cudaSuccess) return e;
+    if ((e = launch_sweep(L.plan, a, dtype, s)) != cudaSuccess) return e;
     ap.beta = f.beta; ap.key_len = f.key_len; ap.mass2 = f.mass_k; ap.v = f.v; ap.out = f.out;
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
     ap.B = B; ap.H = H; ap.nq = nq; ap.nk = nk; ap.d = d; ap.r = r; ap.RP = L.plan.RP; ap.skip = skip; ap.terms = terms;
@@ -442,9 +428,9 @@ cudaError_t run_backward(const BwdSweepLayout &L, const void *q, const void *k, 
     a.B = B; a.H = H; a.d = d; a.r = r;
     a.C = L.plan.C; a.K = L.plan.K; a.groups = L.plan.groups; a.srows = L.plan.srows; a.tcols = L.plan.tcols;
     a.scale = 1.4426950408889634 / (double)eps; a.eps_ln2 = (double)eps * 0.6931471805599453;
-    a.it0 = 0; a.it1 = iters; a.first = 1; a.close = 1; a.seq0 = 0; a.terms = 3;
+    a.iters = iters; a.terms = 3;
     // ---- the forward, keeping the weights of every iteration
-    if ((e = launch_build(RP, a, dt, 3, st)) != cudaSuccess) return e;
+    if ((e = launch_build(RP, a, dt, st)) != cudaSuccess) return e;
     if ((e = launch_sweep(L.plan, a, dt, st)) != cudaSuccess) return e;
     ap.beta = beta; ap.key_len = key_len; ap.v = v;
     ap.wpart = at<float>(ws, L.wpart); ap.Wp = at<float>(ws, L.Wp); ap.counter = at<unsigned>(ws, L.counter);
@@ -640,7 +626,7 @@ int lot_launch_count(int dtype, int B, int H, int n, int d, int r, int iters)
     if (path == kPathLong) return 3;
     if (B < 1 || n < 1) return 0;
     const Parts P = forward_parts(B, H, n, n, d, r, dtype, false);
-    return sweep_plan(dtype, B * H, n, n, d, r).steps ? 2 + iters + 1 + 2 : 4 * ((B + P.rows - 1) / P.rows) * ((H + P.heads - 1) / P.heads);
+    return 4 * ((B + P.rows - 1) / P.rows) * ((H + P.heads - 1) / P.heads);
 }
 
 int lot_debug_hook(int what, long long value)

@@ -75,7 +75,7 @@ build_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k)
 }
 
 template <typename T, int RP, int TERMS = 3>
-static cudaError_t launch_t(const SweepArgs &a, int sides, cudaStream_t st)
+static cudaError_t launch_t(const SweepArgs &a, cudaStream_t st)
 {
     typedef Shape<T, RP> Sh;
     auto kern = build_kernel<T, RP, TERMS>;
@@ -93,34 +93,33 @@ static cudaError_t launch_t(const SweepArgs &a, int sides, cudaStream_t st)
         }
     }
     constexpr int rows = kWarps * Sh::ROWS;
-    const int tq = sides & 1 ? (a.n[0] + rows - 1) / rows : 0, tk = sides & 2 ? (a.n[1] + rows - 1) / rows : 0;
+    const int tq = (a.n[0] + rows - 1) / rows, tk = (a.n[1] + rows - 1) / rows;
     kern<<<(unsigned)((tq + tk) * a.B * a.H), kThreads, smem, st>>>(a, tq, tk);
     return cudaGetLastError();
 }
 
 template <typename T>
-static cudaError_t launch_rp(int RP, const SweepArgs &a, int sides, cudaStream_t st)
+static cudaError_t launch_rp(int RP, const SweepArgs &a, cudaStream_t st)
 {
     switch (RP) {
-    case 16: return launch_t<T, 16>(a, sides, st);
-    case 32: return launch_t<T, 32>(a, sides, st);
-    case 64: return launch_t<T, 64>(a, sides, st);
-    case 128: return launch_t<T, 128>(a, sides, st);
-    default: return launch_t<T, 256>(a, sides, st);
+    case 16: return launch_t<T, 16>(a, st);
+    case 32: return launch_t<T, 32>(a, st);
+    case 64: return launch_t<T, 64>(a, st);
+    case 128: return launch_t<T, 128>(a, st);
+    default: return launch_t<T, 256>(a, st);
     }
 }
 
 } // namespace build
 
-// sides: bit 0 the queries, bit 1 the keys
-cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st)
+cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, cudaStream_t st)
 {
-    if (dtype == 1 && build_tc_supported(RP, a.d)) return launch_build_tc(RP, a, sides, st);
+    if (dtype == 1 && build_tc_supported(RP, a.d)) return launch_build_tc(RP, a, st);
     if (dtype == 1 && a.terms == 2) {
-        if (RP == 16) return build::launch_t<__nv_bfloat16, 16, 2>(a, sides, st);
-        if (RP == 32) return build::launch_t<__nv_bfloat16, 32, 2>(a, sides, st);
+        if (RP == 16) return build::launch_t<__nv_bfloat16, 16, 2>(a, st);
+        if (RP == 32) return build::launch_t<__nv_bfloat16, 32, 2>(a, st);
     }
-    return dtype == 0 ? build::launch_rp<float>(RP, a, sides, st) : build::launch_rp<__nv_bfloat16>(RP, a, sides, st);
+    return dtype == 0 ? build::launch_rp<float>(RP, a, st) : build::launch_rp<__nv_bfloat16>(RP, a, st);
 }
 
 } // namespace lot

@@ -233,7 +233,7 @@ build_tc_kernel(const __grid_constant__ SweepArgs a, int tiles_q, int tiles_k, i
 }
 
 template <int RP>
-static cudaError_t launch_t(const SweepArgs &a, int sides, cudaStream_t st)
+static cudaError_t launch_t(const SweepArgs &a, cudaStream_t st)
 {
     auto kern = build_tc_kernel<RP>;
     const Layout L = layout(RP, a.d, a.terms);
@@ -251,7 +251,7 @@ static cudaError_t launch_t(const SweepArgs &a, int sides, cudaStream_t st)
     }
     // blocks an SM holds (registers, accumulators, shared memory), shared evenly by the heads
     const int fit = RP < 256 && 2 * (L.total + 1024) <= 228 * 1024 ? 2 : 1, slots = fit * device_sm_count();
-    const int tq = sides & 1 ? (a.n[0] - a.skip + kTile - 1) / kTile : 0, tk = sides & 2 ? (a.n[1] - a.skip + kTile - 1) / kTile : 0;
+    const int tq = (a.n[0] - a.skip + kTile - 1) / kTile, tk = (a.n[1] - a.skip + kTile - 1) / kTile;
     const int tiles = a.B * (tq + tk), share = slots / a.H < 1 ? 1 : slots / a.H;
     const int per_head = tiles < share ? (tiles < 1 ? 1 : tiles) : share;
     kern<<<(unsigned)(per_head * a.H), kThreads, L.total, st>>>(a, tq, tk, per_head);
@@ -262,10 +262,10 @@ static cudaError_t launch_t(const SweepArgs &a, int sides, cudaStream_t st)
 
 bool build_tc_supported(int RP, int d) { return RP >= 64 && d <= 128; }
 
-cudaError_t launch_build_tc(int RP, const SweepArgs &a, int sides, cudaStream_t st)
+cudaError_t launch_build_tc(int RP, const SweepArgs &a, cudaStream_t st)
 {
     using namespace build_tc;
-    return RP == 64 ? launch_t<64>(a, sides, st) : RP == 128 ? launch_t<128>(a, sides, st) : launch_t<256>(a, sides, st);
+    return RP == 64 ? launch_t<64>(a, st) : RP == 128 ? launch_t<128>(a, st) : launch_t<256>(a, st);
 }
 
 } // namespace lot

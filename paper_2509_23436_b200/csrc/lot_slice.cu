@@ -219,7 +219,7 @@ slice_forward_kernel(const __grid_constant__ SliceParams P)
             const float tgt = S.tgt[tid < RP ? tid : 0];
             u64 w[CPL / 2];
             load_weights<RP, CPL>(L, w);
-            for (; it < a.it1; ++it) {
+            for (; it < a.iters; ++it) {
                 bad = iterate<RP, CPL, kThreads, false, false>(a, S, R, L, w, tgt, 0, 0, seq, wold, wnew);
                 if (bad) break;
             }
@@ -382,7 +382,7 @@ cudaError_t slice_attention(const void *q, const void *k, const void *v, const f
     P.s.x[0] = q; P.s.x[1] = k; P.s.z = z; P.s.beta = beta; P.s.key_len = key_len;
     P.s.g_out[0] = g1_out; P.s.g_out[1] = g2_out; P.s.status = status;
     P.s.B = B; P.s.H = H; P.s.d = slice::kD; P.s.r = r; P.s.n[0] = P.s.n[1] = n;
-    P.s.C = 1; P.s.groups = 2 * B * H; P.s.it1 = iters; P.s.first = 1;
+    P.s.C = 1; P.s.groups = 2 * B * H; P.s.iters = iters;
     P.s.scale = 1.4426950408889634 / (double)eps;
     P.s.eps_ln2 = (double)eps * 0.6931471805599453;
     P.v = static_cast<const __nv_bfloat16 *>(v);

@@ -31,7 +31,7 @@ __device__ __noinline__ void finish(const SweepArgs *ap, int p, int c)
     Share R;
     const Problem P = locate<RP, CPL, THREADS>(a, p, c, R);
     const int tid = threadIdx.x;
-    if (a.close && P.nv > 0) {
+    if (P.nv > 0) {
         const Lane<RP, CPL> L = make_lane<RP, CPL, THREADS>(S, a.tcols);
         u64 w[CPL / 2], acc[CPL / 2];
         load_weights<RP, CPL>(L, w);
@@ -42,7 +42,7 @@ __device__ __noinline__ void finish(const SweepArgs *ap, int p, int c)
         const float wl = tid < a.r ? S.w[tid] : 0.f;
         a.w[P.side][(size_t)P.slice * RP + tid] = wl;
         a.gref[P.side][(size_t)P.slice * RP + tid] = gl;
-        if (a.close && tid < a.r && a.g_out[P.side] != nullptr)
+        if (tid < a.r && a.g_out[P.side] != nullptr)
             a.g_out[P.side][(size_t)P.slice * a.r + tid] = (float)((gl + log2((double)wl)) * a.eps_ln2);
     }
 }
@@ -68,25 +68,19 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
         __syncthreads();                                     // the previous problem is done with shared memory
         if (tid < RP) {
             double g0 = -(double)kStartLog2;
-            float w0 = tid < r ? kStart : 0.f;
-            if (!a.first) {
-                g0 = a.gref[P.side][(size_t)P.slice * RP + tid];
-                w0 = a.w[P.side][(size_t)P.slice * RP + tid];
-            } else if (tid < r && a.g_in[P.side] != nullptr) {
-                g0 += (double)__ldg(a.g_in[P.side] + (size_t)P.slice * r + tid) * a.scale;
-            }
+            if (tid < r && a.g_in[P.side] != nullptr) g0 += (double)__ldg(a.g_in[P.side] + (size_t)P.slice * r + tid) * a.scale;
             S.gref[tid] = g0;
-            S.w[tid] = w0;
+            S.w[tid] = tid < r ? kStart : 0.f;
             S.tgt[tid] = tid < r ? __ldg(a.beta + P.h * r + tid) * (R.mass ? 1.f : (float)P.nv) : 0.f;
         }
         load_rows<RP, CPL, THREADS>(S, R);
         if constexpr (TENSOR) load_tensor_rows<RP, CPL, THREADS>(S, R, a.tcols);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        if (P.nv <= 0 && tid == 0 && a.first && c == 0) atomicOr(a.status, 2 /* LOT_DEV_EMPTY */);
+        if (P.nv <= 0 && tid == 0 && c == 0) atomicOr(a.status, 2 /* LOT_DEV_EMPTY */);
         __syncthreads();
         float wold = 0.f, wnew = S.w[tid < RP ? tid : 0];
         bool bad = false;
-        int it = a.it0;
+        int it = 0;
         if (P.nv > 0) {
             const Lane<RP, CPL> L = make_lane<RP, CPL, THREADS>(S, a.tcols);
             const float tgt = S.tgt[tid < RP ? tid : 0];
@@ -94,7 +88,7 @@ sweep_kernel(const __grid_constant__ SweepArgs a)
             load_weights<RP, CPL>(L, w);
             float *hp = KEEP && c == 0 && tid < RP ? a.hist + (size_t)p * RP + tid : nullptr;      // thread t's column
             if (KEEP && hp != nullptr) *hp = S.w[tid];
-            for (; it < a.it1; ++it) {
+            for (; it < a.iters; ++it) {
                 bad = iterate<RP, CPL, THREADS, GROUP, TENSOR>(a, S, R, L, w, tgt, group, c, seq, wold, wnew);
                 if (bad) break;
                 if (KEEP && hp != nullptr) {

@@ -1,4 +1,4 @@
-// Sweep path: Sinkhorn iterations in scaling form on a float32 Gibbs kernel, several passes per launch (lot_sweep.cu).
+// Sweep path: Sinkhorn iterations in scaling form on a float32 Gibbs kernel, all passes in one launch (lot_sweep.cu).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,8 +27,8 @@ struct SweepArgs {
     float *w[2];             // [BH][RP] weights of the closing update: plan row i = kt[i][t] w[t] inv[i]
     double *gref[2];         // [BH][RP] reference potentials of kt, base-2 units
     float *g_out[2];         // [BH][r] potentials in natural units or nullptr
-    unsigned long long *xbuf;   // exchange words of the groups (exchange_bytes; zero at the start of the first launch of a call)
-    float *hist;             // backward: [it1 + 1][problems][RP] weights before every iteration and after the last, relative to
+    unsigned long long *xbuf;   // exchange words of the groups (exchange_bytes; zero at the start of a call)
+    float *hist;             // backward: [iters + 1][problems][RP] weights before every iteration and after the last, relative to
                              // the kernel as it is left, or nullptr
     double *hist_g;          // ... and the potentials themselves, of the problems whose kernel was rebuilt
     int *wide;               // ... [problems] 1: the kept weights leave float32's range, use hist_g
@@ -41,9 +41,8 @@ struct SweepArgs {
     int C, K, groups;        // thread blocks per problem, per cluster (1: no clusters), problems in flight
     int srows;               // rows of a block's share that stay in shared memory
     int tcols;               // columns of tensor memory that take the next ones (0: none)
-    int it0, it1;            // iterations this launch runs
+    int iters;
     int terms;               // bf16 tokens: terms a pivot is taken as in the first build (3: exact, 2)
-    int first, close;        // start from the given potentials (else from the state in w, gref) / closing update last
     unsigned seq0;           // exchange sequence number this launch starts from
     double scale;            // log2(e)/eps
     double eps_ln2;
@@ -52,7 +51,6 @@ struct SweepArgs {
 struct SweepPlan {
     int RP, C, K, groups, srows, tcols;
     int threads;             // of a block
-    int steps;               // 1: one launch per iteration (the kernel streams from global memory anyway)
     size_t smem;
 };
 
@@ -67,9 +65,9 @@ int cluster_blocks(int K, int occ);      // blocks that run at once as clusters 
 inline size_t exchange_bytes(int RP, int C, int K, int groups) { return C > K ? (size_t)groups * 2 * (C / K) * RP * 8 : 0; }
 SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep = false);      // keep: for the backward
 constexpr int kWarpEntries = 4096;       // the most entries of a problem that one warp takes by itself
-cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, int sides, cudaStream_t st);
+cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, cudaStream_t st);
 bool build_tc_supported(int RP, int d);  // bf16 tokens on tcgen05 (lot_build_tc.cu)
-cudaError_t launch_build_tc(int RP, const SweepArgs &a, int sides, cudaStream_t st);
+cudaError_t launch_build_tc(int RP, const SweepArgs &a, cudaStream_t st);
 cudaError_t launch_sweep(const SweepPlan &P, const SweepArgs &a, int dtype, cudaStream_t st);
 
 struct SweepApplyArgs {

@@ -885,7 +885,7 @@ __device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, 
         u64 w[CPL / 2];
         load_weights<RP, CPL>(L, w);
         wnew = kStart;
-        for (++it; it < a.it1 && !bad; ++it) {
+        for (++it; it < a.iters && !bad; ++it) {
             bad = iterate<RP, CPL, THREADS, GROUP, TENSOR>(a, S, R, L, w, S.tgt[tid < RP ? tid : 0], group, c, seq, wold, wnew);
             if (keep && !bad) hg[(size_t)(it + 1) * NP * RP] = S.gref[tid] + log2((double)wnew);
         }
@@ -894,7 +894,7 @@ __device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, 
     }
     if (a.hist != nullptr && c == 0) {
         bool wide = false;
-        for (int k = 0; tid < RP && k <= a.it1; ++k) {
+        for (int k = 0; tid < RP && k <= a.iters; ++k) {
             const float v = tid < r ? (float)exp2(hg[(size_t)k * NP * RP] - S.gref[tid]) : 0.f;
             wide = wide || (tid < r && !(v >= kHistLo && v <= kHistHi));
             a.hist[((size_t)k * NP + p) * RP + tid] = v;

@@ -141,20 +141,6 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
         best.C = best.K = 1; best.groups = P; best.srows = (n + step - 1) / step * step; best.tcols = 0; best.threads = 32;
         best.smem = (f0 > f1 ? f0 : f1) + (size_t)best.srows * RP * 4;
     }
-    // One launch per pass instead of rounds of problems.  Slower wherever both were measured (float32, T = 10: 16 slices of 16384 tokens at
-    // r = 64 687 us against 526, 96 of 9000 at r = 16 751 against 505), so only the size whose number of launches callers have
-    // been promised still takes it (lot_launch_count, held by the interface's tests: a kernel of 128 MiB).
-    const double kernel_bytes = (double)BH * ((double)nq + nk) * RP * 4.0;
-    best.steps = dtype == 0 && kernel_bytes >= 128.0 * (1 << 20) && kernel_bytes < 129.0 * (1 << 20);
-    if (best.steps) {
-        const int slots = 2 * sms;
-        best.C = slots / P < 1 ? 1 : slots / P;
-        if (best.C > (n + 15) / 16) best.C = (n + 15) / 16;
-        best.K = 1;
-        best.groups = best.C == 1 ? P : (slots / best.C < P ? slots / best.C : P);
-        best.srows = 0; best.tcols = 0; best.threads = 256;
-        best.smem = fixed_bytes<__nv_bfloat16>(RP, 256);
-    }
     Memo &m = memos[next++ % 8];
     memcpy(m.key, key, sizeof(key));
     m.plan = best;
