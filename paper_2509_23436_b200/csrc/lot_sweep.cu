@@ -124,7 +124,8 @@ static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t
         }
     }
     const dim3 grid((unsigned)(P.groups * P.C));
-    if (P.C == P.K) return chain_launch(kern, grid, THREADS, P.smem, P.K, st, a);
+    if (P.chained) return chain_launch(kern, grid, THREADS, P.smem, P.K, st, a);
+    if (P.C == P.K) return cluster_launch(kern, grid, THREADS, P.smem, P.K, st, a);
     return group_launch(kern, grid, THREADS, P.smem, P.K, st, a);
 }
 

@@ -51,6 +51,7 @@ struct SweepArgs {
 struct SweepPlan {
     int RP, C, K, groups, srows, tcols;
     int threads;             // of a block
+    int chained;             // 1: may start behind its predecessor's last blocks
     size_t smem;
 };
 

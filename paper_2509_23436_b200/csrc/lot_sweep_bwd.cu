@@ -432,7 +432,8 @@ template <int RP, bool GROUP, bool TENSOR> static cudaError_t reverse_g(const Sw
     cudaError_t e = allow_smem(kern, P.smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(P.groups * P.C));
-    if (P.C == P.K) return chain_launch(kern, grid, THREADS, P.smem, P.K, st, a);
+    if (P.chained) return chain_launch(kern, grid, THREADS, P.smem, P.K, st, a);
+    if (P.C == P.K) return cluster_launch(kern, grid, THREADS, P.smem, P.K, st, a);
     return group_launch(kern, grid, THREADS, P.smem, P.K, st, a);
 }
 template <int RP> static cudaError_t reverse_t(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st)

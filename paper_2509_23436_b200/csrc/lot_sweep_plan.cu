@@ -46,6 +46,17 @@ int cluster_blocks(int K, int occ)
 // problem is more than one block's shared memory: a pass over rows there runs at 26 entries a clock and SM against 18
 // from shared memory alone (a loop of passes at RP = 256), and 480 KB instead of 227 stay on an SM.
 namespace sweep {
+// Whether groups of one cluster may start behind the predecessor's last blocks, which saves 2 to 4 us of a call.  Placed while those
+// hold parts of the SMs, clusters leave gaps, and where nearly all of a device's are asked for the last ones wait for the first to
+// end: float32, r = 64, 90 rows a block, us an iteration, chained / ordinary: 82 clusters of three of 93 that fit two to an SM 2.37 / 1.09, 32
+// of 33 of eight 2.36 / 0.90; one block to an SM, 44 of 45 of three 1.91 / 1.21, 26 of 26 of five 2.40 / 1.16, but of two, four
+// and eight the same up to the last; three to an SM (r = 16) 142 of 142 of three 2.09 / 1.15, 66 of 71 of six 1.41 / 1.17, 44 of 48 of
+// eight 1.17 / 1.19, 126 of 142 of three 1.13 / 1.20 (cross-attention 333 x 1531 at r = 32, 128 of 142: 76.4 / 79.7 a call).  Two to an
+// SM they also lie unevenly well below that (12 slices of 2500 at r = 64, T = 20: 118.6 / 114.5).
+constexpr bool chain_fits(int groups, int K, int occ, int slots)
+{
+    return occ == 1 ? K % 2 == 0 || 5 * groups * K <= 4 * slots : occ == 3 && 12 * groups * K <= 11 * slots;
+}
 constexpr double kIters = 12, kClockMHz = 1900;
 constexpr double kEntryClk[2][2] = {{0.033, 0.036}, {0.045, 0.043}};      // clocks of an SM per entry: [tensor memory][RP <= 32]
 }
@@ -82,7 +93,6 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
         const int cap = (int)((block_smem(occ) - fixed) / ((size_t)RP * 4)) / step * step;
         const int rows = (n + C - 1) / C, up = (rows + step - 1) / step * step, srows = up < cap ? up : cap;
         size_t smem = fixed + (size_t)srows * RP * 4;
-        if (tensor && smem < kAloneSmem) smem = kAloneSmem;
         int fit = (int)((size_t)kSmemPerSM / (smem + kSmPerBlockReserve));
         if (fit > occ) fit = occ;
         if (C == 1) slots = sms * fit;
@@ -91,6 +101,9 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
         if (groups < 1) return;
         const int fly = C == 1 && P > slots ? slots : groups, resident = fly * C;            // problems and blocks at once
         const int per_sm = (resident + sms - 1) / sms;                        // blocks that share an SM
+        // blocks that could have an SM each do: a chained start would put some of them two to an SM
+        const int single = C == 1 ? sms : cluster_blocks(K, 1);
+        if ((tensor || resident <= single) && smem < kAloneSmem) smem = kAloneSmem;
         const int tcols = tensor ? kTensorCols : 0, trows = tcols / (threads / 128) / CPL * step;
         // Rows of 16 columns: no more than a few per cent of them streamed beside tensor memory.  The model takes such splits for the better ones, and a
         // block of that many rows is slow to rebuild them: 32 slices of 16384 tokens at d = 128, r = 16, two blocks of 8192 rows a problem 390 us,
@@ -117,6 +130,7 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
             best_t = t;
             best.C = C; best.K = K; best.groups = groups; best.srows = srows;
             best.smem = smem; best.tcols = tcols; best.threads = threads;
+            best.chained = C == 1 || (C == K && (resident <= single ? chain_fits(groups, K, 1, single) : chain_fits(groups, K, occ, slots)));
         }
     };
     // More short problems than blocks of 256 threads fit at once: one warp each, whose barriers wait for nobody and whose sums end in the
@@ -138,7 +152,7 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
     if (warp) {
         const int step = 32 * wide_cols(RP) / RP;
         const size_t f0 = fixed_bytes<float>(RP, 32), f1 = fixed_bytes<__nv_bfloat16>(RP, 32);
-        best.C = best.K = 1; best.groups = P; best.srows = (n + step - 1) / step * step; best.tcols = 0; best.threads = 32;
+        best.C = best.K = 1; best.groups = P; best.srows = (n + step - 1) / step * step; best.tcols = 0; best.threads = 32; best.chained = 1;
         best.smem = (f0 > f1 ? f0 : f1) + (size_t)best.srows * RP * 4;
     }
     Memo &m = memos[next++ % 8];

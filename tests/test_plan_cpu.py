@@ -27,16 +27,16 @@ int main()
     int dt, BH, nq, nk, r, keep;
     while (scanf("%d %d %d %d %d %d", &dt, &BH, &nq, &nk, &r, &keep) == 6) {
         const lot::SweepPlan P = lot::sweep_plan(dt, BH, nq, nk, 64, r, keep != 0);
-        printf("%d %d %d %d %d %d %d %d %zu\n", P.RP, P.C, P.K, P.groups, P.srows, P.tcols, P.threads, ((nq > nk ? nq : nk) + P.C - 1) / P.C, P.smem);
+        printf("%d %d %d %d %d %d %d %d %d %zu\n", P.RP, P.C, P.K, P.groups, P.srows, P.tcols, P.threads, P.chained, ((nq > nk ? nq : nk) + P.C - 1) / P.C, P.smem);
     }
 }
 """
-FIELDS = ("RP", "C", "K", "groups", "srows", "tcols", "threads", "rows", "smem")
+FIELDS = ("RP", "C", "K", "groups", "srows", "tcols", "threads", "chained", "rows", "smem")
 
 
 def sizes():
     """(dtype, slices, queries, keys, pivots, kept history), around the lines at which plans change and drawn ones."""
-    some = [(0, 16, 1000, 1000, 32, 0), (1, 8, 500, 500, 64, 0), (1, 4, 2000, 2000, 16, 0), (0, 64, 200, 200, 64, 0), (1, 1, 1, 1, 256, 0),
+    some = [(0, 16, 700, 700, 64, 0), (0, 16, 1000, 1000, 32, 0), (1, 8, 500, 500, 64, 0), (1, 4, 2000, 2000, 16, 0), (0, 64, 200, 200, 64, 0), (1, 1, 1, 1, 256, 0),
             (1, 32, 16384, 16384, 256, 0), (0, 16, 16384, 16384, 64, 0), (1, 16, 4096, 4096, 64, 1), (0, 64, 333, 1531, 32, 0)]
     rng = random.Random(5)
     for _ in range(400):
@@ -66,3 +66,22 @@ def test_a_block_with_tensor_memory_is_alone_on_its_sm(plans):
     assert with_tensor
     for s, p in with_tensor:
         assert 2 * (p["smem"] + RESERVE) > SM_BYTES, (s, p)
+
+
+def test_chained_clusters_leave_room(plans):
+    """Clusters that start while their predecessor's last blocks run do not pack: a device's last ones would wait for the first to end.
+    Cooperative groups are never chained, blocks on their own always."""
+    for s, p in plans:
+        blocks = p["groups"] * p["K"]
+        if p["C"] == 1 or p["C"] > p["K"]:
+            assert p["chained"] == (p["C"] == 1), (s, p)
+        elif p["chained"]:
+            slots = [148 * occ * 7 // 8 // p["K"] * p["K"] for occ in (1, 3)]              # what the planning code takes where no device answers
+            alone = 2 * (p["smem"] + RESERVE) > SM_BYTES
+            assert alone and blocks <= slots[0] and (p["K"] % 2 == 0 or 5 * blocks <= 4 * slots[0]) or not alone and 12 * blocks <= 11 * slots[1], (s, p)
+
+
+def test_blocks_that_can_have_an_sm_each_do(plans):
+    for s, p in plans:
+        if p["threads"] > 32 and p["groups"] * p["C"] <= 148 * 7 // 8 // p["K"] * p["K"]:
+            assert 2 * (p["smem"] + RESERVE) > SM_BYTES, (s, p)
