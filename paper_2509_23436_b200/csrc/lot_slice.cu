@@ -198,7 +198,7 @@ slice_forward_kernel(const __grid_constant__ SliceParams P)
 {
     constexpr int CPL = wide_cols(RP);
     typedef Lay<RP, CPL> Y;
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const SweepArgs &a = P.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3, mi = lane >> 3;
     const int p = blockIdx.x, n = a.n[0], r = a.r;                 // p even: keys, odd: queries of slice p / 2

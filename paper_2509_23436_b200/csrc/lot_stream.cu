@@ -176,7 +176,7 @@ __device__ __forceinline__ void tile_logits(float (&L)[RP / 8][4], const uint32_
 template <bool REF>
 __device__ __noinline__ void build16(const StreamArgs *ap, int p, int c)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const StreamArgs &a = *ap;
     const Mem m = carve16(smem, a.srows);
     const Part P = locate16(a, p, c);
@@ -500,7 +500,7 @@ __device__ __forceinline__ float log_columns16(const StreamArgs &a, const Mem &m
 template <bool GROUP>
 __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const StreamArgs &a = *ap;
     const Mem m = carve16(smem, a.srows);
     const Part P = locate16(a, p, c);
@@ -524,7 +524,7 @@ __device__ __noinline__ unsigned solve16(const StreamArgs *ap, int p, int group,
 template <bool GROUP>
 __device__ __noinline__ unsigned recover16(const StreamArgs *ap, int p, int group, int c, unsigned seq)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const StreamArgs &a = *ap;
     const Mem m = carve16(smem, a.srows);
     const Part P = locate16(a, p, c);
@@ -571,7 +571,7 @@ template <bool GROUP>
 __global__ void __launch_bounds__(kThreads, 2)
 stream_kernel(const __grid_constant__ StreamArgs a)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, group = GROUP ? blockIdx.x / a.C : blockIdx.x, c = GROUP ? blockIdx.x % a.C : 0;
     unsigned seq = 0;
     const Mem m = carve16(smem, a.srows);

@@ -25,7 +25,7 @@ namespace sweep {
 template <typename T, int RP, int CPL, int THREADS, bool TENSOR>
 __device__ __noinline__ void finish(const SweepArgs *ap, int p, int c)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const SweepArgs &a = *ap;
     const Shared S = carve<T, RP, THREADS>(smem, a.srows);
     Share R;
@@ -52,7 +52,7 @@ template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool TENSOR, boo
 __global__ void __launch_bounds__(THREADS, max_blocks(CPL, THREADS))
 sweep_kernel(const __grid_constant__ SweepArgs a)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, group = GROUP ? blockIdx.x / a.C : blockIdx.x, c = GROUP ? blockIdx.x % a.C : 0;
     const int NP = 2 * a.B * a.H, r = a.r;
     unsigned seq = a.seq0;

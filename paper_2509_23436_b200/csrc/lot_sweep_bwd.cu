@@ -129,7 +129,7 @@ __device__ __forceinline__ void reverse_pass(const Lane<RP, CPL> &L, const Share
     for (int st = 0; st < R.steps; ++st) {
         Row<CPL> k;
 #pragma unroll
-        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.k[v] + st * (STEP * RP * 4));
+        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.template chunk<TENSOR>(st * (STEP * RP * 4), v));
         one(k, L.i0 + st * STEP, R.ns);
     }
     const int on_chip = TENSOR ? R.ns + R.nt : R.ns;
@@ -162,7 +162,7 @@ __device__ __forceinline__ void reverse_pass(const Lane<RP, CPL> &L, const Share
 template <int RP, int CPL, int THREADS, bool GROUP>
 __device__ __noinline__ unsigned reverse_wide(const SweepBwdArgs *ap, int p, int group, int c, unsigned seq, float gam)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     typedef Lay<RP, CPL> Y;
     const SweepArgs &s = ap->s;
     const Shared S = carve<__nv_bfloat16, RP, THREADS>(smem, s.srows);
@@ -240,7 +240,7 @@ template <int RP, int CPL, int THREADS, bool GROUP, bool TENSOR>
 __global__ void __launch_bounds__(THREADS, max_blocks(CPL, THREADS))
 reverse_kernel(const __grid_constant__ SweepBwdArgs a)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     typedef Lay<RP, CPL> Y;
     const SweepArgs &s = a.s;
     const int tid = threadIdx.x, group = GROUP ? blockIdx.x / s.C : blockIdx.x, c = GROUP ? blockIdx.x % s.C : 0;

@@ -56,8 +56,8 @@ __device__ __forceinline__ float lds(uint32_t addr)
 __device__ __forceinline__ void sts(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
 
 // A row of RP columns lies over LPR = RP / CPL adjacent lanes, CPL columns (CPL / 4 chunks of 16 bytes) per lane: chunk v of
-// lane cl is v * LPR + cl.  In shared memory the chunks of a row are permuted so that the eight lanes of a 128-byte
-// phase, which cover 8 / LPR rows, fall on different banks.
+// lane cl is v * LPR + cl.  In shared memory the chunks of a row are permuted so that the eight lanes of a 128-byte phase, which
+// cover 8 / LPR rows, fall on different banks; a row starts at a multiple of its length there (the area is aligned to 1024 bytes).
 template <int RP, int CPL> struct Lay {
     static constexpr int LPR = RP / CPL, RPW = 32 / LPR, CH = RP / 4, NV = CPL / 4;
     static constexpr int RPL = RP >= 32 ? 1 : 32 / RP, SG = LPR >= 8 ? 1 : (8 / LPR / RPL < 1 ? 1 : 8 / LPR / RPL);
@@ -234,6 +234,15 @@ __device__ __forceinline__ float row_step(const Row<CPL> &k, const u64 (&w)[CPL 
 template <int RP, int CPL> struct Lane {
     uint32_t k[CPL / 4], w, red, own, t;
     int i0, cl;
+    // Chunk v of the row `row` bytes (whole steps) behind the first.  ONE: from the first chunk's address alone (the permutation is an
+    // exclusive or within the row): an instruction more and three registers fewer, for the passes beside tensor memory, whose 128
+    // registers do not hold everything.  The forward's iterations then touch no spilled value; with four addresses a warp reloaded 3 to 12 a
+    // pass at r = 32 and 64, more with more rows (13376 x 7341 tokens, 12 slices, r = 32, T = 50: 253.9 us, 256.9; counted by local
+    // memory requests of 5 and 25 iterations).  Left: two reloads an iteration in the backward's two loops, whatever the rows.
+    template <bool ONE> __device__ __forceinline__ uint32_t chunk(uint32_t row, int v) const
+    {
+        return ONE ? (k[0] + row) ^ (v * (Lay<RP, CPL>::LPR * 16)) : k[v] + row;
+    }
 };
 
 // The tensor memory as a second store of kernel rows: a lane's columns of a row are CPL neighbouring columns of its lane there, as
@@ -329,7 +338,7 @@ __device__ __forceinline__ void pass_t(const Lane<RP, CPL> &L, const Share &R, c
     };
     auto load = [&](Row<CPL> &k, int st) {
 #pragma unroll
-        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.k[v] + st * (STEP * RP * 4));
+        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.template chunk<TENSOR>(st * (STEP * RP * 4), v));
     };
     auto fetch = [&](Row<CPL> (&k)[2], int i) {              // two steps' rows from L2
 #pragma unroll
@@ -840,7 +849,7 @@ __device__ __forceinline__ bool iterate(const SweepArgs &a, const Shared &S, con
 template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool TENSOR, size_t WORK = work_bytes<T>(RP, THREADS), size_t REF = ref_bytes(RP, THREADS)>
 __device__ __noinline__ unsigned recover(const SweepArgs *ap, int p, int group, int c, int it, unsigned seq, float wold, float wnew)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     const SweepArgs &a = *ap;
     const Shared S = carve<T, RP, THREADS>(smem, a.srows, WORK, REF);
     Share R;
