@@ -110,7 +110,7 @@ template <typename T, int RP, int CPL, int THREADS, bool GROUP, bool TENSOR, boo
 static cudaError_t launch_g(const SweepPlan &P, const SweepArgs &a, cudaStream_t st)
 {
     auto kern = sweep_kernel<T, RP, CPL, THREADS, GROUP, TENSOR, KEEP>;
-    if (TENSOR && P.smem < kAloneSmem) return cudaErrorInvalidConfiguration;
+    if (P.tcols != 0 && P.smem < kAloneSmem) return cudaErrorInvalidConfiguration;
     static std::mutex mu;
     static bool attr_set[64] = {};
     int dev = 0;
@@ -135,7 +135,7 @@ static cudaError_t launch_k(const SweepPlan &P, const SweepArgs &a, cudaStream_t
     if constexpr (RP <= 32 && !KEEP) {
         if (P.threads == 32) return launch_g<T, RP, wide_cols(RP), 32, false, false, false>(P, a, st);
     }
-    if (P.tcols)
+    if (P.threads == kTensorThreads)
         return P.C > 1 ? launch_g<T, RP, kTensorLane, kTensorThreads, true, true, KEEP>(P, a, st)
                        : launch_g<T, RP, kTensorLane, kTensorThreads, false, true, KEEP>(P, a, st);
     return P.C > 1 ? launch_g<T, RP, wide_cols(RP), 256, true, false, KEEP>(P, a, st) : launch_g<T, RP, wide_cols(RP), 256, false, false, KEEP>(P, a, st);

@@ -428,7 +428,7 @@ template <int RP, bool GROUP, bool TENSOR> static cudaError_t reverse_g(const Sw
 {
     constexpr int THREADS = TENSOR ? kTensorThreads : 256;
     auto kern = reverse_kernel<RP, TENSOR ? kTensorLane : wide_cols(RP), THREADS, GROUP, TENSOR>;
-    if (TENSOR && P.smem < kAloneSmem) return cudaErrorInvalidConfiguration;
+    if (P.tcols != 0 && P.smem < kAloneSmem) return cudaErrorInvalidConfiguration;
     cudaError_t e = allow_smem(kern, P.smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)(P.groups * P.C));
@@ -438,8 +438,8 @@ template <int RP, bool GROUP, bool TENSOR> static cudaError_t reverse_g(const Sw
 }
 template <int RP> static cudaError_t reverse_t(const SweepPlan &P, const SweepBwdArgs &a, cudaStream_t st)
 {
-    if (P.C > 1) return P.tcols ? reverse_g<RP, true, true>(P, a, st) : reverse_g<RP, true, false>(P, a, st);
-    return P.tcols ? reverse_g<RP, false, true>(P, a, st) : reverse_g<RP, false, false>(P, a, st);
+    if (P.C > 1) return P.threads == kTensorThreads ? reverse_g<RP, true, true>(P, a, st) : reverse_g<RP, true, false>(P, a, st);
+    return P.threads == kTensorThreads ? reverse_g<RP, false, true>(P, a, st) : reverse_g<RP, false, false>(P, a, st);
 }
 
 } // namespace sweep

@@ -40,11 +40,14 @@ int cluster_blocks(int K, int occ)
 
 // Blocks per problem and where the rows live: the split with the least modelled time.  In a round all resident groups finish
 // one problem each; it costs the reading of its rows and, per iteration, the larger of one block's chain (latency with
-// the exchange, its own steps) and of what the blocks of an SM need together.  The constants are fitted to the times of whole
-// calls: 40 sizes from 2 problems of 30000 tokens to 512 of 512, each in up to 34 forced splits; over those, the
-// split chosen is on average 1.4 % slower than the best one, 12 % at most.  Rows in tensor memory are what it mostly takes where a
-// problem is more than one block's shared memory: a pass over rows there runs at 26 entries a clock and SM against 18
-// from shared memory alone (a loop of passes at RP = 256), and 480 KB instead of 227 stay on an SM.
+// the exchange, its own steps) and of what the blocks of an SM need together.  The constants are fitted to the times of whole calls of 12
+// iterations: 108 sizes from 2 problems of 300 tokens to 512 of 1100 and 18 of 52000, each in up to 56 forced splits; over those, the
+// split chosen is on average 1.0 % slower than the best one, and in 8 of them more than 5 % (22 % at most: 32 problems of 700 tokens, where
+// clusters of four take 13 us longer than of three for no reason this model knows).
+// Rows in tensor memory are what it mostly takes where a problem is more than one block's shared memory: a pass over rows there
+// runs at 26 entries a clock and SM against 18 from shared memory alone (a loop of passes at RP = 256), and 480 KB instead of 227
+// stay on an SM.  Where all rows fit shared memory, 512 threads are worth it at RP <= 32 with a block a problem (64 slices of 700 at r = 32
+// 47.4 us, 256 threads 49.3) and not for clusters (8 of 500 at r = 64, T = 20: 55.6, 49.6).
 namespace sweep {
 // Whether groups of one cluster may start behind the predecessor's last blocks, which saves 2 to 4 us of a call.  Placed while those
 // hold parts of the SMs, clusters leave gaps, and where nearly all of a device's are asked for the last ones wait for the first to
@@ -58,7 +61,9 @@ constexpr bool chain_fits(int groups, int K, int occ, int slots)
     return occ == 1 ? K % 2 == 0 || 5 * groups * K <= 4 * slots : occ == 3 && 12 * groups * K <= 11 * slots;
 }
 constexpr double kIters = 12, kClockMHz = 1900;
-constexpr double kEntryClk[2][2] = {{0.033, 0.036}, {0.045, 0.043}};      // clocks of an SM per entry: [tensor memory][RP <= 32]
+constexpr double kEntryClk[2][2] = {{0.032, 0.037}, {0.046, 0.041}};      // clocks of an SM per entry: [512 threads][RP <= 32]
+constexpr double kAloneBlock = 1.7;      // times as many where a block of 256 threads has the SM to itself
+constexpr double kOrdinaryStart = 2.9;   // us
 }
 
 SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
@@ -78,10 +83,10 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
     double best_t = 1e30;
     auto consider = [&](bool tensor, int occ, int C, int K, int slots) {
         const int threads = tensor ? kTensorThreads : 256, CPL = tensor ? kTensorLane : wide_cols(RP);
-        const double entry = kEntryClk[tensor][RP <= 32] / kClockMHz * (tensor ? 1.0 : 1.7);
-        double lat = (tensor ? C == 1 ? 0.78 : 0.55 : 0.7) + RP / 256.0;
+        const double entry = kEntryClk[tensor][RP <= 32] / kClockMHz * (tensor ? 1.0 : kAloneBlock);
+        double lat = tensor ? (C == 1 ? 0.88 : 0.98) + RP * (1.2 / 256) : 0.79 + RP * (0.87 / 256);
         if (C > 1) {
-            lat += C == K ? 0.6 : 1.7 + 0.3 * (occ - 1);
+            lat += C == K ? 0.67 + 0.025 * (K - 2) : 2.2 + 0.33 * (occ - 1);
             // most splits are no match for the best so far by this alone (a search of all of them took 60 us)
             if (slots < C) return;
             const int fly = slots / C < P ? slots / C : P, turns = ((nq == nk ? P : BH) + fly - 1) / fly;
@@ -103,34 +108,35 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
         const int per_sm = (resident + sms - 1) / sms;                        // blocks that share an SM
         // blocks that could have an SM each do: a chained start would put some of them two to an SM
         const int single = C == 1 ? sms : cluster_blocks(K, 1);
-        if ((tensor || resident <= single) && smem < kAloneSmem) smem = kAloneSmem;
-        const int tcols = tensor ? kTensorCols : 0, trows = tcols / (threads / 128) / CPL * step;
+        if (resident <= single && smem < kAloneSmem) smem = kAloneSmem;
+        const bool chained = C == 1 || (C == K && (resident <= single ? chain_fits(groups, K, 1, single) : chain_fits(groups, K, occ, slots)));
+        const int tcols = tensor && rows > srows ? kTensorCols : 0, trows = tcols / (threads / 128) / CPL * step;
         // Rows of 16 columns: no more than a few per cent of them streamed beside tensor memory.  The model takes such splits for the better ones, and a
         // block of that many rows is slow to rebuild them: 32 slices of 16384 tokens at d = 128, r = 16, two blocks of 8192 rows a problem 390 us,
-        // peaked 578, four of 4096 384 and 485 (before tensor memory 451 and 498).  At RP = 32 such splits are the
-        // better ones (r = 32, 4096 rows a block: peaked 610, before tensor memory 771).
+        // peaked 578, four of 4096 384 and 485 (before tensor memory 451 and 498).
         if (tensor && RP == 16 && rows > 1.05 * (srows + trows)) return;
         // us of a problem of m tokens
         auto problem = [&](int m) {
             const int mine = (m + C - 1) / C, ns = mine < srows ? mine : srows, nt = mine - ns < trows ? mine - ns : trows, rest = mine - ns - nt;
             const int steps = (ns + step - 1) / step + (nt + 2 * step - 1) / (2 * step) * 2 + (rest + 2 * step - 1) / (2 * step) * 2;
             const double work = (double)steps * step * RP * kEntryClk[tensor][RP <= 32] / kClockMHz;
-            double it = lat + work * (tensor ? 1.0 : 1.7);
+            double it = lat + work * (tensor ? 1.0 : kAloneBlock);
             if (it < per_sm * work) it = per_sm * work;
             if (rest > 0) {
                 const double mb = rest * (RP * 4e-6), all = mb * resident;
-                const double l2 = all / (all > 90 ? 5.0 : 12.0), sm = per_sm * mb / 0.11;
-                it += 0.5 + (l2 > sm ? l2 : sm);
+                const double l2 = all / (all > 60 ? 5.0 : 11.0), sm = per_sm * mb / 0.08;       // TB/s: L2 beyond half of it is no faster than memory
+                it += 0.9 + (l2 > sm ? l2 : sm);
             }
-            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.4 + mine * (RP * 1e-4) + 3.0;
+            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.5 + mine * (RP * 8e-5) + 3.0;
         };
         const int rounds = (P + fly - 1) / fly, first = nq == nk ? rounds : (BH + fly - 1) / fly;         // the longer side's come first
-        const double t = first * problem(n) + (rounds > first ? (rounds - first) * problem(nq < nk ? nq : nk) : 0.0);
+        const double t = first * problem(n) + (rounds > first ? (rounds - first) * problem(nq < nk ? nq : nk) : 0.0) + (chained ? 0.0 : kOrdinaryStart) +
+                         (tensor ? 0.9 : 0.0);
         if (t < best_t) {
             best_t = t;
             best.C = C; best.K = K; best.groups = groups; best.srows = srows;
             best.smem = smem; best.tcols = tcols; best.threads = threads;
-            best.chained = C == 1 || (C == K && (resident <= single ? chain_fits(groups, K, 1, single) : chain_fits(groups, K, occ, slots)));
+            best.chained = chained;
         }
     };
     // More short problems than blocks of 256 threads fit at once: one warp each, whose barriers wait for nobody and whose sums end in the

@@ -85,3 +85,8 @@ def test_blocks_that_can_have_an_sm_each_do(plans):
     for s, p in plans:
         if p["threads"] > 32 and p["groups"] * p["C"] <= 148 * 7 // 8 // p["K"] * p["K"]:
             assert 2 * (p["smem"] + RESERVE) > SM_BYTES, (s, p)
+
+
+def test_tensor_memory_is_taken_only_where_rows_go_there(plans):
+    for s, p in plans:
+        assert (p["tcols"] != 0) == (p["threads"] == 512 and p["rows"] > p["srows"]), (s, p)
