@@ -129,7 +129,7 @@ __device__ __forceinline__ void reverse_pass(const Lane<RP, CPL> &L, const Share
     for (int st = 0; st < R.steps; ++st) {
         Row<CPL> k;
 #pragma unroll
-        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.template chunk<TENSOR>(st * (STEP * RP * 4), v));
+        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.template chunk<TENSOR && RP <= 32>(st * (STEP * RP * 4), v));
         one(k, L.i0 + st * STEP, R.ns);
     }
     const int on_chip = TENSOR ? R.ns + R.nt : R.ns;

@@ -235,10 +235,11 @@ template <int RP, int CPL> struct Lane {
     uint32_t k[CPL / 4], w, red, own, t;
     int i0, cl;
     // Chunk v of the row `row` bytes (whole steps) behind the first.  ONE: from the first chunk's address alone (the permutation is an
-    // exclusive or within the row): an instruction more and three registers fewer, for the passes beside tensor memory, whose 128
-    // registers do not hold everything.  The forward's iterations then touch no spilled value; with four addresses a warp reloaded 3 to 12 a
-    // pass at r = 32 and 64, more with more rows (13376 x 7341 tokens, 12 slices, r = 32, T = 50: 253.9 us, 256.9; counted by local
-    // memory requests of 5 and 25 iterations).  Left: two reloads an iteration in the backward's two loops, whatever the rows.
+    // exclusive or within the row), an instruction more and three registers fewer: for the passes beside tensor memory, whose 128
+    // registers do not hold everything, at r <= 32 (13376 x 7341 tokens, 12 slices, r = 32, T = 50: 254.3 us, 258.1 with four addresses).  At
+    // r = 64 the instruction costs more than the reloads it saves (32 slices of 16384 tokens, T = 20: 975, 941).
+    // Reloads of spilled registers a warp and pass, by local memory requests of 5 and 25 iterations: none at r <= 32, 3 to 9 of 260 to 400
+    // instructions at r = 64, 1 at r = 256; the backward's forward 5 and its reverse steps 2, whatever the rows.
     template <bool ONE> __device__ __forceinline__ uint32_t chunk(uint32_t row, int v) const
     {
         return ONE ? (k[0] + row) ^ (v * (Lay<RP, CPL>::LPR * 16)) : k[v] + row;
@@ -338,7 +339,7 @@ __device__ __forceinline__ void pass_t(const Lane<RP, CPL> &L, const Share &R, c
     };
     auto load = [&](Row<CPL> &k, int st) {
 #pragma unroll
-        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.template chunk<TENSOR>(st * (STEP * RP * 4), v));
+        for (int v = 0; v < Y::NV; ++v) lds2(k.k[2 * v], k.k[2 * v + 1], L.template chunk<TENSOR && RP <= 32>(st * (STEP * RP * 4), v));
     };
     auto fetch = [&](Row<CPL> (&k)[2], int i) {              // two steps' rows from L2
 #pragma unroll
@@ -822,6 +823,7 @@ __device__ __forceinline__ bool iterate(const SweepArgs &a, const Shared &S, con
     __syncthreads();
     float tot = 0.f;
     if (threadIdx.x < RP) {
+        if (TENSOR) { tgt = S.tgt[threadIdx.x]; wnew = S.w[threadIdx.x]; }       // not kept over the pass: three registers
         float o[THREADS / 32];
 #pragma unroll
         for (int i = 0; i < THREADS / 32; ++i) o[i] = lds(L.own + i * (RP * 4));
