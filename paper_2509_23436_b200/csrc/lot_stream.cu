@@ -29,6 +29,9 @@ constexpr int kStage = 2 * RP * kZPitch;   // staged pivots (hi, lo): in the ker
 constexpr int kWork = kThreads / 32 * RP * 4;
 constexpr int kFixed = kWork + kThreads * 4 + RP * 20 + 64 + 2 * kPeers * RP * 4;
 
+constexpr int kRowsCap = (kSmemPerSM / 2 - kSmPerBlockReserve - kFixed) / 128 / kRowsStep * kRowsStep;       // kernel rows a block has room for, two blocks an SM
+constexpr int kMostWords = 80;             // words a column that a thread reads, sixteen at a time
+
 __host__ __device__ constexpr int area_bytes(int srows) { return srows * 128 > kStage ? srows * 128 : kStage; }
 
 struct StreamArgs {
@@ -614,8 +617,14 @@ stream_kernel(const __grid_constant__ StreamArgs a)
 StreamPlan stream_plan(int BH, int n)
 {
     using namespace stream;
+    const int NP = 2 * BH, sms = device_sm_count(), slots = 2 * sms;
+    // asked for by the workspace query and by every call: the last answers are kept
+    struct Memo { int BH, n, sms; StreamPlan plan; };
+    static thread_local Memo memos[4] = {};
+    static thread_local unsigned next = 0;
+    for (const Memo &m : memos)
+        if (m.BH == BH && m.n == n && m.sms == sms) return m.plan;
     StreamPlan L;
-    const int NP = 2 * BH, slots = 2 * device_sm_count();
     const long long npad = ((long long)n + 127) / 128 * 128;
     // problems in flight: all of them, or as many as keep what is iterated on in the L2
     long long fly = 80000000ll / (npad * 128);
@@ -623,29 +632,36 @@ StreamPlan stream_plan(int BH, int n)
     if (fly > NP) fly = NP;
     const int rounds = (int)((NP + fly - 1) / fly), most = (n + 2 * kRowsStep - 1) / (2 * kRowsStep);
     fly = (NP + rounds - 1) / rounds;
-    // Blocks a problem and blocks a cluster: the least time of a pass, us: steps of 64 rows (two blocks share an SM) and the exchange
-    // (group_columns), at least two steps a block.
+    // Blocks a problem and blocks a cluster: the least modelled time of a call of ten iterations, us: steps of 64 rows (more where two blocks share
+    // an SM), rows behind shared memory, the exchange (group_columns: one cluster; else words through L2, sixteen waited for at once,
+    // behind the sums of each cluster of more than one block), and the building; at least two steps a block.  Fitted to 42 sizes
+    // from one slice of 1000 tokens to three of 100000 and 400 of 600 in up to 60 forced splits: 0.7 % above the best of them on average, 7
+    // at most.  Single blocks exchanging through L2 beat clusters of two where a problem has few (12 slices of 9000 tokens 87 / 94), clusters
+    // of eight beat clusters of two and four where those would leave more than 16 words (one of 16384 91 / 108, of 65536 122 / 134).
     L.C = 1; L.K = 1;
     double best = 1e30;
     auto consider = [&](int C, int K, int blocks) {
         if (C > 1 && (C > most || blocks / C < 1)) return;
         const int groups = C == 1 ? (NP < blocks ? NP : blocks) : (blocks / C < NP ? blocks / C : NP), words = C / K;
-        const int steps = ((n + C - 1) / C + kRowsStep - 1) / kRowsStep, turns = (NP + groups - 1) / groups;
-        const double lat = C == 1 ? 0.45 : C == K ? 1.0 : 1.4 + 0.45 * ((words - 1) / (kWords * (words > kWords ? kThreads / RP : 1)));
-        const double t = turns * (steps * 0.25 + lat);
-        if (groups <= fly && t < best) { best = t; L.C = C; L.K = K; }
+        if (groups > fly) return;
+        const int rows = (n + C - 1) / C, steps = (rows + kRowsStep - 1) / kRowsStep, turns = (NP + groups - 1) / groups;
+        const int rest = rows > kRowsCap ? (rows - kRowsCap + kRowsStep - 1) / kRowsStep : 0;
+        const bool two = groups * C > sms;
+        const double lat = C == 1 ? 0.465 : C == K ? 1.1 + 0.018 * (K - 2) : 1.8 + 0.0127 * (words - 2) + 0.477 * ((words - 1) / kWords) + (K > 1 ? 1.05 : 0.0);
+        const double it = lat + steps * (two ? 0.278 : 0.2) + rest * (two ? 0.089 : 0.0445);
+        const double t = turns * (10.5 * it + steps * 0.68 + 4.1);
+        if (t < best) { best = t; L.C = C; L.K = K; L.groups = groups; }
     };
     consider(1, 1, slots);
-    for (int K = 2; K <= kPeers; ++K) {
-        const int blocks = cluster_blocks(K, 2);
-        consider(K, K, blocks);
+    for (int K = 1; K <= kPeers; ++K) {
+        const int blocks = K == 1 ? slots : cluster_blocks(K, 2);
+        if (K > 1) consider(K, K, blocks);
         if ((K & (K - 1)) == 0)
-            for (int M = 2; M * K <= blocks; ++M) consider(M * K, K, blocks);
+            for (int M = 2; M <= kMostWords && M * K <= blocks; ++M) consider(M * K, K, blocks);
     }
-    L.groups = L.C == 1 ? NP : cluster_blocks(L.K, 2) / L.C < NP ? cluster_blocks(L.K, 2) / L.C : NP;
+    if (L.C == 1) L.groups = NP;
     const int rows = (n + L.C - 1) / L.C, up = (rows + kRowsStep - 1) / kRowsStep * kRowsStep;
-    const int cap = (228 * 1024 / 2 - 1024 - kFixed) / 128 / kRowsStep * kRowsStep;
-    L.srows = up < cap ? up : cap;
+    L.srows = up < kRowsCap ? up : kRowsCap;
     L.npad = (int)npad;
     size_t o = 256;
     auto take = [&](size_t bytes) { const size_t at = o; o += (bytes + 255) & ~(size_t)255; return at; };
@@ -656,6 +672,7 @@ StreamPlan stream_plan(int BH, int n)
     L.kt = take((size_t)NP * npad * 128);
     L.wpart = take(stored_apply_wpart_bytes(BH, 1, n));
     L.total = o;
+    memos[next++ % 4] = Memo{BH, n, sms, L};
     return L;
 }
 
