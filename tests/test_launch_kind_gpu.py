@@ -10,8 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 def launches(call):
-    """(cooperative, blocks of a cluster) of every kernel that `call` launches, from a captured graph."""
-    rt = pytest.importorskip("cuda.bindings.runtime")
+    """(cooperative, blocks of a cluster, blocks) of every kernel that `call` launches, from a captured graph."""
+    rt, drv = pytest.importorskip("cuda.bindings.runtime"), pytest.importorskip("cuda.bindings.driver")
     graph = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(graph):
         call()
@@ -25,7 +25,8 @@ def launches(call):
             continue
         ids = rt.cudaLaunchAttributeID
         attr = [rt.cudaGraphKernelNodeGetAttribute(node, i)[1] for i in (ids.cudaLaunchAttributeCooperative, ids.cudaLaunchAttributeClusterDimension)]
-        found.append((bool(attr[0].cooperative), max(1, attr[1].clusterDim.x)))
+        params = drv.cuGraphKernelNodeGetParams(drv.CUgraphNode(int(node)))[1]        # the runtime's form knows only its own copy's kernels
+        found.append((bool(attr[0].cooperative), max(1, attr[1].clusterDim.x), params.gridDimX * params.gridDimY * params.gridDimZ))
     return found
 
 
@@ -41,5 +42,5 @@ def test_only_groups_of_several_clusters_are_cooperative(B, H, n, d, r, dtype, p
     out, ws = lot.lot_attention_fwd_ex(*t, None, x.eps, x.iters)
     torch.cuda.synchronize()
     found = launches(lambda: lot.lot_attention_fwd_ex(*t, None, x.eps, x.iters, out=out, ws=ws))
-    assert any(k > 1 for _, k in found) or not one
-    assert any(coop for coop, _ in found) == (not one)
+    assert any(k > 1 for _, k, _ in found) or not one
+    assert any(coop for coop, _, _ in found) == (not one)
