@@ -63,6 +63,10 @@ grad_kernel(const __grid_constant__ SweepGradArgs ga)
     const float *K = s.kt[side] + (size_t)slice * n * RP, *dC = a.dC[side] + (size_t)slice * n * RP;
     const __nv_bfloat16 *X = static_cast<const __nv_bfloat16 *>(s.x[side]) + (size_t)slice * n * d;
     const float2 *coef = a.coef + (size_t)p * a.T * n;
+    chain_wait();
+    // A wide problem's dC is complete, and its kernel is not to be read: the reverse steps left exponents in place of the rows that were not in
+    // shared memory, -infinity in the columns behind r.
+    const int T = nv == 0 || *reinterpret_cast<const volatile int *>(s.wide + p) != 0 ? 0 : a.T;
     __nv_bfloat16 *dX = static_cast<__nv_bfloat16 *>(ga.dx[side]) + (size_t)slice * n * d;
 
     float4 kr[NP], dr[NP];
@@ -72,7 +76,7 @@ grad_kernel(const __grid_constant__ SweepGradArgs ga)
         for (int u = 0; u < NP; ++u) {
             const int idx = tid + u * kThreads, j = j0 + idx / (RP / 4), t = (idx % (RP / 4)) * 4;
             const bool in = j < nv && j < row1;
-            kr[u] = in ? chain_ld4(K + (size_t)j * RP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+            kr[u] = in && T > 0 ? chain_ld4(K + (size_t)j * RP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
             dr[u] = in ? chain_ld4(dC + (size_t)j * RP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
@@ -92,8 +96,6 @@ grad_kernel(const __grid_constant__ SweepGradArgs ga)
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    chain_wait();
-    const int T = nv == 0 || *reinterpret_cast<const volatile int *>(s.wide + p) != 0 ? 0 : a.T;      // a wide problem's dC is complete
     float acc[NTW][4] = {};
     if (row0 < row1) {
         fetch(row0);

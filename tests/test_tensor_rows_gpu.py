@@ -9,6 +9,7 @@ import pytest
 import torch
 
 from oracle import lot_oracle as O
+from oracle import lot_oracle_grad as OG
 from paper_2509_23436_b200 import binding as lot
 from paper_2509_23436_b200 import synth
 from lot_testutil import TOL, check_slice, gpu_forward, oracle_slices
@@ -16,6 +17,11 @@ from test_backward_gpu import oracle_grads
 
 pytestmark = pytest.mark.gpu
 F32, BF16 = torch.float32, torch.bfloat16
+
+
+def f64(t):
+    return t.float().cpu().double().numpy()
+
 
 # B, H, n, d, r, iters, eps, dtype, key mask, clustered
 FORWARD = [
@@ -111,3 +117,28 @@ def test_a_captured_call_gives_the_same_bits(B, H, n, d, r):
         graph.replay()
         torch.cuda.synchronize()
         assert lot.lot_device_status(ws) == 0 and torch.equal(out, want)
+
+
+# H, n, r: padded ranks, rows in tensor memory and streamed ones
+@pytest.mark.parametrize("H,n,r", [(200, 1500, 48), (200, 4000, 20)])
+def test_backward_reversed_on_exponents_matches_oracle(H, n, r):
+    """Potentials over more than the kept weights' range: such a problem's kernel is overwritten by exponents, -infinity in the padding."""
+    d, eps, iters = 32, 0.01, 3
+    x = synth.make(1, H, n, d, r, seed=9851 + n + r, dtype=BF16, eps=eps, iters=iters, qk="mixture")
+    dout = synth.cotangent(x)
+    f, w, h = x.f64(), np.full(n, 1.0 / n), H - 1
+    fw = OG.head_forward(f["q"][0, h], f["k"][0, h], f["v"][0, h], f["z"][h], f["beta"][h], w, w, eps, iters)
+    for trace, g in ((fw["tr1"], fw["g1"]), (fw["tr2"], fw["g2"])):
+        all_g = np.array([g0 for g0, _ in trace] + [g]) / (eps * np.log(2))
+        assert np.ptp(all_g, axis=0).max() > 230               # weights between 2^-115 and 2^115 cannot hold them
+    dev = torch.device("cuda:0")
+    t = [getattr(x, name).to(dev) for name in ("q", "k", "v", "z", "beta")]
+    res = lot.lot_attention_bwd(*t, None, dout.to(dev), eps, iters)
+    assert lot.lot_device_status(res[5]) == 0
+    for name, got in zip(("dq", "dk", "dv", "dz", "dbeta"), res):
+        assert bool(torch.isfinite(got.float()).all()), name
+    ref = OG.head_backward(fw, f64(dout[0, h]))
+    for name, got in zip(("dq", "dk", "dv"), res):
+        check_slice(f64(got[0, h]), ref[name], TOL[BF16], name)
+    check_slice(f64(res[3][h]), ref["dz"], TOL[BF16], "dz")
+    check_slice(f64(res[4][h])[None, :], ref["dbeta"][None, :], TOL[BF16], "dbeta")
