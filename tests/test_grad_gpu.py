@@ -55,5 +55,11 @@ def test_a_batch_row_without_keys_has_finite_gradients():
     ws = torch.full((lot.lot_bwd_workspace_bytes(2, 2, 130, 64, 32, lot.LOT_BF16, 4),), 0xFF, dtype=torch.uint8, device=dev)
     res = lot.lot_attention_bwd(*t, torch.tensor([0, 130], dtype=torch.int32, device=dev), synth.cotangent(x).to(dev), 0.1, 4, ws=ws)
     assert np.all(res[1][0].float().cpu().numpy() == 0) and np.all(res[2][0].float().cpu().numpy() == 0)
-    for g in (res[0][1], res[1], res[2][1]):
+    for g in res[:5]:
         assert bool(torch.isfinite(g.float()).all())
+    assert np.all(res[0][0].float().cpu().numpy() == 0)
+    # the sums over the batch are the other row's: float32 sums of at most 130 tokens in another order, through four reverse steps
+    one = lot.lot_attention_bwd(*(g[1:].contiguous() for g in t[:3]), *t[3:], None, synth.cotangent(x)[1:].contiguous().to(dev), 0.1, 4)
+    for i, name in ((3, "dz"), (4, "dbeta")):
+        for h in range(2):
+            check_slice(res[i][h].cpu().double().numpy(), one[i][h].cpu().double().numpy(), 1e-4, f"{name} head {h}")
