@@ -513,23 +513,28 @@ __device__ __forceinline__ void send(uint32_t dst, float v, uint32_t bar)
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst), "r"(__float_as_uint(v)), "r"(bar)
                  : "memory");
 }
-// Wait for the bytes of a set of sends (at most a second, then the call is flagged and every later wait gives up at once).
-__device__ __forceinline__ void wait_sends(uint32_t bar, unsigned parity, volatile int *dead, int *status)
+// Whether the bytes of a set of sends have arrived.
+__device__ __forceinline__ bool sends_arrived(uint32_t bar, unsigned parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Wait for them (at most a second, then the call is flagged and every later wait gives up at once); false if they did not come.
+__device__ __forceinline__ bool wait_sends(uint32_t bar, unsigned parity, volatile int *dead, int *status)
 {
     u64 start = 0;
     for (unsigned spin = 1;; ++spin) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return;
+        if (sends_arrived(bar, parity)) return true;
         if ((spin & 63u) != 0) continue;
         const u64 now = global_timer_ns();
         if (start == 0) start = now;
         if (*dead || now - start > kWaitNs) {
             if (!*dead) atomicOr(status, 4 /* LOT_DEV_TIMEOUT */);
             *dead = 1;
-            return;
+            return false;
         }
     }
 }
@@ -597,6 +602,11 @@ __device__ __forceinline__ float group_columns(const Args &a, const Shared &S, f
 {
     const int C = a.C, K = a.K, tid = threadIdx.x;
     if (C == 1) return part;
+    // A wait of the block gave up: the call is flagged, its results are void.  Nothing is sent, waited for or armed any more, so no barrier is
+    // armed whose phase is still open (its count would be undefined) and none counts more bytes than a few exchanges bring.
+    // (The flag is read behind the sends, its latency under theirs: in front of them they waited 0.09 us for it.)
+    constexpr unsigned kGaveUp = ~0u;
+    if (seq == kGaveUp) return part;
     const unsigned nth = seq - a.seq0;                       // of this launch
     ++seq;
     const unsigned tag = seq;
@@ -617,10 +627,11 @@ __device__ __forceinline__ float group_columns(const Args &a, const Shared &S, f
     if (C == K) {
         if (tid < RP) {
             for (int o = 0; o < K; ++o) send(in_peer(mine + (c * RP + tid) * 4, o), part, in_peer(bar, o));
-            wait_sends(bar, parity, S.flag, a.status);
+            const bool dead = *S.flag, all = wait_sends(bar, parity, S.flag, a.status);
             part = add_up(RP);
+            if (tid == 0 && all) sm100::mbar_arrive_expect_tx(bar, peer_bytes(RP, C, K) / 2);      // for the exchange after the next
+            if (dead || !all) seq = kGaveUp;
         }
-        if (tid == 0) sm100::mbar_arrive_expect_tx(bar, peer_bytes(RP, C, K) / 2);      // for the exchange after the next
         return part;
     }
     const int M = C / K, m = c / K, rank = c % K;
@@ -634,12 +645,13 @@ __device__ __forceinline__ float group_columns(const Args &a, const Shared &S, f
             send(in_peer(mine + (rank * own + (tid & (own - 1))) * 4, to), part, in_peer(bar, to));
         }
         if (tid < own) {
-            wait_sends(bar, parity, S.flag, a.status);
-            put_word(X + (size_t)m * RP + rank * own + tid, add_up(own), tag);
+            const bool all = wait_sends(bar, parity, S.flag, a.status);
+            if (all) put_word(X + (size_t)m * RP + rank * own + tid, add_up(own), tag);
+            if (tid == 0 && all) sm100::mbar_arrive_expect_tx(bar, peer_bytes(RP, C, K) / 2);
         }
-        if (tid == 0) sm100::mbar_arrive_expect_tx(bar, peer_bytes(RP, C, K) / 2);
     }
     float tot = none;
+    bool dead = *S.flag;
     if (tid < RP)
         for (int m0 = 0; m0 < M; m0 += kWords) {
             const u64 *p = X + (size_t)m0 * RP + tid;
@@ -661,12 +673,14 @@ __device__ __forceinline__ float group_columns(const Args &a, const Shared &S, f
                 if (*S.flag || now - start > kWaitNs) {
                     if (!*S.flag) atomicOr(a.status, 4 /* LOT_DEV_TIMEOUT */);
                     *S.flag = 1;
+                    dead = true;
                     break;
                 }
             }
 #pragma unroll
             for (int u = 0; u < kWords; ++u) tot = join(tot, __uint_as_float((unsigned)wd[u]));
         }
+    if (dead) seq = kGaveUp;
     return tot;
 }
 
