@@ -77,6 +77,7 @@ __host__ __device__ constexpr int max_blocks(int cpl, int threads) { return (cpl
 constexpr int kTensorThreads = 512, kTensorCols = 512, kTensorLane = 16;
 constexpr size_t kAloneSmem = kSmemPerSM / 2;
 static_assert(2 * (kAloneSmem + kSmPerBlockReserve) > (size_t)kSmemPerSM && kAloneSmem <= (size_t)kSmemPerBlock, "one such block an SM");
+__host__ __device__ constexpr int lane_sharers(int threads) { return threads < 128 ? 1 : threads / 128; }       // warps that share a quarter of the lanes
 
 // shared memory: [kernel rows | gref | work area (staged pivots, or the column reduction) | refs | weights, targets | flags,
 // barriers | columns from the blocks of the cluster]
@@ -254,7 +255,7 @@ template <int THREADS> __device__ __forceinline__ uint32_t tensor_rows(const Sha
     uint32_t base;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(base) : "r"(S.tmem) : "memory");
     const uint32_t warp = threadIdx.x >> 5;
-    return base + ((warp & 3) << 21) + (warp >> 2) * (tcols / (THREADS / 128));
+    return base + ((warp & 3) << 21) + (warp >> 2) * (tcols / lane_sharers(THREADS));
 }
 // N = 16 or 32 columns of the lane as packed pairs; to be used behind settle().
 template <int N> __device__ __forceinline__ void tensor_load(u64 (&v)[N / 2], uint32_t t)
@@ -788,7 +789,7 @@ __device__ __forceinline__ Problem locate(const SweepArgs &a, int p, int c, Shar
     P.row0 += a.skip;                                        // from here on within the slice's tokens
     R.ns = min(R.nrows, a.srows);
     R.steps = (R.ns + STEP - 1) / STEP;
-    R.nt = min(R.nrows - R.ns, a.tcols / (THREADS / 128) / CPL * STEP);
+    R.nt = min(R.nrows - R.ns, a.tcols / lane_sharers(THREADS) / CPL * STEP);
     R.tsteps = (R.nt + 2 * STEP - 1) / (2 * STEP) * 2;
     R.g = a.kt[P.side] ? a.kt[P.side] + ((size_t)P.slice * P.n + P.row0) * RP : nullptr;
     R.mass = a.mass[P.side] ? a.mass[P.side] + (size_t)P.slice * P.n + P.row0 : nullptr;
