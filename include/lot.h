@@ -235,9 +235,10 @@ LOT_API int lot_attention_fwd_ex(const void *q, const void *k, const void *v,
  *   beta is treated as r free positive numbers per head (no simplex constraint: a softmax parametrisation is the
  *   caller's chain rule); dz and dbeta are summed over the batch.
  * The forward is recomputed in the general path's arithmetic (float32 for bf16 tensors, float64 for float32 tensors);
- * of its iterations only the pivot potentials are kept.  bf16 tensors: 13 kernel launches; the workspace holds, per token
+ * of its iterations only the pivot potentials are kept.  bf16 tensors: 9 kernel launches up to r = 64 and
+ * d = 128, else 13 (12 without iterations); the workspace holds, per token
  * and side, two float32 numbers for each of the r pivots (r padded to a power of two from 16 on) and two for each iteration;
- * calls that would need more than 8 GiB run their slices in parts of at most that, 13 launches each (a slice is never split).
+ * calls that would need more than 8 GiB run their slices in parts of at most that, as many launches each (a slice is never split).
  * float32 tensors: 2*iters + 15 launches.
  * ws: lot_bwd_workspace_bytes(...) bytes of device scratch, 256-byte aligned, owned by the caller; the device
  * status word of the recomputed forward sits at its start (lot_device_status).

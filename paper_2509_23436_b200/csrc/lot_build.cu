@@ -114,7 +114,7 @@ static cudaError_t launch_rp(int RP, const SweepArgs &a, cudaStream_t st)
 
 cudaError_t launch_build(int RP, const SweepArgs &a, int dtype, cudaStream_t st)
 {
-    if (dtype == 1 && build_tc_supported(RP, a.d)) return launch_build_tc(RP, a, st);
+    if (dtype == 1 && build_tc_supported(RP, a.d)) return launch_build_tc(RP, a, st);       // whatever the number of tiles: lot_build_tc.cu
     if (dtype == 1 && a.terms == 2) {
         if (RP == 16) return build::launch_t<__nv_bfloat16, 16, 2>(a, st);
         if (RP == 32) return build::launch_t<__nv_bfloat16, 32, 2>(a, st);

@@ -9,6 +9,9 @@
 // memory for 16 tokens (75% of its bandwidth, tensor cores at 39%): B = 4, H = 8, n = 16384, d = 128, r = 256, 1.07 GB of kernel,
 // 985 us, now 388; 16 x 17 tiles of d = 128, r = 256 36 us, now 24; n = 4096, H = 16, d = 64, r = 64 24 us, now 20.  The potentials' error
 // against float64 is half of what it was (rms in units of eps at d = 128, r = 256: 8e-7, before 2e-6).
+// Taken however few the tiles are: at r <= 64, d <= 64 and fewer than 400 tiles a call is up to 2 us slower than with warp-level products
+// (16 slices of 120 tokens 24.8 us, 22.9; 64 of 384 43.3, 41.3; faster from 512 tiles on, and nearly everywhere at d = 128 or r > 64), but its
+// potentials have two thirds of the error there too (16 slices of 64 tokens at r = 64 9.7e-7 and 1.5e-6 of eps).
 #include "lot_chain.cuh"
 #include "lot_internal.h"
 #include "lot_logits.cuh"

@@ -10,8 +10,10 @@
 // the current potentials; when a column sum itself leaves float32's range that iteration is redone in the log domain
 // (column maxima first), so any spread of the potentials is exact.
 // What bounds a pass: the latency of rows in flight (16 warps an SM: 18 entries a clock and SM from shared memory, 26 with tensor
-// memory) and, for C > 1, the exchange.  64 problems of 16384 rows at RP = 256, 20 iterations: 3410 us with rows in shared
-// memory and L2, 49 blocks a problem and words exchanged through L2; 1790 with 36 blocks a problem, clusters of two.
+// memory) and, for C > 1, the exchange.  64 problems of 16384 rows at RP = 256, 20 iterations: this kernel 3410 us with rows in shared
+// memory and L2, 49 blocks a problem and words exchanged through L2; 1883 with six problems at once, 24 blocks each in clusters of two.
+// The call with that split, the one chosen, 3305 us; with 18 blocks a problem 3618, 28 3584, 32 3571 (clusters of four 3553, of eight
+// 4097), 24 in clusters of four 3807.
 #include "lot_chain.cuh"
 #include "lot_sweep_core.cuh"
 
