@@ -64,6 +64,12 @@ constexpr double kIters = 12, kClockMHz = 1900;
 constexpr double kEntryClk[2][2] = {{0.032, 0.037}, {0.046, 0.041}};      // clocks of an SM per entry: [512 threads][RP <= 32]
 constexpr double kAloneBlock = 1.7;      // times as many where a block of 256 threads has the SM to itself
 constexpr double kOrdinaryStart = 2.9;   // us
+// What a block's rows may cost to rebuild, us per row, column and channel with 256 threads, weighed by how seldom calls do: the fit's calls never
+// did, and without it peaked ones were given few blocks of many rows (39 slices of 3059 at r = 32, eps 0.02 205 us before that fit, 323 with it;
+// 12 of 1047 at d = 128, r = 16 64 and 80).  Over 774 drawn calls, a quarter of them peaked, against the splits before: peaked 2.6 % faster
+// on average with it and 1.4 without, others 3.1 and 3.1; 30 in all instead of 48 more than 2 % slower.  A third and one and a half
+// times of it are no better.
+constexpr double kRebuild = 3e-6;
 }
 
 SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
@@ -127,7 +133,7 @@ SweepPlan sweep_plan(int dtype, int BH, int nq, int nk, int d, int r, bool keep)
                 const double l2 = all / (all > 60 ? 5.0 : 11.0), sm = per_sm * mb / 0.08;       // TB/s: L2 beyond half of it is no faster than memory
                 it += 0.9 + (l2 > sm ? l2 : sm);
             }
-            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.5 + mine * (RP * 8e-5) + 3.0;
+            return (kIters + 0.7) * it + resident * (double)(ns + nt) * (RP * 4e-6) / 7.5 + mine * (RP * 8e-5) + (double)mine * RP * d * (kRebuild * 256 / threads) + 3.0;
         };
         const int rounds = (P + fly - 1) / fly, first = nq == nk ? rounds : (BH + fly - 1) / fly;         // the longer side's come first
         const double t = first * problem(n) + (rounds > first ? (rounds - first) * problem(nq < nk ? nq : nk) : 0.0) + (chained ? 0.0 : kOrdinaryStart) +
